@@ -43,3 +43,26 @@ def test_rotated_append(Hq, Hkv, d, theta):
     assert ulp_diff(got_pool[:, 0][differs], ref_pool[:, 0][differs]).max(initial=0) <= 1
     dq = got_q != q_rot
     assert dq.mean() < 1e-3 and ulp_diff(got_q[dq], q_rot[dq]).max(initial=0) <= 1
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,rotate_q", [(64, 8, 128, True), (8, 8, 128, False), (1, 1, 64, True), (128, 16, 64, True)])
+def test_rotated_append_over_head_counts(Hq, Hkv, d, rotate_q):
+    """One CTA rotates all heads of a token: fewer heads than a warp has room for, and more than one pass."""
+    import torch
+    from gpu_util import to_bits, to_dev
+    shape = W.Shape(Hq, Hkv, d, 16)
+    wl = W.make_single_step("rope_heads", shape, [0, 131071, 40], [3, 2, 17], seed=32, poison_unused=True)
+    st = wl.steps[0]
+    pool_dev, q_dev = to_dev(wl.kv_pool), to_dev(st.q)
+    plan = B.asynclm_plan(shape, wl.num_pages, st.q_indptr, st.kv_len_before, st.page_indptr, st.page_indices)
+    B.asynclm_kv_append_rope(plan, to_dev(st.k_new), to_dev(st.v_new), pool_dev, q_dev if rotate_q else None, 500000.0)
+    torch.cuda.synchronize()
+    pos = np.concatenate([np.arange(c, c + n) for c, n in zip(st.kv_len_before, st.q_len)])
+    rot = lambda bits: W.f32_to_bf16_bits(rope.rotate(W.bf16_bits_to_f64(bits), pos, 500000.0).astype(np.float32))
+    ref_pool = wl.kv_pool.copy()
+    oracle.kv_append(ref_pool, st.q_indptr, st.kv_len_before, st.page_indptr, st.page_indices, rot(st.k_new), st.v_new)
+    # the two sides evaluate pow / sin / cos with different libraries: a value on a rounding boundary may go either way
+    for got, ref in ((to_bits(pool_dev)[:, 0], ref_pool[:, 0]), (to_bits(q_dev), rot(st.q) if rotate_q else st.q)):
+        diff = got != ref
+        assert diff.mean() < 1e-3 and ulp_diff(got[diff], ref[diff]).max(initial=0) <= 1
+    assert np.array_equal(to_bits(pool_dev)[:, 1], ref_pool[:, 1])
