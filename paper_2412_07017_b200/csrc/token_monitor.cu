@@ -6,8 +6,9 @@
 // which interrupts are deferred, Section 3.2).
 //
 // The logits are streamed once (16-byte loads, several CTAs per sequence): the kernel is bound by HBM,
-// vocab * element size bytes per sequence.  The mask costs nothing per element: the scan takes the
-// plain maximum, and only a row whose maximum is a token its state forbids is looked at a second time.
+// vocab * element size bytes per sequence.  The mask costs nothing per element: the scan leaves the five
+// CML tokens out, which only the few vectors that hold one have to look at, and the CML tokens that the
+// state allows, two at most, are fetched by their ids and compete at the end.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -45,7 +46,7 @@ template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16
 // goes in complemented.  Key 0 means "nothing yet" (no real candidate maps to it: -NaN patterns never
 // enter, and -inf maps to 0x007fffff in the upper half).
 __device__ __forceinline__ unsigned long long pack_key(float v, int i) {
-    const unsigned u = __float_as_uint(v);
+    const unsigned u = __float_as_uint(v + 0.f);      // -0 becomes +0: the two are equal, so the lower id wins
     const unsigned ord = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
     return ((unsigned long long)ord << 32) | (unsigned)(0x7fffffff - i);
 }
@@ -83,34 +84,39 @@ template <> struct Vec<float> {
     }
 };
 
-// Largest element of vectors [j_begin, j_end) of a row (stride of the CTA's threads), lowest id among
-// equals; `skip`: leave the five CML tokens out.  Per vector only its maximum is computed; the
-// position inside the best vector is found at the end by looking at that one vector again.
+// Largest ordinary element (no CML token) of vectors [j_begin, j_end) of a row (stride of the CTA's
+// threads), lowest id among equals.  Per vector only its maximum is computed; the position inside the
+// best vector is found at the end by looking at that one vector again.
 template <typename T>
-__device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, const asynclm_cml_tokens& tok, bool skip) {
+__device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, const asynclm_cml_tokens& tok) {
     constexpr int VEC = Vec<T>::N;
     const uint4* v4 = reinterpret_cast<const uint4*>(row);
+    const int sv[5] = {tok.call / VEC, tok.intr / VEC, tok.trap / VEC, tok.end / VEC, tok.head / VEC};
     float bv = -INFINITY;
     int bj = -1;
-    for (int j0 = j_begin + threadIdx.x; j0 < j_end; j0 += kMonVecs * kMonThreads) {
+    for (int b0 = j_begin; b0 < j_end; b0 += kMonVecs * kMonThreads) {
+        const int j0 = b0 + threadIdx.x;
         uint4 w[kMonVecs];
 #pragma unroll
         for (int u = 0; u < kMonVecs; ++u) {
             const int j = j0 + u * kMonThreads;
+            w[u] = make_uint4(0, 0, 0, 0);
             if (j < j_end) w[u] = ldg_nc_v4(v4 + j);
         }
+        bool special = false;      // does this stretch of vectors hold a CML token? (the same for all threads)
+#pragma unroll
+        for (int a = 0; a < 5; ++a) special |= (unsigned)(sv[a] - b0) < (unsigned)(kMonVecs * kMonThreads);
 #pragma unroll
         for (int u = 0; u < kMonVecs; ++u) {
             const int j = j0 + u * kMonThreads;
-            if (j >= j_end) break;
             float m = Vec<T>::vmax(w[u]);
-            if (skip) {      // (the rare second pass) recompute without the CML tokens this vector may hold
+            if (special) {
                 m = -INFINITY;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k)
                     if (!is_special(j * VEC + k, tok)) m = fmaxf(m, Vec<T>::at(w[u], k));
             }
-            if (m > bv) { bv = m; bj = j; }      // a thread's vectors come in increasing order: the first one wins a tie
+            if (j < j_end && m > bv) { bv = m; bj = j; }      // a thread's vectors come in increasing order: the first one wins a tie
         }
     }
     Best best{-INFINITY, INT_MAX};
@@ -118,7 +124,7 @@ __device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, c
         const uint4 w = ldg_nc_v4(v4 + bj);
 #pragma unroll
         for (int k = VEC - 1; k >= 0; --k)
-            if (Vec<T>::at(w, k) == bv && !(skip && is_special(bj * VEC + k, tok))) best = Best{bv, bj * VEC + k};
+            if (Vec<T>::at(w, k) == bv && !is_special(bj * VEC + k, tok)) best = Best{bv, bj * VEC + k};
     }
     return best;
 }
@@ -131,7 +137,6 @@ __device__ __forceinline__ Best block_best(Best best, float* sv, int* si) {
         const int i = __shfl_xor_sync(0xffffffffu, best.i, off);
         if (better(v, i, best)) best = Best{v, i};
     }
-    __syncthreads();      // (sv / si may still be read from an earlier call)
     if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best.v; si[threadIdx.x >> 5] = best.i; }
     __syncthreads();
     if (threadIdx.x == 0)
@@ -140,13 +145,12 @@ __device__ __forceinline__ Best block_best(Best best, float* sv, int* si) {
     return best;
 }
 
-// Grid: (slices, batch).  Every CTA scans one slice of a sequence's row, ALL tokens alike, and folds its
-// best into the row's key with one atomic max; the CTA that arrives last (per-row counter) finishes the
-// row.  If the row's largest logit belongs to an ordinary token or to a CML token the state allows, that
-// token is the answer (an allowed token that beats everything beats everything allowed).  Only if it
-// belongs to a CML token the state forbids, a "hallucinated" [INTR] say, the last CTA scans the row once
-// more without the CML tokens and lets the allowed ones compete.  Then the state machine advances and
-// the two workspace words go back to zero.  The result does not depend on arrival order.
+// Grid: (slices, batch).  Every CTA scans one slice of a sequence's row and folds its best ordinary token
+// into the row's key with one atomic max; the CTA that arrives last (per-row counter) lets the CML tokens
+// that the state allows compete, advances the state machine and puts the two workspace words back to zero.
+// The result does not depend on arrival order.  (Scanning all tokens alike and looking at a row a second
+// time when a forbidden token had won kept one CTA busy with a whole row after all others had left:
+// 256 rows of 128 256 bf16 with a few such rows took 31 us a call, 21 us now.)
 template <typename T>
 __global__ void __launch_bounds__(kMonThreads)
 token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, asynclm_cml_tokens tok,
@@ -156,10 +160,10 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
     constexpr int VEC = Vec<T>::N;
     __shared__ float sv[kMonThreads / 32];
     __shared__ int si[kMonThreads / 32];
-    __shared__ int s_rescan;
     const int seq = blockIdx.y;
     const T* row = logits + (int64_t)seq * row_stride;
-    if (state_in[seq] == kTrap) {
+    const int state = state_in[seq];
+    if (state == kTrap) {
         // [TRAP] is followed by [END] whatever the logits say: nothing to read
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             token_out[seq] = tok.end;
@@ -168,61 +172,35 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
         }
         return;
     }
+    // the CML tokens this state allows (INT_MAX: none) and their logits, for the thread that may finish the row
+    const int spec0 = state == kText ? tok.call : tok.end, spec1 = state == kText ? tok.trap : state == kCall ? tok.head : INT_MAX;
+    float spec_v0 = 0.f, spec_v1 = 0.f;
+    if (threadIdx.x == 0) {
+        spec_v0 = to_f32<T>(row[spec0]);
+        if (spec1 != INT_MAX) spec_v1 = to_f32<T>(row[spec1]);
+    }
     const int nvec = vocab / VEC;
     const int per = (nvec + gridDim.x - 1) / gridDim.x;
-    Best best = scan_row<T>(row, blockIdx.x * per, min(nvec, (int)(blockIdx.x + 1) * per), tok, false);
+    Best best = scan_row<T>(row, blockIdx.x * per, min(nvec, (int)(blockIdx.x + 1) * per), tok);
     if (blockIdx.x == gridDim.x - 1)      // the row's ragged end, element by element
         for (int i = nvec * VEC + threadIdx.x; i < vocab; i += kMonThreads) {
             const float v = to_f32<T>(row[i]);
-            if (better(v, i, best)) best = Best{v, i};
+            if (!is_special(i, tok) && better(v, i, best)) best = Best{v, i};
         }
     best = block_best(best, sv, si);
-    unsigned long long* key = ws + 2 * (size_t)seq;
-    unsigned* arrived = reinterpret_cast<unsigned*>(key + 1);
-    const int state = state_in[seq];
-    auto allowed_special = [&](int id) {
-        return (state == kText && (id == tok.call || id == tok.trap)) || (state == kCall && (id == tok.head || id == tok.end)) ||
-               ((state == kBody || state == kTrap) && id == tok.end);
-    };
-    if (threadIdx.x == 0) {
-        s_rescan = -1;      // -1: this CTA is not the last one of its row
+    if (threadIdx.x != 0) return;
+    if (gridDim.x > 1) {
+        unsigned long long* key = ws + 2 * (size_t)seq;
+        unsigned* arrived = reinterpret_cast<unsigned*>(key + 1);
         if (best.i != INT_MAX) atomicMax(key, pack_key(best.v, best.i));
         __threadfence();
-        if (atomicAdd(arrived, 1u) == gridDim.x - 1) {
-            __threadfence();
-            best = unpack_key(atomicExch(key, 0ull));
-            *arrived = 0;
-            const bool ordinary = best.i != INT_MAX && !is_special(best.i, tok);
-            // ordinary tokens are allowed everywhere but in a trap block
-            const bool settled = best.i != INT_MAX && best.v > -INFINITY &&
-                                 (ordinary ? state != kTrap : allowed_special(best.i));
-            s_rescan = settled ? 0 : 1;
-        }
+        if (atomicAdd(arrived, 1u) != gridDim.x - 1) return;      // not the last CTA of its row
+        __threadfence();
+        best = unpack_key(atomicExch(key, 0ull));
+        *arrived = 0;
     }
-    __syncthreads();
-    if (s_rescan < 0) return;
-    if (s_rescan == 1) {
-        // the row's best ordinary token (none in a trap block), then the CML tokens the state allows
-        Best ord{-INFINITY, INT_MAX};
-        if (state != kTrap) {
-            ord = scan_row<T>(row, 0, nvec, tok, true);
-            for (int i = nvec * VEC + threadIdx.x; i < vocab; i += kMonThreads) {
-                const float v = to_f32<T>(row[i]);
-                if (!is_special(i, tok) && better(v, i, ord)) ord = Best{v, i};
-            }
-        }
-        ord = block_best(ord, sv, si);
-        if (threadIdx.x == 0) {
-            best = ord;
-            const int ids[5] = {tok.call, tok.trap, tok.head, tok.end, tok.intr};
-            for (int a = 0; a < 5; ++a)
-                if (allowed_special(ids[a])) {
-                    const float v = to_f32<T>(row[ids[a]]);
-                    if (better(v, ids[a], best)) best = Best{v, ids[a]};
-                }
-        }
-    }
-    if (threadIdx.x != 0) return;
+    if (better(spec_v0, spec0, best)) best = Best{spec_v0, spec0};
+    if (spec1 != INT_MAX && better(spec_v1, spec1, best)) best = Best{spec_v1, spec1};
     Best pick = best;
     if (pick.i == INT_MAX || pick.v == -INFINITY) {
         // no allowed token has a logit above -inf (all NaN or -inf): the lowest allowed id is taken
@@ -231,12 +209,10 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
         if (state == kText) low = min(low, min(tok.call, tok.trap));
         if (state == kCall) low = min(low, min(tok.head, tok.end));
         if (state == kBody) low = min(low, tok.end);
-        if (state == kTrap) low = tok.end;
         pick.i = low;
     }
     int next = state, flags = 0;
     if (state == kText) next = pick.i == tok.call ? kCall : pick.i == tok.trap ? kTrap : kText;
-    else if (state == kTrap) { next = kText; flags = ASYNCLM_MONITOR_TRAP; }
     else if (pick.i == tok.end) { next = kText; flags = ASYNCLM_MONITOR_CALL; }
     else if (state == kCall && pick.i == tok.head) next = kBody;
     if (next == kCall || next == kBody) flags |= ASYNCLM_MONITOR_CRITICAL;

@@ -101,3 +101,20 @@ def test_degenerate_rows():
     tok, nxt, fl = run(vals, states, special, False)
     rt, rn, rf = M.step(vals.astype(np.float64), states, special)
     assert np.array_equal(tok, rt) and np.array_equal(nxt, rn) and np.array_equal(fl, rf)
+
+
+@pytest.mark.parametrize("Bsz,vocab,bf16", [(1, 128256, True), (3, 40963, True), (2, 16385, False), (300, 2051, False)])
+def test_cml_tokens_at_the_edges_of_the_scan(Bsz, vocab, bf16):
+    """The CML tokens sit in the first and last vector, next to a slice boundary and in the ragged end of the
+    row; each in turn has the largest logit, beside a runner-up that ties across the row, zeros of both
+    signs among them."""
+    special = {"CALL": 0, "INTR": vocab - 1, "TRAP": 2048, "END": vocab // 2, "HEAD": 2047}
+    for k, name in enumerate(special):
+        vals = np.full((Bsz, vocab), -5.0)
+        vals[:, [1, 2046, 2049, vocab - 2]] = [-0.0, 0.0, -0.0, 0.0] if k % 2 else 1.0
+        vals[:, special[name]] = 9.0
+        bits = W.f32_to_bf16_bits(vals.astype(np.float32)) if bf16 else vals.astype(np.float32)
+        states = (np.arange(Bsz) + k) % 4
+        tok, nxt, fl = run(bits, states, special, bf16)
+        rt, rn, rf = M.step(vals, states, special)
+        assert np.array_equal(tok, rt) and np.array_equal(nxt, rn) and np.array_equal(fl, rf), name
