@@ -7,36 +7,36 @@
 // (row r = token r / G, head r % G) and S = Q K^T and O += P V run on the tensor cores.
 //
 // A work item covers up to 256 query rows (two row tiles) of one (sequence, kv head) and a range of
-// keys.  One persistent CTA per SM, twelve working warps:
-//   warps 0-3, 4-7  two softmax groups, one thread per query row of a tile.  Each group owns one S
-//                   accumulator (128 fp32 columns of tensor memory) and one O accumulator.
+// keys, 64 to a KV tile.  One persistent CTA per SM, twelve warps:
+//   warps 0-3, 4-7  two softmax groups, one thread per query row of a tile.  Each group owns two S
+//                   accumulators (64 fp32 columns of tensor memory each) and one O accumulator.
 //                     * items with more than 128 rows ("dual"): group b owns row tile b and both
 //                       groups consume every KV tile, so K and V are fetched once for 256 rows;
 //                     * items with at most 128 rows: the groups take alternate KV tiles of the one
 //                       row tile and their (max, sum, O) states are merged in the epilogue like two
 //                       KV splits.
-//                   The softmax runs in place: a thread reads its row of S 64 columns at a time and
-//                   writes P as packed bf16 pairs over the columns it has already read; P V then
-//                   takes its A operand from tensor memory.  The reference maximum only moves when
-//                   a score exceeds it by 2^8; then O, the running sum and the half of P already
-//                   written are rescaled.  With one softmax warp per scheduler the stage is bound
-//                   by issue slots and dependent latency, so the arithmetic around the exponentials
-//                   is packed two values to an instruction and reductions run in independent chains.
+//                   The softmax runs in place: a thread reads its row of S and writes P as packed bf16
+//                   pairs over columns it has already read; P V then takes its A operand from tensor
+//                   memory.  The reference maximum only moves when a score exceeds it by 2^8; then O and
+//                   the running sum are rescaled.  The arithmetic around the exponentials is packed two
+//                   values to an instruction and reductions run in independent chains.
 //                   At the end of an item the rows go out through the group's (now idle) Q tile in
 //                   shared memory, so that every global store writes whole 128-byte lines.
 //   warps 8, 10     producers of K tiles and of V tiles: 16-byte cp.async copies (fully coalesced,
-//                   two 256-byte rows per warp instruction) that write the 128-byte-swizzled operand
-//                   layout and complete on the slot's mbarrier.  K and V share one ring of five
-//                   32 KiB slots, filled in the order the tensor core consumes them
-//                   (K0 K1 V0 K2 V1 K3 ...): a V tile is needed one softmax later than the K tile
-//                   of the same keys, and a shared ring lets whichever is due use the free slots.
-//   warp 9          one thread issues all MMAs, a group at a time (P V of its tile, then Q K^T of its
-//                   next tile), so that the groups' softmaxes alternate instead of colliding on the
-//                   exponential unit.  The warp owns the tensor-memory allocation.
-//   warp 11         idle, except when the kernel appends the step's new K/V rows itself
-//                   (asynclm_step): then it runs ahead of the producers and copies, item by item, the
-//                   new rows the item reads into their page slots; the producers wait for an item's
-//                   rows before they fetch its first tile.
+//                   whole rows, 512 bytes per warp instruction) that write the 128-byte-swizzled operand
+//                   layout and complete on the slot's mbarrier.  K and V share one ring of 160 KiB, filled
+//                   in the order the tensor core consumes the tiles (see ring_pos_k).  For asynclm_step
+//                   the K warp also puts an item's new K/V rows into their page slots, before the first
+//                   tile that holds one.
+//   warps 9, 11     issue the MMAs, one warp per softmax group.  Warp 9 owns the tensor-memory allocation.
+// Why tiles of 64 keys: with two S buffers per group, the Q K^T of the tile after next is issued behind the
+// P V of the current one, and the softmax of the next tile, whose S is complete, runs meanwhile; with
+// 128-key tiles tensor memory holds one S per group (at head_dim 128) and each group's softmax and MMAs
+// took turns.  Per 64 keys of both row tiles (cycles): the exponential unit needs 1024, the tensor pipe
+// 1280 (64-column Q K^T is bound by its operands in shared memory), a lone group's softmax 1130, and a tile
+// pair takes 1900-2000: the MMA warps need about 100 cycles to issue an MMA, and the groups' exponentials
+// collide in part.  8192 tokens of one sequence (32 / 8 heads, head_dim 128): 522 us, 530 before;
+// head_dim 64 had no tensor-core body before (32 sequences, 8 spans: 163 -> 56 us).
 // All hand-offs are mbarriers with bounded waits; a wait that runs out sets the plan's status word
 // and a CTA-wide abort flag, every role falls through to the common exit, and the tensor memory is
 // released there.
@@ -51,43 +51,49 @@ namespace asynclm {
 namespace tc {
 
 constexpr int kThreads = 384;
-constexpr int kProducerWarpK = 8, kMmaWarp = 9, kProducerWarpV = 10, kAppendWarp = 11;
-constexpr int kD = 128;
-constexpr int kTile = 128;                       // keys per K/V ring slot and query rows per row tile
-constexpr int kSub = 64;                         // keys the softmax handles at a time (half an S tile)
-// Pairs (of the 16 of a quarter) whose exponentials are evaluated by polynomial instead of ex2.approx.
-#ifndef ASYNCLM_POLY_MASK
-#define ASYNCLM_POLY_MASK 0x4924u
-#endif
-constexpr uint32_t kPolyMask = ASYNCLM_POLY_MASK;
-constexpr int kRing = 5;                         // K/V ring slots
-constexpr uint32_t kHalfBytes = 128 * 128;       // one 64-value half of a 128-row tile
-constexpr uint32_t kTileBytes = 2 * kHalfBytes;  // 32 KiB
+constexpr int kProducerWarpK = 8, kMmaWarp = 9, kProducerWarpV = 10;      // 11: the second MMA warp
+constexpr int kRows = 128;                       // query rows per row tile
+constexpr int kTile = 64;                        // keys per KV tile: a K or V ring slot, an S buffer
 constexpr float kRescaleThreshold = 8.f;
 constexpr long long kWaitCycles = 2000000000ll;
+constexpr long long kGroupSkewCycles = 600;
 
-// shared memory map (offsets from a 1024-byte aligned base)
-constexpr uint32_t kOffQ = 0;                           // Q[0], Q[1]
-constexpr uint32_t kOffRing = kOffQ + 2 * kTileBytes;
-constexpr uint32_t kOffBar = kOffRing + kRing * kTileBytes;
-// S, P V and P hand-offs exist per group b: index 2 * b
-enum Bar { kQFull = 0, kStats, kOFree, kPFull0, kPvDone0 = kPFull0 + 4, kSFull0 = kPvDone0 + 4,
-           kRingFull0 = kSFull0 + 4, kRingEmpty0 = kRingFull0 + kRing, kMmaDrain = kRingEmpty0 + kRing,
-           kNumBars };
-constexpr uint32_t kOffTmemPtr = kOffBar + 8 * kNumBars;
-constexpr uint32_t kOffAbort = kOffTmemPtr + 8;
-constexpr uint32_t kOffAppended = kOffAbort + 8;      // items of this CTA whose new K/V rows are in the pool
-constexpr uint32_t kSmemBytes = kOffAppended + 8 + 1024;
-static_assert(kSmemBytes <= 232448, "shared memory budget");
+// Per head_dim: shared memory map (offsets from a 1024-byte aligned base) and barriers.
+template <int D>
+struct Geometry {
+    static constexpr int HALVES = D / 64;                                  // 128-byte pieces of a row
+    static constexpr uint32_t QHALF_BYTES = kRows * 128;                   // one 64-value half of a Q tile
+    static constexpr uint32_t QTILE_BYTES = HALVES * QHALF_BYTES;
+    static constexpr uint32_t HALF_BYTES = kTile * 128;                    // one 64-value half of a K or V tile
+    static constexpr uint32_t SLOT_BYTES = HALVES * HALF_BYTES;
+    static constexpr int RING = 20 / HALVES;                               // K/V ring slots: 160 KiB
+    static constexpr uint32_t OFF_Q = 0;                                   // Q[0], Q[1]
+    static constexpr uint32_t OFF_RING = OFF_Q + 2 * QTILE_BYTES;
+    // The barriers lie behind everything the warp body uses when the CTA goes on to it: arrivals that nobody
+    // waits for (an item's last on kOFree and on the ring's empty barriers) may still be queued in the shared
+    // memory pipe then, and would change whatever has been copied there since.
+    static constexpr uint32_t OFF_BAR = 224 * 1024;
+    static_assert(OFF_RING + RING * SLOT_BYTES <= OFF_BAR, "barriers behind the tiles");
+    // S, P and last-P-V hand-offs exist per group b and buffer s: index 2 * b + s
+    enum Bar { kQFull = 0, kStats, kOFree, kPFull0, kPvDone0 = kPFull0 + 4, kSFull0 = kPvDone0 + 4,
+               kRingFull0 = kSFull0 + 4, kRingEmpty0 = kRingFull0 + RING, kMmaDrain = kRingEmpty0 + RING, kNumBars };
+    static constexpr uint32_t OFF_TMEM_PTR = OFF_BAR + 8 * kNumBars;
+    static constexpr uint32_t OFF_ABORT = OFF_TMEM_PTR + 8;
+    static constexpr uint32_t OFF_APPENDED = OFF_ABORT + 8;      // items of this CTA whose new K/V rows are in the pool
+    static constexpr uint32_t SMEM_BYTES = OFF_APPENDED + 8 + 1024;
+    static_assert(SMEM_BYTES <= 232448, "shared memory budget");
+};
 
 // tensor memory columns
-constexpr uint32_t kColS = 0;      // S[0], S[1]: 128 columns each; P[b] overlays the first 64 of S[b]
-constexpr uint32_t kColO = 256;    // O[0], O[1]: 128 columns each
+constexpr uint32_t kColS = 0;      // S[b][s]: 64 columns each at 128 b + 64 s; P[b][s] overlays the first 32 of S[b][s]
+constexpr uint32_t kColO = 256;    // O[b]: head_dim columns each
 constexpr uint32_t kTmemCols = 512;
 
-// Ring position of the K tile and of the V tile of the CTA's g-th KV tile: K0 K1 V0 K2 V1 K3 ...
-__device__ __forceinline__ int ring_pos_k(int g) { return g == 0 ? 0 : 2 * g - 1; }
-__device__ __forceinline__ int ring_pos_v(int g) { return 2 * g + 2; }
+// Ring positions, relative to the item's first slot, of the K tile and of the V tile of its g-th KV tile
+// (of n): the order in which the tensor core consumes them.  The first `lead` K tiles go ahead, then a V
+// tile and the K tile `lead` further take turns: K0 K1 V0 K2 V1 K3 ... for a lead of two.
+__device__ __forceinline__ int ring_pos_k(int g, int lead) { return g < lead ? g : 2 * g - lead + 1; }
+__device__ __forceinline__ int ring_pos_v(int g, int n, int lead) { return g + min(n, g + lead); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -95,6 +101,9 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t count) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
@@ -165,14 +174,15 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes,
 }
 // Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = n; b_mn = 1 when B is stored with N
 // contiguous (the V tile), 0 when K is contiguous.
-__device__ __forceinline__ uint32_t instr_desc(uint32_t n, uint32_t b_mn) {
+__host__ __device__ constexpr uint32_t instr_desc(uint32_t n, uint32_t b_mn) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn << 16) | ((n >> 3) << 17) | ((128u >> 4) << 24);
 }
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+// `el`: 1 in the lane that issues, 0 in the others (the warp stays converged, so that operands are uniform).
+__device__ __forceinline__ void mma_f16(uint32_t el, uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc), "r"(el) : "memory");
 }
 // True in exactly one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
@@ -180,8 +190,9 @@ __device__ __forceinline__ bool elect_one() {
     asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(pred));
     return pred != 0;
 }
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void mma_commit(uint32_t el, uint32_t bar) {
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(el) : "memory");
 }
 
 #define TC_R32(r) \
@@ -248,27 +259,11 @@ __device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t a, uint32_t b)
 }
 // D (+)= A B with A taken from tensor memory: row i of A is lane i, its 16 bf16 values of one K step
 // are 8 consecutive 32-bit columns (two values per column, the lower index in the low half).
-__device__ __forceinline__ void mma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16_ta(uint32_t el, uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
-}
-
-// 2^x for two finite values on the FMA pipe: n = round(x) through the 1.5 * 2^23 trick, a cubic for
-// 2^(x - n) on [-1/2, 1/2] (relative error 7.5e-5, below the bf16 rounding of P), n added to the
-// exponent field.  x is clamped at -125 so that the exponent cannot wrap.
-__device__ __forceinline__ float2 poly_exp2(float2 x) {
-    const float kMagic = 12582912.f;
-    const float2 xc = make_float2(fmaxf(x.x, -125.f), fmaxf(x.y, -125.f));
-    const float2 t = __fadd2_rn(xc, make_float2(kMagic, kMagic));
-    const float2 n = __fadd2_rn(t, make_float2(-kMagic, -kMagic));
-    const float2 f = __ffma2_rn(n, make_float2(-1.f, -1.f), xc);
-    float2 r = __ffma2_rn(f, make_float2(0.0551716685f, 0.0551716685f), make_float2(0.2426111251f, 0.2426111251f));
-    r = __ffma2_rn(r, f, make_float2(0.6932609677f, 0.6932609677f));
-    r = __ffma2_rn(r, f, make_float2(0.9999280572f, 0.9999280572f));
-    return make_float2(__int_as_float(__float_as_int(r.x) + (__float_as_int(t.x) << 23)),
-                       __int_as_float(__float_as_int(r.y) + (__float_as_int(t.y) << 23)));
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc), "r"(el) : "memory");
 }
 
 __device__ __forceinline__ float fmax3(float a, float b, float c) {
@@ -295,17 +290,18 @@ __device__ __forceinline__ TItem load_titem(const Work* rec, bool valid) {
 }
 
 // The whole kernel body, called by all twelve warps with `smem` 1024-byte aligned.
-template <int G, bool APPEND>
+template <int D, int G, bool APPEND>
 __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* __restrict__ q,
                                         const __nv_bfloat16* pool,
                                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                                         uint8_t* smem, const AppendSrc& app) {
+    using Geo = Geometry<D>;
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar0 = sbase + kOffBar;
+    const uint32_t bar0 = sbase + Geo::OFF_BAR;
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    volatile uint32_t* tmem_ptr = (volatile uint32_t*)(smem + kOffTmemPtr);
-    volatile int* abort_flag = (volatile int*)(smem + kOffAbort);
-    volatile int* appended = (volatile int*)(smem + kOffAppended);
+    volatile uint32_t* tmem_ptr = (volatile uint32_t*)(smem + Geo::OFF_TMEM_PTR);
+    volatile int* abort_flag = (volatile int*)(smem + Geo::OFF_ABORT);
+    volatile int* appended = (volatile int*)(smem + Geo::OFF_APPENDED);
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -317,16 +313,16 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
     const Work* head_work = reinterpret_cast<const Work*>(head + kHeadWorkTensor);      // = p.works[i0]
 
     if (threadIdx.x == 0) {
-        mbar_init(bar(kQFull), 256);
-        mbar_init(bar(kStats), 256);
-        mbar_init(bar(kOFree), 256);
+        mbar_init(bar(Geo::kQFull), 256);
+        mbar_init(bar(Geo::kStats), 256);
+        mbar_init(bar(Geo::kOFree), 256);
         for (int b = 0; b < 4; ++b) {
-            mbar_init(bar(kPFull0 + b), 4);      // one arrival per warp of the group
-            mbar_init(bar(kPvDone0 + b), 1);
-            mbar_init(bar(kSFull0 + b), 1);
+            mbar_init(bar(Geo::kPFull0 + b), 4);      // one arrival per warp of the group
+            mbar_init(bar(Geo::kPvDone0 + b), 1);
+            mbar_init(bar(Geo::kSFull0 + b), 1);
         }
-        for (int s = 0; s < kRing; ++s) { mbar_init(bar(kRingFull0 + s), 32); mbar_init(bar(kRingEmpty0 + s), 1); }
-        mbar_init(bar(kMmaDrain), 1);
+        for (int s = 0; s < Geo::RING; ++s) { mbar_init(bar(Geo::kRingFull0 + s), 32); mbar_init(bar(Geo::kRingEmpty0 + s), 2); }
+        mbar_init(bar(Geo::kMmaDrain), 2);
         *abort_flag = 0;
         *appended = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -334,7 +330,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
     }
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(sbase + kOffTmemPtr), "r"(kTmemCols) : "memory");
+                     ::"r"(sbase + Geo::OFF_TMEM_PTR), "r"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
@@ -346,16 +342,18 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
       if (warp == kProducerWarpK || warp == kProducerWarpV) {
         // ------------------------------------------------------------------ producer warps
         const int which = warp == kProducerWarpV ? 1 : 0;       // 0: K tiles, 1: V tiles
-        const uint32_t ring = sbase + kOffRing;
+        const uint32_t ring = sbase + Geo::OFF_RING;
         auto load_pages = [&](const TItem& it, int first_page) {
             const int npg = (it.kv_end - it.kv0 + kPage - 1) / kPage;
             const int idx = first_page + lane;
             return idx < npg ? __ldg(p.page_indices + it.page0 + idx) : 0;
         };
-        constexpr int kPagesPerTile = kTile / kPage;          // 8
-        constexpr int kGroupTiles = 32 / kPagesPerTile;       // 4
+        constexpr int kPagesPerTile = kTile / kPage;          // 4
+        constexpr int kGroupTiles = 32 / kPagesPerTile;       // 8
+        constexpr int kChunks = D / 8, kRowsPerOp = 32 / kChunks;      // 16-byte chunks of a row; rows a warp instruction moves
         bool ok = true;
         int n = 0;                                             // KV tiles issued so far (all items)
+        int base = 0;                                          // ring position of the item's first slot
         int last_pos = -1;
         int ev = 0;      // time-stamp build: event log position (lane 0 of a producer)
         TItem cur = load_titem(head_work, i0 < i1), nxt = load_titem(p.works + i0 + 1, i0 + 1 < i1);
@@ -364,8 +362,9 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         for (int ii = i0; cur.kv_end > 0 && ok; ++ii) {
             const TItem after = load_titem(p.works + ii + 2, ii + 2 < i1);
             const int ntiles = (cur.kv_end - cur.kv0 + kTile - 1) / kTile;
-            // APPEND: the first key position of the item that this step appends; tiles up to it are
-            // fetched at once, the others only when the append warp has put the rows in the pool
+            const int lead = cur.ntok * G > kRows ? 2 : 4;
+            // APPEND: the first key position of the item that this step appends; tiles up to it are fetched at
+            // once, before the others the K warp puts the item's new rows in the pool
             int first_new = INT_MAX;
             if constexpr (APPEND) {
                 const int q_seq0 = ii == i0 ? head_work->q_seq0 : __ldg(&p.works[ii].q_seq0);
@@ -380,6 +379,12 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                     const int npages = (rows + kPage - 1) / kPage;
                     if constexpr (APPEND) {
                         if (!appended_seen && cur.kv0 + t * kTile + rows > first_new) {
+                            if (which == 0) {
+                                append_rows_of_item(p, app, ii == i0 ? *head_work : p.works[ii], lane);
+                                __threadfence();      // the rows are visible before the count moves
+                                __syncwarp();
+                                if (lane == 0) *appended = ii - i0 + 1;
+                            }
                             const long long t_wait = clock64();
                             while (*appended <= ii - i0 && ok) {
                                 __nanosleep(64);
@@ -396,37 +401,36 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                             appended_seen = true;
                         }
                     }
-                    const int pos = which ? ring_pos_v(n) : ring_pos_k(n);
-                    const int s = pos % kRing;
-                    if (lane == 0) trace_event(9 + which, ev, 40);
-                    ok = mbar_wait_warp(bar(kRingEmpty0 + s), ((uint32_t)(pos / kRing) & 1u) ^ 1u, abort_flag, p.status, 11 + which);
+                    const int pos = base + (which ? ring_pos_v(t, ntiles, lead) : ring_pos_k(t, lead));
+                    const int s = pos % Geo::RING;
+                    if (lane == 0 && which == 0) trace_event(9, ev, 40);
+                    ok = mbar_wait_warp(bar(Geo::kRingEmpty0 + s), ((uint32_t)(pos / Geo::RING) & 1u) ^ 1u, abort_flag, p.status, 11 + which);
                     if (!ok) break;
-                    if (lane == 0) trace_event(9 + which, ev, 42);
+                    if (lane == 0 && which == 0) trace_event(9, ev, 42);
                     last_pos = pos;
-                    // lane -> 16-byte chunk c of row 2*rr + (lane >> 4) of each page: a warp instruction
-                    // moves two whole 256-byte rows
-                    const int c = lane & 15;
-                    const uint32_t dst_half = ring + s * kTileBytes + (uint32_t)(c >> 3) * kHalfBytes;
+                    // lane -> 16-byte chunk c of a row: a warp instruction moves whole rows, 512 bytes in all
+                    const int c = lane % kChunks;
+                    const uint32_t dst_half = ring + s * Geo::SLOT_BYTES + (uint32_t)(c >> 3) * Geo::HALF_BYTES;
                     for (int pg = 0; pg < npages; ++pg) {
                         int64_t page = __shfl_sync(0xffffffffu, pages_cur, (t - t0) * kPagesPerTile + pg);
                         const bool page_good = page_ok(page, p.num_pages, p.status, kStatusBadPageSpan);      // checked build only
                         if (!page_good) page = 0;      // the tile gets zeros in its place
                         const uint8_t* src_page = reinterpret_cast<const uint8_t*>(
-                            pool + pool_row_offset(page, which, cur.kv_head, 0, Hkv, kD));
+                            pool + pool_row_offset(page, which, cur.kv_head, 0, Hkv, D));
 #pragma unroll
-                        for (int rr = 0; rr < kPage / 2; ++rr) {
-                            const int slot = rr * 2 + (lane >> 4);
+                        for (int rr = 0; rr < kPage / kRowsPerOp; ++rr) {
+                            const int slot = rr * kRowsPerOp + lane / kChunks;
                             const int row = pg * kPage + slot;
                             cp_async16(dst_half + (uint32_t)row * 128u + (uint32_t)(((c & 7) ^ (row & 7)) << 4),
-                                       src_page + slot * (kD * 2) + c * 16, (row < rows && page_good) ? 16u : 0u);
+                                       src_page + slot * (D * 2) + c * 16, (row < rows && page_good) ? 16u : 0u);
                         }
                     }
 #ifdef ASYNCLM_DEBUG
                     // checked build: a test may ask for one hand-off to be left out, to see a bounded wait run out
                     if (!(which == 0 && blockIdx.x == 0 && p.debug_stall_tile == n + 1))
 #endif
-                    cp_async_arrive(bar(kRingFull0 + s));
-                    if (lane == 0) trace_event(9 + which, ev, 44);
+                    cp_async_arrive(bar(Geo::kRingFull0 + s));
+                    if (lane == 0 && which == 0) trace_event(9, ev, 44);
                     // page ids of the next group of tiles (or of the next item), requested only after this
                     // group's first tile is on its way: the next item's descriptor may still be in flight
                     if (t == t0) {
@@ -436,6 +440,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 }
                 pages_cur = pages_nxt;
             }
+            base += 2 * ntiles;
             cur = nxt;
             nxt = after;
         }
@@ -443,160 +448,113 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             // aborted: let the loads already issued land before shared memory goes away
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
-      } else if (warp == kAppendWarp) {
-        // ------------------------------------------------------------------ append warp (asynclm_step only)
-        if constexpr (APPEND) {
-            pdl_wait();
-            for (int ii = i0; ii < i1; ++ii) {
-                const Work rec = ii == i0 ? *head_work : p.works[ii];
-                append_rows_of_item(p, app, rec, lane);
-                __threadfence();      // the rows are visible device-wide before the count moves
-                __syncwarp();
-                if (lane == 0) *appended = ii - i0 + 1;
-            }
-        }
-    } else if (warp == kMmaWarp) {
-        // ------------------------------------------------------------------ MMA issuer
-        // One warp, running convergently, issues every MMA of the CTA through an elected lane (operands then
-        // stay in uniform registers: under a lane-0 branch each MMA took the lone thread 85-110 cycles to
-        // issue, against 64 cycles on the tensor core), in an order that lets the two softmax groups work
-        // in turns: after the P V of a group's tile it issues the Q K^T of the same group's next tile
-        // at once (MMAs of one thread execute in issue order, so the new S may overwrite the P that the
-        // P V in front of it reads), then it turns to the other group.  While the tensor core works
-        // for one group, the other group's softmax has the exponential unit to itself.
-        // Q K^T is issued 128 keys wide (8 instructions per tile and group, 64 cycles each on the tensor
-        // core): narrower instructions cost nearly as much to issue.
-        {
-            bool ok = true;
-            int gt = 0;               // KV tiles before this item (all items): ring position
-            int cnt0 = 0, cnt1 = 0;   // tiles whose P V has been issued, per group: phase of the P hand-off
-            int item_no = 0;
-            const uint32_t idesc_pv = instr_desc(128, 1);
-            TItem it_next = load_titem(head_work, i0 < i1);
-            const long long t_loop = trace_clock();
-            long long tr_p = 0, tr_kv = 0, tr_item = 0, tr_qk = 0, tr_pv = 0;      // time-stamp build: cycles waiting for P, for K/V, for an item's Q and O
-            int ev = 0;                                                            // time-stamp build: event log position
-            for (int ii = i0; ii < i1 && ok; ++ii, ++item_no) {
-                const TItem it = it_next;
-                it_next = load_titem(p.works + ii + 1, ii + 1 < i1);      // in flight while this item runs
-                const int ntiles = (it.kv_end - it.kv0 + kTile - 1) / kTile;
-                const bool dual = it.ntok * G > kTile;
-                const long long t_item = trace_clock();
-                if (lane == 0) trace_event(0, ev, 1);
-                ok = mbar_wait_spin(bar(kQFull), (uint32_t)item_no & 1u, abort_flag, p.status, 22);
-                // S and O of the previous item are in use until its epilogue is over
-                if (ok && item_no > 0) ok = mbar_wait_spin(bar(kOFree), (uint32_t)(item_no - 1) & 1u, abort_flag, p.status, 27);
-                tr_item += trace_clock() - t_item;
-                if (lane == 0) trace_event(0, ev, 2);
-                if (ok) tc_fence_after();
-                auto tile_pages = [&](int j) { return (min(kTile, it.kv_end - (it.kv0 + j * kTile)) + kPage - 1) / kPage; };
-                // Hand-offs the MMAs of a turn wait for.  K/V tiles first (they are normally there already),
-                // P last, so that nothing stands between its arrival and the first MMA.
-                auto wait_k = [&](int j) {
-                    const int pos = ring_pos_k(gt + j), s = pos % kRing;
+      } else {
+        // ------------------------------------------------------------------ MMA issuers
+        // One warp per softmax group, running convergently, issues the group's MMAs through an elected lane.
+        // (One warp for both groups was the limit: 3000 cycles for the turns of a tile pair, 2000 with two.)  A
+        // turn is one KV tile of the group: its P V and the Q K^T of the group's next tile
+        // but one into the S buffer that the P V has just read (MMAs of one thread execute in issue order).
+        // While the tensor core works on a turn, the group runs the softmax of its other buffer: neither
+        // waits for the other as long as both keep up.
+        const int b = warp == kMmaWarp ? 0 : 1;
+        const uint32_t el = elect_one() ? 1u : 0u;
+        bool ok = true;
+        int base = 0;             // ring position of the item's first slot
+        int cnt = 0;              // tiles of the group before this item: S buffer and phase of the hand-offs
+        int item_no = 0;
+        constexpr uint32_t idesc_pv = instr_desc(D, 1);
+        const uint32_t ocol = tmem + kColO + (uint32_t)(D * b);
+        TItem it_next = load_titem(head_work, i0 < i1);
+        const long long t_loop = trace_clock();
+        long long tr_p = 0, tr_kv = 0, tr_item = 0;      // time-stamp build: cycles waiting for P, for K/V, for an item's Q and O
+        int ev = 0;                                      // time-stamp build: event log position
+        for (int ii = i0; ii < i1 && ok; ++ii, ++item_no) {
+            const TItem it = it_next;
+            it_next = load_titem(p.works + ii + 1, ii + 1 < i1);      // in flight while this item runs
+            const int ntiles = (it.kv_end - it.kv0 + kTile - 1) / kTile;
+            const bool dual = it.ntok * G > kRows;      // both groups on every tile, group b on row tile b; otherwise alternate tiles
+            const int lead = dual ? 2 : 4, mine = dual ? ntiles : (ntiles + 1 - b) / 2;
+            const long long t_item = trace_clock();
+            ok = mbar_wait_spin(bar(Geo::kQFull), (uint32_t)item_no & 1u, abort_flag, p.status, 22);
+            // S and O of the previous item are in use until its epilogue is over
+            if (ok && item_no > 0) ok = mbar_wait_spin(bar(Geo::kOFree), (uint32_t)(item_no - 1) & 1u, abort_flag, p.status, 27);
+            tr_item += trace_clock() - t_item;
+            if (ok) tc_fence_after();
+            const uint64_t qd = smem_desc(sbase + Geo::OFF_Q + (dual ? (uint32_t)b * Geo::QTILE_BYTES : 0u), 16, 1024);
+            auto tile_pages = [&](int j) { return (min(kTile, it.kv_end - (it.kv0 + j * kTile)) + kPage - 1) / kPage; };
+            auto wait_slot = [&](int pos, int code) {
+                const long long tw = trace_clock();
+                ok = ok && mbar_wait_spin(bar(Geo::kRingFull0 + pos % Geo::RING), (uint32_t)(pos / Geo::RING) & 1u, abort_flag, p.status, code);
+                tr_kv += trace_clock() - tw;
+            };
+            auto slot_addr = [&](int pos) { return sbase + Geo::OFF_RING + (uint32_t)(pos % Geo::RING) * Geo::SLOT_BYTES; };
+            // u = -2, -1: the Q K^T of the group's first two tiles; u >= 0: the turn of its u-th tile, the P V of
+            // tile j and the Q K^T of tile j + lead back to back once everything they read is there.  K/V tiles
+            // are waited for first (they are normally there already), P last, so that nothing stands between
+            // its arrival and the first MMA.  One commit per turn: it tells the group that its next S is complete
+            // and, because MMAs complete in issue order, that every MMA in front of it is done as well (the
+            // group releases ring slots on that knowledge; a commit costs the tensor pipe ~90 cycles).  Where no
+            // next tile is left the P V is committed by itself: the last turn on either buffer ends on kPvDone.
+            for (int u = -2; u < mine && ok; ++u) {
+                const int c = cnt + u;
+                const bool pv = u >= 0, qk = u + 2 < mine;
+                if (!pv && !qk) continue;
+                const int j = dual ? u : 2 * u + b, jn = j + lead;
+                const int pos_v = base + ring_pos_v(j, ntiles, lead), pos_k = base + ring_pos_k(jn, lead);
+                if (lane == 0) trace_event(b ? 10 : 0, ev, 20 + b);
+                if (pv) wait_slot(pos_v, 24);
+                if (qk) wait_slot(pos_k, 21);
+                const uint32_t buf = tmem + kColS + 128u * (uint32_t)b + 64u * (uint32_t)(c & 1);      // S and P
+                const uint64_t vd = smem_desc(slot_addr(pos_v), Geo::HALF_BYTES, 1024);
+                const uint64_t kd = smem_desc(slot_addr(pos_k), 16, 1024);
+                const uint32_t idesc_qk = instr_desc(16u * (uint32_t)tile_pages(jn), 0);
+                const int npg = tile_pages(j);
+                const uint32_t done = bar((qk ? Geo::kSFull0 : Geo::kPvDone0) + 2 * b + (c & 1));
+                if (pv) {
                     const long long tw = trace_clock();
-                    ok = ok && mbar_wait_spin(bar(kRingFull0 + s), (uint32_t)(pos / kRing) & 1u, abort_flag, p.status, 21);
-                    tr_kv += trace_clock() - tw;
-                };
-                auto wait_v = [&](int j) {
-                    const int pos = ring_pos_v(gt + j), s = pos % kRing;
-                    const long long tw = trace_clock();
-                    ok = ok && mbar_wait_spin(bar(kRingFull0 + s), (uint32_t)(pos / kRing) & 1u, abort_flag, p.status, 24);
-                    tr_kv += trace_clock() - tw;
-                };
-                auto wait_p = [&](int b) {
-                    const long long tw = trace_clock();
-                    ok = ok && mbar_wait_spin(bar(kPFull0 + 2 * b), (uint32_t)(b ? cnt1 : cnt0) & 1u, abort_flag, p.status, 26);
+                    ok = ok && mbar_wait_spin(bar(Geo::kPFull0 + 2 * b + (c & 1)), (uint32_t)(c >> 1) & 1u, abort_flag, p.status, 26);
                     tr_p += trace_clock() - tw;
-                };
-                // S[b] <- Q[qt] K_j^T, then one commit: it tells group b that S[b] is complete and, because MMAs
-                // complete in issue order, that every MMA in front of it is done as well (the group releases
-                // the ring slots on that knowledge: a second commit per batch costs the tensor pipe ~90 cycles)
-                auto emit_qk = [&](int j, int b) {
-                    const long long ti = trace_clock();
-                    const int s = ring_pos_k(gt + j) % kRing;
-                    const uint32_t idesc = instr_desc(16u * (uint32_t)tile_pages(j), 0);
-                    const uint32_t d = tmem + kColS + 128u * (uint32_t)b;
-                    const uint64_t qd = smem_desc(sbase + kOffQ + (dual ? (uint32_t)b * kTileBytes : 0u), 16, 1024);
-                    const uint64_t kd = smem_desc(sbase + kOffRing + s * kTileBytes, 16, 1024);
-#pragma unroll
-                    for (int ks = 0; ks < kD / 16; ++ks) {
-                        // the address field counts 16-byte units and cannot carry out of its 14 bits here
-                        const uint64_t off = (uint64_t)(((uint32_t)(ks >> 2) * kHalfBytes + (uint32_t)(ks & 3) * 32u) >> 4);
-                        if (elect_one()) mma_f16(d, qd + off, kd + off, idesc, ks > 0);
-                    }
-                    if (elect_one()) mma_commit(bar(kSFull0 + 2 * b));
-                    tr_qk += trace_clock() - ti;
-                    if (lane == 0) trace_event(0, ev, 14 + b);
-                };
-                // O[b] (+)= P[b] V_j with P[b] in tensor memory; fresh: first P V of the item into O[b];
-                // last: the group's last tile of the item, the only one whose completion is signalled by itself
-                auto emit_pv = [&](int j, int b, bool fresh, bool last) {
-                    const long long ti = trace_clock();
-                    const int s = ring_pos_v(gt + j) % kRing;
-                    const int npg = tile_pages(j);
-                    const uint32_t pcol = tmem + kColS + 128u * (uint32_t)b;
-                    const uint64_t vd = smem_desc(sbase + kOffRing + s * kTileBytes, kHalfBytes, 1024);
-                    const uint32_t ocol = tmem + kColO + 128u * (uint32_t)b;
+                }
+                if (lane == 0) trace_event(b ? 10 : 0, ev, 22 + b);
+                if (!ok) break;
+                tc_fence_after();
+                if (pv) {
+                    // O[b] (+)= P[b] V_j with P[b] in tensor memory
                     if (npg == kTile / kPage) {
 #pragma unroll
                         for (int ks = 0; ks < kTile / kPage; ++ks)
-                            if (elect_one()) mma_f16_ta(ocol, pcol + 8u * (uint32_t)ks, vd + (uint64_t)(ks * 128), idesc_pv, (!fresh || ks > 0) ? 1u : 0u);
+                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)(ks * 128), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
                     } else {
                         for (int ks = 0; ks < npg; ++ks)
-                            if (elect_one()) mma_f16_ta(ocol, pcol + 8u * (uint32_t)ks, vd + (uint64_t)(ks * 128), idesc_pv, (!fresh || ks > 0) ? 1u : 0u);
+                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)(ks * 128), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
                     }
-                    if (last && elect_one()) mma_commit(bar(kPvDone0 + 2 * b));
-                    if (b) ++cnt1; else ++cnt0;
-                    tr_pv += trace_clock() - ti;
-                    if (lane == 0) trace_event(0, ev, 26 + b);
-                };
-                auto first_qk = [&](int j, int b) {
-                    wait_k(j);
-                    if (!ok) return;
-                    tc_fence_after();
-                    emit_qk(j, b);
-                };
-                // One turn of group b: the P V of its tile j and at once the Q K^T of its next tile jn (-1: none),
-                // sixteen MMAs issued back to back once everything they read is there.
-                auto turn = [&](int j, int b, bool fresh, int jn) {
-                    if (lane == 0) trace_event(0, ev, 20 + b);
-                    wait_v(j);
-                    if (jn >= 0) wait_k(jn);
-                    wait_p(b);
-                    if (lane == 0) trace_event(0, ev, 22 + b);
-                    if (!ok) return;
-                    tc_fence_after();
-                    emit_pv(j, b, fresh, jn < 0);
-                    if (jn >= 0) emit_qk(jn, b);
-                };
-                if (dual) {
-                    // both groups on every tile: group b owns row tile b
-                    first_qk(0, 0);
-                    if (ok) first_qk(0, 1);
-                    for (int j = 0; j < ntiles && ok; ++j)
-                        for (int b = 0; b < 2 && ok; ++b) turn(j, b, j == 0, j + 1 < ntiles ? j + 1 : -1);
-                } else {
-                    // one row tile: the groups take alternate KV tiles
-                    first_qk(0, 0);
-                    if (ok && ntiles > 1) first_qk(1, 1);
-                    for (int j = 0; j < ntiles && ok; ++j) turn(j, j & 1, j < 2, j + 2 < ntiles ? j + 2 : -1);
                 }
-                gt += ntiles;
+                if (qk) {
+                    // S[b] <- Q[b] K^T
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        // the address field counts 16-byte units and cannot carry out of its 14 bits here
+                        const uint64_t qoff = (uint64_t)(((uint32_t)(ks >> 2) * Geo::QHALF_BYTES + (uint32_t)(ks & 3) * 32u) >> 4);
+                        const uint64_t koff = (uint64_t)(((uint32_t)(ks >> 2) * Geo::HALF_BYTES + (uint32_t)(ks & 3) * 32u) >> 4);
+                        mma_f16(el, buf, qd + qoff, kd + koff, idesc_qk, ks > 0);
+                    }
+                }
+                mma_commit(el, done);
+                if (lane == 0) trace_event(b ? 10 : 0, ev, 26 + b);
             }
-            if (lane == 0) {
-                trace_set(8, tr_p);
-                trace_set(9, tr_kv);
-                trace_set(10, trace_clock() - t_loop);
-                trace_set(14, tr_item);
-                trace_set(2, tr_qk);
-                trace_set(3, tr_pv);
-            }
-            // make sure nothing is still running on the tensor core before tensor memory is released
-            if (elect_one()) mma_commit(bar(kMmaDrain));
-            const long long t0 = clock64();
-            while (!mbar_try_wait(bar(kMmaDrain), 0) && clock64() - t0 < kWaitCycles) {}
+            cnt += mine;
+            base += 2 * ntiles;
         }
+        if (lane == 0 && b == 0) {
+            trace_set(8, tr_p);
+            trace_set(9, tr_kv);
+            trace_set(10, trace_clock() - t_loop);
+            trace_set(14, tr_item);
+        }
+        // make sure nothing is still running on the tensor core before tensor memory is released
+        mma_commit(el, bar(Geo::kMmaDrain));
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar(Geo::kMmaDrain), 0) && clock64() - t0 < kWaitCycles) {}
         __syncwarp();
       }
     } else {
@@ -605,179 +563,164 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         const int m = threadIdx.x & 127;           // row of the group's tile = tensor-memory lane
         const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t s_addr = lane_addr + kColS + 128u * (uint32_t)b;      // + 64 * buffer
-        const uint32_t o_addr = lane_addr + kColO + 128u * (uint32_t)b;
+        const uint32_t o_addr = lane_addr + kColO + (uint32_t)(D * b);
         const float qscale = p.sm_scale * kLog2e;
         const float2 qscale2 = make_float2(qscale, qscale);
         int cnt = 0;         // tiles this group has processed before this item
-        int gt = 0;          // KV tiles of the CTA before this item (both groups): ring position
-        int pv_cnt = 0;      // items so far in which this group had tiles: phase of its "last P V done" barrier
+        int ring_base = 0;   // ring position of the item's first slot
+        uint32_t pv_phase = 0;      // bit s: parity of the next phase of this group's kPvDone of buffer s
         int item_no = 0;
         bool ok = true;
         long long tr_wait = 0, tr_work = 0, tr_tiles = 0;      // time-stamp build: cycles waiting for S, cycles from S to P, tiles
         int ev = 0;                                            // time-stamp build: event log position (lane 0 of each warp)
-        // This thread's share of an item's Q.  Dual items: the whole row 128 b + m (16 chunks of 16
-        // bytes) into Q[b]; otherwise value half b of row m (8 chunks) into Q[0].  The next item's Q is
+        // This thread's share of an item's Q.  Dual items: the whole row 128 b + m (kQV chunks of 16
+        // bytes) into Q[b]; otherwise value half b of row m (kQV / 2 chunks) into Q[0].  The next item's Q is
         // fetched at the end of the current item's KV loop, ahead of the epilogue.
-        auto load_q = [&](const TItem& x, uint4 (&w)[16]) {
-            const bool dual = x.ntok * G > kTile;
+        constexpr int kQV = D / 8;
+        auto load_q = [&](const TItem& x, uint4 (&w)[kQV]) {
+            const bool dual = x.ntok * G > kRows;
             const int r = dual ? 128 * b + m : m;
             const bool valid = x.kv_end > 0 && r / G < x.ntok;
             const uint4* src = reinterpret_cast<const uint4*>(
-                q + ((size_t)(x.q_row0 + r / G) * Hq + (size_t)x.kv_head * G + r % G) * kD) + (dual ? 0 : 8 * b);
+                q + ((size_t)(x.q_row0 + r / G) * Hq + (size_t)x.kv_head * G + r % G) * D) + (dual ? 0 : kQV / 2 * b);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) w[c] = valid ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
+            for (int c = 0; c < kQV / 2; ++c) w[c] = valid ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-            for (int c = 8; c < 16; ++c) w[c] = (valid && dual) ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
+            for (int c = kQV / 2; c < kQV; ++c) w[c] = (valid && dual) ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
         };
+        // A ring slot is free again after two arrivals: one of each group in a dual item, else two of its only reader.
+        auto release = [&](int s, bool dual) { mbar_arrive_n(bar(Geo::kRingEmpty0 + s), dual ? 1u : 2u); };
         TItem it_next = load_titem(head_work, i0 < i1);
-        uint4 q_next[16];
+        uint4 q_next[kQV];
         pdl_wait();
         load_q(it_next, q_next);
         for (int ii = i0; ii < i1 && ok; ++ii, ++item_no) {
             const TItem it = it_next;
             const int ntiles = (it.kv_end - it.kv0 + kTile - 1) / kTile;
-            const bool dual = it.ntok * G > kTile;
+            const bool dual = it.ntok * G > kRows;
+            const int lead = dual ? 2 : 4;
+            const int mine = dual ? ntiles : (ntiles + 1 - b) / 2;      // KV tiles of this group
             const int r = dual ? 128 * b + m : m;      // query row of the item
             const int t = r / G, g = r % G;
             const bool row_valid = t < it.ntok;
             // ---- stage Q with the 128-byte swizzle the MMA descriptor expects (the previous item's
             // epilogue used the Q tiles as its output staging area: wait until every warp is through)
             if (item_no > 0) {
-                ok = mbar_wait_warp(bar(kOFree), (uint32_t)(item_no - 1) & 1u, abort_flag, p.status, 36);
+                ok = mbar_wait_warp(bar(Geo::kOFree), (uint32_t)(item_no - 1) & 1u, abort_flag, p.status, 36);
                 if (!ok) break;
             }
-            if (dual) {
 #pragma unroll
-                for (int c = 0; c < 16; ++c)
-                    *reinterpret_cast<uint4*>(smem + kOffQ + b * kTileBytes + (c >> 3) * kHalfBytes + m * 128 +
-                                              (((c & 7) ^ (m & 7)) << 4)) = q_next[c];
-            } else {
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                    *reinterpret_cast<uint4*>(smem + kOffQ + b * kHalfBytes + m * 128 + ((c ^ (m & 7)) << 4)) = q_next[c];
-            }
+            for (int c = 0; c < kQV; ++c)
+                if (dual || c < kQV / 2) {
+                    const int cc = dual ? c : c + kQV / 2 * b;      // chunk of the row
+                    *reinterpret_cast<uint4*>(smem + Geo::OFF_Q + (dual ? b * Geo::QTILE_BYTES : 0u) + (cc >> 3) * Geo::QHALF_BYTES + m * 128 +
+                                              (((cc & 7) ^ (m & 7)) << 4)) = q_next[c];
+                }
             fence_async_smem();
-            mbar_arrive(bar(kQFull));
+            mbar_arrive(bar(Geo::kQFull));
             if (lane == 0) trace_event(1 + warp, ev, 37);
             it_next = load_titem(p.works + ii + 1, ii + 1 < i1);
             const int lim_row = row_valid ? min(it.kv_limit0 + t, it.kv_end) : 0;   // keys [0, lim_row) visible
             float m_ref = -INFINITY;                     // reference maximum (log2 domain)
             float2 l2 = make_float2(0.f, 0.f), l2b = make_float2(0.f, 0.f);      // running sum of P, four partial sums
-            int mine = 0;                                // tiles of this group so far in this item
-            for (int j = dual ? 0 : b; j < ntiles && ok; j += dual ? 1 : 2, ++mine) {
+            for (int u = 0; u < mine && ok; ++u) {
+                const int j = dual ? u : 2 * u + b, ct = cnt + u;
                 const int npg = (min(kTile, it.kv_end - (it.kv0 + j * kTile)) + kPage - 1) / kPage;
-                // S[b] complete; it was issued after the P V of this group's previous tile finished, so
-                // O[b] is at rest as well
+                const uint32_t sb = s_addr + 64u * (uint32_t)(ct & 1);
                 const long long tw = trace_clock();
                 if (lane == 0) trace_event(1 + warp, ev, 30);
-                ok = __all_sync(0xffffffffu, mbar_wait_spin(bar(kSFull0 + 2 * b), (uint32_t)(cnt + mine) & 1u, abort_flag, p.status, 31));
+                ok = __all_sync(0xffffffffu, mbar_wait_spin(bar(Geo::kSFull0 + 2 * b + (ct & 1)), (uint32_t)(ct >> 1) & 1u, abort_flag, p.status, 31));
                 const long long ts = trace_clock();
                 if (lane == 0) trace_event(1 + warp, ev, 31);
                 tr_wait += ts - tw;
                 ++tr_tiles;
                 if (!ok) break;
                 tc_fence_after();
-                // S[b] of tile j complete means every MMA issued before it is complete.  The group that is
-                // last to use a ring slot gives it back to the producers: the K tile of j now, and the V tile
-                // of the group's previous tile (its P V was issued in front of this Q K^T).
-                if (m == 0 && (!dual || b == 1)) {
-                    mbar_arrive(bar(kRingEmpty0 + ring_pos_k(gt + j) % kRing));
-                    if (mine > 0) mbar_arrive(bar(kRingEmpty0 + ring_pos_v(gt + j - (dual ? 1 : 2)) % kRing));
+                const int base = it.kv0 + j * kTile;
+                const int vis = max(0, min(kTile, lim_row - base));      // visible columns of this row
+                uint32_t rr[64];
+                tmem_ld32(sb, *reinterpret_cast<uint32_t(*)[32]>(&rr[0]));
+                tmem_ld32(sb + 32u, *reinterpret_cast<uint32_t(*)[32]>(&rr[32]));
+                // This S complete means every MMA issued for the group before it is complete: the ring slots they
+                // read go back to the producers, the K tile of j now, and the V tile of j - lead (its P V was
+                // issued in front of this Q K^T).
+                if (m == 0) {
+                    release((ring_base + ring_pos_k(j, lead)) % Geo::RING, dual);
+                    if (u >= 2) release((ring_base + ring_pos_v(j - lead, ntiles, lead)) % Geo::RING, dual);
                 }
-                // the tile is handled in two halves of 64 keys (register budget)
-                for (int h = 0; h * 4 < npg; ++h) {
-                    const int base = it.kv0 + j * kTile + h * kSub;
-                    const int vis = max(0, min(kSub, lim_row - base));      // visible columns of this row
-                    const uint32_t sb = s_addr + 64u * (uint32_t)h;
-                    uint32_t rr[64];
-                    tmem_ld32(sb, *reinterpret_cast<uint32_t(*)[32]>(&rr[0]));
-                    tmem_ld32(sb + 32u, *reinterpret_cast<uint32_t(*)[32]>(&rr[32]));
-                    tmem_wait_ld();
-                    // x = S * scale - m_ref (log2 domain), two values per instruction
-                    const float m_use = m_ref == -INFINITY ? 0.f : m_ref;
-                    const float2 nm2 = make_float2(-m_use, -m_use);
-                    float2 x[32];
+                tmem_wait_ld();
+                if (!__all_sync(0xffffffffu, vis == kTile)) {
 #pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        x[e] = __ffma2_rn(make_float2(__uint_as_float(rr[2 * e]), __uint_as_float(rr[2 * e + 1])), qscale2, nm2);
-                    if (!__all_sync(0xffffffffu, vis == kSub)) {
+                    for (int e = 0; e < 64; ++e)
+                        if (e >= vis) rr[e] = 0xff800000u;      // -inf
+                }
+                // row maximum of the raw scores (the scale is positive): four independent chains of 3-input
+                // maxima (a lone warp per scheduler cannot hide one long dependent chain)
+                auto sv = [&](int k) { return __uint_as_float(rr[k]); };
+                float cm[4];
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            if (2 * e >= vis) x[e].x = -INFINITY;
-                            if (2 * e + 1 >= vis) x[e].y = -INFINITY;
-                        }
-                    }
-                    // row maximum of the half: four independent chains of 3-input maxima (a lone warp per
-                    // scheduler cannot hide one long dependent chain)
-                    auto xv = [&](int k) { return (k & 1) ? x[k >> 1].y : x[k >> 1].x; };
-                    float cm[4];
+                for (int c = 0; c < 4; ++c) cm[c] = fmax3(sv(16 * c), sv(16 * c + 1), sv(16 * c + 2));
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) cm[c] = fmax3(xv(16 * c), xv(16 * c + 1), xv(16 * c + 2));
+                for (int k = 3; k < 15; k += 2) {
 #pragma unroll
-                    for (int k = 3; k < 15; k += 2) {
+                    for (int c = 0; c < 4; ++c) cm[c] = fmax3(cm[c], sv(16 * c + k), sv(16 * c + k + 1));
+                }
 #pragma unroll
-                        for (int c = 0; c < 4; ++c) cm[c] = fmax3(cm[c], xv(16 * c + k), xv(16 * c + k + 1));
-                    }
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) cm[c] = fmaxf(cm[c], xv(16 * c + 15));
-                    const float cmax = fmax3(fmaxf(cm[0], cm[1]), cm[2], cm[3]);
-                    // x is relative to m_ref (to 0 while the row has no reference yet: then any visible key sets it)
-                    if (__any_sync(0xffffffffu, cmax > (m_ref == -INFINITY ? -INFINITY : kRescaleThreshold))) {
-                        // Move the reference maximum (rare after the first tile): rescale the running sum, the
-                        // half of P already written for this tile and O[b], and shift this half's x.
-                        const float m_new = cmax == -INFINITY ? m_ref : fmaxf(m_ref, m_use + cmax);
-                        const float scale = m_new == -INFINITY ? 1.f : fast_exp2(m_ref - m_new);
-                        const float shift = (m_new == -INFINITY ? 0.f : m_new) - m_use;
-                        m_ref = m_new;
-                        l2.x *= scale;
-                        l2.y *= scale;
-                        l2b.x *= scale;
-                        l2b.y *= scale;
-                        const float2 ns2 = make_float2(-shift, -shift);
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) x[e] = __fadd2_rn(x[e], ns2);
-                        tmem_wait_st();
-                        if (h > 0) {
+                for (int c = 0; c < 4; ++c) cm[c] = fmaxf(cm[c], sv(16 * c + 15));
+                const float cmax = fmax3(fmaxf(cm[0], cm[1]), cm[2], cm[3]) * qscale;      // log2 domain
+                if (__any_sync(0xffffffffu, cmax > m_ref + kRescaleThreshold)) {
+                    // Move the reference maximum (rare after the first tile; a row without one takes any visible
+                    // key's): rescale the running sum and O[b].  O[b] is at rest once the P V of the group's
+                    // previous tile is done, which its commit tells: the next S of the other buffer, or kPvDone.
+                    const float m_new = fmaxf(m_ref, cmax);
+                    const float scale = m_new == -INFINITY ? 1.f : fast_exp2(m_ref - m_new);
+                    m_ref = m_new;
+                    l2.x *= scale;
+                    l2.y *= scale;
+                    l2b.x *= scale;
+                    l2b.y *= scale;
+                    if (u > 0) {
+                        const int ob = (ct + 1) & 1, pb = (u + 1 < mine ? Geo::kSFull0 : Geo::kPvDone0) + 2 * b + ob;
+                        const uint32_t pp = u + 1 < mine ? (uint32_t)((ct + 1) >> 1) & 1u : (pv_phase >> ob) & 1u;
+                        ok = __all_sync(0xffffffffu, mbar_wait_spin(bar(pb), pp, abort_flag, p.status, 32));
+                        if (!ok) break;
+                        tc_fence_after();
 #pragma unroll 1
-                            for (int cc = 0; cc < 2; ++cc) {
-                                uint32_t pk[16];
-                                tmem_ld16(s_addr + 16u * cc, pk);
-                                tmem_wait_ld();
+                        for (int cc = 0; cc < D / 16; ++cc) {
+                            uint32_t ro[16];
+                            tmem_ld16(o_addr + 16u * cc, ro);
+                            tmem_wait_ld();
 #pragma unroll
-                                for (int e = 0; e < 16; ++e)
-                                    pk[e] = pack_bf16x2(bf16_lo(pk[e]) * scale, bf16_hi(pk[e]) * scale);
-                                tmem_st16(s_addr + 16u * cc, pk);
-                            }
-                        }
-                        if (mine > 0) {
-#pragma unroll 1
-                            for (int cc = 0; cc < 8; ++cc) {
-                                uint32_t ro[16];
-                                tmem_ld16(o_addr + 16u * cc, ro);
-                                tmem_wait_ld();
-#pragma unroll
-                                for (int e = 0; e < 16; ++e) ro[e] = __float_as_uint(__uint_as_float(ro[e]) * scale);
-                                tmem_st16(o_addr + 16u * cc, ro);
-                            }
+                            for (int e = 0; e < 16; ++e) ro[e] = __float_as_uint(__uint_as_float(ro[e]) * scale);
+                            tmem_st16(o_addr + 16u * cc, ro);
                         }
                         tmem_wait_st();
                     }
-                    // P = exp2(x) as packed bf16: half h of the tile goes to columns [32 h, 32 h + 32) of
-                    // the buffer, which this thread has already read
-                    uint32_t pk[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) {
-                        const float2 pe = make_float2(fast_exp2(x[e].x), fast_exp2(x[e].y));
-                        if (e & 1) l2b = __fadd2_rn(l2b, pe); else l2 = __fadd2_rn(l2, pe);
-                        pk[e] = pack_bf16x2(pe.x, pe.y);
-                    }
-                    tmem_st16(s_addr + 32u * (uint32_t)h, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));
-                    tmem_st16(s_addr + 32u * (uint32_t)h + 16u, *reinterpret_cast<uint32_t(*)[16]>(&pk[16]));
                 }
+                // Both groups of a dual item get their first S together and would stay in step, both on the
+                // exponential unit at once and both off it: the second group starts half a tile later.
+                if (dual && b == 1 && u == 0) {
+                    const long long t0 = clock64();
+                    while (clock64() - t0 < kGroupSkewCycles) {}
+                }
+                // P = exp2(S * scale - m_ref) as packed bf16 goes to the first 32 columns of the buffer, which this
+                // thread has read
+                const float m_use = m_ref == -INFINITY ? 0.f : m_ref;
+                const float2 nm2 = make_float2(-m_use, -m_use);
+                uint32_t pk[32];
+#pragma unroll
+                for (int e = 0; e < 32; ++e) {
+                    const float2 x = __ffma2_rn(make_float2(__uint_as_float(rr[2 * e]), __uint_as_float(rr[2 * e + 1])), qscale2, nm2);
+                    const float2 pe = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                    if (e & 1) l2b = __fadd2_rn(l2b, pe); else l2 = __fadd2_rn(l2, pe);
+                    pk[e] = pack_bf16x2(pe.x, pe.y);
+                }
+                tmem_st16(sb, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));
+                tmem_st16(sb + 16u, *reinterpret_cast<uint32_t(*)[16]>(&pk[16]));
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();      // 128 arrivals on one barrier word would take turns; the warp's lanes are ordered here instead
-                if (lane == 0) mbar_arrive(bar(kPFull0 + 2 * b));
+                if (lane == 0) mbar_arrive(bar(Geo::kPFull0 + 2 * b + (ct & 1)));
                 tr_work += trace_clock() - ts;
                 if (lane == 0) trace_event(1 + warp, ev, 32);
             }
@@ -787,21 +730,21 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             if (lane == 0) trace_event(1 + warp, ev, 33);
             // ---- epilogue.  The groups' (max, sum) go through columns 0-1 of their S buffers, which are
             // idle from the group's last P V until the next item's first Q K^T.
-            if (mine > 0) {
-                ok = mbar_wait_warp(bar(kPvDone0 + 2 * b), (uint32_t)pv_cnt & 1u, abort_flag, p.status, 34);
-                if (!ok) break;
-                ++pv_cnt;
-                tc_fence_after();
-                if (lane == 0) trace_event(1 + warp, ev, 34);
-                // the V tile of the group's last tile goes back to the producers
-                if (m == 0 && (!dual || b == 1))
-                    mbar_arrive(bar(kRingEmpty0 + ring_pos_v(gt + (dual ? ntiles - 1 : b + 2 * (mine - 1))) % kRing));
+            for (int u = max(0, mine - 2); u < mine && ok; ++u) {
+                const int sb = (cnt + u) & 1;
+                ok = mbar_wait_warp(bar(Geo::kPvDone0 + 2 * b + sb), (pv_phase >> sb) & 1u, abort_flag, p.status, 34);
+                pv_phase ^= 1u << sb;
+                // the V tiles of the group's last tiles go back to the producers
+                if (ok && m == 0) release((ring_base + ring_pos_v(dual ? u : 2 * u + b, ntiles, lead)) % Geo::RING, dual);
             }
+            if (!ok) break;
+            tc_fence_after();
+            if (lane == 0) trace_event(1 + warp, ev, 34);
             tmem_st2(s_addr, __float_as_uint(m_ref), __float_as_uint(l_sum));
             tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(bar(kStats));
-            ok = mbar_wait_warp(bar(kStats), (uint32_t)item_no & 1u, abort_flag, p.status, 35);
+            mbar_arrive(bar(Geo::kStats));
+            ok = mbar_wait_warp(bar(Geo::kStats), (uint32_t)item_no & 1u, abort_flag, p.status, 35);
             if (!ok) break;
             tc_fence_after();
             if (lane == 0) trace_event(1 + warp, ev, 35);
@@ -814,9 +757,10 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 w0 = b == 0 ? inv : 0.f;
                 w1 = b == 1 ? inv : 0.f;
                 lse2 = l_sum > 0.f ? m_ref + log2f(l_sum) : -INFINITY;
-                c_begin = 0; c_end = 4;
+                c_begin = 0; c_end = D / 32;
             } else {
-                // the two groups hold two KV splits of the same rows: merge them; group b writes value half b
+                // the two groups hold two KV splits of the same rows: merge them; a group writes slices of 64 values,
+                // group b the b-th (head_dim 64 has only one)
                 uint32_t x0, y0, x1, y1;
                 tmem_ld2(lane_addr + kColS, x0, y0);
                 tmem_ld2(lane_addr + kColS + 128u, x1, y1);
@@ -831,14 +775,14 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 w0 = a0 * inv;
                 w1 = a1 * inv;
                 lse2 = L > 0.f ? M + log2f(L) : -INFINITY;
-                c_begin = 2 * b; c_end = 2 * b + 2;
+                c_begin = 2 * b; c_end = min(2 * b + 2, D / 32);
             }
             const bool use0 = __any_sync(0xffffffffu, w0 != 0.f), use1 = __any_sync(0xffffffffu, w1 != 0.f);
             // A thread holds one row, but a row-per-thread store touches 32 lines per instruction: the
             // warp passes each 128-byte slice of its 32 rows through shared memory (its own rows of the Q
             // tile, which no MMA reads any more; 16-byte pieces XOR-swizzled by row) and writes whole lines.
             const int w4 = warp & 3;
-            uint8_t* stage = smem + kOffQ + (dual ? b * kTileBytes : b * kHalfBytes) + w4 * 32 * 128;
+            uint8_t* stage = smem + Geo::OFF_Q + b * (dual ? Geo::QTILE_BYTES : Geo::QHALF_BYTES) + w4 * 32 * 128;
             const int row_base = (dual ? 128 * b : 0) + 32 * w4;      // item row of the warp's first thread
             const bool final_out = it.partial_row0 < 0;
             auto flush = [&](int byte0) {      // byte0: offset of the slice inside an output row
@@ -850,8 +794,8 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                     const int ri = row_base + row, tt = ri / G, gg = ri % G;
                     if (tt < it.ntok) {
                         uint8_t* dst = final_out
-                            ? reinterpret_cast<uint8_t*>(out + ((size_t)(it.q_row0 + tt) * Hq + (size_t)it.kv_head * G + gg) * kD)
-                            : reinterpret_cast<uint8_t*>(p.partial_o + (((size_t)it.partial_row0 + tt) * G + gg) * kD);
+                            ? reinterpret_cast<uint8_t*>(out + ((size_t)(it.q_row0 + tt) * Hq + (size_t)it.kv_head * G + gg) * D)
+                            : reinterpret_cast<uint8_t*>(p.partial_o + (((size_t)it.partial_row0 + tt) * G + gg) * D);
                         *reinterpret_cast<uint4*>(dst + byte0 + pc * 16) = v;
                     }
                 }
@@ -873,7 +817,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 }
                 if (use1) {
                     uint32_t ro[32];
-                    tmem_ld32(lane_addr + kColO + 128u + 32u * c, ro);
+                    tmem_ld32(lane_addr + kColO + (uint32_t)D + 32u * c, ro);
                     tmem_wait_ld();
                     if (w1 != 0.f) {
 #pragma unroll
@@ -906,10 +850,10 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 }
             }
             tc_fence_before();
-            mbar_arrive(bar(kOFree));
+            mbar_arrive(bar(Geo::kOFree));
             if (lane == 0) trace_event(1 + warp, ev, 36);
             cnt += mine;
-            gt += ntiles;
+            ring_base += 2 * ntiles;
         }
         if ((threadIdx.x & 127) == 0) {
             trace_set(b ? 15 : 11, tr_wait);

@@ -179,7 +179,7 @@ struct Geometry {
 };
 
 template <int D>
-size_t smem_bytes(int stages) {
+constexpr size_t smem_bytes(int stages) {
     using Geo = Geometry<D>;
     return (size_t)stages * (Geo::STAGE_BYTES + Geo::Q_BYTES + sizeof(TileDesc) + 16) +
            (size_t)(kHandoffs + kMergeReqs) * (sizeof(TileDesc) + 8) + kMergeReqs * 8 + sizeof(NextItem) + 16 +

@@ -8,9 +8,10 @@
 //                          start-up and tail per kernel at 148 CTAs) is paid once, and a CTA that is
 //                          done with its span tiles early moves on to decode rows at once.
 //   attn_append_tc_kernel  steps that have span tiles only
-//   attn_decode_kernel     steps without span tiles, and head_dim 64
+//   attn_decode_kernel     steps without span tiles
 // All are launched with programmatic stream serialization and wait for the kernel in front of them
 // (normally the KV append) right before they first touch the pool.
+#include <algorithm>
 #include <atomic>
 
 #include "attn_append_tc.cuh"
@@ -36,7 +37,7 @@ attn_decode_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const 
     dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, aligned_smem(smem_raw), app);
 }
 
-template <int G, bool APPEND>
+template <int D, int G, bool APPEND>
 __global__ void __launch_bounds__(tc::kThreads, 1)
 attn_append_tc_kernel(DevPlan p, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* pool,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse, AppendSrc app) {
@@ -46,11 +47,11 @@ attn_append_tc_kernel(DevPlan p, const __nv_bfloat16* __restrict__ q, const __nv
         trace_mark(0);
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<G, APPEND>(p, q, pool, out, lse, aligned_smem(smem_raw), app);
+    tc::tc_body<D, G, APPEND>(p, q, pool, out, lse, aligned_smem(smem_raw), app);
     if (threadIdx.x == 0) trace_mark(1);
 }
 
-template <int G, bool APPEND>
+template <int D, int G, bool APPEND>
 __global__ void __launch_bounds__(tc::kThreads, 1)
 attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* pool, __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
@@ -66,17 +67,17 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(&kv_map));
     if (head[0] == head[1]) {
         // no span tiles for this CTA: straight to its decode rows, without the tensor-memory set-up
-        dec::decode_body<tc::kD, G, APPEND>(p, &kv_map, q, out, lse, S, smem, app);
+        dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, smem, app);
         return;
     }
     if (threadIdx.x == 0) {
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<G, APPEND>(p, q, pool, out, lse, smem, app);
+    tc::tc_body<D, G, APPEND>(p, q, pool, out, lse, smem, app);
     if (threadIdx.x == 0) trace_mark(1);
     if (head[2] == head[3] && p.queue_count == 0) return;      // nothing left for the warp body
     __syncthreads();      // tensor memory released, shared memory free for the second phase
-    dec::decode_body<tc::kD, G, APPEND>(p, &kv_map, q, out, lse, S, smem, app);
+    dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, smem, app);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -146,8 +147,8 @@ cudaError_t cached_kv_map(const DevPlan& p, const void* pool, CUtensorMap* map) 
 }
 
 template <int D>
-int decode_stages() {
-    int S = 6;
+constexpr int decode_stages() {
+    int S = dec::kMaxStages;
     while (S > 2 && dec::smem_bytes<D>(S) > (size_t)kMaxSmem) --S;
     return S;
 }
@@ -166,88 +167,68 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
                       (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
-template <int G, bool APPEND>
+template <int D, int G, bool APPEND>
 cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, void* out, float* lse,
                           cudaStream_t stream, AppendSrc app) {
-    cudaError_t e = allow_smem<attn_append_tc_kernel<G, APPEND>>(tc::kSmemBytes);
+    constexpr size_t smem = tc::Geometry<D>::SMEM_BYTES;
+    cudaError_t e = allow_smem<attn_append_tc_kernel<D, G, APPEND>>(smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_append_tc_kernel<G, APPEND>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), tc::kSmemBytes, stream,
+    return launch_pdl(attn_append_tc_kernel<D, G, APPEND>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
                       p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, app);
 }
 
-template <int G, bool APPEND>
+template <int D, int G, bool APPEND>
 cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void* out, float* lse,
                          cudaStream_t stream, AppendSrc app) {
-    const int S = decode_stages<tc::kD>();
-    const size_t smem = dec::smem_bytes<tc::kD>(S) > tc::kSmemBytes ? dec::smem_bytes<tc::kD>(S) : tc::kSmemBytes;
-    cudaError_t e = allow_smem<attn_fused_kernel<G, APPEND>>(smem);
+    constexpr int S = decode_stages<D>();
+    constexpr size_t smem = std::max<size_t>(dec::smem_bytes<D>(S), tc::Geometry<D>::SMEM_BYTES);
+    static_assert(dec::smem_bytes<D>(S) - 1024 <= tc::Geometry<D>::OFF_BAR, "the span body's barriers stay clear of the warp body");
+    cudaError_t e = allow_smem<attn_fused_kernel<D, G, APPEND>>(smem);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     e = cached_kv_map(p, pool, &map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_fused_kernel<G, APPEND>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, map,
+    return launch_pdl(attn_fused_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, map,
                       (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S, app);
 }
 
+template <int D, int G, bool APPEND>
+cudaError_t launch_attention_impl(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
+                                  cudaStream_t stream, AppendSrc app) {
+    const bool has_tensor = p.num_items_tensor > 0, has_cuda = p.num_items_cuda > 0;
+    if (has_tensor && has_cuda && p.num_ctas_tensor == p.num_ctas_cuda)
+        return launch_fused<D, G, APPEND>(p, q, kv_pool, out, lse, stream, app);
+    if (has_tensor)
+        if (cudaError_t e = launch_tensor<D, G, APPEND>(p, q, kv_pool, out, lse, stream, app)) return e;
+    // a decode kernel behind a tensor kernel would have to wait for it to finish (pdl_wait), which is what
+    // stream order gives anyway
+    return has_cuda ? launch_decode<D, G, APPEND>(p, q, kv_pool, out, lse, stream, app) : cudaSuccess;
+}
+
 template <int D, bool APPEND>
-cudaError_t launch_decode_d(const DevPlan& p, const void* q, const void* pool, void* out, float* lse,
-                            cudaStream_t stream, AppendSrc app) {
+cudaError_t launch_attention_d(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
+                               cudaStream_t stream, AppendSrc app) {
     switch (p.group) {
-        case 1: return launch_decode<D, 1, APPEND>(p, q, pool, out, lse, stream, app);
-        case 2: return launch_decode<D, 2, APPEND>(p, q, pool, out, lse, stream, app);
-        case 4: return launch_decode<D, 4, APPEND>(p, q, pool, out, lse, stream, app);
-        case 8: return launch_decode<D, 8, APPEND>(p, q, pool, out, lse, stream, app);
+        case 1: return launch_attention_impl<D, 1, APPEND>(p, q, kv_pool, out, lse, stream, app);
+        case 2: return launch_attention_impl<D, 2, APPEND>(p, q, kv_pool, out, lse, stream, app);
+        case 4: return launch_attention_impl<D, 4, APPEND>(p, q, kv_pool, out, lse, stream, app);
+        case 8: return launch_attention_impl<D, 8, APPEND>(p, q, kv_pool, out, lse, stream, app);
         default: return cudaErrorInvalidValue;
     }
 }
 
 }  // namespace
 
-bool tensor_path_compiled(int head_dim) { return head_dim == tc::kD; }
-
-namespace {
-
-template <bool APPEND>
-cudaError_t launch_attention_impl(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
-                                  cudaStream_t stream, AppendSrc app) {
-    const bool has_tensor = p.num_items_tensor > 0, has_cuda = p.num_items_cuda > 0;
-    if (has_tensor && p.head_dim != tc::kD) return cudaErrorInvalidValue;
-    if (has_tensor && has_cuda && p.num_ctas_tensor == p.num_ctas_cuda) {
-        switch (p.group) {
-            case 1: return launch_fused<1, APPEND>(p, q, kv_pool, out, lse, stream, app);
-            case 2: return launch_fused<2, APPEND>(p, q, kv_pool, out, lse, stream, app);
-            case 4: return launch_fused<4, APPEND>(p, q, kv_pool, out, lse, stream, app);
-            case 8: return launch_fused<8, APPEND>(p, q, kv_pool, out, lse, stream, app);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (has_tensor) {
-        cudaError_t e;
-        switch (p.group) {
-            case 1: e = launch_tensor<1, APPEND>(p, q, kv_pool, out, lse, stream, app); break;
-            case 2: e = launch_tensor<2, APPEND>(p, q, kv_pool, out, lse, stream, app); break;
-            case 4: e = launch_tensor<4, APPEND>(p, q, kv_pool, out, lse, stream, app); break;
-            case 8: e = launch_tensor<8, APPEND>(p, q, kv_pool, out, lse, stream, app); break;
-            default: e = cudaErrorInvalidValue;
-        }
-        if (e != cudaSuccess) return e;
-    }
-    if (has_cuda) {
-        // a decode kernel behind a tensor kernel would have to wait for it to finish (pdl_wait), which
-        // is what stream order gives anyway
-        if (p.head_dim == 128) return launch_decode_d<128, APPEND>(p, q, kv_pool, out, lse, stream, app);
-        if (p.head_dim == 64) return launch_decode_d<64, APPEND>(p, q, kv_pool, out, lse, stream, app);
-        return cudaErrorInvalidValue;
-    }
-    return cudaSuccess;
-}
-
-}  // namespace
-
 cudaError_t launch_attention(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
                              cudaStream_t stream, AppendSrc app) {
-    return app.k_new != nullptr ? launch_attention_impl<true>(p, q, kv_pool, out, lse, stream, app)
-                                : launch_attention_impl<false>(p, q, kv_pool, out, lse, stream, app);
+    const bool append = app.k_new != nullptr;
+    if (p.head_dim == 128)
+        return append ? launch_attention_d<128, true>(p, q, kv_pool, out, lse, stream, app)
+                      : launch_attention_d<128, false>(p, q, kv_pool, out, lse, stream, app);
+    if (p.head_dim == 64)
+        return append ? launch_attention_d<64, true>(p, q, kv_pool, out, lse, stream, app)
+                      : launch_attention_d<64, false>(p, q, kv_pool, out, lse, stream, app);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace asynclm

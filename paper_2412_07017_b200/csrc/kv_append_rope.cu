@@ -56,7 +56,7 @@ kv_append_rope_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* _
     const int r0 = blockIdx.x * tokens, n = min(tokens, p.total_q - r0);
     pdl_wait();      // the rows and the pool belong to the kernels in front until those have completed
     auto load = [&](int i, int h) {
-        RopeRow x;
+        RopeRow x{};
         if (i >= n) return x;
         if (h < heads_k) {
             const size_t at = ((size_t)(r0 + i) * heads_k + h) * (2 * half_vecs) + v;

@@ -47,8 +47,8 @@ int tensor_tile_tokens(int group) { return 256 / group; }
 // Rows (G * q_len) from which a (sequence, kv head) goes to the span body (tcgen05).  Below it the
 // warp body reads the keys once per 8 (token, head) columns, which costs less than a span item's
 // start-up; decode rows (G rows) always stay on the warp body, which runs at the memory rate for
-// every supported G.
-static int default_tensor_min_rows(int) { return 32; }
+// every supported G.  At head_dim 64 a re-read of the keys costs half as much.
+static int default_tensor_min_rows(int head_dim) { return head_dim == 64 ? 64 : 32; }
 
 // Sizes of the sections of the packed blob (identical offsets on host and device).
 struct BlobLayout {
@@ -336,7 +336,8 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         // themselves (span CTAs draw little bandwidth, and one SM streams only so much)
         const int64_t stream_ctas = limit > kStartNs
             ? (warp_tiles * kWarpCost.tile_ns * kStreamShare64 / 64 + (limit - kStartNs) - 1) / (limit - kStartNs) : n_ctas;
-        const int64_t span_ctas = ids_warp.empty() ? n_ctas : n_ctas - stream_ctas;
+        // (a lone CTA does both)
+        const int64_t span_ctas = ids_warp.empty() || n_ctas == 1 ? n_ctas : n_ctas - stream_ctas;
         if (!order.empty() && span_ctas < 1) return false;
         // what a span CTA may be given: the span work spread over those CTAs with some slack for the
         // packing, at most the load limit less the safety margin.  Spreading the spans thin costs little (a
@@ -551,10 +552,9 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     }
 
     // ---- units ------------------------------------------------------------------------------
-    const bool tensor_ok = !(opts && (opts->flags & ASYNCLM_PLAN_NO_TENSOR_PATH)) &&
-                           tensor_path_compiled(shape->head_dim);
+    const bool tensor_ok = !(opts && (opts->flags & ASYNCLM_PLAN_NO_TENSOR_PATH));
     const int tensor_min_rows =
-        (opts && opts->tensor_min_rows > 0) ? opts->tensor_min_rows : default_tensor_min_rows(G);
+        (opts && opts->tensor_min_rows > 0) ? opts->tensor_min_rows : default_tensor_min_rows(shape->head_dim);
     const int TQ = tensor_tile_tokens(G);
     std::vector<UnitBuild> units;
     std::vector<int> ids_cuda, ids_tensor;

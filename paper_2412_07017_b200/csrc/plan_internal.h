@@ -15,9 +15,6 @@ constexpr int kCudaSlotsPerSm = 1;
 constexpr int kCudaItemOverheadTiles = 1;
 constexpr int kTensorItemOverheadTiles = 4;   // measured: an item boundary costs the tensor kernel about 4 tiles
 
-// True when the tensor-core attention kernel exists for this head_dim.
-bool tensor_path_compiled(int head_dim);
-
 int tensor_tile_tokens(int group);
 
 }  // namespace asynclm

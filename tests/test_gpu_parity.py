@@ -301,3 +301,43 @@ def test_sequences_that_share_prefix_pages():
             st.page_indices[st.page_indptr[0]:st.page_indptr[0] + shared]
     _, _, plan = run_and_check(wl, what="shared prefix pages", flags=B.PLAN_REJECT_ALIASED_WRITES)
     assert plan.info["num_items_tensor"] > 0
+
+
+@pytest.mark.parametrize("Hq,Hkv,ctx,ql", [
+    (32, 8, [700, 64, 0, 129], [64, 33, 64, 40]),
+    (32, 8, [1000], [200]),
+    (16, 2, [300, 55], [32, 17]),
+    (4, 4, [500, 20], [256, 130]),
+    (8, 2, [0, 16, 32, 48, 64, 65, 127, 193], [16, 16, 20, 31, 32, 40, 33, 64]),      # 1 .. 5 KV tiles, 1 .. 4 pages in the last
+])
+def test_spans_at_head_dim_64(Hq, Hkv, ctx, ql):
+    shape = W.Shape(Hq, Hkv, 64, 16)
+    wl = W.make_single_step("dim64", shape, ctx, ql, seed=640 + Hq + len(ctx), interleave_pages=True, poison_unused=True)
+    _, _, plan = run_and_check(wl, what=f"head_dim 64, {Hq}/{Hkv}")
+    assert plan.info["num_items_tensor"] == plan.info["num_items"]
+    run_and_check(wl, what="fixed chunks", kv_chunk_tokens=64)
+    wl = W.make_single_step("dim64", shape, ctx + [900, 40, 2000], ql + [1, 1, 1], seed=641 + Hq + len(ctx))
+    _, _, plan = run_and_check(wl, what="beside decode rows", num_sms=3)
+    assert 0 < plan.info["num_items_tensor"] < plan.info["num_items"]
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("ql", [17, 33])      # one row tile (the groups take alternate KV tiles), two
+def test_reference_maximum_moves_in_every_tile(d, ql):
+    """Scores that rise from tile to tile, over contexts of one to six KV tiles with full and ragged last
+    tiles: the accumulator is rescaled while the tensor core may still be adding an earlier tile to it."""
+    shape = W.Shape(8, 2, d, 16)
+    ctx = [0, 47, 48, 64, 111, 128, 175, 192, 200, 256, 300, 367]
+    wl = W.make_single_step("rising", shape, ctx, [ql] * len(ctx), seed=92)
+    st = wl.steps[0]
+    for b, c in enumerate(ctx):
+        alpha = (np.arange(c + ql, dtype=np.float32) / 64 * 12.0 - 20.0) / np.sqrt(d)
+        for pos in range(c):
+            pg = st.page_indices[st.page_indptr[b] + pos // 16]
+            wl.kv_pool[pg, 0, :, pos % 16, :] = W.f32_to_bf16_bits(np.full(d, alpha[pos], np.float32))
+        for i in range(ql):
+            st.k_new[st.q_indptr[b] + i] = W.f32_to_bf16_bits(np.full(d, alpha[c + i], np.float32))
+    st.q[:] = W.f32_to_bf16_bits(np.ones(d, np.float32))
+    _, _, plan = run_and_check(wl, what="rising scores", tensor_min_rows=1)
+    assert plan.info["num_items_tensor"] == plan.info["num_items"]
+    run_and_check(wl, what="rising scores, one CTA", tensor_min_rows=1, num_sms=1)

@@ -283,3 +283,12 @@ def test_host_workspace_must_be_16_byte_aligned():
                             None, ctypes.byref(out)) == 0
     assert lib.asynclm_plan(ctypes.byref(cs), ctypes.byref(co), ctypes.byref(cb), ok + 8, 1 << 16, None, 0,
                             None, ctypes.byref(out)) == -1
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("sms", [1, 2])
+def test_spans_beside_decode_rows_on_one_or_two_ctas(d, sms):
+    """A lone CTA holds the span work and the queue: there is no other CTA to stream the queue."""
+    wl = W.make_single_step("few", W.Shape(8, 2, d, 16), [0, 700, 33, 5], [40, 1, 90, 1], seed=2)
+    items = check_cover(wl, plan(wl, num_sms=sms))
+    assert {0, 1} == set(items["path"].tolist())
