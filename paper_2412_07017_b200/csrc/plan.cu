@@ -92,6 +92,16 @@ static size_t partial_bytes(int64_t rows, int group, int head_dim) {
 // kTailChunksPerCta per CTA and never shorter than kMinChunkTiles tiles (see deal_dynamic).
 constexpr int kTailChunksPerCta = 2;
 constexpr int kMinChunkTiles = 4;
+// The other units are cut into pieces of at most kBulkTiles tiles (70-110 us) or an eighth of a CTA's share: with
+// contexts of 10^5 tokens, pieces of two fifths of the step, which used to be the only limit, left some CTAs on
+// a last piece of half a millisecond.  32 and 128 tiles measure the same.
+constexpr int kBulkTiles = 64;
+// Span units of two row tiles are cut by keys instead of divided by rows where the pieces are at least this
+// long, because the divided halves each stream the keys: a 128-key tile takes a CTA 2.3 us for two row tiles
+// and 1.5 us for one, when all CTAs stream.  (8 sequences of 32-131 K tokens, two 256-token spans: 1080 us a
+// step with divided units, 887 with cut ones.)  Below, the partial rows and their merge cost more than they save
+// (32 sequences of up to 4 K tokens, 8 spans: 65 us divided, 72 cut).
+constexpr int kLongPieceTiles = 64;
 // Tokens of one warp-body unit: its MMAs have 8 (token, head) columns.
 static int warp_unit_tokens(int group) { return 8 / group; }
 
@@ -252,8 +262,12 @@ constexpr PathCost kWarpCost{128, 1050, 400, 2000};
 constexpr int64_t kDramBytesPerUs = 6000000;
 // A span CTA that finishes early joins the queue; one that finishes late delays the whole step, and the
 // span body slows down by up to 15 % when the warp-body CTAs saturate the memory.  So the span CTAs
-// are filled to the load limit divided by this margin (in 1/64).
-constexpr int64_t kSpanMargin64 = 72;
+// are filled to the load limit divided by this margin (in 1/64).  (128 sequences of 64 / 8 heads, 13 spans:
+// 524 us a step at 72, 495 at 80, 479 at 88, 482 at 96; smaller batches do not care.)
+constexpr int64_t kSpanMargin64 = 88;
+// The same, for the decision to divide a unit by rows: a unit just above the span CTAs' share is better cut by
+// the packing than divided, its halves would stream the keys twice.
+constexpr int64_t kDivideMargin64 = 72;
 // Share (in 1/64) of the queue that the CTAs without span work must be able to stream by themselves.
 constexpr int64_t kStreamShare64 = 58;
 constexpr int64_t kStartNs = 3000;
@@ -295,7 +309,7 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         int64_t work = warp_ns;
         for (int id : ids_tensor)
             work += tc.item_ns + tiles_of(units[id].n_keys, tc.gran) * (units[id].u.ntok * group > 128 ? dual_tile_ns : tc.tile_ns);
-        const int64_t limit0 = std::max(work / n_ctas, kStartNs + kv_bytes * 1000 / kDramBytesPerUs) * 64 / kSpanMargin64;
+        const int64_t limit0 = std::max(work / n_ctas, kStartNs + kv_bytes * 1000 / kDramBytesPerUs) * 64 / kDivideMargin64;
         const int half = 128 / group;      // tokens of one row tile
         const size_t n0 = ids_tensor.size();
         for (size_t i = 0; i < n0; ++i) {
@@ -303,6 +317,7 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
             UnitBuild& ub = units[(size_t)id];
             if (ub.u.ntok * group <= 128) continue;
             if (tc.phase_ns + tc.item_ns + tiles_of(ub.n_keys, tc.gran) * dual_tile_ns <= limit0) continue;
+            if (limit0 - tc.phase_ns - tc.item_ns >= kLongPieceTiles * dual_tile_ns) continue;      // cut by keys below
             UnitBuild second = ub;
             second.u.q_row0 += half;
             second.u.ntok -= half;
@@ -331,6 +346,8 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     // the queue.  With emit == false only the verdict is computed (the bisection's probes).
     int64_t span_work = 0;      // all span items without the per-CTA start
     for (int id : order) span_work += tc.item_ns + tiles[(size_t)id] * tns[(size_t)id];
+    const int64_t floor_ns = kStartNs + kv_bytes * 1000 / kDramBytesPerUs;
+    const int64_t bound = std::max<int64_t>(std::max<int64_t>(1, (warp_ns + span_work) / n_ctas), floor_ns);      // of the load limit
     auto fill = [&](int64_t limit, bool emit) {
         // CTAs that may hold span work: the others have to be able to stream most of the queue by
         // themselves (span CTAs draw little bandwidth, and one SM streams only so much)
@@ -343,7 +360,10 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         // packing, at most the load limit less the safety margin.  Spreading the spans thin costs little (a
         // span CTA that is done early joins the queue), filling span CTAs to the brim risks a late finish.
         const int64_t thin = order.empty() ? 0 : span_work / span_ctas * 5 / 4 + tc.phase_ns + tc.item_ns + dual_tile_ns;
-        const int64_t cap = std::min(limit * 64 / kSpanMargin64, std::max(thin, 2 * (tc.phase_ns + tc.item_ns)));
+        // (Past twice the lower bound the spread is given up: items of more than half of `thin` take a CTA each,
+        // and there may be more of them than CTAs.)
+        const int64_t full = limit * 64 / kSpanMargin64;
+        const int64_t cap = limit > 2 * bound ? full : std::min(full, std::max(thin, 2 * (tc.phase_ns + tc.item_ns)));
         pieces_out.clear();
         std::fill(load.begin(), load.end(), (int64_t)0);
         used = 0;
@@ -386,9 +406,7 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
             room += std::max<int64_t>(0, limit - load[(size_t)k] - kWarpCost.phase_ns);
         return fits && used <= span_ctas && room >= warp_ns;
     };
-    const int64_t total = warp_ns + span_work;
-    const int64_t floor_ns = kStartNs + kv_bytes * 1000 / kDramBytesPerUs;
-    int64_t lo = std::max<int64_t>(std::max<int64_t>(1, total / n_ctas), floor_ns);
+    int64_t lo = bound;
     int64_t hi = lo + lo / 4 + tc.item_ns + tc.phase_ns + kWarpCost.phase_ns;
     while (!fill(hi, false)) { lo = hi; hi += hi / 2; }
     for (int iter = 0; iter < 24 && hi - lo > std::max<int64_t>(50, hi / 128); ++iter) {      // to 0.8 %
@@ -408,7 +426,8 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
                      [&](int x, int y) { return units[x].n_keys > units[y].n_keys; });
     std::vector<Item> chunks, tail;
     chunks.reserve(ids_warp.size() + (size_t)n_ctas * 4);
-    const int64_t bulk_max = std::max<int64_t>(kMinChunkTiles, hi * 2 / 5 / kWarpCost.tile_ns);
+    const int64_t bulk_max = std::max<int64_t>(kMinChunkTiles, std::min<int64_t>(hi * 2 / 5 / kWarpCost.tile_ns,
+                                                                              std::max<int64_t>(kBulkTiles, warp_tiles / (8 * (int64_t)n_ctas))));
     const int64_t tail_target = warp_tiles / 6;
     const int64_t tail_chunk = std::max<int64_t>(kMinChunkTiles, tail_target / ((int64_t)n_ctas * kTailChunksPerCta));
     // which units are cut short: first those of up to four chunks (their merge is one round trip to

@@ -292,3 +292,38 @@ def test_spans_beside_decode_rows_on_one_or_two_ctas(d, sms):
     wl = W.make_single_step("few", W.Shape(8, 2, d, 16), [0, 700, 33, 5], [40, 1, 90, 1], seed=2)
     items = check_cover(wl, plan(wl, num_sms=sms))
     assert {0, 1} == set(items["path"].tolist())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_more_long_span_units_than_ctas_beside_a_decode_row(d):
+    """200 equal span units that fill most of a CTA each, and a decode row: they do not fit under a load
+    limit spread evenly over the CTAs, so the planner has to give that spread up."""
+    n = 26
+    ctx, ql = np.full(n, 5000), np.full(n, 64)
+    ql[-1] = 1
+    need = -(-(ctx + ql) // 16)
+    q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+    p = B.plan_host(W.Shape(32, 8, d, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=148)
+    items = p.items()
+    span = items[items["path"] == 1]
+    assert len(span) >= 200 and span["cta"].max() < 148 and (items["path"] == 0).sum() >= 8
+
+
+def test_long_decode_units_are_cut_into_many_pieces():
+    """Contexts of 10^5 tokens beside long spans: no piece of the queue is longer than 64 tiles (or an eighth of a
+    CTA's share), and the partial rows stay within the workspace that the size call reports."""
+    ctx, ql = np.array([120000, 60000, 110000, 90000]), np.array([256, 1, 1, 1])
+    need = -(-(ctx + ql) // 16)
+    q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+    shape = W.Shape(32, 8, 128, 16)
+    for sms in (148, 8, 1):
+        p = B.plan_host(shape, int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
+        items = p.items()
+        dec = items[items["path"] == 0]
+        tiles = -(-(dec["kv1"] - dec["kv0"]) // 128)
+        assert tiles.max() <= 1.5 * max(64, tiles.sum() // (8 * sms))
+        host_bytes, dev_bytes = B.workspace_size(shape, int(need.sum()), 4, int(ql.sum()), int(need.sum()), num_sms=sms)
+        assert p.info["device_bytes_used"] <= dev_bytes and p.info["host_bytes_used"] <= host_bytes
+        for b in (1, 2, 3):
+            segs = sorted((int(a), int(c)) for a, c, s, h in zip(dec["kv0"], dec["kv1"], dec["seq"], dec["kv_head"]) if s == b and h == 3)
+            assert segs[0][0] == 0 and segs[-1][1] == ctx[b] + 1 and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
