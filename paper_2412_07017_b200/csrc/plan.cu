@@ -272,6 +272,14 @@ constexpr int64_t kDivideMargin64 = 72;
 constexpr int64_t kStreamShare64 = 58;
 constexpr int64_t kStartNs = 3000;
 
+// How span units and long decode units are cut.  The default is the fastest; asynclm_plan asks for fewer cuts
+// where the partial results would outgrow the fixed array of asynclm_attn_mixed_static.
+struct CutPolicy {
+    int64_t span_margin64 = kSpanMargin64;
+    int units_by_keys = INT_MAX;      // long span units (kLongPieceTiles) that may be cut by keys, the longest first
+    bool bound_pieces = true;         // kBulkTiles
+};
+
 // Default policy for the fused kernel.
 //   Span units (tensor-core body) are compute-heavy and predictable: they are packed whole onto as few
 // persistent CTAs as the load limit allows (largest first, each into the fullest CTA that still has
@@ -286,7 +294,8 @@ constexpr int64_t kStartNs = 3000;
 //   The load limit is the smallest one under which the span units fit and the room left on all CTAs
 // covers the modelled time of the queue; it is found by bisection.
 void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp,
-                  std::vector<UnitBuild>& units, int group, int64_t kv_bytes, int n_ctas, std::vector<Item>& items,
+                  std::vector<UnitBuild>& units, int group, int64_t kv_bytes, int n_ctas, const CutPolicy& policy,
+                  std::vector<Item>& items,
                   std::vector<int32_t>& cta_indptr_warp, std::vector<int32_t>& cta_indptr_tensor,
                   std::vector<int32_t>& item_cta, int32_t* queue_first, int32_t* queue_count) {
     struct Piece { Item it; int32_t cta; };
@@ -311,13 +320,24 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
             work += tc.item_ns + tiles_of(units[id].n_keys, tc.gran) * (units[id].u.ntok * group > 128 ? dual_tile_ns : tc.tile_ns);
         const int64_t limit0 = std::max(work / n_ctas, kStartNs + kv_bytes * 1000 / kDramBytesPerUs) * 64 / kDivideMargin64;
         const int half = 128 / group;      // tokens of one row tile
+        // which of them are left to be cut by keys (below): the longest, because a divided half stays whole and would
+        // be a CTA's longest item
+        std::vector<char> by_keys;
+        if (policy.units_by_keys > 0 && limit0 - tc.phase_ns - tc.item_ns >= kLongPieceTiles * dual_tile_ns) {
+            std::vector<int> longest(ids_tensor);
+            std::stable_sort(longest.begin(), longest.end(), [&](int x, int y) { return units[x].n_keys > units[y].n_keys; });
+            by_keys.assign(units.size(), 0);
+            int n = 0;
+            for (int id : longest)
+                if (units[(size_t)id].u.ntok * group > 128 && n < policy.units_by_keys) by_keys[(size_t)id] = 1, ++n;
+        }
         const size_t n0 = ids_tensor.size();
         for (size_t i = 0; i < n0; ++i) {
             const int id = ids_tensor[i];
             UnitBuild& ub = units[(size_t)id];
             if (ub.u.ntok * group <= 128) continue;
             if (tc.phase_ns + tc.item_ns + tiles_of(ub.n_keys, tc.gran) * dual_tile_ns <= limit0) continue;
-            if (limit0 - tc.phase_ns - tc.item_ns >= kLongPieceTiles * dual_tile_ns) continue;      // cut by keys below
+            if (!by_keys.empty() && by_keys[(size_t)id]) continue;
             UnitBuild second = ub;
             second.u.q_row0 += half;
             second.u.ntok -= half;
@@ -362,7 +382,7 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         const int64_t thin = order.empty() ? 0 : span_work / span_ctas * 5 / 4 + tc.phase_ns + tc.item_ns + dual_tile_ns;
         // (Past twice the lower bound the spread is given up: items of more than half of `thin` take a CTA each,
         // and there may be more of them than CTAs.)
-        const int64_t full = limit * 64 / kSpanMargin64;
+        const int64_t full = limit * 64 / policy.span_margin64;
         const int64_t cap = limit > 2 * bound ? full : std::min(full, std::max(thin, 2 * (tc.phase_ns + tc.item_ns)));
         pieces_out.clear();
         std::fill(load.begin(), load.end(), (int64_t)0);
@@ -426,8 +446,9 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
                      [&](int x, int y) { return units[x].n_keys > units[y].n_keys; });
     std::vector<Item> chunks, tail;
     chunks.reserve(ids_warp.size() + (size_t)n_ctas * 4);
-    const int64_t bulk_max = std::max<int64_t>(kMinChunkTiles, std::min<int64_t>(hi * 2 / 5 / kWarpCost.tile_ns,
-                                                                              std::max<int64_t>(kBulkTiles, warp_tiles / (8 * (int64_t)n_ctas))));
+    int64_t bulk_max = hi * 2 / 5 / kWarpCost.tile_ns;
+    if (policy.bound_pieces) bulk_max = std::min(bulk_max, std::max<int64_t>(kBulkTiles, warp_tiles / (8 * (int64_t)n_ctas)));
+    bulk_max = std::max<int64_t>(bulk_max, kMinChunkTiles);
     const int64_t tail_target = warp_tiles / 6;
     const int64_t tail_chunk = std::max<int64_t>(kMinChunkTiles, tail_target / ((int64_t)n_ctas * kTailChunksPerCta));
     // which units are cut short: first those of up to four chunks (their merge is one round trip to
@@ -571,76 +592,109 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     }
 
     // ---- units ------------------------------------------------------------------------------
-    const bool tensor_ok = !(opts && (opts->flags & ASYNCLM_PLAN_NO_TENSOR_PATH));
+    const bool tensor_wanted = !(opts && (opts->flags & ASYNCLM_PLAN_NO_TENSOR_PATH));
     const int tensor_min_rows =
         (opts && opts->tensor_min_rows > 0) ? opts->tensor_min_rows : default_tensor_min_rows(shape->head_dim);
     const int TQ = tensor_tile_tokens(G);
-    std::vector<UnitBuild> units;
-    std::vector<int> ids_cuda, ids_tensor;
-    for (int b = 0; b < B; ++b) {
-        const int ql = q_indptr[b + 1] - q_indptr[b];
-        if (ql == 0) continue;
-        const int ctx = batch->kv_len_before[b];
-        const bool tensor = tensor_ok && (int64_t)G * ql >= tensor_min_rows;
-        const int step = tensor ? TQ : warp_unit_tokens(G);
-        for (int h = 0; h < Hkv; ++h) {
-            for (int t0 = 0; t0 < ql; t0 += step) {
-                UnitBuild ub{};
-                ub.u.seq = b;
-                ub.u.kv_head = h;
-                ub.u.q_row0 = q_indptr[b] + t0;
-                ub.u.ntok = std::min(step, ql - t0);
-                ub.u.kv_limit0 = ctx + t0 + 1;
-                ub.u.n_chunks = 0;
-                ub.u.partial_base = -1;
-                ub.u.page_base = page_indptr[b];
-                ub.path = tensor ? kPathTensor : kPathCuda;
-                ub.n_keys = (int64_t)ub.u.kv_limit0 + ub.u.ntok - 1;
-                (tensor ? ids_tensor : ids_cuda).push_back((int)units.size());
-                units.push_back(ub);
-            }
-        }
-    }
-
-    // ---- items and CTA assignment --------------------------------------------------------------
     const int fixed_chunk = opts ? opts->kv_chunk_tokens : 0;
     const int ctas_cuda = n_sms * kCudaSlotsPerSm;
     const int ctas_tensor = n_sms;
+    std::vector<UnitBuild> units;
+    std::vector<int> ids_cuda, ids_tensor;
     std::vector<Item> items;
     std::vector<int32_t> item_cta, cta_indptr_cuda, cta_indptr_tensor;
     int n_items_cuda = 0;
     int32_t queue_first = 0, queue_count = 0;
-    if (fixed_chunk > 0 || ctas_cuda != ctas_tensor) {
-        cut_and_deal(ids_cuda, units, fixed_chunk, ctas_cuda, kCudaItemOverheadTiles, items,
-                     cta_indptr_cuda, item_cta);
-        n_items_cuda = (int)items.size();
-        cut_and_deal(ids_tensor, units, fixed_chunk, ctas_tensor, kTensorItemOverheadTiles, items,
-                     cta_indptr_tensor, item_cta);
-    } else {
-        // bytes of K and V the step has to read, each (sequence, kv head) counted once
-        const int64_t kv_bytes = total_kv * Hkv * 4 * shape->head_dim;
-        deal_dynamic(ids_tensor, ids_cuda, units, G, kv_bytes, ctas_cuda, items, cta_indptr_cuda, cta_indptr_tensor, item_cta,
-                     &queue_first, &queue_count);
-        n_items_cuda = queue_first + queue_count;
-    }
-    const int n_items = (int)items.size();
-
-    // ---- partial rows ------------------------------------------------------------------------
     std::vector<int32_t> split_units, merge_blocks;   // merge block: 4 (token, head) rows of a split unit
     int64_t partial_rows = 0;
-    for (size_t i = 0; i < units.size(); ++i) {
-        if (units[i].u.n_chunks > 1) {
-            units[i].u.partial_base = (int32_t)partial_rows;
-            partial_rows += (int64_t)units[i].u.n_chunks * units[i].u.ntok;
-            split_units.push_back((int32_t)i);
-            if (i >= (size_t)(INT32_MAX >> 6)) return ASYNCLM_ERR_WORKSPACE_TOO_SMALL;
-            // split units of the warp body are merged inside the attention kernel; those of the span
-            // body by the merge kernel
-            if (units[i].path == kPathTensor)
-                for (int rb = 0; rb * 4 < units[i].u.ntok * G; ++rb) merge_blocks.push_back((int32_t)((i << 6) | (size_t)rb));
-            if (partial_rows > INT32_MAX / 2) return ASYNCLM_ERR_WORKSPACE_TOO_SMALL;
+    auto deal = [&](const CutPolicy& policy, bool tensor_on) -> int {
+        units.clear(); ids_cuda.clear(); ids_tensor.clear(); items.clear(); item_cta.clear();
+        split_units.clear(); merge_blocks.clear();
+        n_items_cuda = queue_first = queue_count = 0;
+        partial_rows = 0;
+        for (int b = 0; b < B; ++b) {
+            const int ql = q_indptr[b + 1] - q_indptr[b];
+            if (ql == 0) continue;
+            const int ctx = batch->kv_len_before[b];
+            const bool tensor = tensor_on && (int64_t)G * ql >= tensor_min_rows;
+            const int step = tensor ? TQ : warp_unit_tokens(G);
+            for (int h = 0; h < Hkv; ++h) {
+                for (int t0 = 0; t0 < ql; t0 += step) {
+                    UnitBuild ub{};
+                    ub.u.seq = b;
+                    ub.u.kv_head = h;
+                    ub.u.q_row0 = q_indptr[b] + t0;
+                    ub.u.ntok = std::min(step, ql - t0);
+                    ub.u.kv_limit0 = ctx + t0 + 1;
+                    ub.u.n_chunks = 0;
+                    ub.u.partial_base = -1;
+                    ub.u.page_base = page_indptr[b];
+                    ub.path = tensor ? kPathTensor : kPathCuda;
+                    ub.n_keys = (int64_t)ub.u.kv_limit0 + ub.u.ntok - 1;
+                    (tensor ? ids_tensor : ids_cuda).push_back((int)units.size());
+                    units.push_back(ub);
+                }
+            }
         }
+
+        // ---- items and CTA assignment --------------------------------------------------------------
+        if (fixed_chunk > 0 || ctas_cuda != ctas_tensor) {
+            cut_and_deal(ids_cuda, units, fixed_chunk, ctas_cuda, kCudaItemOverheadTiles, items,
+                         cta_indptr_cuda, item_cta);
+            n_items_cuda = (int)items.size();
+            cut_and_deal(ids_tensor, units, fixed_chunk, ctas_tensor, kTensorItemOverheadTiles, items,
+                         cta_indptr_tensor, item_cta);
+        } else {
+            // bytes of K and V the step has to read, each (sequence, kv head) counted once
+            const int64_t kv_bytes = total_kv * Hkv * 4 * shape->head_dim;
+            deal_dynamic(ids_tensor, ids_cuda, units, G, kv_bytes, ctas_cuda, policy, items, cta_indptr_cuda, cta_indptr_tensor, item_cta,
+                         &queue_first, &queue_count);
+            n_items_cuda = queue_first + queue_count;
+        }
+
+        // ---- partial rows ------------------------------------------------------------------------
+        for (size_t i = 0; i < units.size(); ++i) {
+            if (units[i].u.n_chunks > 1) {
+                units[i].u.partial_base = (int32_t)partial_rows;
+                partial_rows += (int64_t)units[i].u.n_chunks * units[i].u.ntok;
+                split_units.push_back((int32_t)i);
+                if (i >= (size_t)(INT32_MAX >> 6)) return ASYNCLM_ERR_WORKSPACE_TOO_SMALL;
+                // split units of the warp body are merged inside the attention kernel; those of the span
+                // body by the merge kernel
+                if (units[i].path == kPathTensor)
+                    for (int rb = 0; rb * 4 < units[i].u.ntok * G; ++rb) merge_blocks.push_back((int32_t)((i << 6) | (size_t)rb));
+                if (partial_rows > INT32_MAX / 2) return ASYNCLM_ERR_WORKSPACE_TOO_SMALL;
+            }
+        }
+        return ASYNCLM_OK;
+    };
+    // The fastest cuts, as long as their partial results fit the fixed array of asynclm_attn_mixed_static; else as
+    // many of the long span units cut by keys as it has room for, none of them, long pieces in the queue as
+    // well, and at head_dim 64 no span units at all (warp units have far fewer partial rows).  If nothing fits,
+    // the fastest again: that call then refuses the plan.
+    auto fits_static = [&]() { return partial_bytes(partial_rows, G, shape->head_dim) <= ASYNCLM_STATIC_SCRATCH_BYTES; };
+    const CutPolicy fastest;
+    rc = deal(fastest, tensor_wanted);
+    if (rc == ASYNCLM_OK && !fits_static()) {
+        if (fixed_chunk == 0) {
+            int64_t span_rows = 0, span_units = 0;
+            for (int id : split_units)
+                if (units[(size_t)id].path == kPathTensor) {
+                    span_rows += (int64_t)units[(size_t)id].u.n_chunks * units[(size_t)id].u.ntok;
+                    ++span_units;
+                }
+            const int64_t room = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float))) - (partial_rows - span_rows);
+            CutPolicy fewer;
+            fewer.units_by_keys = room <= 0 ? 0 : (int)(span_units * room / std::max<int64_t>(1, span_rows) * 15 / 16);
+            if (fewer.units_by_keys > 0) rc = deal(fewer, tensor_wanted);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, true}, tensor_wanted);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, false}, tensor_wanted);
+        }
+        if (rc == ASYNCLM_OK && !fits_static() && tensor_wanted && shape->head_dim == 64) rc = deal(CutPolicy{kDivideMargin64, 0, false}, false);
+        if (rc == ASYNCLM_OK && !fits_static()) rc = deal(fastest, tensor_wanted);
     }
+    if (rc != ASYNCLM_OK) return rc;
+    const int n_items = (int)items.size();
 
     const int n_split = (int)split_units.size();
 

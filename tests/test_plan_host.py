@@ -327,3 +327,20 @@ def test_long_decode_units_are_cut_into_many_pieces():
         for b in (1, 2, 3):
             segs = sorted((int(a), int(c)) for a, c, s, h in zip(dec["kv0"], dec["kv1"], dec["seq"], dec["kv_head"]) if s == b and h == 3)
             assert segs[0][0] == 0 and segs[-1][1] == ctx[b] + 1 and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
+
+
+@pytest.mark.parametrize("d,ctx,ql", [
+    (128, [131072, 98000, 65000, 60000, 50000, 40000, 33000, 70000], [256, 256, 1, 1, 1, 1, 1, 1]),
+    (128, [120000] * 4, [1000, 1000, 1, 1]),
+    (64, [120000] * 4, [1000, 1000, 1, 1]),
+    (64, [120000] * 6, [256] * 6),
+])
+def test_long_cuts_stay_within_the_fixed_scratch_array(d, ctx, ql):
+    """Partial results of a plan fit asynclm_attn_mixed_static's array wherever fewer cuts make them fit."""
+    ctx, ql = np.array(ctx), np.array(ql)
+    need = -(-(ctx + ql) // 16)
+    q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+    p = B.plan_host(W.Shape(32, 8, d, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=148)
+    rows = p.info["partial_rows"]
+    up = lambda x: -(-x // 256) * 256
+    assert up(rows * 4 * d * 4) + up(rows * 4 * 4) <= B.static_scratch_bytes()
