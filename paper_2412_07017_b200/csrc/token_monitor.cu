@@ -148,14 +148,17 @@ __device__ __forceinline__ Best block_best(Best best, float* sv, int* si) {
 // Grid: (slices, batch).  Every CTA scans one slice of a sequence's row and folds its best ordinary token
 // into the row's key with one atomic max; the CTA that arrives last (per-row counter) lets the CML tokens
 // that the state allows compete, advances the state machine and puts the two workspace words back to zero.
+// The CTAs of a row in the TRAP state read no logits but arrive all the same: state_out may be state_in, so
+// nothing is written before every slice of the row has read the state (a CTA arrives behind a block-wide
+// barrier, and the two state pointers are not __restrict__).
 // The result does not depend on arrival order.  (Scanning all tokens alike and looking at a row a second
 // time when a forbidden token had won kept one CTA busy with a whole row after all others had left:
 // 256 rows of 128 256 bf16 with a few such rows took 31 us a call, 21 us now.)
 template <typename T>
 __global__ void __launch_bounds__(kMonThreads)
 token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, asynclm_cml_tokens tok,
-                     const int32_t* __restrict__ state_in, int32_t* __restrict__ token_out,
-                     int32_t* __restrict__ state_out, int32_t* __restrict__ flags_out,
+                     const int32_t* state_in, int32_t* __restrict__ token_out,
+                     int32_t* state_out, int32_t* __restrict__ flags_out,
                      unsigned long long* __restrict__ ws) {
     constexpr int VEC = Vec<T>::N;
     __shared__ float sv[kMonThreads / 32];
@@ -163,31 +166,27 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
     const int seq = blockIdx.y;
     const T* row = logits + (int64_t)seq * row_stride;
     const int state = state_in[seq];
-    if (state == kTrap) {
-        // [TRAP] is followed by [END] whatever the logits say: nothing to read
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            token_out[seq] = tok.end;
-            state_out[seq] = kText;
-            flags_out[seq] = ASYNCLM_MONITOR_TRAP;
-        }
-        return;
-    }
     // the CML tokens this state allows (INT_MAX: none) and their logits, for the thread that may finish the row
     const int spec0 = state == kText ? tok.call : tok.end, spec1 = state == kText ? tok.trap : state == kCall ? tok.head : INT_MAX;
     float spec_v0 = 0.f, spec_v1 = 0.f;
-    if (threadIdx.x == 0) {
-        spec_v0 = to_f32<T>(row[spec0]);
-        if (spec1 != INT_MAX) spec_v1 = to_f32<T>(row[spec1]);
-    }
-    const int nvec = vocab / VEC;
-    const int per = (nvec + gridDim.x - 1) / gridDim.x;
-    Best best = scan_row<T>(row, blockIdx.x * per, min(nvec, (int)(blockIdx.x + 1) * per), tok);
-    if (blockIdx.x == gridDim.x - 1)      // the row's ragged end, element by element
-        for (int i = nvec * VEC + threadIdx.x; i < vocab; i += kMonThreads) {
-            const float v = to_f32<T>(row[i]);
-            if (!is_special(i, tok) && better(v, i, best)) best = Best{v, i};
+    Best best{-INFINITY, INT_MAX};
+    if (state != kTrap) {
+        if (threadIdx.x == 0) {
+            spec_v0 = to_f32<T>(row[spec0]);
+            if (spec1 != INT_MAX) spec_v1 = to_f32<T>(row[spec1]);
         }
-    best = block_best(best, sv, si);
+        const int nvec = vocab / VEC;
+        const int per = (nvec + gridDim.x - 1) / gridDim.x;
+        best = scan_row<T>(row, blockIdx.x * per, min(nvec, (int)(blockIdx.x + 1) * per), tok);
+        if (blockIdx.x == gridDim.x - 1)      // the row's ragged end, element by element
+            for (int i = nvec * VEC + threadIdx.x; i < vocab; i += kMonThreads) {
+                const float v = to_f32<T>(row[i]);
+                if (!is_special(i, tok) && better(v, i, best)) best = Best{v, i};
+            }
+        best = block_best(best, sv, si);
+    } else {
+        __syncthreads();      // every thread has read the state
+    }
     if (threadIdx.x != 0) return;
     if (gridDim.x > 1) {
         unsigned long long* key = ws + 2 * (size_t)seq;
@@ -198,6 +197,13 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
         __threadfence();
         best = unpack_key(atomicExch(key, 0ull));
         *arrived = 0;
+    }
+    if (state == kTrap) {
+        // [TRAP] is followed by [END] whatever the logits say
+        token_out[seq] = tok.end;
+        state_out[seq] = kText;
+        flags_out[seq] = ASYNCLM_MONITOR_TRAP;
+        return;
     }
     if (better(spec_v0, spec0, best)) best = Best{spec_v0, spec0};
     if (spec1 != INT_MAX && better(spec_v1, spec1, best)) best = Best{spec_v1, spec1};

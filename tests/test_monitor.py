@@ -118,3 +118,31 @@ def test_cml_tokens_at_the_edges_of_the_scan(Bsz, vocab, bf16):
         tok, nxt, fl = run(bits, states, special, bf16)
         rt, rn, rf = M.step(vals, states, special)
         assert np.array_equal(tok, rt) and np.array_equal(nxt, rn) and np.array_equal(fl, rf), name
+
+
+@pytest.mark.parametrize("Bsz,vocab,bf16", [(4, 128256, True), (16, 32000, False), (40, 128256, True), (300, 4099, False)])
+def test_states_advanced_in_place(Bsz, vocab, bf16):
+    """state_out is state_in, over several steps, most rows in the TRAP state at some of them, rows of one and of
+    many slices: no slice of a row may see the state that another has already written, and every step leaves
+    the workspace zero."""
+    import torch
+    special = {"CALL": 11, "INTR": 700, "TRAP": 1500, "END": 1501, "HEAD": vocab - 1}
+    g = np.random.default_rng(Bsz)
+    vals32 = g.normal(size=(Bsz, vocab)).astype(np.float32)
+    wants_trap = g.random(Bsz) < 0.8
+    vals32[wants_trap, special["TRAP"]] = 30.0      # TEXT -> TRAP -> TEXT -> TRAP ...
+    vals32[~wants_trap, special["CALL"]] = 30.0     # TEXT -> CALL, and there an ordinary token
+    stride = -(-vocab // 8) * 8
+    full = torch.zeros((Bsz, stride), dtype=torch.bfloat16 if bf16 else torch.float32, device="cuda")
+    full[:, :vocab] = torch.from_numpy(vals32).cuda().to(full.dtype)
+    vals = full[:, :vocab].float().cpu().numpy().astype(np.float64)
+    states = np.where(np.arange(Bsz) % 3 == 0, 3, 0).astype(np.int32)
+    st = torch.from_numpy(states).cuda()
+    tok, fl = torch.full_like(st, -7), torch.full_like(st, -7)
+    ws = torch.zeros(B.token_monitor_workspace_bytes(Bsz), dtype=torch.uint8, device="cuda")
+    for _ in range(6):
+        B.asynclm_token_monitor_step(full[:, :vocab], special, st, tok, st, fl, ws)
+        torch.cuda.synchronize()
+        rt, states, rf = M.step(vals, states, special)
+        assert int(ws.max()) == 0
+        assert np.array_equal(tok.cpu().numpy(), rt) and np.array_equal(st.cpu().numpy(), states) and np.array_equal(fl.cpu().numpy(), rf)
