@@ -167,12 +167,13 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
     const T* row = logits + (int64_t)seq * row_stride;
     const int state = state_in[seq];
     // the CML tokens this state allows (INT_MAX: none) and their logits, for the thread that may finish the row
-    const int spec0 = state == kText ? tok.call : tok.end, spec1 = state == kText ? tok.trap : state == kCall ? tok.head : INT_MAX;
+    const int spec0 = state == kText ? tok.call : state == kCall || state == kBody ? tok.end : INT_MAX;
+    const int spec1 = state == kText ? tok.trap : state == kCall ? tok.head : INT_MAX;
     float spec_v0 = 0.f, spec_v1 = 0.f;
     Best best{-INFINITY, INT_MAX};
     if (state != kTrap) {
         if (threadIdx.x == 0) {
-            spec_v0 = to_f32<T>(row[spec0]);
+            if (spec0 != INT_MAX) spec_v0 = to_f32<T>(row[spec0]);
             if (spec1 != INT_MAX) spec_v1 = to_f32<T>(row[spec1]);
         }
         const int nvec = vocab / VEC;
@@ -205,7 +206,7 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
         flags_out[seq] = ASYNCLM_MONITOR_TRAP;
         return;
     }
-    if (better(spec_v0, spec0, best)) best = Best{spec_v0, spec0};
+    if (spec0 != INT_MAX && better(spec_v0, spec0, best)) best = Best{spec_v0, spec0};
     if (spec1 != INT_MAX && better(spec_v1, spec1, best)) best = Best{spec_v1, spec1};
     Best pick = best;
     if (pick.i == INT_MAX || pick.v == -INFINITY) {

@@ -146,3 +146,16 @@ def test_states_advanced_in_place(Bsz, vocab, bf16):
         rt, states, rf = M.step(vals, states, special)
         assert int(ws.max()) == 0
         assert np.array_equal(tok.cpu().numpy(), rt) and np.array_equal(st.cpu().numpy(), states) and np.array_equal(fl.cpu().numpy(), rf)
+
+
+def test_a_state_outside_the_grammar_allows_ordinary_tokens_only():
+    """Such a state is not one of the four; it keeps its value and no CML token is chosen in it."""
+    special = {"CALL": 3, "INTR": 4, "TRAP": 5, "END": 6, "HEAD": 7}
+    vals = np.random.default_rng(1).normal(size=(6, 20011)).astype(np.float32)
+    vals[:, 3:8] = 40.0
+    vals[4:, [0, 1, 2]] = np.nan
+    vals[4:, 8:] = -np.inf
+    states = np.array([4, 7, -1, 2, 4, -9])
+    tok, nxt, fl = run(vals, states, special, False)
+    rt, rn, rf = M.step(vals.astype(np.float64), states, special)
+    assert np.array_equal(tok, rt) and np.array_equal(nxt, rn) and np.array_equal(fl, rf)
