@@ -24,8 +24,8 @@
 //                   shared memory, so that every global store writes whole 128-byte lines.
 //   warps 8, 10     producers of K tiles and of V tiles: 16-byte cp.async copies (fully coalesced,
 //                   whole rows, 512 bytes per warp instruction) that write the 128-byte-swizzled operand
-//                   layout and complete on the slot's mbarrier.  K and V share one ring of 160 KiB, filled
-//                   in the order the tensor core consumes the tiles (see ring_pos_k).  For asynclm_step
+//                   layout and complete on the slot's mbarrier.  K and V have a ring of 80 KiB each
+//                   (see span_ring.h).  For asynclm_step
 //                   the K warp also puts an item's new K/V rows into their page slots, before the first
 //                   tile that holds one.
 //   warps 9, 11     issue the MMAs, one warp per softmax group.  Warp 9 owns the tensor-memory allocation.
@@ -45,6 +45,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "span_ring.h"
 
 namespace asynclm {
 
@@ -66,17 +67,17 @@ struct Geometry {
     static constexpr uint32_t QTILE_BYTES = HALVES * QHALF_BYTES;
     static constexpr uint32_t HALF_BYTES = kTile * 128;                    // one 64-value half of a K or V tile
     static constexpr uint32_t SLOT_BYTES = HALVES * HALF_BYTES;
-    static constexpr int RING = 20 / HALVES;                               // K/V ring slots: 160 KiB
+    static constexpr int RING = ring_slots(D);                             // slots of the K ring and of the V ring
     static constexpr uint32_t OFF_Q = 0;                                   // Q[0], Q[1]
     static constexpr uint32_t OFF_RING = OFF_Q + 2 * QTILE_BYTES;
     // The barriers lie behind everything the warp body uses when the CTA goes on to it: arrivals that nobody
     // waits for (an item's last on kOFree and on the ring's empty barriers) may still be queued in the shared
     // memory pipe then, and would change whatever has been copied there since.
     static constexpr uint32_t OFF_BAR = 224 * 1024;
-    static_assert(OFF_RING + RING * SLOT_BYTES <= OFF_BAR, "barriers behind the tiles");
+    static_assert(OFF_RING + 2 * RING * SLOT_BYTES <= OFF_BAR, "barriers behind the tiles");
     // S, P and last-P-V hand-offs exist per group b and buffer s: index 2 * b + s
     enum Bar { kQFull = 0, kStats, kOFree, kPFull0, kPvDone0 = kPFull0 + 4, kSFull0 = kPvDone0 + 4,
-               kRingFull0 = kSFull0 + 4, kRingEmpty0 = kRingFull0 + RING, kMmaDrain = kRingEmpty0 + RING, kNumBars };
+               kRingFull0 = kSFull0 + 4, kRingEmpty0 = kRingFull0 + 2 * RING, kMmaDrain = kRingEmpty0 + 2 * RING, kNumBars };
     static constexpr uint32_t OFF_TMEM_PTR = OFF_BAR + 8 * kNumBars;
     static constexpr uint32_t OFF_ABORT = OFF_TMEM_PTR + 8;
     static constexpr uint32_t OFF_APPENDED = OFF_ABORT + 8;      // items of this CTA whose new K/V rows are in the pool
@@ -88,12 +89,6 @@ struct Geometry {
 constexpr uint32_t kColS = 0;      // S[b][s]: 64 columns each at 128 b + 64 s; P[b][s] overlays the first 32 of S[b][s]
 constexpr uint32_t kColO = 256;    // O[b]: head_dim columns each
 constexpr uint32_t kTmemCols = 512;
-
-// Ring positions, relative to the item's first slot, of the K tile and of the V tile of its g-th KV tile
-// (of n): the order in which the tensor core consumes them.  The first `lead` K tiles go ahead, then a V
-// tile and the K tile `lead` further take turns: K0 K1 V0 K2 V1 K3 ... for a lead of two.
-__device__ __forceinline__ int ring_pos_k(int g, int lead) { return g < lead ? g : 2 * g - lead + 1; }
-__device__ __forceinline__ int ring_pos_v(int g, int n, int lead) { return g + min(n, g + lead); }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
@@ -321,7 +316,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             mbar_init(bar(Geo::kPvDone0 + b), 1);
             mbar_init(bar(Geo::kSFull0 + b), 1);
         }
-        for (int s = 0; s < Geo::RING; ++s) { mbar_init(bar(Geo::kRingFull0 + s), 32); mbar_init(bar(Geo::kRingEmpty0 + s), 2); }
+        for (int s = 0; s < 2 * Geo::RING; ++s) { mbar_init(bar(Geo::kRingFull0 + s), 32); mbar_init(bar(Geo::kRingEmpty0 + s), 2); }
         mbar_init(bar(Geo::kMmaDrain), 2);
         *abort_flag = 0;
         *appended = 0;
@@ -352,9 +347,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         constexpr int kGroupTiles = 32 / kPagesPerTile;       // 8
         constexpr int kChunks = D / 8, kRowsPerOp = 32 / kChunks;      // 16-byte chunks of a row; rows a warp instruction moves
         bool ok = true;
-        int n = 0;                                             // KV tiles issued so far (all items)
-        int base = 0;                                          // ring position of the item's first slot
-        int last_pos = -1;
+        int n = 0;                                             // tiles issued so far (all items)
         int ev = 0;      // time-stamp build: event log position (lane 0 of a producer)
         TItem cur = load_titem(head_work, i0 < i1), nxt = load_titem(p.works + i0 + 1, i0 + 1 < i1);
         int pages_cur = head[kHeadPagesTensor + lane];      // the first item's first 32 page ids (0 beyond its end)
@@ -362,7 +355,6 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         for (int ii = i0; cur.kv_end > 0 && ok; ++ii) {
             const TItem after = load_titem(p.works + ii + 2, ii + 2 < i1);
             const int ntiles = (cur.kv_end - cur.kv0 + kTile - 1) / kTile;
-            const int lead = cur.ntok * G > kRows ? 2 : 4;
             // APPEND: the first key position of the item that this step appends; tiles up to it are fetched at
             // once, before the others the K warp puts the item's new rows in the pool
             int first_new = INT_MAX;
@@ -401,13 +393,11 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                             appended_seen = true;
                         }
                     }
-                    const int pos = base + (which ? ring_pos_v(t, ntiles, lead) : ring_pos_k(t, lead));
-                    const int s = pos % Geo::RING;
+                    const int s = ring_slot(which, n, Geo::RING);
                     if (lane == 0 && which == 0) trace_event(9, ev, 40);
-                    ok = mbar_wait_warp(bar(Geo::kRingEmpty0 + s), ((uint32_t)(pos / Geo::RING) & 1u) ^ 1u, abort_flag, p.status, 11 + which);
+                    ok = mbar_wait_warp(bar(Geo::kRingEmpty0 + s), ((uint32_t)ring_use(n, Geo::RING) & 1u) ^ 1u, abort_flag, p.status, 11 + which);
                     if (!ok) break;
                     if (lane == 0 && which == 0) trace_event(9, ev, 42);
-                    last_pos = pos;
                     // lane -> 16-byte chunk c of a row: a warp instruction moves whole rows, 512 bytes in all
                     const int c = lane % kChunks;
                     const uint32_t dst_half = ring + s * Geo::SLOT_BYTES + (uint32_t)(c >> 3) * Geo::HALF_BYTES;
@@ -440,11 +430,10 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 }
                 pages_cur = pages_nxt;
             }
-            base += 2 * ntiles;
             cur = nxt;
             nxt = after;
         }
-        if (!ok && last_pos >= 0) {
+        if (!ok) {
             // aborted: let the loads already issued land before shared memory goes away
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
@@ -459,7 +448,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         const int b = warp == kMmaWarp ? 0 : 1;
         const uint32_t el = elect_one() ? 1u : 0u;
         bool ok = true;
-        int base = 0;             // ring position of the item's first slot
+        int base = 0;             // KV tiles before this item
         int cnt = 0;              // tiles of the group before this item: S buffer and phase of the hand-offs
         int item_no = 0;
         constexpr uint32_t idesc_pv = instr_desc(D, 1);
@@ -482,12 +471,12 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             if (ok) tc_fence_after();
             const uint64_t qd = smem_desc(sbase + Geo::OFF_Q + (dual ? (uint32_t)b * Geo::QTILE_BYTES : 0u), 16, 1024);
             auto tile_pages = [&](int j) { return (min(kTile, it.kv_end - (it.kv0 + j * kTile)) + kPage - 1) / kPage; };
-            auto wait_slot = [&](int pos, int code) {
+            auto wait_tile = [&](int which, int t, int code) {
                 const long long tw = trace_clock();
-                ok = ok && mbar_wait_spin(bar(Geo::kRingFull0 + pos % Geo::RING), (uint32_t)(pos / Geo::RING) & 1u, abort_flag, p.status, code);
+                ok = ok && mbar_wait_spin(bar(Geo::kRingFull0 + ring_slot(which, t, Geo::RING)), (uint32_t)ring_use(t, Geo::RING) & 1u, abort_flag, p.status, code);
                 tr_kv += trace_clock() - tw;
             };
-            auto slot_addr = [&](int pos) { return sbase + Geo::OFF_RING + (uint32_t)(pos % Geo::RING) * Geo::SLOT_BYTES; };
+            auto tile_addr = [&](int which, int t) { return sbase + Geo::OFF_RING + (uint32_t)ring_slot(which, t, Geo::RING) * Geo::SLOT_BYTES; };
             // u = -2, -1: the Q K^T of the group's first two tiles; u >= 0: the turn of its u-th tile, the P V of
             // tile j and the Q K^T of tile j + lead back to back once everything they read is there.  K/V tiles
             // are waited for first (they are normally there already), P last, so that nothing stands between
@@ -500,13 +489,12 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 const bool pv = u >= 0, qk = u + 2 < mine;
                 if (!pv && !qk) continue;
                 const int j = dual ? u : 2 * u + b, jn = j + lead;
-                const int pos_v = base + ring_pos_v(j, ntiles, lead), pos_k = base + ring_pos_k(jn, lead);
                 if (lane == 0) trace_event(b ? 10 : 0, ev, 20 + b);
-                if (pv) wait_slot(pos_v, 24);
-                if (qk) wait_slot(pos_k, 21);
+                if (pv) wait_tile(1, base + j, 24);
+                if (qk) wait_tile(0, base + jn, 21);
                 const uint32_t buf = tmem + kColS + 128u * (uint32_t)b + 64u * (uint32_t)(c & 1);      // S and P
-                const uint64_t vd = smem_desc(slot_addr(pos_v), Geo::HALF_BYTES, 1024);
-                const uint64_t kd = smem_desc(slot_addr(pos_k), 16, 1024);
+                const uint64_t vd = smem_desc(tile_addr(1, base + max(j, 0)), Geo::HALF_BYTES, 1024);
+                const uint64_t kd = smem_desc(tile_addr(0, base + jn), 16, 1024);
                 const uint32_t idesc_qk = instr_desc(16u * (uint32_t)tile_pages(jn), 0);
                 const int npg = tile_pages(j);
                 const uint32_t done = bar((qk ? Geo::kSFull0 : Geo::kPvDone0) + 2 * b + (c & 1));
@@ -543,7 +531,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 if (lane == 0) trace_event(b ? 10 : 0, ev, 26 + b);
             }
             cnt += mine;
-            base += 2 * ntiles;
+            base += ntiles;
         }
         if (lane == 0 && b == 0) {
             trace_set(8, tr_p);
@@ -567,7 +555,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         const float qscale = p.sm_scale * kLog2e;
         const float2 qscale2 = make_float2(qscale, qscale);
         int cnt = 0;         // tiles this group has processed before this item
-        int ring_base = 0;   // ring position of the item's first slot
+        int kv_base = 0;     // KV tiles of the CTA before this item (both groups)
         uint32_t pv_phase = 0;      // bit s: parity of the next phase of this group's kPvDone of buffer s
         int item_no = 0;
         bool ok = true;
@@ -589,7 +577,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             for (int c = kQV / 2; c < kQV; ++c) w[c] = (valid && dual) ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
         };
         // A ring slot is free again after two arrivals: one of each group in a dual item, else two of its only reader.
-        auto release = [&](int s, bool dual) { mbar_arrive_n(bar(Geo::kRingEmpty0 + s), dual ? 1u : 2u); };
+        auto release = [&](int which, int t, bool dual) { mbar_arrive_n(bar(Geo::kRingEmpty0 + ring_slot(which, t, Geo::RING)), dual ? 1u : 2u); };
         TItem it_next = load_titem(head_work, i0 < i1);
         uint4 q_next[kQV];
         pdl_wait();
@@ -645,8 +633,8 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 // read go back to the producers, the K tile of j now, and the V tile of j - lead (its P V was
                 // issued in front of this Q K^T).
                 if (m == 0) {
-                    release((ring_base + ring_pos_k(j, lead)) % Geo::RING, dual);
-                    if (u >= 2) release((ring_base + ring_pos_v(j - lead, ntiles, lead)) % Geo::RING, dual);
+                    release(0, kv_base + j, dual);
+                    if (u >= 2) release(1, kv_base + j - lead, dual);
                 }
                 tmem_wait_ld();
                 if (!__all_sync(0xffffffffu, vis == kTile)) {
@@ -735,7 +723,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 ok = mbar_wait_warp(bar(Geo::kPvDone0 + 2 * b + sb), (pv_phase >> sb) & 1u, abort_flag, p.status, 34);
                 pv_phase ^= 1u << sb;
                 // the V tiles of the group's last tiles go back to the producers
-                if (ok && m == 0) release((ring_base + ring_pos_v(dual ? u : 2 * u + b, ntiles, lead)) % Geo::RING, dual);
+                if (ok && m == 0) release(1, kv_base + (dual ? u : 2 * u + b), dual);
             }
             if (!ok) break;
             tc_fence_after();
@@ -853,7 +841,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             mbar_arrive(bar(Geo::kOFree));
             if (lane == 0) trace_event(1 + warp, ev, 36);
             cnt += mine;
-            ring_base += 2 * ntiles;
+            kv_base += ntiles;
         }
         if ((threadIdx.x & 127) == 0) {
             trace_set(b ? 15 : 11, tr_wait);

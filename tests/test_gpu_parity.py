@@ -341,3 +341,19 @@ def test_reference_maximum_moves_in_every_tile(d, ql):
     _, _, plan = run_and_check(wl, what="rising scores", tensor_min_rows=1)
     assert plan.info["num_items_tensor"] == plan.info["num_items"]
     run_and_check(wl, what="rising scores, one CTA", tensor_min_rows=1, num_sms=1)
+
+
+@pytest.mark.parametrize("d", [128, 64])
+@pytest.mark.parametrize("group", [4, 8])
+def test_one_cta_runs_span_items_of_one_to_twelve_tiles(d, group):
+    """All span items on one CTA, in the order of the sequences: one row tile (the groups take alternate 64-key
+    tiles) and two, short items between long ones, so that the K and V rings wrap in every relation to them."""
+    half = 128 // group                              # tokens of one row tile
+    tiles = [7, 1, 12, 12, 2, 11, 1, 3, 1, 9, 5, 2, 1, 1, 1, 10, 8, 6, 4, 7, 2, 12, 1, 7, 2, 9]
+    dual = [0, 0, 0, 1, 0, 0, 1, 0, 0, 1, 0, 1, 0, 0, 0, 0, 1, 0, 1, 0, 0, 1, 1, 1, 0, 0]
+    ql = [half + 1 + (5 * i) % (min(half, 63 - half)) if two else 1 + (7 * i) % half for i, two in enumerate(dual)]
+    ctx = [64 * t - n - (3 * i) % 20 if 64 * t - n >= 20 else 0 for i, (t, n) in enumerate(zip(tiles, ql))]
+    wl = W.make_single_step("one cta", W.Shape(group, 1, d, 16), ctx, ql, seed=640 + d + group, interleave_pages=True, poison_unused=True)
+    _, _, plan = run_and_check(wl, what="whole items", num_sms=1, tensor_min_rows=1, kv_chunk_tokens=1 << 20)
+    assert plan.info["num_items_tensor"] == plan.info["num_items"] == len(tiles)
+    run_and_check(wl, what="items of three tiles at most", num_sms=1, tensor_min_rows=1, kv_chunk_tokens=192)

@@ -1,0 +1,156 @@
+"""Order of the span body's hand-offs (csrc/span_ring.h, csrc/attn_append_tc.cuh), on the CPU.
+
+A barrier wait names only the parity of a phase: it tells phase k from phase k - 1, not from phase k - 2.
+The model below builds, for a CTA's sequence of items, the order that the kernel's waits and program order
+enforce among fills, tensor-core turns, softmax steps and releases, with the slots and use counts taken
+from the kernel's own header, and checks for every wait on a ring barrier that the phase before the one it
+waits for is over whatever the warps' relative speed.
+"""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2412_07017_b200 import build as lib_build
+
+PROBE = """
+#include "span_ring.h"
+using namespace asynclm::tc;
+extern "C" int slots_of(int head_dim) { return ring_slots(head_dim); }
+extern "C" int slot_of(int which, int t, int slots) { return ring_slot(which, t, slots); }
+extern "C" int use_of(int t, int slots) { return ring_use(t, slots); }
+"""
+
+
+@pytest.fixture(scope="module")
+def ring(tmp_path_factory):
+    d = tmp_path_factory.mktemp("ring")
+    src, lib = os.path.join(d, "probe.cpp"), os.path.join(d, "probe.so")
+    with open(src, "w") as f:
+        f.write(PROBE)
+    subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", "-I", lib_build.CSRC, "-o", lib, src], check=True)
+    return ctypes.CDLL(lib)
+
+
+def placed_by_kernel(ring, head_dim):
+    """(kind, tile, its item's first tile, item's tiles, dual) -> (slot, uses of that slot before)"""
+    n = ring.slots_of(head_dim)
+    return lambda which, t, first, tiles, dual: (ring.slot_of(which, t, n), ring.use_of(t, n))
+
+
+def placed_in_one_ring(slots):
+    """K and V tiles in one ring in the order of consumption, restarted with every item: the mistake."""
+    def place(which, t, first, tiles, dual):
+        lead, g = 2 if dual else 4, t - first
+        pos = 2 * first + (g + min(tiles, g + lead) if which else (g if g < lead else 2 * g - lead + 1))
+        return pos % slots, pos // slots
+    return place
+
+
+def ambiguous_waits(items, place):
+    """items: (64-key tiles, dual) in the order a CTA runs them.  Returns the waits that could pass early."""
+    before = {}          # node -> nodes known to come before it
+
+    def after(node, *prev):
+        before.setdefault(node, set()).update(p for p in prev if p is not None)
+        return node
+
+    waits = []           # (where the warp stands when it waits, what has to be over, description)
+    used = {}            # slot -> {use: (kind, tile, groups that read it)}
+    last = {}            # program order of each warp: its latest node
+    first, opened = 0, None
+    for i, (n, dual) in enumerate(items):
+        for t in range(first, first + n):
+            for which in (0, 1):
+                slot, use = place(which, t, first, n, dual)
+                used.setdefault(slot, {})[use] = (which, t, (0, 1) if dual else ((t - first) & 1,))
+        first += n
+    first = 0
+    for i, (n, dual) in enumerate(items):
+        where = {(w, t): place(w, t, first, n, dual) for w in (0, 1) for t in range(first, first + n)}
+        for which in (0, 1):                                   # producers: not tied to the items' ends
+            for t in range(first, first + n):
+                slot, use = where[which, t]
+                here = last.get(("prod", which))
+                if use >= 2:
+                    w0, t0, groups = used[slot][use - 2]
+                    waits += [(here, ("free", w0, t0, b), ("empty", which, t)) for b in groups]
+                fill = after(("fill", which, t), here)
+                if use >= 1:
+                    w0, t0, groups = used[slot][use - 1]
+                    after(fill, *[("free", w0, t0, b) for b in groups])
+                last["prod", which] = fill
+                # a lane's arrival comes after all of its earlier copies
+                after(("full", which, t), fill, ("full", which, t - 1) if t else None)
+        ends = []
+        for b in (0, 1):
+            mine = [first + j for j in range(n) if dual or j % 2 == b]
+            last["mma", b] = after(("open", i, b), last.get(("mma", b)), opened)
+            last["soft", b] = after(("q", i, b), last.get(("soft", b)), opened)
+            for u in range(-2, len(mine)):
+                if u >= 0:                                     # softmax of tile u: its scores came with turn u - 2
+                    s = after(("soft", i, b, u), last["soft", b], ("turn", i, b, u - 2))
+                    after(("free", 0, mine[u], b), s)
+                    if u >= 2:
+                        after(("free", 1, mine[u - 2], b), s)
+                    last["soft", b] = s
+                reads = ([(1, mine[u])] if u >= 0 else []) + ([(0, mine[u + 2])] if u + 2 < len(mine) else [])
+                if not reads:
+                    continue
+                here = last["mma", b]
+                turn = after(("turn", i, b, u), here, ("soft", i, b, u) if u >= 0 else None)
+                for which, t in reads:
+                    slot, use = where[which, t]
+                    if use >= 1:
+                        w0, t0, _ = used[slot][use - 1]
+                        waits.append((here, ("full", w0, t0), ("full", which, t)))
+                    after(turn, ("full", which, t))
+                last["mma", b] = turn
+            end = after(("end", i, b), last["soft", b], last["mma", b])
+            for t in mine[-2:]:
+                after(("free", 1, t, b), end)
+            last["soft", b] = end
+            ends.append(end)
+        opened = after(("opened", i), *ends)
+        first += n
+    # ancestors as bit sets, in an order in which everything comes after what precedes it
+    index, anc, stack = {}, {}, []
+    for root in before:
+        stack.append(root)
+        while stack:
+            node = stack[-1]
+            todo = [p for p in before.get(node, ()) if p not in anc]
+            if node in anc or not todo:
+                stack.pop()
+                if node not in anc:
+                    index[node] = len(index)
+                    bits = 1 << index[node]
+                    for p in before.get(node, ()):
+                        bits |= anc[p]
+                    anc[node] = bits
+            else:
+                stack.extend(todo)
+    return [what for here, need, what in waits if here is None or need not in index or not (anc[here] >> index[need]) & 1]
+
+
+def three_items():
+    for n1 in range(1, 13):
+        for n2 in range(1, 13):
+            for modes in range(8):
+                yield [(n1, bool(modes & 1)), (n2, bool(modes & 2)), (12, bool(modes & 4))]
+
+
+@pytest.mark.parametrize("head_dim", [128, 64])
+def test_no_wait_on_a_ring_barrier_can_pass_a_phase_early(ring, head_dim):
+    place = placed_by_kernel(ring, head_dim)
+    for items in three_items():
+        assert not ambiguous_waits(items, place), items
+    assert not ambiguous_waits([(1, False)] * 30 + [(9, True), (2, False), (40, True)], place)
+
+
+def test_the_model_finds_the_early_wait_of_a_shared_ring():
+    """V5 of the first item frees a slot for the V producer while V0, two uses earlier, may be unread."""
+    found = ambiguous_waits([(7, False), (1, False), (12, False)], placed_in_one_ring(10))
+    assert any(kind == "empty" for kind, _, _ in found)
+    assert not any(kind == "empty" for kind, _, _ in ambiguous_waits([(40, True)], placed_in_one_ring(10)))
