@@ -492,6 +492,10 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                 if (lane == 0) trace_event(b ? 10 : 0, ev, 20 + b);
                 if (pv) wait_tile(1, base + j, 24);
                 if (qk) wait_tile(0, base + jn, 21);
+                // The tiles were written by cp.async, through the generic proxy; the MMAs read them through the
+                // asynchronous one.  The full barriers order the two, the fence makes the bytes visible across;
+                // it stands before the wait for P, which hides it.
+                fence_async_smem();
                 const uint32_t buf = tmem + kColS + 128u * (uint32_t)b + 64u * (uint32_t)(c & 1);      // S and P
                 const uint64_t vd = smem_desc(tile_addr(1, base + max(j, 0)), Geo::HALF_BYTES, 1024);
                 const uint64_t kd = smem_desc(tile_addr(0, base + jn), 16, 1024);

@@ -154,3 +154,14 @@ def test_the_model_finds_the_early_wait_of_a_shared_ring():
     found = ambiguous_waits([(7, False), (1, False), (12, False)], placed_in_one_ring(10))
     assert any(kind == "empty" for kind, _, _ in found)
     assert not any(kind == "empty" for kind, _, _ in ambiguous_waits([(40, True)], placed_in_one_ring(10)))
+
+
+def test_the_proxy_fence_stands_between_the_tiles_arrival_and_the_mmas_that_read_them():
+    """K and V tiles are generic-proxy writes (cp.async), tcgen05.mma reads shared memory through the asynchronous
+    proxy: without a proxy fence behind the full barriers' waits nothing says that it sees them.  A missing
+    one need not show in any result, so the order of the statements is what is checked."""
+    with open(os.path.join(lib_build.CSRC, "attn_append_tc.cuh")) as f:
+        turn = f.read().split("for (int u = -2; u < mine && ok; ++u) {", 1)[1].split("mma_commit(el, done);", 1)[0]
+    steps = ["wait_tile(1, ", "wait_tile(0, ", "fence_async_smem();", "mma_f16_ta(", "mma_f16("]
+    at = [turn.index(s) for s in steps]
+    assert at == sorted(at) and turn.count("fence_async_smem();") == 1 and "cp_async16(" not in turn
