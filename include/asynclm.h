@@ -15,7 +15,7 @@
  *     asynclm_plan       (host integer work + one async host->device copy of the plan)
  *     asynclm_kv_append  (scatter the new K/V rows into their page slots)
  *     asynclm_attn_mixed (attention of every new row over its sequence's pages)
- * or, instead of the last two, asynclm_step, which does both in one launch.
+ * or, instead of the last two, asynclm_step, which does both in one call.
  * A plan depends only on the lengths and the page table, so a multi-layer model builds it once per
  * step and reuses it for every layer's pool.
  *
@@ -235,14 +235,16 @@ int asynclm_attn_mixed(const asynclm_plan_t* plan, const void* q, const void* kv
 
 /*
  * The whole step in one call: asynclm_kv_append followed by asynclm_attn_mixed, with the same
- * arguments, results and bit-exact pool contents, but without a separate append launch.  The
- * interrupt block still goes to the end of the context first (Section 3.2) and is then processed
- * with the other sequences' decodes (Section 5.3): every work item of the attention kernel copies
- * the new K/V rows it is about to read into their page slots itself, right before it fetches the
- * pages that hold them, so no part of the kernel waits for another, and every new row is written
- * (each new token attends to itself).  Items that read the same new rows write the same bytes; for
- * a step with a span of more than 64 tokens (the trap handler's recompute, say) that duplication
- * would dominate, and the call runs the append as a kernel of its own instead.
+ * arguments, results and bit-exact pool contents.  The interrupt block still goes to the end of the
+ * context first (Section 3.2) and is then processed with the other sequences' decodes (Section 5.3).
+ * In a step whose items all run on the warp body (asynclm_plan_info.num_items_tensor is 0: decode rows
+ * and short spans) with no span of more than 64 tokens there is no separate append launch: every work
+ * item of the attention kernel copies the new K/V rows it is about to read into their page slots
+ * itself, right before it fetches the pages that hold them, so no part of the kernel waits for another,
+ * and every new row is written (each new token attends to itself).  Items that read the same new rows
+ * write the same bytes.  Where the span body is used, that copy would stand in front of its loads, and
+ * for long spans the duplication would dominate: then the append is a kernel of its own, as in the two
+ * calls.
  *
  *   q             device, bf16 [T][num_q_heads][head_dim]
  *   k_new, v_new  device, bf16 [T][num_kv_heads][head_dim]

@@ -43,7 +43,8 @@ extern "C" const char* asynclm_strerror(int status) {
     }
 }
 
-// Longest span for which asynclm_step appends inside the attention kernel.
+// Longest span (of units that all run on the warp body) for which asynclm_step appends inside the
+// attention kernel.
 constexpr int kStepFusedMaxSpan = 64;
 
 static bool runnable(const asynclm_plan_t* plan) {
@@ -85,10 +86,14 @@ extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const voi
     if (int rc = check_plan_device(plan->device)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     int rc;
-    if (plan->max_q_len > kStepFusedMaxSpan) {
-        // In the fused kernel every item copies the new rows it reads, so the units of one long span
-        // copy its first rows again and again (quadratic in the span length): beyond a few hundred
-        // tokens the separate append kernel, which copies every row once, is the better first half.
+    if (plan->dev.num_items_tensor > 0 || plan->max_q_len > kStepFusedMaxSpan) {
+        // With the append fused in, every item copies the new rows it reads, so the units of one long span
+        // copy its first rows again and again (quadratic in the span length), and in the span body the
+        // copy stands in front of the loads: the separate append kernel, which copies every row once, is
+        // the better first half.  (us a layer, fused | separate: 32 sequences with 8 spans of up to 64 tokens
+        // 90 | 65, the same at head_dim 64 85 | 59, 24 sequences with a span each 122 | 72.  Steps without
+        // span tiles keep the fused form: 4 decoding sequences 15.5 | 17.7, 16 with 8 spans of up to 7
+        // tokens 49.5 | 49.9.)
         rc = cuda_status(launch_kv_append(plan->dev, k_new, v_new, kv_pool, s));
         if (rc != ASYNCLM_OK) return rc;
         rc = cuda_status(launch_attention(plan->dev, q, kv_pool, out, lse, s));

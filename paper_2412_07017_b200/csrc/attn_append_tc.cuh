@@ -25,9 +25,7 @@
 //   warps 8, 10     producers of K tiles and of V tiles: 16-byte cp.async copies (fully coalesced,
 //                   whole rows, 512 bytes per warp instruction) that write the 128-byte-swizzled operand
 //                   layout and complete on the slot's mbarrier.  K and V have a ring of 80 KiB each
-//                   (see span_ring.h).  For asynclm_step
-//                   the K warp also puts an item's new K/V rows into their page slots, before the first
-//                   tile that holds one.
+//                   (see span_ring.h).
 //   warps 9, 11     issue the MMAs, one warp per softmax group.  Warp 9 owns the tensor-memory allocation.
 // Why tiles of 64 keys: with two S buffers per group, the Q K^T of the tile after next is issued behind the
 // P V of the current one, and the softmax of the next tile, whose S is complete, runs meanwhile; with
@@ -80,8 +78,7 @@ struct Geometry {
                kRingFull0 = kSFull0 + 4, kRingEmpty0 = kRingFull0 + 2 * RING, kMmaDrain = kRingEmpty0 + 2 * RING, kNumBars };
     static constexpr uint32_t OFF_TMEM_PTR = OFF_BAR + 8 * kNumBars;
     static constexpr uint32_t OFF_ABORT = OFF_TMEM_PTR + 8;
-    static constexpr uint32_t OFF_APPENDED = OFF_ABORT + 8;      // items of this CTA whose new K/V rows are in the pool
-    static constexpr uint32_t SMEM_BYTES = OFF_APPENDED + 8 + 1024;
+    static constexpr uint32_t SMEM_BYTES = OFF_ABORT + 8 + 1024;
     static_assert(SMEM_BYTES <= 232448, "shared memory budget");
 };
 
@@ -285,18 +282,17 @@ __device__ __forceinline__ TItem load_titem(const Work* rec, bool valid) {
 }
 
 // The whole kernel body, called by all twelve warps with `smem` 1024-byte aligned.
-template <int D, int G, bool APPEND>
+template <int D, int G>
 __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* __restrict__ q,
                                         const __nv_bfloat16* pool,
                                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
-                                        uint8_t* smem, const AppendSrc& app) {
+                                        uint8_t* smem) {
     using Geo = Geometry<D>;
     const uint32_t sbase = smem_u32(smem);
     const uint32_t bar0 = sbase + Geo::OFF_BAR;
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
     volatile uint32_t* tmem_ptr = (volatile uint32_t*)(smem + Geo::OFF_TMEM_PTR);
     volatile int* abort_flag = (volatile int*)(smem + Geo::OFF_ABORT);
-    volatile int* appended = (volatile int*)(smem + Geo::OFF_APPENDED);
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
@@ -319,7 +315,6 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         for (int s = 0; s < 2 * Geo::RING; ++s) { mbar_init(bar(Geo::kRingFull0 + s), 32); mbar_init(bar(Geo::kRingEmpty0 + s), 2); }
         mbar_init(bar(Geo::kMmaDrain), 2);
         *abort_flag = 0;
-        *appended = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
@@ -355,44 +350,12 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         for (int ii = i0; cur.kv_end > 0 && ok; ++ii) {
             const TItem after = load_titem(p.works + ii + 2, ii + 2 < i1);
             const int ntiles = (cur.kv_end - cur.kv0 + kTile - 1) / kTile;
-            // APPEND: the first key position of the item that this step appends; tiles up to it are fetched at
-            // once, before the others the K warp puts the item's new rows in the pool
-            int first_new = INT_MAX;
-            if constexpr (APPEND) {
-                const int q_seq0 = ii == i0 ? head_work->q_seq0 : __ldg(&p.works[ii].q_seq0);
-                first_new = cur.kv_limit0 - 1 - (cur.q_row0 - q_seq0);
-            }
-            bool appended_seen = false;
             for (int t0 = 0; t0 < ntiles && ok; t0 += kGroupTiles) {
                 int pages_nxt = 0;
                 const int t1 = min(t0 + kGroupTiles, ntiles);
                 for (int t = t0; t < t1 && ok; ++t, ++n) {
                     const int rows = min(kTile, cur.kv_end - (cur.kv0 + t * kTile));
                     const int npages = (rows + kPage - 1) / kPage;
-                    if constexpr (APPEND) {
-                        if (!appended_seen && cur.kv0 + t * kTile + rows > first_new) {
-                            if (which == 0) {
-                                append_rows_of_item(p, app, ii == i0 ? *head_work : p.works[ii], lane);
-                                __threadfence();      // the rows are visible before the count moves
-                                __syncwarp();
-                                if (lane == 0) *appended = ii - i0 + 1;
-                            }
-                            const long long t_wait = clock64();
-                            while (*appended <= ii - i0 && ok) {
-                                __nanosleep(64);
-                                if (*abort_flag) ok = false;
-                                else if (clock64() - t_wait > kWaitCycles) {
-                                    *abort_flag = 1;
-                                    atomicCAS(p.status, 0, 13);
-                                    ok = false;
-                                }
-                            }
-                            ok = __all_sync(0xffffffffu, ok);
-                            if (!ok) break;
-                            __threadfence();
-                            appended_seen = true;
-                        }
-                    }
                     const int s = ring_slot(which, n, Geo::RING);
                     if (lane == 0 && which == 0) trace_event(9, ev, 40);
                     ok = mbar_wait_warp(bar(Geo::kRingEmpty0 + s), ((uint32_t)ring_use(n, Geo::RING) & 1u) ^ 1u, abort_flag, p.status, 11 + which);

@@ -37,25 +37,25 @@ attn_decode_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const 
     dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, aligned_smem(smem_raw), app);
 }
 
-template <int D, int G, bool APPEND>
+template <int D, int G>
 __global__ void __launch_bounds__(tc::kThreads, 1)
 attn_append_tc_kernel(DevPlan p, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* pool,
-                      __nv_bfloat16* __restrict__ out, float* __restrict__ lse, AppendSrc app) {
+                      __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
     extern __shared__ uint8_t smem_raw[];
     pdl_trigger();      // the kernel behind this one may start its prologue; it waits for this grid to complete
     if (threadIdx.x == 0) {
         trace_mark(0);
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<D, G, APPEND>(p, q, pool, out, lse, aligned_smem(smem_raw), app);
+    tc::tc_body<D, G>(p, q, pool, out, lse, aligned_smem(smem_raw));
     if (threadIdx.x == 0) trace_mark(1);
 }
 
-template <int D, int G, bool APPEND>
+template <int D, int G>
 __global__ void __launch_bounds__(tc::kThreads, 1)
 attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const __nv_bfloat16* __restrict__ q,
                   const __nv_bfloat16* pool, __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
-                  int S, AppendSrc app) {
+                  int S) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = aligned_smem(smem_raw);
     pdl_trigger();      // the split-KV merge behind this kernel may start its prologue
@@ -67,17 +67,17 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(&kv_map));
     if (head[0] == head[1]) {
         // no span tiles for this CTA: straight to its decode rows, without the tensor-memory set-up
-        dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, smem, app);
+        dec::decode_body<D, G, false>(p, &kv_map, q, out, lse, S, smem, AppendSrc{});
         return;
     }
     if (threadIdx.x == 0) {
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<D, G, APPEND>(p, q, pool, out, lse, smem, app);
+    tc::tc_body<D, G>(p, q, pool, out, lse, smem);
     if (threadIdx.x == 0) trace_mark(1);
     if (head[2] == head[3] && p.queue_count == 0) return;      // nothing left for the warp body
     __syncthreads();      // tensor memory released, shared memory free for the second phase
-    dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, smem, app);
+    dec::decode_body<D, G, false>(p, &kv_map, q, out, lse, S, smem, AppendSrc{});
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -167,52 +167,52 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
                       (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
-template <int D, int G, bool APPEND>
-cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, void* out, float* lse,
-                          cudaStream_t stream, AppendSrc app) {
+template <int D, int G>
+cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, void* out, float* lse, cudaStream_t stream) {
     constexpr size_t smem = tc::Geometry<D>::SMEM_BYTES;
-    cudaError_t e = allow_smem<attn_append_tc_kernel<D, G, APPEND>>(smem);
+    cudaError_t e = allow_smem<attn_append_tc_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_append_tc_kernel<D, G, APPEND>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
-                      p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, app);
+    return launch_pdl(attn_append_tc_kernel<D, G>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
+                      p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
 }
 
-template <int D, int G, bool APPEND>
-cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void* out, float* lse,
-                         cudaStream_t stream, AppendSrc app) {
+template <int D, int G>
+cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void* out, float* lse, cudaStream_t stream) {
     constexpr int S = decode_stages<D>();
     constexpr size_t smem = std::max<size_t>(dec::smem_bytes<D>(S), tc::Geometry<D>::SMEM_BYTES);
     static_assert(dec::smem_bytes<D>(S) - 1024 <= tc::Geometry<D>::OFF_BAR, "the span body's barriers stay clear of the warp body");
-    cudaError_t e = allow_smem<attn_fused_kernel<D, G, APPEND>>(smem);
+    cudaError_t e = allow_smem<attn_fused_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     e = cached_kv_map(p, pool, &map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_fused_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, map,
-                      (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S, app);
+    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, map,
+                      (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S);
 }
 
-template <int D, int G, bool APPEND>
+template <int D, int G>
 cudaError_t launch_attention_impl(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
                                   cudaStream_t stream, AppendSrc app) {
     const bool has_tensor = p.num_items_tensor > 0, has_cuda = p.num_items_cuda > 0;
+    if (app.k_new != nullptr)      // the warp body only
+        return has_tensor || !has_cuda ? cudaErrorInvalidValue : launch_decode<D, G, true>(p, q, kv_pool, out, lse, stream, app);
     if (has_tensor && has_cuda && p.num_ctas_tensor == p.num_ctas_cuda)
-        return launch_fused<D, G, APPEND>(p, q, kv_pool, out, lse, stream, app);
+        return launch_fused<D, G>(p, q, kv_pool, out, lse, stream);
     if (has_tensor)
-        if (cudaError_t e = launch_tensor<D, G, APPEND>(p, q, kv_pool, out, lse, stream, app)) return e;
+        if (cudaError_t e = launch_tensor<D, G>(p, q, kv_pool, out, lse, stream)) return e;
     // a decode kernel behind a tensor kernel would have to wait for it to finish (pdl_wait), which is what
     // stream order gives anyway
-    return has_cuda ? launch_decode<D, G, APPEND>(p, q, kv_pool, out, lse, stream, app) : cudaSuccess;
+    return has_cuda ? launch_decode<D, G, false>(p, q, kv_pool, out, lse, stream, app) : cudaSuccess;
 }
 
-template <int D, bool APPEND>
+template <int D>
 cudaError_t launch_attention_d(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
                                cudaStream_t stream, AppendSrc app) {
     switch (p.group) {
-        case 1: return launch_attention_impl<D, 1, APPEND>(p, q, kv_pool, out, lse, stream, app);
-        case 2: return launch_attention_impl<D, 2, APPEND>(p, q, kv_pool, out, lse, stream, app);
-        case 4: return launch_attention_impl<D, 4, APPEND>(p, q, kv_pool, out, lse, stream, app);
-        case 8: return launch_attention_impl<D, 8, APPEND>(p, q, kv_pool, out, lse, stream, app);
+        case 1: return launch_attention_impl<D, 1>(p, q, kv_pool, out, lse, stream, app);
+        case 2: return launch_attention_impl<D, 2>(p, q, kv_pool, out, lse, stream, app);
+        case 4: return launch_attention_impl<D, 4>(p, q, kv_pool, out, lse, stream, app);
+        case 8: return launch_attention_impl<D, 8>(p, q, kv_pool, out, lse, stream, app);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -221,13 +221,8 @@ cudaError_t launch_attention_d(const DevPlan& p, const void* q, const void* kv_p
 
 cudaError_t launch_attention(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
                              cudaStream_t stream, AppendSrc app) {
-    const bool append = app.k_new != nullptr;
-    if (p.head_dim == 128)
-        return append ? launch_attention_d<128, true>(p, q, kv_pool, out, lse, stream, app)
-                      : launch_attention_d<128, false>(p, q, kv_pool, out, lse, stream, app);
-    if (p.head_dim == 64)
-        return append ? launch_attention_d<64, true>(p, q, kv_pool, out, lse, stream, app)
-                      : launch_attention_d<64, false>(p, q, kv_pool, out, lse, stream, app);
+    if (p.head_dim == 128) return launch_attention_d<128>(p, q, kv_pool, out, lse, stream, app);
+    if (p.head_dim == 64) return launch_attention_d<64>(p, q, kv_pool, out, lse, stream, app);
     return cudaErrorInvalidValue;
 }
 

@@ -10,8 +10,9 @@ cudaError_t launch_kv_append(const DevPlan& p, const void* k_new, const void* v_
                              cudaStream_t stream);
 
 // All attention kernels of a step: span tiles and warp-body items (one fused launch when the step
-// has both), writing final rows to `out` and split rows to the plan's partials.  With app.k_new set
-// the kernels first put every new K/V row they are about to read into its page slot themselves.
+// has both), writing final rows to `out` and split rows to the plan's partials.  With app.k_new set,
+// only for steps without span tiles, the kernel first puts every new K/V row it is about to read into its
+// page slot itself.
 cudaError_t launch_attention(const DevPlan& p, const void* q, const void* kv_pool, void* out, float* lse,
                              cudaStream_t stream, AppendSrc app = AppendSrc{nullptr, nullptr, nullptr});
 

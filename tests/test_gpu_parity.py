@@ -357,3 +357,38 @@ def test_one_cta_runs_span_items_of_one_to_twelve_tiles(d, group):
     _, _, plan = run_and_check(wl, what="whole items", num_sms=1, tensor_min_rows=1, kv_chunk_tokens=1 << 20)
     assert plan.info["num_items_tensor"] == plan.info["num_items"] == len(tiles)
     run_and_check(wl, what="items of three tiles at most", num_sms=1, tensor_min_rows=1, kv_chunk_tokens=192)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("ctx,ql,tensor,append_launches", [
+    ([300, 90, 700, 40], [1, 1, 1, 1], False, 0),           # decode rows: the attention kernel appends
+    ([300, 90, 700, 40], [7, 1, 0, 3], False, 0),           # and short spans
+    ([300, 90, 700, 40], [40, 1, 1, 1], True, 1),           # span tiles: an append kernel in front
+    ([300, 0], [64, 33], True, 1),
+    ([300, 90], [65, 1], False, 1),                         # a long span kept on the warp body
+])
+def test_launches_of_a_step(api, d, ctx, ql, tensor, append_launches):
+    from cuda.bindings import runtime
+    opts = {} if tensor else {"flags": B.PLAN_NO_TENSOR_PATH}
+    wl = W.make_single_step("launches", W.Shape(32, 8, d, 16), ctx, ql, seed=5)
+    _, _, plan = run_and_check(wl, what="one call", **opts)
+    assert (plan.info["num_items_tensor"] > 0) == tensor
+    st = wl.steps[0]
+    q, kn, vn, pool = to_dev(st.q), to_dev(st.k_new), to_dev(st.v_new), to_dev(wl.kv_pool)
+    out = torch.empty_like(q)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        if api == "step":
+            B.asynclm_step(plan, q, kn, vn, pool, out, None)
+        else:
+            append_launches = plan.info["launches_append"]
+            B.asynclm_kv_append(plan, kn, vn, pool)
+            B.asynclm_attn_mixed(plan, q, pool, out, None)
+    err, _, nodes = runtime.cudaGraphGetNodes(runtime.cudaGraph_t(graph.raw_cuda_graph()))
+    assert int(err) == 0 and nodes == append_launches + plan.info["launches_attn"]
+    graph.instantiate()
+    graph.replay()
+    torch.cuda.synchronize()
+    ref_pool, ref_out, _ = oracle_step(wl, st)
+    assert np.array_equal(to_bits(pool), ref_pool)
+    assert_close(to_bits(out), None, ref_out, None, what="replayed")
