@@ -293,9 +293,11 @@ struct CutPolicy {
 // and merged in chunk order, so the output does not depend on which CTA ran what.
 //   The load limit is the smallest one under which the span units fit and the room left on all CTAs
 // covers the modelled time of the queue; it is found by bisection.
-void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp,
+//   Returns false, with only the units (their division and n_chunks) filled in, if the cuts leave more than
+// max_partial_rows partial rows.
+bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp,
                   std::vector<UnitBuild>& units, int group, int64_t kv_bytes, int n_ctas, const CutPolicy& policy,
-                  std::vector<Item>& items,
+                  int64_t max_partial_rows, std::vector<Item>& items,
                   std::vector<int32_t>& cta_indptr_warp, std::vector<int32_t>& cta_indptr_tensor,
                   std::vector<int32_t>& item_cta, int32_t* queue_first, int32_t* queue_count) {
     struct Piece { Item it; int32_t cta; };
@@ -434,7 +436,7 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         if (fill(mid, false)) hi = mid; else lo = mid;
     }
     fill(hi, true);
-    std::stable_sort(pieces_out.begin(), pieces_out.end(), [](const Piece& x, const Piece& y) { return x.cta < y.cta; });
+    for (const Piece& pz : pieces_out) units[pz.it.unit].u.n_chunks = std::max(units[pz.it.unit].u.n_chunks, pz.it.chunk + 1);
 
     // ---- warp-body chunks.  An item boundary costs time and a split unit costs partial rows and a
     // merge, so most of the work stays in long pieces: a few units, a sixth of all tiles, are cut into
@@ -477,6 +479,10 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         }
         units[id].u.n_chunks = (int32_t)pieces;
     }
+    int64_t partial_rows = 0;
+    for (const UnitBuild& ub : units)
+        if (ub.u.n_chunks > 1) partial_rows += (int64_t)ub.u.n_chunks * ub.u.ntok;
+    if (partial_rows > max_partial_rows) return false;
     auto longer = [](const Item& x, const Item& y) { return x.kv1 - x.kv0 > y.kv1 - y.kv0; };
     std::stable_sort(chunks.begin(), chunks.end(), longer);
     std::stable_sort(tail.begin(), tail.end(), longer);
@@ -496,12 +502,12 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     *queue_first = n_start;
     *queue_count = (int32_t)chunks.size() - n_start;
     const int32_t first = (int32_t)items.size();
+    std::stable_sort(pieces_out.begin(), pieces_out.end(), [](const Piece& x, const Piece& y) { return x.cta < y.cta; });
     std::vector<int32_t> count((size_t)n_ctas, 0);
     for (const Piece& pz : pieces_out) {
         items.push_back(pz.it);
         item_cta.push_back(pz.cta);
         count[(size_t)pz.cta]++;
-        units[pz.it.unit].u.n_chunks = std::max(units[pz.it.unit].u.n_chunks, pz.it.chunk + 1);
     }
     int32_t at = first;
     for (int k = 0; k < n_ctas; ++k) {
@@ -509,6 +515,7 @@ void deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         at += count[(size_t)k];
     }
     cta_indptr_tensor[(size_t)n_ctas] = at;
+    return true;
 }
 
 }  // namespace
@@ -607,7 +614,9 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     int32_t queue_first = 0, queue_count = 0;
     std::vector<int32_t> split_units, merge_blocks;   // merge block: 4 (token, head) rows of a split unit
     int64_t partial_rows = 0;
-    auto deal = [&](const CutPolicy& policy, bool tensor_on) -> int {
+    // (too_many: the cuts leave more than max_partial_rows partial rows, and nothing is dealt)
+    bool too_many = false;
+    auto deal = [&](const CutPolicy& policy, bool tensor_on, int64_t max_partial_rows) -> int {
         units.clear(); ids_cuda.clear(); ids_tensor.clear(); items.clear(); item_cta.clear();
         split_units.clear(); merge_blocks.clear();
         n_items_cuda = queue_first = queue_count = 0;
@@ -647,8 +656,9 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
         } else {
             // bytes of K and V the step has to read, each (sequence, kv head) counted once
             const int64_t kv_bytes = total_kv * Hkv * 4 * shape->head_dim;
-            deal_dynamic(ids_tensor, ids_cuda, units, G, kv_bytes, ctas_cuda, policy, items, cta_indptr_cuda, cta_indptr_tensor, item_cta,
-                         &queue_first, &queue_count);
+            too_many = !deal_dynamic(ids_tensor, ids_cuda, units, G, kv_bytes, ctas_cuda, policy, max_partial_rows, items,
+                                     cta_indptr_cuda, cta_indptr_tensor, item_cta, &queue_first, &queue_count);
+            if (too_many) return ASYNCLM_OK;
             n_items_cuda = queue_first + queue_count;
         }
 
@@ -671,27 +681,31 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     // The fastest cuts, as long as their partial results fit the fixed array of asynclm_attn_mixed_static; else as
     // many of the long span units cut by keys as it has room for, none of them, long pieces in the queue as
     // well, and at head_dim 64 no span units at all (warp units have far fewer partial rows).  If nothing fits,
-    // the fastest again: that call then refuses the plan.
-    auto fits_static = [&]() { return partial_bytes(partial_rows, G, shape->head_dim) <= ASYNCLM_STATIC_SCRATCH_BYTES; };
+    // the fastest again: that call then refuses the plan.  A try that does not fit ends when its cuts are
+    // known, before the items are sorted and dealt.
+    int64_t static_rows = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float)));
+    while (partial_bytes(static_rows, G, shape->head_dim) > ASYNCLM_STATIC_SCRATCH_BYTES) --static_rows;
+    auto fits_static = [&]() { return !too_many && partial_rows <= static_rows; };
     const CutPolicy fastest;
-    rc = deal(fastest, tensor_wanted);
+    rc = deal(fastest, tensor_wanted, static_rows);
     if (rc == ASYNCLM_OK && !fits_static()) {
         if (fixed_chunk == 0) {
-            int64_t span_rows = 0, span_units = 0;
-            for (int id : split_units)
-                if (units[(size_t)id].path == kPathTensor) {
-                    span_rows += (int64_t)units[(size_t)id].u.n_chunks * units[(size_t)id].u.ntok;
-                    ++span_units;
-                }
-            const int64_t room = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float))) - (partial_rows - span_rows);
+            int64_t span_rows = 0, span_units = 0, warp_rows = 0;
+            for (const UnitBuild& ub : units) {
+                const int64_t rows = ub.u.n_chunks > 1 ? (int64_t)ub.u.n_chunks * ub.u.ntok : 0;
+                if (ub.path != kPathTensor) warp_rows += rows;
+                else if (rows > 0) span_rows += rows, ++span_units;
+            }
+            const int64_t room = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float))) - warp_rows;
             CutPolicy fewer;
             fewer.units_by_keys = room <= 0 ? 0 : (int)(span_units * room / std::max<int64_t>(1, span_rows) * 15 / 16);
-            if (fewer.units_by_keys > 0) rc = deal(fewer, tensor_wanted);
-            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, true}, tensor_wanted);
-            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, false}, tensor_wanted);
+            if (fewer.units_by_keys > 0) rc = deal(fewer, tensor_wanted, static_rows);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, true}, tensor_wanted, static_rows);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, false}, tensor_wanted, static_rows);
         }
-        if (rc == ASYNCLM_OK && !fits_static() && tensor_wanted && shape->head_dim == 64) rc = deal(CutPolicy{kDivideMargin64, 0, false}, false);
-        if (rc == ASYNCLM_OK && !fits_static()) rc = deal(fastest, tensor_wanted);
+        if (rc == ASYNCLM_OK && !fits_static() && tensor_wanted && shape->head_dim == 64)
+            rc = deal(CutPolicy{kDivideMargin64, 0, false}, false, static_rows);
+        if (rc == ASYNCLM_OK && !fits_static()) rc = deal(fastest, tensor_wanted, INT64_MAX);
     }
     if (rc != ASYNCLM_OK) return rc;
     const int n_items = (int)items.size();

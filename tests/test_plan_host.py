@@ -344,3 +344,33 @@ def test_long_cuts_stay_within_the_fixed_scratch_array(d, ctx, ql):
     rows = p.info["partial_rows"]
     up = lambda x: -(-x // 256) * 256
     assert up(rows * 4 * d * 4) + up(rows * 4 * 4) <= B.static_scratch_bytes()
+
+
+@pytest.mark.parametrize("shape,ctx,ql,sms,spans", [
+    ((16, 4, 128), [50926, 57166, 121457], [1, 1000, 1], 148, True),               # fewer units cut by keys
+    ((16, 2, 128), [38674], [1000], 148, True),
+    ((64, 8, 128), [58080, 125149], [128, 1], 148, True),                         # none
+    ((64, 8, 64), [59781], [256], 600, False),                                    # no span units
+    ((32, 8, 64), [74994, 46782, 53037, 121102], [1, 512, 1, 128], 600, False),
+    ((64, 8, 128), [24651], [256], 264, True),                                    # nothing fits: the fastest cuts
+])
+def test_every_step_of_the_way_to_fewer_cuts_covers_the_batch(shape, ctx, ql, sms, spans):
+    """Whatever the planner falls back to, each (sequence, kv head, token range) keeps every key exactly once, in
+    order, and the workspaces stay within the reported sizes."""
+    ctx, ql, shape = np.array(ctx), np.array(ql), W.Shape(*shape, 16)
+    need = -(-(ctx + ql) // 16)
+    q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+    p = B.plan_host(shape, int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
+    host_bytes, dev_bytes = B.workspace_size(shape, int(need.sum()), len(ctx), int(ql.sum()), int(need.sum()), num_sms=sms)
+    assert p.info["device_bytes_used"] <= dev_bytes and p.info["host_bytes_used"] <= host_bytes
+    assert (p.info["num_items_tensor"] > 0) == spans
+    units = {}
+    for it in p.items():
+        units.setdefault((it["seq"], it["kv_head"], it["tok0"], it["ntok"]), []).append((it["kv0"], it["kv1"]))
+    for (b, _, tok0, ntok), segs in units.items():
+        segs.sort()
+        assert segs[0][0] == 0 and segs[-1][1] == ctx[b] + tok0 + ntok and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
+    for b in range(len(ctx)):
+        for h in range(shape.num_kv_heads):
+            toks = sorted((t, t + n) for s, hh, t, n in units if s == b and hh == h)
+            assert toks[0][0] == 0 and toks[-1][1] == ql[b] and all(x[1] == y[0] for x, y in zip(toks, toks[1:]))
