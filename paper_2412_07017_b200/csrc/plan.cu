@@ -7,6 +7,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <climits>
 #include <cstring>
 #include <vector>
@@ -846,7 +847,9 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     d.head_dim = shape->head_dim;
     d.group = G;
     d.num_pages = shape->num_pages;
-    d.sm_scale = shape->sm_scale > 0.f ? shape->sm_scale : 1.0f / sqrtf((float)shape->head_dim);
+    // at least the smallest normal number: the kernels flush smaller ones to zero, and the span body scales masked
+    // scores (-inf) as well
+    d.sm_scale = shape->sm_scale > 0.f ? std::max(shape->sm_scale, FLT_MIN) : 1.0f / sqrtf((float)shape->head_dim);
 
     asynclm_plan_info& info = plan->info;
     info.total_q = T;

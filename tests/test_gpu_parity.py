@@ -392,3 +392,16 @@ def test_launches_of_a_step(api, d, ctx, ql, tensor, append_launches):
     ref_pool, ref_out, _ = oracle_step(wl, st)
     assert np.array_equal(to_bits(pool), ref_pool)
     assert_close(to_bits(out), None, ref_out, None, what="replayed")
+
+
+# (no scale above the default ones: where one key dominates, outputs reach 4, where half a bf16 step is 0.008 and the
+# rounding of P as much again, which is more than the bar of 1e-2)
+@pytest.mark.parametrize("sm_scale", [1e-42, 1e-37, 0.05])
+@pytest.mark.parametrize("d", [64, 128])
+def test_any_positive_scale(d, sm_scale):
+    """A scale below the smallest normal number makes every visible key count alike; none of the hidden ones may."""
+    wl = W.make_single_step("scale", W.Shape(8, 2, d, 16), [100, 0, 700, 20], [40, 70, 1, 3], seed=11, poison_unused=True)
+    _, out_bits, lse, plan = gpu_step(wl, wl.steps[0], sm_scale=sm_scale)
+    _, ref_out, ref_lse = oracle_step(wl, wl.steps[0], sm_scale=sm_scale)
+    assert_close(out_bits, lse, ref_out, ref_lse, what=f"scale {sm_scale}")
+    assert 0 < plan.info["num_items_tensor"] < plan.info["num_items"]
