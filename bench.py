@@ -617,9 +617,7 @@ def run_timeline(args):
             "group1_waits_for_S": round(float(t[span, 15].mean())),
             "group0_softmax_of_tiles": round(float(t[span, 12].mean())),
             "group0_tiles": round(float(t[span, 13].mean()), 1),
-            "mma_thread_waits_for_item_start": round(float(t[span, 14].mean())),
-            "mma_thread_issues_QK (tensor-only kernel)": round(float(t[span, 2].mean())) if args.spans_only else None,
-            "mma_thread_issues_PV (tensor-only kernel)": round(float(t[span, 3].mean())) if args.spans_only else None},
+            "mma_thread_waits_for_item_start": round(float(t[span, 14].mean()))},
         "plan": {k: plan.info[k] for k in ("num_items", "num_items_tensor", "num_split_units")}}))
 
 

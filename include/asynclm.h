@@ -75,8 +75,8 @@ typedef struct asynclm_plan_options {
                                  the work items roughly fill the machine; a value >= the longest
                                  context disables splitting */
     int32_t tensor_min_rows;  /* new tokens of a sequence use the span body (tcgen05 MMA, 128
-                                 query rows to a tile) when G * q_len >= this; 0 = default: 32.
-                                 Below it they use the warp body (warp-level MMA with the keys
+                                 query rows to a tile) when G * q_len >= this; 0 = default: 32
+                                 at head_dim 128, 64 at head_dim 64.  Below it they use the warp body (warp-level MMA with the keys
                                  on the M axis, 8 / G tokens to a unit), which streams K/V at
                                  the memory rate for every supported G and is where decode
                                  rows always go by default.  INT32_MAX keeps every row on the
@@ -157,11 +157,18 @@ int asynclm_plan_workspace_size(const asynclm_shape* shape, const asynclm_plan_o
  * (long contexts are split; partial results are merged by log-sum-exp inside asynclm_attn_mixed),
  * and decides who runs what: span tiles are packed whole where possible, largest first, onto as
  * few persistent CTAs as a load limit allows (a span of two row tiles that does not fit is divided
- * by rows before it is cut by keys); decode rows and short spans are cut into chunks (long pieces
- * first, short ones from a few units at the end) that the CTAs take from a queue at run time, one
- * atomic add per chunk, so that no cost model has to predict how fast each SM streams.  Results do
- * not depend on which CTA ran which chunk: partial results are indexed by chunk and merged in
- * chunk order.  Then ONE host->device copy of the packed plan is enqueued on `stream`.
+ * by rows, or cut by keys where the pieces are long, from about 8 K keys); decode rows and short
+ * spans are cut into chunks (long pieces first, short ones from a few units at the end) that the CTAs
+ * take from a queue at run time, one atomic add per chunk, so that no cost model has to predict how
+ * fast each SM streams.  Results do not depend on which CTA ran which chunk: partial results are
+ * indexed by chunk and merged in chunk order.  Then ONE host->device copy of the packed plan is
+ * enqueued on `stream`.
+ *
+ * Where the cuts would leave more partial results than asynclm_attn_mixed_static has room for, fewer of
+ * the long spans are cut by keys, so that the plan serves that call too (a span divided by rows instead
+ * reads its keys twice).  If none at all is still too much, the decode queue gets longer pieces, and at
+ * head_dim 64 spans run on the warp body; a plan that fits in no way is made without regard to that
+ * call.
  *
  * A plan holds a few counters in its device workspace (queue position, arrivals per split unit)
  * that every launch leaves at zero; launches that use the same plan must therefore not overlap on

@@ -32,9 +32,10 @@
 // 128-key tiles tensor memory holds one S per group (at head_dim 128) and each group's softmax and MMAs
 // took turns.  Per 64 keys of both row tiles (cycles): the exponential unit needs 1024, the tensor pipe
 // 1280 (64-column Q K^T is bound by its operands in shared memory), a lone group's softmax 1130, and a tile
-// pair takes 1900-2000: the MMA warps need about 100 cycles to issue an MMA, and the groups' exponentials
-// collide in part.  8192 tokens of one sequence (32 / 8 heads, head_dim 128): 522 us, 530 before;
-// head_dim 64 had no tensor-core body before (32 sequences, 8 spans: 163 -> 56 us).
+// pair takes 2060 on a CTA alone and 2370 when all CTAs stream: the MMA warps need about 100 cycles to issue
+// an MMA, and the groups' exponentials collide in part.  Attention of 8192 tokens of one sequence (32 / 8 heads,
+// head_dim 128): 530-575 us, the power cap moves it; head_dim 64 had no tensor-core body before (32 sequences,
+// 8 spans: 163 -> 58 us).
 // All hand-offs are mbarriers with bounded waits; a wait that runs out sets the plan's status word
 // and a CTA-wide abort flag, every role falls through to the common exit, and the tensor memory is
 // released there.

@@ -1,8 +1,8 @@
 // The attention kernels' entry points and launchers.
 //
-// Three kernels are built from two bodies (attn_append_tc.cuh: tensor-core span tiles,
-// attn_decode.cuh: CUDA-core decode rows):
-//   attn_fused_kernel      a persistent CTA first runs its tensor-core items, then its CUDA-core items
+// Three kernels are built from two bodies (attn_append_tc.cuh: span tiles on tcgen05, attn_decode.cuh: decode
+// rows and short spans on warp-level MMAs):
+//   attn_fused_kernel      a persistent CTA first runs its span items, then takes warp-body items
 //                          (a CTA without span tiles skips the tensor-memory set-up altogether).
 //                          One launch instead of two: the fixed cost of a launch (about 10 us of
 //                          start-up and tail per kernel at 148 CTAs) is paid once, and a CTA that is

@@ -93,23 +93,32 @@ static size_t partial_bytes(int64_t rows, int group, int head_dim) {
 // kTailChunksPerCta per CTA and never shorter than kMinChunkTiles tiles (see deal_dynamic).
 constexpr int kTailChunksPerCta = 2;
 constexpr int kMinChunkTiles = 4;
-// The other units are cut into pieces of at most kBulkTiles tiles (70-110 us) or an eighth of a CTA's share: with
+// The other units are cut into pieces of at most kBulkTiles tiles (50-90 us) or an eighth of a CTA's share: with
 // contexts of 10^5 tokens, pieces of two fifths of the step, which used to be the only limit, left some CTAs on
-// a last piece of half a millisecond.  32 and 128 tiles measure the same.
+// a last piece of half a millisecond.  (8 sequences of 32-131 K tokens, two 256-token spans: 1083 us of attention
+// a layer without this limit, 910-970 with it, run to run; 32 and 128 tiles the same; 128 sequences of 64 / 8
+// heads 489 at 32 tiles, 480 at 64 and 128.)
 constexpr int kBulkTiles = 64;
 // Span units of two row tiles are cut by keys instead of divided by rows where the pieces are at least this
-// long, because the divided halves each stream the keys: a 128-key tile takes a CTA 2.3 us for two row tiles
-// and 1.5 us for one, when all CTAs stream.  (8 sequences of 32-131 K tokens, two 256-token spans: 1080 us a
-// step with divided units, 887 with cut ones.)  Below, the partial rows and their merge cost more than they save
-// (32 sequences of up to 4 K tokens, 8 spans: 65 us divided, 72 cut).
+// long, because the divided halves each stream the keys: 128 keys take a CTA 2.4 us for two row tiles and
+// 1.55 us for one, when all CTAs stream.  (8 sequences of 32-131 K tokens, two 256-token spans: 1065-1096 us of
+// attention a layer with divided units, 910-970 with as many cut ones as the fixed array has room for.)  Below,
+// the partial rows and their merge cost more than they save (32 sequences of up to 4 K tokens, 8 spans: 62.5 us
+// divided, 68.7 cut).
 constexpr int kLongPieceTiles = 64;
 // Tokens of one warp-body unit: its MMAs have 8 (token, head) columns.
 static int warp_unit_tokens(int group) { return 8 / group; }
 
-// Upper bounds on what the automatic policy produces.  Warp body: the short chunks are at least
-// (all tiles) / (12 CTAs) long, so even a single unit that holds all the work yields at most 12 per
-// CTA; a long piece is at least two fifths of a CTA's share.  Span body: a unit is cut only where it
-// is larger than a CTA's share.
+// Upper bounds on what the automatic policy produces, for C CTAs and W tiles of warp-body work in all.
+//   Warp body, only units longer than 1.5 pieces are cut, into ceil(t / piece) <= 1.5 t / piece pieces (the
+// worst is just over two).  A long piece is at least min(2/5 of a CTA's share, max(kBulkTiles, an eighth of
+// it)) >= W / (8 C) tiles: at most 12 C pieces.  A short one is at least W / (12 C) less the rounding, and
+// never below kMinChunkTiles, so below 1.25 times as many: 15 C pieces if one unit holds all the work; a unit
+// goes to the short ones only until they hold a sixth of W, so all but the last add at most 1.5 * 15 C / 6.
+// The worst mixture, a sixth of W in small units and the rest in the last one, stays below 17 C.
+//   Span body: a unit is cut only if it is longer than what a fresh CTA takes, into pieces longer than half of
+// that (or of one tile, which each need a CTA of their own), so a CTA holds fewer than three.
+//   A unit that is not cut is one item, and a divided unit is two; only cut units hold partial rows.
 static int64_t auto_item_bound(int64_t units, int ctas) { return 2 * units + (int64_t)20 * ctas; }
 static int64_t auto_partial_row_bound(int ctas, int group) {
     return (int64_t)20 * ctas * warp_unit_tokens(group) + (int64_t)3 * ctas * tensor_tile_tokens(group);
@@ -237,7 +246,11 @@ void cut_and_deal(const std::vector<int>& unit_ids, std::vector<UnitBuild>& unit
 }
 
 
-// Measured costs of the attention kernels on B200, in nanoseconds, used only to size the span CTAs.
+// Costs of the attention kernels on B200 as the packing sees them, in nanoseconds, used only to size the span
+// CTAs.  The span body's were measured at head_dim 128 on a form of it with 128-key tiles, and the margins below
+// were chosen with them.  The present body takes, per 128 keys with one | two row tiles: 1.27 | 2.10 us on a CTA
+// alone, 1.34 | 2.11 on 74, 1.55 | 2.42 on all 148, and 3.5 | 4.3 us to pass from one item to the next; at
+// head_dim 64 1.08 | 1.70, 1.15 | 2.03, 1.17 | 2.02 and 2.1 | 2.5.
 struct PathCost {
     int gran;            // tokens per tile of the path (cuts fall on multiples of it)
     int64_t tile_ns;     // one tile in steady state
@@ -251,9 +264,10 @@ constexpr int64_t kTensorDualTileNs = 2435;   // a KV tile of an item with two r
 // the memory system (64 KB per tile and SM); the producers run ahead across item boundaries.
 constexpr PathCost kTensorOnlyCost{128, 1543, 8000, 2400};
 constexpr int64_t kTensorOnlyDualTileNs = 3126;
-// Warp body: 64 KB per 128-key tile.  It is bound by memory, so its tile time depends on how many SMs
-// stream at once: 1.45 us when all 148 do, 1.05 us (62 KB/us, about what one SM can stream) when
-// half of them run span tiles, which draw little bandwidth.  The model takes the latter figure.
+// Warp body: 64 KB per 128-key tile (32 KB at head_dim 64).  It is bound by memory, so its tile time depends on
+// how many SMs stream at once: 1.39 us when all 148 do, 1.05 us (62 KB/us) when half of them run span tiles,
+// which draw some bandwidth too, 0.77 us for 74 and 0.68 for one by themselves; at head_dim 64 0.77, 0.75 and
+// 0.67.  The model takes the second figure.
 constexpr PathCost kWarpCost{128, 1050, 400, 2000};
 // No step ends before its bytes have crossed the memory bus: K/V pages stream at about 6 bytes per
 // nanosecond on this access pattern (4 KB runs through a shuffled page table), after about 3 us in
@@ -263,8 +277,10 @@ constexpr PathCost kWarpCost{128, 1050, 400, 2000};
 constexpr int64_t kDramBytesPerUs = 6000000;
 // A span CTA that finishes early joins the queue; one that finishes late delays the whole step, and the
 // span body slows down by up to 15 % when the warp-body CTAs saturate the memory.  So the span CTAs
-// are filled to the load limit divided by this margin (in 1/64).  (128 sequences of 64 / 8 heads, 13 spans:
-// 524 us a step at 72, 495 at 80, 479 at 88, 482 at 96; smaller batches do not care.)
+// are filled to the load limit divided by this margin (in 1/64).  Attention of a layer in us at 72 | 80 | 88 | 96:
+// 128 sequences of 64 / 8 heads with 13 spans 520 | 490 | 480 | 482, 32 sequences of 32 / 8 heads with 8 spans 63
+// | 62 | 63 | 63, at head_dim 64 53 | 53 | 58 | 53 (the costs above are head_dim 128's: how many span CTAs come out
+// there, 68 at 88 and 96 or 104 at the others, is chance).
 constexpr int64_t kSpanMargin64 = 88;
 // The same, for the decision to divide a unit by rows: a unit just above the span CTAs' share is better cut by
 // the packing than divided, its halves would stream the keys twice.
@@ -314,9 +330,9 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     const int64_t warp_ns = warp_tiles * kWarpCost.tile_ns + (int64_t)ids_warp.size() * 2 * kWarpCost.item_ns;
 
     // ---- span units with two row tiles that would not fit a CTA whole are divided by rows into two
-    // units of one row tile each (same CTA-time in total, and the second reader of the keys finds most
-    // of them in L2) rather than by keys, which would cost fp32 partial rows and a merge.  The limit
-    // used for the decision is the lower bound of the one found below.
+    // units of one row tile each (the second reader of the keys finds most of them in L2) rather than by
+    // keys, which would cost fp32 partial rows and a merge, unless the pieces would be long (kLongPieceTiles).
+    // The limit used for the decision is the lower bound of the one found below.
     {
         int64_t work = warp_ns;
         for (int id : ids_tensor)
@@ -442,8 +458,8 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     // ---- warp-body chunks.  An item boundary costs time and a split unit costs partial rows and a
     // merge, so most of the work stays in long pieces: a few units, a sixth of all tiles, are cut into
     // short chunks that go to the END of the queue, where they even out the CTAs' finishing times;
-    // every other unit stays whole unless it is longer than two fifths of the step, in which case it is
-    // cut into equal pieces.  The queue holds the long pieces longest first, then the short chunks.
+    // every other unit stays whole unless it is longer than two fifths of the step (or than kBulkTiles tiles
+    // and an eighth of a CTA's share), in which case it is cut into equal pieces.  The queue holds the long pieces longest first, then the short chunks.
     std::vector<int> warp_order(ids_warp);
     std::stable_sort(warp_order.begin(), warp_order.end(),
                      [&](int x, int y) { return units[x].n_keys > units[y].n_keys; });
@@ -864,7 +880,7 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     info.num_ctas_tensor = ctas_tensor;
     info.num_items_tensor = d.num_items_tensor;
     info.launches_append = T > 0 ? 1 : 0;
-    // span tiles and decode rows share one fused launch when a step has both (head_dim 128)
+    // span tiles and decode rows share one fused launch when a step has both
     info.launches_attn = ((n_items_cuda > 0 || d.num_items_tensor > 0) ? 1 : 0) + (merge_blocks.empty() ? 0 : 1);
     info.num_sms = n_sms;
     info.total_kv_tokens = total_kv;

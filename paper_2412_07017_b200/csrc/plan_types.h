@@ -74,7 +74,7 @@ struct DevPlan {
     const int32_t* row_seq;          // [T] sequence of each new token row
     const int64_t* row_slot;         // [T] page * 16 + slot where the row's K/V go (resolved by the planner)
     const Unit* units;
-    const Item* items;               // CUDA-core items first (grouped by CTA), then tensor items
+    const Item* items;               // warp-body items first, then span items (grouped by CTA)
     const Work* works;               // [num_items] the same items, resolved for the kernels
     const int32_t* cta_heads;        // [num_ctas][kHeadWords], see above
     const int32_t* cta_indptr_cuda;  // [num_ctas_cuda + 1] into items

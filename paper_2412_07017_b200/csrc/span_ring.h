@@ -11,6 +11,9 @@
 //     order, ahead of a tile of this item that the same MMA warp has waited for.
 // One ring for both kinds does not have the first property: a slot would pass from V to K and back to V
 // without the V producer having waited for the tile in between, whose fill and release it does not see.
+// Five slots each at head_dim 128 hold as many tiles, in the order of consumption, as one ring of ten (24 sequences
+// with spans of up to 96 tokens, four layers: 399 us a pass with one ring, 390 with two; 32 layers of a mixed
+// batch: 2284 and 2245-2275).
 #pragma once
 
 #ifdef __CUDACC__

@@ -374,3 +374,25 @@ def test_every_step_of_the_way_to_fewer_cuts_covers_the_batch(shape, ctx, ql, sm
         for h in range(shape.num_kv_heads):
             toks = sorted((t, t + n) for s, hh, t, n in units if s == b and hh == h)
             assert toks[0][0] == 0 and toks[-1][1] == ql[b] and all(x[1] == y[0] for x, y in zip(toks, toks[1:]))
+
+
+def test_random_batches_stay_within_the_reported_workspaces():
+    """Partial rows and items against the planner's bounds, over shapes, SM counts and lengths: contexts from
+    nothing to 131 K, decode rows, short and long spans, paused sequences."""
+    rng = np.random.default_rng(97)
+    for _ in range(80):
+        hq, hkv = [(8, 8), (8, 4), (32, 8), (16, 2), (8, 1)][rng.integers(5)]
+        shape = W.Shape(hq, hkv, int(rng.choice([64, 128])), 16)
+        n = int(rng.choice([1, 2, 5, 17, 40]))
+        hi = int(rng.choice([60, 2000, 20000, 131072] if n < 17 else [60, 2000, 20000]))
+        ctx = rng.integers(0, hi + 1, n)
+        ql = np.where(rng.random(n) < 0.4, rng.integers(0, int(rng.choice([4, 40, 600])) + 1, n), 1)
+        need = -(-(ctx + ql) // 16)
+        q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+        sms = int(rng.choice([1, 2, 9, 148, 160]))
+        p = B.plan_host(shape, int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
+        host_bytes, dev_bytes = B.workspace_size(shape, int(need.sum()), n, int(ql.sum()), int(need.sum()), num_sms=sms)
+        what = (shape, ctx.tolist(), ql.tolist(), sms)
+        assert p.info["device_bytes_used"] <= dev_bytes and p.info["host_bytes_used"] <= host_bytes, what
+        assert p.info["partial_rows"] <= 20 * sms * (8 // shape.group) + 3 * sms * (256 // shape.group), what
+        assert p.info["num_items"] <= 2 * int(ql.sum()) * hkv + 20 * sms, what
