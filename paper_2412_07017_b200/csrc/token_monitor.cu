@@ -86,12 +86,16 @@ template <> struct Vec<float> {
 
 // Largest ordinary element (no CML token) of vectors [j_begin, j_end) of a row (stride of the CTA's
 // threads), lowest id among equals.  Per vector only its maximum is computed; the position inside the
-// best vector is found at the end by looking at that one vector again.
+// best vector is found at the end by looking at that one vector again.  Only the vectors that hold a CML token
+// have their elements looked at: when all vectors of a stretch with one were, the CTA that had it finished
+// last (bf16 rows of 128 256 without a forbidden winner, 256 | 32 | 8 | 1 of them, us a call from a graph:
+// 20.5 | 9.0 | 6.9 | 5.8, 15.8 | 7.1 | 6.0 | 4.9 now).
 template <typename T>
 __device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, const asynclm_cml_tokens& tok) {
     constexpr int VEC = Vec<T>::N;
     const uint4* v4 = reinterpret_cast<const uint4*>(row);
     const int sv[5] = {tok.call / VEC, tok.intr / VEC, tok.trap / VEC, tok.end / VEC, tok.head / VEC};
+    auto holds_special = [&](int j) { return j == sv[0] || j == sv[1] || j == sv[2] || j == sv[3] || j == sv[4]; };
     float bv = -INFINITY;
     int bj = -1;
     for (int b0 = j_begin; b0 < j_end; b0 += kMonVecs * kMonThreads) {
@@ -110,7 +114,7 @@ __device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, c
         for (int u = 0; u < kMonVecs; ++u) {
             const int j = j0 + u * kMonThreads;
             float m = Vec<T>::vmax(w[u]);
-            if (special) {
+            if (special && holds_special(j)) {
                 m = -INFINITY;
 #pragma unroll
                 for (int k = 0; k < VEC; ++k)
@@ -122,9 +126,10 @@ __device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, c
     Best best{-INFINITY, INT_MAX};
     if (bj >= 0) {
         const uint4 w = ldg_nc_v4(v4 + bj);
+        const bool mixed = holds_special(bj);
 #pragma unroll
         for (int k = VEC - 1; k >= 0; --k)
-            if (Vec<T>::at(w, k) == bv && !is_special(bj * VEC + k, tok)) best = Best{bv, bj * VEC + k};
+            if (Vec<T>::at(w, k) == bv && !(mixed && is_special(bj * VEC + k, tok))) best = Best{bv, bj * VEC + k};
     }
     return best;
 }
@@ -153,7 +158,7 @@ __device__ __forceinline__ Best block_best(Best best, float* sv, int* si) {
 // barrier, and the two state pointers are not __restrict__).
 // The result does not depend on arrival order.  (Scanning all tokens alike and looking at a row a second
 // time when a forbidden token had won kept one CTA busy with a whole row after all others had left:
-// 256 rows of 128 256 bf16 with a few such rows took 31 us a call, 21 us now.)
+// 256 rows of 128 256 bf16 with a few such rows took 40 us a call on cold inputs, 25 now.)
 template <typename T>
 __global__ void __launch_bounds__(kMonThreads)
 token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride, asynclm_cml_tokens tok,
