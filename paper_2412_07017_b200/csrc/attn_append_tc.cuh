@@ -22,24 +22,30 @@
 //                   values to an instruction and reductions run in independent chains.
 //                   At the end of an item the rows go out through the group's (now idle) Q tile in
 //                   shared memory, so that every global store writes whole 128-byte lines.
-//   warps 8, 10     producers of K tiles and of V tiles: 16-byte cp.async copies (fully coalesced,
-//                   whole rows, 512 bytes per warp instruction) that write the 128-byte-swizzled operand
-//                   layout and complete on the slot's mbarrier.  K and V have a ring of 80 KiB each
-//                   (see span_ring.h).
-//   warps 9, 11     issue the MMAs, one warp per softmax group.  Warp 9 owns the tensor-memory allocation.
+//   warps 8, 10     producers of K tiles and of V tiles: one TMA copy a page, completing on the slot's mbarrier (an
+//                   unfinished last V page goes row by row through cp.async, with zeros behind the end).  K and V
+//                   have a ring of 80 KiB each (see span_ring.h).
+//   warps 9, 11     issue the MMAs, one warp per softmax group, by turns.  Warp 9 owns the tensor-memory allocation.
 // Why tiles of 64 keys: with two S buffers per group, the Q K^T of the tile after next is issued behind the
 // P V of the current one, and the softmax of the next tile, whose S is complete, runs meanwhile; with
 // 128-key tiles tensor memory holds one S per group (at head_dim 128) and each group's softmax and MMAs
-// took turns.  Per 64 keys of both row tiles (cycles): the exponential unit needs 1024, the tensor pipe
-// 1280 (64-column Q K^T is bound by its operands in shared memory), a lone group's softmax 1130, and a tile
-// pair takes 2060 on a CTA alone and 2370 when all CTAs stream: the MMA warps need about 100 cycles to issue
-// an MMA, and the groups' exponentials collide in part.  Attention of 8192 tokens of one sequence (32 / 8 heads,
-// head_dim 128): 530-575 us, the power cap moves it; head_dim 64 had no tensor-core body before (32 sequences,
-// 8 spans: 163 -> 58 us).
+// took turns.  Per 64 keys of both row tiles (cycles, head_dim 128): the exponential unit needs 1024, the tensor pipe
+// 1280 (64-column Q K^T is bound by its operands in shared memory), a lone group's softmax about 1150.
+// Why the MMA warps take turns: the pipe serves two warps that issue at once in turn about, so both were done
+// at the same time, and then both waited for tiles and scores while the pipe ran dry; the groups' exponentials
+// fell together as well.  Turns keep the groups half a period apart.  What a turn has to work out in
+// front of its first MMA counts, too: positions in the rings are carried along instead of divided out.
+// A tile pair takes 1500-1640 cycles on a CTA alone (2050 with both warps issuing at once and cp.async copies), a
+// tile of one row tile 890 (1250; with a copy for each half of a page 1150: see tma_page); at head_dim 64 1520
+// (1700) and 900-940 (1070).  When all CTAs stream, power holds the clock at about 1.5 GHz: attention of 8192 tokens
+// of one sequence (32 / 8 heads, head_dim 128) 530-570 -> 490-520 us, 24 sequences with spans of 33-96 tokens over 1-3 K keys
+// 82 -> 71-74 us a layer.
 // All hand-offs are mbarriers with bounded waits; a wait that runs out sets the plan's status word
 // and a CTA-wide abort flag, every role falls through to the common exit, and the tensor memory is
 // released there.
 #pragma once
+#include <cuda.h>
+
 #include <climits>
 
 #include "common.cuh"
@@ -64,8 +70,12 @@ struct Geometry {
     static constexpr int HALVES = D / 64;                                  // 128-byte pieces of a row
     static constexpr uint32_t QHALF_BYTES = kRows * 128;                   // one 64-value half of a Q tile
     static constexpr uint32_t QTILE_BYTES = HALVES * QHALF_BYTES;
-    static constexpr uint32_t HALF_BYTES = kTile * 128;                    // one 64-value half of a K or V tile
-    static constexpr uint32_t SLOT_BYTES = HALVES * HALF_BYTES;
+    // A K or V tile is its pages one after the other, a page its two groups of 8 rows, a group its halves of 64 values
+    // (8 rows of 128 bytes, swizzled): so one TMA copy lands a whole page, and groups still lie at one stride.
+    static constexpr uint32_t ATOM_BYTES = 8 * 128;                        // one half of a group
+    static constexpr uint32_t GROUP_BYTES = HALVES * ATOM_BYTES;
+    static constexpr uint32_t PAGE_BYTES = 2 * GROUP_BYTES;
+    static constexpr uint32_t SLOT_BYTES = kTile / kPage * PAGE_BYTES;
     static constexpr int RING = ring_slots(D);                             // slots of the K ring and of the V ring
     static constexpr uint32_t OFF_Q = 0;                                   // Q[0], Q[1]
     static constexpr uint32_t OFF_RING = OFF_Q + 2 * QTILE_BYTES;
@@ -75,7 +85,8 @@ struct Geometry {
     static constexpr uint32_t OFF_BAR = 224 * 1024;
     static_assert(OFF_RING + 2 * RING * SLOT_BYTES <= OFF_BAR, "barriers behind the tiles");
     // S, P and last-P-V hand-offs exist per group b and buffer s: index 2 * b + s
-    enum Bar { kQFull = 0, kStats, kOFree, kPFull0, kPvDone0 = kPFull0 + 4, kSFull0 = kPvDone0 + 4,
+    // (kToken0 + b: it is the turn of group b's MMA warp)
+    enum Bar { kQFull = 0, kStats, kOFree, kToken0, kPFull0 = kToken0 + 2, kPvDone0 = kPFull0 + 4, kSFull0 = kPvDone0 + 4,
                kRingFull0 = kSFull0 + 4, kRingEmpty0 = kRingFull0 + 2 * RING, kMmaDrain = kRingEmpty0 + 2 * RING, kNumBars };
     static constexpr uint32_t OFF_TMEM_PTR = OFF_BAR + 8 * kNumBars;
     static constexpr uint32_t OFF_ABORT = OFF_TMEM_PTR + 8;
@@ -158,6 +169,16 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32
 // Arrive on the mbarrier once all cp.async copies issued so far by this thread have landed.
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// A page's 16 K or V rows of one kv head, `block` = (2 * page + K|V) * Hkv + head, land as [2 groups of 8 rows][halves]
+// [8 rows][128 bytes], 16-byte pieces XOR-swizzled by row (see make_kv_maps).  One SM's TMA unit takes about as long
+// for a copy of 2 KB (35 ns) as for one of 4 KB (44 ns): with a copy for each half of a page, one SM
+// streamed 57 KB/us, with one for both 92.  No multicast.
+__device__ __forceinline__ void tma_page(uint32_t dst, const CUtensorMap* map, int block, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+        ::"r"(dst), "l"(map), "r"(0), "r"(0), "r"(0), "r"(0), "r"(block), "r"(bar) : "memory");
 }
 
 // Shared-memory matrix descriptor, 128-byte swizzle, descriptor version 1.
@@ -284,7 +305,7 @@ __device__ __forceinline__ TItem load_titem(const Work* rec, bool valid) {
 
 // The whole kernel body, called by all twelve warps with `smem` 1024-byte aligned.
 template <int D, int G>
-__device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* __restrict__ q,
+__device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* span_map, const __nv_bfloat16* __restrict__ q,
                                         const __nv_bfloat16* pool,
                                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                                         uint8_t* smem) {
@@ -308,17 +329,23 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         mbar_init(bar(Geo::kQFull), 256);
         mbar_init(bar(Geo::kStats), 256);
         mbar_init(bar(Geo::kOFree), 256);
+        mbar_init(bar(Geo::kToken0), 1);
+        mbar_init(bar(Geo::kToken0 + 1), 1);
         for (int b = 0; b < 4; ++b) {
             mbar_init(bar(Geo::kPFull0 + b), 4);      // one arrival per warp of the group
             mbar_init(bar(Geo::kPvDone0 + b), 1);
             mbar_init(bar(Geo::kSFull0 + b), 1);
         }
-        for (int s = 0; s < 2 * Geo::RING; ++s) { mbar_init(bar(Geo::kRingFull0 + s), 32); mbar_init(bar(Geo::kRingEmpty0 + s), 2); }
+        for (int s = 0; s < 2 * Geo::RING; ++s) {
+            mbar_init(bar(Geo::kRingFull0 + s), s < Geo::RING ? 1 : 33);      // V tiles: see the producers
+            mbar_init(bar(Geo::kRingEmpty0 + s), 2);
+        }
         mbar_init(bar(Geo::kMmaDrain), 2);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
+    if (threadIdx.x == kProducerWarpK * 32) asm volatile("prefetch.tensormap [%0];" ::"l"(span_map));
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(sbase + Geo::OFF_TMEM_PTR), "r"(kTmemCols) : "memory");
@@ -341,7 +368,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         };
         constexpr int kPagesPerTile = kTile / kPage;          // 4
         constexpr int kGroupTiles = 32 / kPagesPerTile;       // 8
-        constexpr int kChunks = D / 8, kRowsPerOp = 32 / kChunks;      // 16-byte chunks of a row; rows a warp instruction moves
+        constexpr int kChunks = D / 8, kRowsPerOp = 32 / kChunks;      // cp.async: 16-byte chunks of a row; rows a warp instruction moves
         bool ok = true;
         int n = 0;                                             // tiles issued so far (all items)
         int ev = 0;      // time-stamp build: event log position (lane 0 of a producer)
@@ -362,28 +389,43 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
                     ok = mbar_wait_warp(bar(Geo::kRingEmpty0 + s), ((uint32_t)ring_use(n, Geo::RING) & 1u) ^ 1u, abort_flag, p.status, 11 + which);
                     if (!ok) break;
                     if (lane == 0 && which == 0) trace_event(9, ev, 42);
-                    // lane -> 16-byte chunk c of a row: a warp instruction moves whole rows, 512 bytes in all
-                    const int c = lane % kChunks;
-                    const uint32_t dst_half = ring + s * Geo::SLOT_BYTES + (uint32_t)(c >> 3) * Geo::HALF_BYTES;
-                    for (int pg = 0; pg < npages; ++pg) {
-                        int64_t page = __shfl_sync(0xffffffffu, pages_cur, (t - t0) * kPagesPerTile + pg);
-                        const bool page_good = page_ok(page, p.num_pages, p.status, kStatusBadPageSpan);      // checked build only
-                        if (!page_good) page = 0;      // the tile gets zeros in its place
-                        const uint8_t* src_page = reinterpret_cast<const uint8_t*>(
-                            pool + pool_row_offset(page, which, cur.kv_head, 0, Hkv, D));
+                    const uint32_t full = bar(Geo::kRingFull0 + s), slot_addr = ring + s * Geo::SLOT_BYTES;
+                    // Slots past the item's end hold anything.  K's only reach scores that the softmax masks, but 0 * NaN
+                    // would poison P V, so the item's last V page, if it is not full, is copied row by row with zeros
+                    // behind the end.  A V barrier takes 33 arrivals: one with the byte count of the TMA copies, and one
+                    // of each lane's cp.async copies or all 32 at once where there are none.
+                    const bool ragged = which == 1 && (rows & (kPage - 1)) != 0;
+                    const int npages_tma = npages - (ragged ? 1 : 0);
+#ifdef ASYNCLM_DEBUG
+                    // checked build: a test may ask for one hand-off to be left out, to see a bounded wait run out
+                    const bool stall = which == 0 && blockIdx.x == 0 && p.debug_stall_tile == n + 1;
+#else
+                    constexpr bool stall = false;
+#endif
+                    if (lane == 0 && !stall) {
+                        mbar_arrive_expect_tx(full, (uint32_t)npages_tma * Geo::PAGE_BYTES);
+                        if (which == 1 && !ragged) mbar_arrive_n(full, 32);
+                    }
+                    __syncwarp();
+                    int page = __shfl_sync(0xffffffffu, pages_cur, (t - t0) * kPagesPerTile + min(lane, npages - 1));
+                    // checked build only: a bad id is replaced by page 0 (the copy must happen: the barrier counts its bytes)
+                    if (lane < npages && !page_ok(page, p.num_pages, p.status, kStatusBadPageSpan)) page = 0;
+                    if (lane < npages_tma && !stall)
+                        tma_page(slot_addr + (uint32_t)lane * Geo::PAGE_BYTES, span_map, (2 * page + which) * Hkv + cur.kv_head, full);
+                    if (ragged) {
+                        page = __shfl_sync(0xffffffffu, page, npages - 1);
+                        const uint8_t* src_page = reinterpret_cast<const uint8_t*>(pool + pool_row_offset(page, which, cur.kv_head, 0, Hkv, D));
+                        // lane -> 16-byte chunk c of a row: a warp instruction moves whole rows, 512 bytes in all
+                        const int c = lane % kChunks;
 #pragma unroll
                         for (int rr = 0; rr < kPage / kRowsPerOp; ++rr) {
                             const int slot = rr * kRowsPerOp + lane / kChunks;
-                            const int row = pg * kPage + slot;
-                            cp_async16(dst_half + (uint32_t)row * 128u + (uint32_t)(((c & 7) ^ (row & 7)) << 4),
-                                       src_page + slot * (D * 2) + c * 16, (row < rows && page_good) ? 16u : 0u);
+                            cp_async16(slot_addr + (uint32_t)(npages - 1) * Geo::PAGE_BYTES + (uint32_t)(slot >> 3) * Geo::GROUP_BYTES +
+                                           (uint32_t)(c >> 3) * Geo::ATOM_BYTES + (uint32_t)(slot & 7) * 128u + (uint32_t)(((c & 7) ^ (slot & 7)) << 4),
+                                       src_page + slot * (D * 2) + c * 16, (npages - 1) * kPage + slot < rows ? 16u : 0u);
                         }
+                        cp_async_arrive(full);
                     }
-#ifdef ASYNCLM_DEBUG
-                    // checked build: a test may ask for one hand-off to be left out, to see a bounded wait run out
-                    if (!(which == 0 && blockIdx.x == 0 && p.debug_stall_tile == n + 1))
-#endif
-                    cp_async_arrive(bar(Geo::kRingFull0 + s));
                     if (lane == 0 && which == 0) trace_event(9, ev, 44);
                     // page ids of the next group of tiles (or of the next item), requested only after this
                     // group's first tile is on its way: the next item's descriptor may still be in flight
@@ -400,11 +442,14 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         if (!ok) {
             // aborted: let the loads already issued land before shared memory goes away
             asm volatile("cp.async.wait_all;" ::: "memory");
+            const long long t0 = clock64();
+            for (int k = max(0, n - Geo::RING); k < n; ++k)
+                while (!mbar_try_wait(bar(Geo::kRingFull0 + ring_slot(which, k, Geo::RING)), (uint32_t)ring_use(k, Geo::RING) & 1u) &&
+                       clock64() - t0 < kWaitCycles) {}
         }
       } else {
         // ------------------------------------------------------------------ MMA issuers
-        // One warp per softmax group, running convergently, issues the group's MMAs through an elected lane.
-        // (One warp for both groups was the limit: 3000 cycles for the turns of a tile pair, 2000 with two.)  A
+        // One warp per softmax group, running convergently, issues the group's MMAs through an elected lane.  A
         // turn is one KV tile of the group: its P V and the Q K^T of the group's next tile
         // but one into the S buffer that the P V has just read (MMAs of one thread execute in issue order).
         // While the tensor core works on a turn, the group runs the softmax of its other buffer: neither
@@ -415,6 +460,14 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
         int base = 0;             // KV tiles before this item
         int cnt = 0;              // tiles of the group before this item: S buffer and phase of the hand-offs
         int item_no = 0;
+        // The warps take turns, group 0 first, whether they have MMAs to issue or not: turn n of warp 1 follows turn n of
+        // warp 0, turn n of warp 0 follows turn n - 1 of warp 1.
+        int turn_no = 0;
+        auto take_token = [&](bool& good) {
+            good = good && (b + turn_no == 0 || mbar_wait_spin(bar(Geo::kToken0 + b), (uint32_t)(turn_no + b + 1) & 1u, abort_flag, p.status, 28));
+            ++turn_no;
+        };
+        auto pass_token = [&]() { if (lane == 0) mbar_arrive(bar(Geo::kToken0 + (b ^ 1))); };
         constexpr uint32_t idesc_pv = instr_desc(D, 1);
         const uint32_t ocol = tmem + kColO + (uint32_t)(D * b);
         TItem it_next = load_titem(head_work, i0 < i1);
@@ -434,13 +487,22 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             tr_item += trace_clock() - t_item;
             if (ok) tc_fence_after();
             const uint64_t qd = smem_desc(sbase + Geo::OFF_Q + (dual ? (uint32_t)b * Geo::QTILE_BYTES : 0u), 16, 1024);
-            auto tile_pages = [&](int j) { return (min(kTile, it.kv_end - (it.kv0 + j * kTile)) + kPage - 1) / kPage; };
-            auto wait_tile = [&](int which, int t, int code) {
+            const int last_pages = (it.kv_end - (it.kv0 + (ntiles - 1) * kTile) + kPage - 1) / kPage;      // of the item's last tile
+            const uint32_t idesc_last = instr_desc(16u * (uint32_t)last_pages, 0);
+            const bool ragged = (it.kv_end & (kPage - 1)) != 0;
+            // where the group's next K and V tile lie: slot, and the parity of its phase
+            struct Place { int slot; uint32_t parity; };
+            Place kp{ring_slot(0, base + (dual ? 0 : b), Geo::RING), (uint32_t)ring_use(base + (dual ? 0 : b), Geo::RING) & 1u}, vp = kp;
+            auto next_place = [&](Place& x) {
+                x.slot += dual ? 1 : 2;
+                if (x.slot >= Geo::RING) { x.slot -= Geo::RING; x.parity ^= 1u; }
+            };
+            auto wait_tile = [&](int which, const Place& x, int code) {
                 const long long tw = trace_clock();
-                ok = ok && mbar_wait_spin(bar(Geo::kRingFull0 + ring_slot(which, t, Geo::RING)), (uint32_t)ring_use(t, Geo::RING) & 1u, abort_flag, p.status, code);
+                ok = ok && mbar_wait_spin(bar(Geo::kRingFull0 + which * Geo::RING + x.slot), x.parity, abort_flag, p.status, code);
                 tr_kv += trace_clock() - tw;
             };
-            auto tile_addr = [&](int which, int t) { return sbase + Geo::OFF_RING + (uint32_t)ring_slot(which, t, Geo::RING) * Geo::SLOT_BYTES; };
+            auto tile_addr = [&](int which, const Place& x) { return sbase + Geo::OFF_RING + (uint32_t)(which * Geo::RING + x.slot) * Geo::SLOT_BYTES; };
             // u = -2, -1: the Q K^T of the group's first two tiles; u >= 0: the turn of its u-th tile, the P V of
             // tile j and the Q K^T of tile j + lead back to back once everything they read is there.  K/V tiles
             // are waited for first (they are normally there already), P last, so that nothing stands between
@@ -451,52 +513,64 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const __nv_bfloat16* _
             for (int u = -2; u < mine && ok; ++u) {
                 const int c = cnt + u;
                 const bool pv = u >= 0, qk = u + 2 < mine;
-                if (!pv && !qk) continue;
+                if (!pv && !qk) {
+                    take_token(ok);
+                    pass_token();
+                    continue;
+                }
                 const int j = dual ? u : 2 * u + b, jn = j + lead;
                 if (lane == 0) trace_event(b ? 10 : 0, ev, 20 + b);
-                if (pv) wait_tile(1, base + j, 24);
-                if (qk) wait_tile(0, base + jn, 21);
-                // The tiles were written by cp.async, through the generic proxy; the MMAs read them through the
-                // asynchronous one.  The full barriers order the two, the fence makes the bytes visible across;
-                // it stands before the wait for P, which hides it.
-                fence_async_smem();
+                if (pv) wait_tile(1, vp, 24);
+                if (qk) wait_tile(0, kp, 21);
+                // The tiles were written by TMA copies, but for the rows of an unfinished last V page: those came by cp.async,
+                // through the generic proxy, and the MMAs read through the asynchronous one.  The full barrier orders
+                // the two, the fence makes the bytes visible across.
+                if (pv && ragged && j == ntiles - 1) fence_async_smem();
                 const uint32_t buf = tmem + kColS + 128u * (uint32_t)b + 64u * (uint32_t)(c & 1);      // S and P
-                const uint64_t vd = smem_desc(tile_addr(1, base + max(j, 0)), Geo::HALF_BYTES, 1024);
-                const uint64_t kd = smem_desc(tile_addr(0, base + jn), 16, 1024);
-                const uint32_t idesc_qk = instr_desc(16u * (uint32_t)tile_pages(jn), 0);
-                const int npg = tile_pages(j);
+                const uint64_t vd = smem_desc(tile_addr(1, vp), Geo::ATOM_BYTES, Geo::GROUP_BYTES);
+                const uint64_t kd = smem_desc(tile_addr(0, kp), 16, Geo::GROUP_BYTES);
+                const uint32_t idesc_qk = jn == ntiles - 1 ? idesc_last : instr_desc(kTile, 0);
                 const uint32_t done = bar((qk ? Geo::kSFull0 : Geo::kPvDone0) + 2 * b + (c & 1));
                 if (pv) {
                     const long long tw = trace_clock();
                     ok = ok && mbar_wait_spin(bar(Geo::kPFull0 + 2 * b + (c & 1)), (uint32_t)(c >> 1) & 1u, abort_flag, p.status, 26);
                     tr_p += trace_clock() - tw;
                 }
+                take_token(ok);
                 if (lane == 0) trace_event(b ? 10 : 0, ev, 22 + b);
                 if (!ok) break;
                 tc_fence_after();
                 if (pv) {
                     // O[b] (+)= P[b] V_j with P[b] in tensor memory
-                    if (npg == kTile / kPage) {
+                    if (j < ntiles - 1 || last_pages == kTile / kPage) {
 #pragma unroll
                         for (int ks = 0; ks < kTile / kPage; ++ks)
-                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)(ks * 128), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
+                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)ks * (Geo::PAGE_BYTES >> 4), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
                     } else {
-                        for (int ks = 0; ks < npg; ++ks)
-                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)(ks * 128), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
+                        for (int ks = 0; ks < last_pages; ++ks)
+                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)ks * (Geo::PAGE_BYTES >> 4), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
                     }
                 }
                 if (qk) {
                     // S[b] <- Q[b] K^T
 #pragma unroll
                     for (int ks = 0; ks < D / 16; ++ks) {
+                        if (ks == D / 16 - 2) pass_token();      // the other warp's first MMA queues behind the last two
                         // the address field counts 16-byte units and cannot carry out of its 14 bits here
                         const uint64_t qoff = (uint64_t)(((uint32_t)(ks >> 2) * Geo::QHALF_BYTES + (uint32_t)(ks & 3) * 32u) >> 4);
-                        const uint64_t koff = (uint64_t)(((uint32_t)(ks >> 2) * Geo::HALF_BYTES + (uint32_t)(ks & 3) * 32u) >> 4);
+                        const uint64_t koff = (uint64_t)(((uint32_t)(ks >> 2) * Geo::ATOM_BYTES + (uint32_t)(ks & 3) * 32u) >> 4);
                         mma_f16(el, buf, qd + qoff, kd + koff, idesc_qk, ks > 0);
                     }
                 }
                 mma_commit(el, done);
+                if (!qk) pass_token();
+                if (pv) next_place(vp);
+                if (qk) next_place(kp);
                 if (lane == 0) trace_event(b ? 10 : 0, ev, 26 + b);
+            }
+            if (!dual && b == 1 && (ntiles & 1) != 0) {      // group 0 has a turn more
+                take_token(ok);
+                pass_token();
             }
             cnt += mine;
             base += ntiles;

@@ -39,7 +39,7 @@ attn_decode_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const 
 
 template <int D, int G>
 __global__ void __launch_bounds__(tc::kThreads, 1)
-attn_append_tc_kernel(DevPlan p, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* pool,
+attn_append_tc_kernel(DevPlan p, const __grid_constant__ CUtensorMap span_map, const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* pool,
                       __nv_bfloat16* __restrict__ out, float* __restrict__ lse) {
     extern __shared__ uint8_t smem_raw[];
     pdl_trigger();      // the kernel behind this one may start its prologue; it waits for this grid to complete
@@ -47,14 +47,14 @@ attn_append_tc_kernel(DevPlan p, const __nv_bfloat16* __restrict__ q, const __nv
         trace_mark(0);
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<D, G>(p, q, pool, out, lse, aligned_smem(smem_raw));
+    tc::tc_body<D, G>(p, &span_map, q, pool, out, lse, aligned_smem(smem_raw));
     if (threadIdx.x == 0) trace_mark(1);
 }
 
 template <int D, int G>
 __global__ void __launch_bounds__(tc::kThreads, 1)
-attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const __nv_bfloat16* __restrict__ q,
-                  const __nv_bfloat16* pool, __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
+attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const __grid_constant__ CUtensorMap span_map,
+                  const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* pool, __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                   int S) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = aligned_smem(smem_raw);
@@ -73,7 +73,7 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 0) {
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<D, G>(p, q, pool, out, lse, smem);
+    tc::tc_body<D, G>(p, &span_map, q, pool, out, lse, smem);
     if (threadIdx.x == 0) trace_mark(1);
     if (head[2] == head[3] && p.queue_count == 0) return;      // nothing left for the warp body
     __syncthreads();      // tensor memory released, shared memory free for the second phase
@@ -84,10 +84,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// The pool as a 5-D tensor (64 values, 16 slots, d / 64 row halves, Hkv, pages x K|V) with a box of
-// one page's K and V blocks of one kv head, landed with the 128-byte swizzle (see dec::tma_page_kv).
+// The pool as the two bodies read it, landed with the 128-byte swizzle:
+//   kv    (64 values, 16 slots, d / 64 row halves, Hkv, pages x K|V), a box is one page's K and V blocks of one kv head
+//         (dec::tma_page_kv)
+//   span  (64 values, 8 slots, d / 64 row halves, 2 groups of 8 slots, pages x K|V x Hkv), a box is one block (tc::tma_page)
+struct KvMaps { CUtensorMap kv, span; };
+
+constexpr int64_t kMaxMapPages = 0x3fffffff;
+
 // The driver entry point is looked up once per process.
-cudaError_t make_kv_map(const DevPlan& p, const void* pool, CUtensorMap* map) {
+cudaError_t make_kv_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
     static std::atomic<EncodeTiledFn> encode_fn{nullptr};
     EncodeTiledFn encode = encode_fn.load(std::memory_order_acquire);
     if (encode == nullptr) {
@@ -100,15 +106,20 @@ cudaError_t make_kv_map(const DevPlan& p, const void* pool, CUtensorMap* map) {
         encode_fn.store(encode, std::memory_order_release);
     }
     const cuuint64_t d = (cuuint64_t)p.head_dim, hkv = (cuuint64_t)p.num_kv_heads;
-    if (p.num_pages <= 0 || p.num_pages > 0x3fffffff) return cudaErrorInvalidValue;
-    const cuuint64_t dims[5] = {64, kPage, d / 64, hkv, 2 * (cuuint64_t)p.num_pages};
-    const cuuint64_t strides[4] = {d * 2, 128, kPage * d * 2, hkv * kPage * d * 2};
-    const cuuint32_t box[5] = {64, kPage, (cuuint32_t)(d / 64), 1, 2};
+    if (p.num_pages <= 0) return cudaErrorInvalidValue;
+    // (the pages that a tensor map can count hold more than any device's memory)
+    const cuuint64_t blocks = 2 * (cuuint64_t)std::min(p.num_pages, kMaxMapPages);
+    const cuuint64_t dims_kv[5] = {64, kPage, d / 64, hkv, blocks}, strides_kv[4] = {d * 2, 128, kPage * d * 2, hkv * kPage * d * 2};
+    const cuuint64_t dims_span[5] = {64, 8, d / 64, 2, std::min<cuuint64_t>(blocks * hkv, INT32_MAX)};
+    const cuuint64_t strides_span[4] = {d * 2, 128, 8 * d * 2, kPage * d * 2};
+    const cuuint32_t box_kv[5] = {64, kPage, (cuuint32_t)(d / 64), 1, 2}, box_span[5] = {64, 8, (cuuint32_t)(d / 64), 2, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pool), dims, strides, box,
-                              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                              CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    auto make = [&](CUtensorMap* map, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+        return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pool), dims, strides, box,
+                      estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    return make(&maps->kv, dims_kv, strides_kv, box_kv) && make(&maps->span, dims_span, strides_span, box_span) ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device instead of once per launch.
@@ -127,20 +138,22 @@ cudaError_t allow_smem(size_t bytes) {
     return e;
 }
 
-// The tensor map of a pool depends on its address and shape only: the last few are kept per thread.
-cudaError_t cached_kv_map(const DevPlan& p, const void* pool, CUtensorMap* map) {
-    struct Entry { const void* pool; int64_t pages; int hkv, d; CUtensorMap map; };
+// The tensor maps of a pool depend on its address and shape only: the last few are kept per thread.
+cudaError_t cached_kv_maps(const DevPlan& p, const void* pool, const KvMaps** maps) {
+    struct Entry { const void* pool; int64_t pages; int hkv, d; KvMaps maps; };
     constexpr int kEntries = 8;
     thread_local Entry cache[kEntries] = {};
     thread_local int next = 0;
     for (int i = 0; i < kEntries; ++i)
         if (cache[i].pool == pool && cache[i].pages == p.num_pages && cache[i].hkv == p.num_kv_heads && cache[i].d == p.head_dim) {
-            *map = cache[i].map;
+            *maps = &cache[i].maps;
             return cudaSuccess;
         }
-    const cudaError_t e = make_kv_map(p, pool, map);
+    Entry fresh{pool, p.num_pages, p.num_kv_heads, p.head_dim, {}};
+    const cudaError_t e = make_kv_maps(p, pool, &fresh.maps);
     if (e == cudaSuccess) {
-        cache[next] = Entry{pool, p.num_pages, p.num_kv_heads, p.head_dim, *map};
+        cache[next] = fresh;
+        *maps = &cache[next].maps;
         next = (next + 1) % kEntries;
     }
     return e;
@@ -160,10 +173,11 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
     const size_t smem = dec::smem_bytes<D>(S);
     cudaError_t e = allow_smem<attn_decode_kernel<D, G, APPEND>>(smem);
     if (e != cudaSuccess) return e;
-    CUtensorMap map;
-    e = cached_kv_map(p, pool, &map);
+    const KvMaps* maps;
+    if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
+    e = cached_kv_maps(p, pool, &maps);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, map,
+    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, maps->kv,
                       (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
@@ -172,8 +186,11 @@ cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, voi
     constexpr size_t smem = tc::Geometry<D>::SMEM_BYTES;
     cudaError_t e = allow_smem<attn_append_tc_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
+    const KvMaps* maps;
+    e = cached_kv_maps(p, pool, &maps);
+    if (e != cudaSuccess) return e;
     return launch_pdl(attn_append_tc_kernel<D, G>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
-                      p, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
+                      p, maps->span, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
 }
 
 template <int D, int G>
@@ -183,10 +200,11 @@ cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void
     static_assert(dec::smem_bytes<D>(S) - 1024 <= tc::Geometry<D>::OFF_BAR, "the span body's barriers stay clear of the warp body");
     cudaError_t e = allow_smem<attn_fused_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
-    CUtensorMap map;
-    e = cached_kv_map(p, pool, &map);
+    const KvMaps* maps;
+    if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
+    e = cached_kv_maps(p, pool, &maps);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, map,
+    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, maps->kv, maps->span,
                       (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S);
 }
 

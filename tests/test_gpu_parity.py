@@ -405,3 +405,16 @@ def test_any_positive_scale(d, sm_scale):
     _, ref_out, ref_lse = oracle_step(wl, wl.steps[0], sm_scale=sm_scale)
     assert_close(out_bits, lse, ref_out, ref_lse, what=f"scale {sm_scale}")
     assert 0 < plan.info["num_items_tensor"] < plan.info["num_items"]
+
+
+@pytest.mark.parametrize("d", [128, 64])
+@pytest.mark.parametrize("ql", [9, 40])      # one row tile, two
+def test_span_tiles_that_end_at_any_slot(d, ql):
+    """The last K/V tile of an item ends at each slot of each of its pages, after none or some full tiles; slots and
+    pages behind the end hold NaN patterns (a span tile is copied page by page, V's last page with zeros behind the end)."""
+    shape = W.Shape(8, 2, d, 16)
+    ends = [64 * k + e for k in (0, 1, 5) for e in range(41, 105, 3)]
+    wl = W.make_single_step("ends", shape, [e - ql for e in ends], [ql] * len(ends), seed=2024 + d, poison_unused=True,
+                            extra_pages=[i % 2 for i in range(len(ends))])
+    _, _, plan = run_and_check(wl, what=f"span ends, head_dim {d}, {ql} tokens", tensor_min_rows=1)
+    assert plan.info["num_items_tensor"] == plan.info["num_items"]
