@@ -33,6 +33,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <climits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -51,6 +53,7 @@ constexpr int kMaxStages = 6;
 constexpr int kHandoffs = kMaxStages + 2;    // item hand-offs in flight: a stage each, so at most kMaxStages
 constexpr int kCols = 8;                     // (token, head) columns of a unit: the N of the MMAs
 constexpr int kTileTok = kWarps * kPage;     // keys per ring stage
+constexpr int kPrefetchMinPages = 24;        // of a first item that is brought into L2 ahead
 constexpr float kRescaleThreshold = 8.f;     // log2 units a score may exceed the reference max by
 constexpr long long kWaitCycles = 2000000000ll;
 
@@ -182,7 +185,7 @@ template <int D>
 constexpr size_t smem_bytes(int stages) {
     using Geo = Geometry<D>;
     return (size_t)stages * (Geo::STAGE_BYTES + Geo::Q_BYTES + sizeof(TileDesc) + 16) +
-           (size_t)(kHandoffs + kMergeReqs) * (sizeof(TileDesc) + 8) + kMergeReqs * 8 + sizeof(NextItem) + 16 +
+           (size_t)(kHandoffs + kMergeReqs) * (sizeof(TileDesc) + 8) + kMergeReqs * 8 + sizeof(NextItem) + 24 +
            16 + 1024;
 }
 
@@ -385,7 +388,7 @@ __device__ __forceinline__ void merge_loop(const DevPlan& p, __nv_bfloat16* __re
 // The whole kernel body: warps 0-7 consume, warp 8 produces, warps 9 and 10 are the epilogue and the
 // merge warp, any further warps of the CTA return at once (the fused kernel has twelve).
 template <int D, int GT, bool APPEND>
-__device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap* kv_map,
+__device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap* kv_map, const __nv_bfloat16* pool,
                                             const __nv_bfloat16* __restrict__ q,
                                             __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                                             int S, uint8_t* smem, const AppendSrc& app) {
@@ -398,14 +401,14 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
     TileDesc* handoff = desc + S;                // what the epilogue warp needs to know about a finished item
     TileDesc* merge_req = handoff + kHandoffs;   // completed split units on their way to the merge warp
     NextItem* next_item = (NextItem*)(merge_req + kMergeReqs);
-    uint64_t* bars = (uint64_t*)(next_item + 1);   // full[S], empty[S], done[kHandoffs], req, reqfree, next full, free
-    volatile int* abort_flag = (volatile int*)(bars + 2 * S + kHandoffs + 2 * kMergeReqs + 2);
+    uint64_t* bars = (uint64_t*)(next_item + 1);   // full[S], empty[S], done[kHandoffs], req, reqfree, next full, free, appended
+    volatile int* abort_flag = (volatile int*)(bars + 2 * S + kHandoffs + 2 * kMergeReqs + 3);
 
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + S), done0 = smem_u32(bars + 2 * S);
     const uint32_t req0 = done0 + 8 * kHandoffs, reqfree0 = req0 + 8 * kMergeReqs;
-    const uint32_t next_full = reqfree0 + 8 * kMergeReqs, next_free = next_full + 8;
+    const uint32_t next_full = reqfree0 + 8 * kMergeReqs, next_free = next_full + 8, appended = next_free + 8;
 
     if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(kv_map));
     if (threadIdx.x == 0) {
@@ -414,7 +417,7 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             mbar_init(empty0 + 8 * s, kWarps);
         }
         for (int h = 0; h < kHandoffs; ++h) mbar_init(done0 + 8 * h, kWarps);
-        for (int j = 0; j < 2 * kMergeReqs + 2; ++j) mbar_init(req0 + 8 * j, 1);
+        for (int j = 0; j < 2 * kMergeReqs + 3; ++j) mbar_init(req0 + 8 * j, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -429,7 +432,7 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
         // Its own first item (if the planner gave it one) comes inline in the CTA's header with its
         // first 32 page ids, so that the first copies leave after one round trip to memory; every
         // later item arrives from the fetch warp through shared memory, ready to issue.
-        struct PItem { int kv0, kv_end, q_row0, ntok, kv_limit0, kv_head, partial_row, page0, unit, n_chunks, partial_base; };
+        struct PItem { int kv0, kv_end, q_row0, ntok, kv_limit0, kv_head, partial_row, page0, unit, n_chunks, partial_base, q_seq0; };
         int n = 0;
         const int32_t* head = p.cta_heads + (size_t)blockIdx.x * kHeadWords;
         const int i0 = head[2], i1 = head[3];
@@ -437,7 +440,7 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             PItem r;
             r.kv0 = w[0]; r.kv_end = w[1]; r.q_row0 = w[2]; r.ntok = w[3];
             r.kv_limit0 = w[4]; r.kv_head = w[5]; r.partial_row = w[6]; r.page0 = w[7];
-            r.unit = w[8]; r.n_chunks = w[9]; r.partial_base = w[10];
+            r.unit = w[8]; r.n_chunks = w[9]; r.partial_base = w[10]; r.q_seq0 = w[11];
             return r;
         };
         auto load_pages = [&](const PItem& it, int first_page) {
@@ -452,7 +455,7 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
         int pages_cur = 0;
         // next item from the fetch warp (kv_end == 0: none); also sets pages_cur to its first 32 page ids
         auto take = [&]() {
-            PItem r{0, 0, 0, 0, 0, 0, -1, 0, 0, 1, -1};
+            PItem r{0, 0, 0, 0, 0, 0, -1, 0, 0, 1, -1, 0};
             ok = mbar_wait(next_full, (uint32_t)taken & 1u, abort_flag, p.status, 6);
             if (ok) {
                 r = unpack(next_item->work);
@@ -463,10 +466,15 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             }
             return r;
         };
-        PItem cur{0, 0, 0, 0, 0, 0, -1, 0, 0, 1, -1};
-        if (i0 < i1 && !APPEND) {      // (with the append fused in, every item passes the fetch warp)
+        PItem cur{0, 0, 0, 0, 0, 0, -1, 0, 0, 1, -1, 0};
+        // With the append fused in, the fetch warp puts the first item's new rows into their slots meanwhile: the first
+        // stage that holds one of them waits for that, the stages in front do not (14.7 -> 13.5 us a layer for 4 decoding
+        // sequences, from a graph).  Later items are handed over with their rows in place.
+        int unappended_from = INT_MAX;
+        if (i0 < i1) {
             cur = unpack(head + kHeadWorkCuda);
             pages_cur = head[kHeadPagesCuda + lane];
+            if constexpr (APPEND) unappended_from = cur.kv_limit0 - 1 - (cur.q_row0 - cur.q_seq0);
         }
         // The plan was uploaded before the kernel in front of this one started, so all of the above
         // overlaps that kernel's tail; the pool, Q and the queue are touched only from here on.
@@ -486,6 +494,13 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
                     const int rows = min(kTileTok, cur.kv_end - base);
                     const int npages = (rows + kPage - 1) / kPage;
                     const bool first = t == 0;
+                    if constexpr (APPEND) {
+                        if (base + rows > unappended_from) {
+                            ok = mbar_wait(appended, 0, abort_flag, p.status, 8);
+                            if (!ok) break;
+                            unappended_from = INT_MAX;
+                        }
+                    }
                     if (lane == 0) {
                         TileDesc d;
                         d.flags = (first ? kFlagFirst : 0) | (t == ntiles - 1 ? kFlagLast : 0);
@@ -525,6 +540,7 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
                 }
                 pages_cur = pages_nxt;
             }
+            unappended_from = INT_MAX;
             if (ok) cur = take();
         }
         if (ok) {
@@ -567,8 +583,17 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
         // it has not started.
         const int32_t* head = p.cta_heads + (size_t)blockIdx.x * kHeadWords;
         const int i1 = head[3];
-        int own = head[2] < i1 && !APPEND ? head[2] + 1 : head[2];
+        int own = head[2] < i1 ? head[2] + 1 : head[2];
         pdl_wait();      // the queue's counter belongs to the launch in front until that has completed
+        if constexpr (APPEND) {
+            // asynclm_step: the new rows of the CTA's first item (see the producer)
+            if (head[2] < i1) {
+                append_rows_of_item(p, app, *reinterpret_cast<const Work*>(head + kHeadWorkCuda), lane);
+                asm volatile("fence.proxy.async.global;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) mbar_arrive(appended);
+            }
+        }
         for (int j = 0;; ++j) {
             if (j > 0 && !mbar_wait(next_free, (uint32_t)(j - 1) & 1u, abort_flag, p.status, 7)) break;
             int idx = -1;
@@ -610,6 +635,16 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
     }
 
     // ---------------------------------------------------------------------- consumer warps
+    // Pages ahead of the ring, only where they pay: in steps without span tiles, and for items that are not all latency.
+    // (us a layer from a graph, without | with: 4 decoding sequences over 0.5-4 K keys 13.6 | 12.6, 64 over 1-3 K 87.3 | 85.7; with
+    // span tiles, where a longer append kernel in front competes for the memory, 32 sequences with 8 spans 69.9 |
+    // 70.6, and for the span tiles themselves 24 sequences with a span each 74.6 | 78.9; 4 sequences of 100-300 keys 8.4 | 8.7.)
+    if (p.num_items_tensor == 0) {
+        const int32_t* head = p.cta_heads + (size_t)blockIdx.x * kHeadWords;
+        const Work* w = reinterpret_cast<const Work*>(head + kHeadWorkCuda);
+        const int pages = head[2] < head[3] ? (w->kv_end - w->kv0 + kPage - 1) / kPage : 0;
+        if (pages >= kPrefetchMinPages) prefetch_first_pages<D>(p, pool, head + kHeadPagesCuda, pages, w->kv_head, warp, kWarps, lane);
+    }
     pdl_wait();
     const int g = lane >> 2, t4 = lane & 3;      // fragment coordinates
     const float qscale = p.sm_scale * kLog2e;

@@ -29,12 +29,12 @@ __device__ __forceinline__ uint8_t* aligned_smem(uint8_t* raw) {
 
 template <int D, int G, bool APPEND>
 __global__ void __launch_bounds__(dec::kThreads, 1)
-attn_decode_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const __nv_bfloat16* __restrict__ q,
+attn_decode_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const __nv_bfloat16* pool, const __nv_bfloat16* __restrict__ q,
                    __nv_bfloat16* __restrict__ out, float* __restrict__ lse, int S, AppendSrc app) {
     extern __shared__ uint8_t smem_raw[];
     pdl_trigger();      // the split-KV merge behind this kernel may start its prologue
     if (threadIdx.x == 0) { trace_mark(0); trace_set(1, 0); trace_set(5, 0); trace_set(6, 0); trace_set(7, 0); }
-    dec::decode_body<D, G, APPEND>(p, &kv_map, q, out, lse, S, aligned_smem(smem_raw), app);
+    dec::decode_body<D, G, APPEND>(p, &kv_map, pool, q, out, lse, S, aligned_smem(smem_raw), app);
 }
 
 template <int D, int G>
@@ -67,7 +67,7 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(&kv_map));
     if (head[0] == head[1]) {
         // no span tiles for this CTA: straight to its decode rows, without the tensor-memory set-up
-        dec::decode_body<D, G, false>(p, &kv_map, q, out, lse, S, smem, AppendSrc{});
+        dec::decode_body<D, G, false>(p, &kv_map, pool, q, out, lse, S, smem, AppendSrc{});
         return;
     }
     if (threadIdx.x == 0) {
@@ -77,7 +77,7 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 0) trace_mark(1);
     if (head[2] == head[3] && p.queue_count == 0) return;      // nothing left for the warp body
     __syncthreads();      // tensor memory released, shared memory free for the second phase
-    dec::decode_body<D, G, false>(p, &kv_map, q, out, lse, S, smem, AppendSrc{});
+    dec::decode_body<D, G, false>(p, &kv_map, pool, q, out, lse, S, smem, AppendSrc{});
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -178,7 +178,7 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
     e = cached_kv_maps(p, pool, &maps);
     if (e != cudaSuccess) return e;
     return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, maps->kv,
-                      (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
+                      (const __nv_bfloat16*)pool, (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
 template <int D, int G>

@@ -113,6 +113,26 @@ __device__ __forceinline__ size_t pool_row_offset(int64_t page, int which, int k
             (size_t)slot) * (size_t)head_dim;
 }
 
+// While the kernel in front finishes (its last CTAs merge, most SMs are idle), the memory can bring the first pages of
+// a CTA's first item into L2: pages first, first + step, ... of the 32 in its header, K and V block of kv head
+// `kv_head`.  A hint: nothing is read, so it may come before the kernels in front have completed.  Done with ordinary
+// prefetch instructions of warps that have nothing to do yet, because the copy unit would take its 40-60 ns for each
+// page and the first copies stand behind that (a step of 4 sequences over 100-300 keys 8.4 -> 10.4 us).
+template <int D>
+__device__ __forceinline__ void prefetch_first_pages(const DevPlan& p, const __nv_bfloat16* pool, const int32_t* pages, int num_pages, int kv_head,
+                                                     int first, int step, int lane) {
+    constexpr int kLines = kPage * D * 2 / 128;      // of a block: 32 or 16
+    for (int k = first; k < min(num_pages, 32); k += step) {
+        const int page = __ldg(pages + k);
+        if (page < 0 || page >= p.num_pages) continue;      // (the checked build reports it where it is copied)
+#pragma unroll
+        for (int l = lane; l < 2 * kLines; l += 32) {
+            const __nv_bfloat16* line = pool + pool_row_offset(page, l / kLines, kv_head, 0, p.num_kv_heads, D) + (l % kLines) * 64;
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(line));
+        }
+    }
+}
+
 // Interrupt append inside an attention kernel (paper Section 3.2: the block goes to the end of the
 // context): one warp copies, bit for bit, the new K/V rows of one kv head that an item is about to
 // read, positions [max(kv0, ctx), kv_end) of its sequence, from k_new / v_new into their page slots.
