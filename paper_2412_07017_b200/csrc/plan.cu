@@ -90,9 +90,17 @@ static size_t partial_bytes(int64_t rows, int group, int head_dim) {
 }
 
 // Warp-body units: a sixth of the work is cut into short chunks for the end of the queue, about
-// kTailChunksPerCta per CTA and never shorter than kMinChunkTiles tiles (see deal_dynamic).
+// kTailChunksPerCta per CTA and never shorter than kMinChunkTiles tiles (see deal_dynamic), unless the shortest
+// units, which stand at the end of the queue anyway, are short enough to even out the CTAs' finishing times: those
+// that make up a sixth of the work are no longer than kShortUnitShare of a CTA's share.  Cutting costs item boundaries,
+// partial rows and merges, and a CTA that is late streams faster once others have left the memory to it (which takes
+// kSaturatingCtas to begin with).  (us of attention a layer, cut | not: 64 decoding sequences of 1-3 K keys 85.3 | 83.4, 256 of
+// 0.3-2 K with 5 spans 192 | 186, 32 of 0.5-4 K with 8 spans 62.1 | 60.0, 40 of 64/8 heads with 8 123 | 114; the longest of the
+// shortest sixth has 0.05 to 0.6 of a share there.  Near a share, cutting wins: 19 of 3 K keys 45.4 | 50.)
 constexpr int kTailChunksPerCta = 2;
 constexpr int kMinChunkTiles = 4;
+constexpr int kShortUnitShareNum = 2, kShortUnitShareDen = 3;
+constexpr int kSaturatingCtas = 74;      // stream 6.2 TB/s of pages, 148 6.6, 37 4.4
 // The other units are cut into pieces of at most kBulkTiles tiles (50-90 us) or an eighth of a CTA's share: with
 // contexts of 10^5 tokens, pieces of two fifths of the step, which used to be the only limit, left some CTAs on
 // a last piece of half a millisecond.  (8 sequences of 32-131 K tokens, two 256-token spans: 1083 us of attention
@@ -247,10 +255,10 @@ void cut_and_deal(const std::vector<int>& unit_ids, std::vector<UnitBuild>& unit
 
 
 // Costs of the attention kernels on B200 as the packing sees them, in nanoseconds, used only to size the span
-// CTAs.  The span body's were measured at head_dim 128 on a form of it with 128-key tiles, and the margins below
-// were chosen with them.  The present body takes, per 128 keys with one | two row tiles: 1.27 | 2.10 us on a CTA
-// alone, 1.34 | 2.11 on 74, 1.55 | 2.42 on all 148, and 3.5 | 4.3 us to pass from one item to the next; at
-// head_dim 64 1.08 | 1.70, 1.15 | 2.03, 1.17 | 2.02 and 2.1 | 2.5.
+// CTAs.  At head_dim 128 they are those of an earlier form of the span body with 128-key tiles, which the margins
+// below were chosen with; the present body takes, per 128 keys with one | two row tiles, 0.9 | 1.55 us on a CTA
+// alone and 1.4 | 2.4 on all 148, where memory and power bound it (with 900 | 1800 here, 48 sequences with 6 spans took
+// 120 us instead of 112).  At head_dim 64 it takes 0.93 | 1.55 alone and 1.0 | 1.9 on all.
 struct PathCost {
     int gran;            // tokens per tile of the path (cuts fall on multiples of it)
     int64_t tile_ns;     // one tile in steady state
@@ -275,13 +283,14 @@ constexpr PathCost kWarpCost{128, 1050, 400, 2000};
 // that too few were left streaming to keep the memory busy (one SM streams 60-75 KB/us at most).
 // Each (sequence, kv head) counts once: the row tiles of a long span re-read it, mostly from L2.
 constexpr int64_t kDramBytesPerUs = 6000000;
-// A span CTA that finishes early joins the queue; one that finishes late delays the whole step, and the
-// span body slows down by up to 15 % when the warp-body CTAs saturate the memory.  So the span CTAs
-// are filled to the load limit divided by this margin (in 1/64).  Attention of a layer in us at 72 | 80 | 88 | 96:
-// 128 sequences of 64 / 8 heads with 13 spans 520 | 490 | 480 | 482, 32 sequences of 32 / 8 heads with 8 spans 63
-// | 62 | 63 | 63, at head_dim 64 53 | 53 | 58 | 53 (the costs above are head_dim 128's: how many span CTAs come out
-// there, 68 at 88 and 96 or 104 at the others, is chance).
-constexpr int64_t kSpanMargin64 = 88;
+// A span CTA that finishes early joins the queue; one that finishes late delays the whole step, so the span CTAs
+// are filled to the load limit divided by this margin (in 1/64).  The costs above are head_dim 128's of a
+// slower body, which leaves a margin by itself.  Attention of a layer in us at 66 | 68 | 72 | 88, head_dim 128: 32
+// sequences with 8 spans 60.0 | 61.5 | 61.4 | 61.6, 64 with 12 73.3 | 73.1 | 72.8 | 79.2, 40 of 16/8 heads with 10 65.1 | 64.7 |
+// 64.5 | 69.2, 40 of 64/8 heads with 8 114 | 121 | 120 | 122, 128 of 64/8 heads with 13 492 | 489 | 488 | 479 (469 | 465 | 463 |
+// 463 at best: power); at head_dim 64, 64 | 72 | 76 | 88: 32 with 8 50.0 | 49.8 | 49.4 | 55.4, 64 with 16 83.3 | 81.1 | 80.7 |
+// 80.2, 64 of 8/8 heads with 8 103 | 103 | 104 | 106, 100 of 8/2 heads with 20 48.1 | 50.4 | 50.7 | 55.1.
+constexpr int64_t span_margin64(int head_dim) { return head_dim == 64 ? 72 : 66; }
 // The same, for the decision to divide a unit by rows: a unit just above the span CTAs' share is better cut by
 // the packing than divided, its halves would stream the keys twice.
 constexpr int64_t kDivideMargin64 = 72;
@@ -292,7 +301,7 @@ constexpr int64_t kStartNs = 3000;
 // How span units and long decode units are cut.  The default is the fastest; asynclm_plan asks for fewer cuts
 // where the partial results would outgrow the fixed array of asynclm_attn_mixed_static.
 struct CutPolicy {
-    int64_t span_margin64 = kSpanMargin64;
+    int64_t span_margin64;
     int units_by_keys = INT_MAX;      // long span units (kLongPieceTiles) that may be cut by keys, the longest first
     bool bound_pieces = true;         // kBulkTiles
 };
@@ -456,9 +465,9 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     for (const Piece& pz : pieces_out) units[pz.it.unit].u.n_chunks = std::max(units[pz.it.unit].u.n_chunks, pz.it.chunk + 1);
 
     // ---- warp-body chunks.  An item boundary costs time and a split unit costs partial rows and a
-    // merge, so most of the work stays in long pieces: a few units, a sixth of all tiles, are cut into
-    // short chunks that go to the END of the queue, where they even out the CTAs' finishing times;
-    // every other unit stays whole unless it is longer than two fifths of the step (or than kBulkTiles tiles
+    // merge, so most of the work stays in long pieces: where the shortest units are long themselves (kShortUnitShare), a
+    // few units, a sixth of all tiles, are cut into short chunks that go to the END of the queue, where they even out
+    // the CTAs' finishing times; every other unit stays whole unless it is longer than two fifths of the step (or than kBulkTiles tiles
     // and an eighth of a CTA's share), in which case it is cut into equal pieces.  The queue holds the long pieces longest first, then the short chunks.
     std::vector<int> warp_order(ids_warp);
     std::stable_sort(warp_order.begin(), warp_order.end(),
@@ -473,8 +482,19 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     // which units are cut short: first those of up to four chunks (their merge is one round trip to
     // L2), longest first; longer ones only if that does not give a sixth of the tiles
     std::vector<char> to_tail(units.size(), 0);
+    bool cut_tail = n_ctas < kSaturatingCtas;
+    int64_t shortest = 0;
+    for (size_t i = warp_order.size(); i-- > 0 && shortest < tail_target && !cut_tail;) {
+        const int64_t t = tiles_of(units[(size_t)warp_order[i]].n_keys, kWarpCost.gran);
+        shortest += t;
+        cut_tail = t * n_ctas * kShortUnitShareDen > warp_tiles * kShortUnitShareNum;
+    }
+    int64_t decode_tiles = 0;
+    for (int id : ids_warp)
+        if (units[(size_t)id].u.ntok == 1) decode_tiles += tiles_of(units[(size_t)id].n_keys, kWarpCost.gran);
+    cut_tail = cut_tail || 2 * decode_tiles < warp_tiles;      // (spans on the warp body: not measured without)
     int64_t tail_tiles = 0;
-    for (int pass = 0; pass < 2 && tail_tiles < tail_target; ++pass)
+    for (int pass = 0; pass < 2 && cut_tail && tail_tiles < tail_target; ++pass)
         for (int id : warp_order) {
             const int64_t t = tiles_of(units[id].n_keys, kWarpCost.gran);
             if (tail_tiles >= tail_target) break;
@@ -703,7 +723,8 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     int64_t static_rows = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float)));
     while (partial_bytes(static_rows, G, shape->head_dim) > ASYNCLM_STATIC_SCRATCH_BYTES) --static_rows;
     auto fits_static = [&]() { return !too_many && partial_rows <= static_rows; };
-    const CutPolicy fastest;
+    const int64_t margin = span_margin64(shape->head_dim), fuller = std::min(margin, kDivideMargin64);
+    const CutPolicy fastest{margin};
     rc = deal(fastest, tensor_wanted, static_rows);
     if (rc == ASYNCLM_OK && !fits_static()) {
         if (fixed_chunk == 0) {
@@ -714,14 +735,14 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
                 else if (rows > 0) span_rows += rows, ++span_units;
             }
             const int64_t room = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float))) - warp_rows;
-            CutPolicy fewer;
+            CutPolicy fewer{margin};
             fewer.units_by_keys = room <= 0 ? 0 : (int)(span_units * room / std::max<int64_t>(1, span_rows) * 15 / 16);
             if (fewer.units_by_keys > 0) rc = deal(fewer, tensor_wanted, static_rows);
-            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, true}, tensor_wanted, static_rows);
-            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{kDivideMargin64, 0, false}, tensor_wanted, static_rows);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{fuller, 0, true}, tensor_wanted, static_rows);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{fuller, 0, false}, tensor_wanted, static_rows);
         }
         if (rc == ASYNCLM_OK && !fits_static() && tensor_wanted && shape->head_dim == 64)
-            rc = deal(CutPolicy{kDivideMargin64, 0, false}, false, static_rows);
+            rc = deal(CutPolicy{fuller, 0, false}, false, static_rows);
         if (rc == ASYNCLM_OK && !fits_static()) rc = deal(fastest, tensor_wanted, INT64_MAX);
     }
     if (rc != ASYNCLM_OK) return rc;

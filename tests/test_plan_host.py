@@ -396,3 +396,24 @@ def test_random_batches_stay_within_the_reported_workspaces():
         assert p.info["device_bytes_used"] <= dev_bytes and p.info["host_bytes_used"] <= host_bytes, what
         assert p.info["partial_rows"] <= 20 * sms * (8 // shape.group) + 3 * sms * (256 // shape.group), what
         assert p.info["num_items"] <= 2 * int(ql.sum()) * hkv + 20 * sms, what
+
+
+@pytest.mark.parametrize("ctx,sms,cut", [
+    (list(range(1000, 3048, 32)), 148, False),      # the shortest units are short beside a CTA's share
+    (list(range(1000, 3048, 32)), 73, True),        # too few CTAs to saturate the memory
+    ([3050] * 19, 148, True),                       # every unit is a CTA's share
+])
+def test_short_chunks_only_where_the_shortest_units_are_long(ctx, sms, cut):
+    ctx, ql = np.array(ctx), np.ones(len(ctx), dtype=np.int64)
+    need = -(-(ctx + ql) // 16)
+    q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+    p = B.plan_host(W.Shape(32, 8, 128, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
+    items = p.items()
+    assert (p.info["num_split_units"] > 0) == cut
+    keys = {}
+    for it in items:
+        keys.setdefault((it["seq"], it["kv_head"]), []).append((it["kv0"], it["kv1"]))
+    assert len(keys) == 8 * len(ctx)
+    for (b, _), segs in keys.items():
+        segs.sort()
+        assert segs[0][0] == 0 and segs[-1][1] == ctx[b] + 1 and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
