@@ -265,10 +265,11 @@ def asynclm_plan(shape, num_pages, q_indptr, kv_len_before, page_indptr, page_in
 
 
 def _stream_ptr(stream):
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    # (the raw handle of the current stream, without a Stream object around it)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def asynclm_kv_append(plan: Plan, k_new, v_new, kv_pool, stream=None) -> None:

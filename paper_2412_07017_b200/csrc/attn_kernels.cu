@@ -84,6 +84,20 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
+
+// The driver's entry points are looked up once per process.
+template <typename Fn>
+cudaError_t driver_function(const char* name, Fn* fn) {
+    void* sym = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    cudaError_t e = cudaGetDriverEntryPoint(name, &sym, cudaEnableDefault, &qres);
+    if (e != cudaSuccess) return e;
+    if (qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+    *fn = (Fn)sym;
+    return cudaSuccess;
+}
+
 // The pool as the two bodies read it, landed with the 128-byte swizzle:
 //   kv    (64 values, 16 slots, d / 64 row halves, Hkv, pages x K|V), a box is one page's K and V blocks of one kv head
 //         (dec::tma_page_kv)
@@ -92,17 +106,12 @@ struct KvMaps { CUtensorMap kv, span; };
 
 constexpr int64_t kMaxMapPages = 0x3fffffff;
 
-// The driver entry point is looked up once per process.
 cudaError_t make_kv_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
     static std::atomic<EncodeTiledFn> encode_fn{nullptr};
     EncodeTiledFn encode = encode_fn.load(std::memory_order_acquire);
     if (encode == nullptr) {
-        void* sym = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &qres);
+        cudaError_t e = driver_function("cuTensorMapEncodeTiled", &encode);
         if (e != cudaSuccess) return e;
-        if (qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-        encode = (EncodeTiledFn)sym;
         encode_fn.store(encode, std::memory_order_release);
     }
     const cuuint64_t d = (cuuint64_t)p.head_dim, hkv = (cuuint64_t)p.num_kv_heads;
@@ -138,22 +147,29 @@ cudaError_t allow_smem(size_t bytes) {
     return e;
 }
 
-// The tensor maps of a pool depend on its address and shape only: the last few are kept per thread.
-cudaError_t cached_kv_maps(const DevPlan& p, const void* pool, const KvMaps** maps) {
-    struct Entry { const void* pool; int64_t pages; int hkv, d; KvMaps maps; };
-    constexpr int kEntries = 8;
+// A pool's tensor maps: those of its shape, of which the last few are kept per thread, with its address put in.
+// (The layers of a model have a pool each; encoding a launch's maps anew takes longer than the address.)
+cudaError_t pool_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
+    struct Entry { int64_t pages; int hkv, d; KvMaps maps; };
+    constexpr int kEntries = 4;
     thread_local Entry cache[kEntries] = {};
     thread_local int next = 0;
+    static std::atomic<ReplaceAddressFn> replace_fn{nullptr};
+    ReplaceAddressFn replace = replace_fn.load(std::memory_order_acquire);
+    if (replace == nullptr) {
+        cudaError_t e = driver_function("cuTensorMapReplaceAddress", &replace);
+        if (e != cudaSuccess) return e;
+        replace_fn.store(replace, std::memory_order_release);
+    }
     for (int i = 0; i < kEntries; ++i)
-        if (cache[i].pool == pool && cache[i].pages == p.num_pages && cache[i].hkv == p.num_kv_heads && cache[i].d == p.head_dim) {
-            *maps = &cache[i].maps;
-            return cudaSuccess;
+        if (cache[i].pages == p.num_pages && cache[i].hkv == p.num_kv_heads && cache[i].d == p.head_dim) {
+            *maps = cache[i].maps;
+            void* addr = const_cast<void*>(pool);
+            return replace(&maps->kv, addr) == CUDA_SUCCESS && replace(&maps->span, addr) == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
         }
-    Entry fresh{pool, p.num_pages, p.num_kv_heads, p.head_dim, {}};
-    const cudaError_t e = make_kv_maps(p, pool, &fresh.maps);
+    const cudaError_t e = make_kv_maps(p, pool, maps);
     if (e == cudaSuccess) {
-        cache[next] = fresh;
-        *maps = &cache[next].maps;
+        cache[next] = Entry{p.num_pages, p.num_kv_heads, p.head_dim, *maps};
         next = (next + 1) % kEntries;
     }
     return e;
@@ -173,11 +189,11 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
     const size_t smem = dec::smem_bytes<D>(S);
     cudaError_t e = allow_smem<attn_decode_kernel<D, G, APPEND>>(smem);
     if (e != cudaSuccess) return e;
-    const KvMaps* maps;
+    KvMaps maps;
     if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
-    e = cached_kv_maps(p, pool, &maps);
+    e = pool_maps(p, pool, &maps);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, maps->kv,
+    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, maps.kv,
                       (const __nv_bfloat16*)pool, (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
@@ -186,11 +202,11 @@ cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, voi
     constexpr size_t smem = tc::Geometry<D>::SMEM_BYTES;
     cudaError_t e = allow_smem<attn_append_tc_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
-    const KvMaps* maps;
-    e = cached_kv_maps(p, pool, &maps);
+    KvMaps maps;
+    e = pool_maps(p, pool, &maps);
     if (e != cudaSuccess) return e;
     return launch_pdl(attn_append_tc_kernel<D, G>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
-                      p, maps->span, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
+                      p, maps.span, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
 }
 
 template <int D, int G>
@@ -200,11 +216,11 @@ cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void
     static_assert(dec::smem_bytes<D>(S) - 1024 <= tc::Geometry<D>::OFF_BAR, "the span body's barriers stay clear of the warp body");
     cudaError_t e = allow_smem<attn_fused_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
-    const KvMaps* maps;
+    KvMaps maps;
     if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
-    e = cached_kv_maps(p, pool, &maps);
+    e = pool_maps(p, pool, &maps);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, maps->kv, maps->span,
+    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, maps.kv, maps.span,
                       (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S);
 }
 

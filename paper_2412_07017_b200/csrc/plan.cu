@@ -298,6 +298,27 @@ constexpr int64_t kDivideMargin64 = 72;
 constexpr int64_t kStreamShare64 = 58;
 constexpr int64_t kStartNs = 3000;
 
+// Sorts `v` by falling key, equal keys in the order they stand in.  What stands here comes in runs of equal keys (the
+// kv heads of a sequence, a unit's pieces), so the runs are sorted and written out again.
+template <typename T, typename Key>
+void sort_falling(std::vector<T>& v, Key key) {
+    struct Run { int64_t key; uint32_t at, count; };
+    std::vector<Run> runs;
+    runs.reserve(v.size() / 4 + 8);
+    for (size_t i = 0; i < v.size(); ++i) {
+        const int64_t k = key(v[i]);
+        if (!runs.empty() && runs.back().key == k) ++runs.back().count;
+        else runs.push_back(Run{k, (uint32_t)i, 1});
+    }
+    auto before = [](const Run& x, const Run& y) { return x.key != y.key ? x.key > y.key : x.at < y.at; };
+    if (std::is_sorted(runs.begin(), runs.end(), before)) return;
+    std::sort(runs.begin(), runs.end(), before);
+    std::vector<T> sorted;
+    sorted.reserve(v.size());
+    for (const Run& r : runs) sorted.insert(sorted.end(), v.begin() + r.at, v.begin() + r.at + r.count);
+    v.swap(sorted);
+}
+
 // How span units and long decode units are cut.  The default is the fastest; asynclm_plan asks for fewer cuts
 // where the partial results would outgrow the fixed array of asynclm_attn_mixed_static.
 struct CutPolicy {
@@ -384,10 +405,17 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         tiles[(size_t)id] = tiles_of(units[id].n_keys, tc.gran);
         tns[(size_t)id] = units[id].u.ntok * group > 128 ? dual_tile_ns : tc.tile_ns;
     }
-    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-        return tiles[(size_t)x] * tns[(size_t)x] > tiles[(size_t)y] * tns[(size_t)y];
-    });
-    std::vector<int64_t> load((size_t)n_ctas);
+    sort_falling(order, [&](int id) { return tiles[(size_t)id] * tns[(size_t)id]; });
+    // units of the same cost one after the other: (first in `order`, how many)
+    struct Batch { int64_t tiles, ns; uint32_t at, count; };
+    std::vector<Batch> batches;
+    for (size_t i = 0; i < order.size(); ++i) {
+        const int64_t t = tiles[(size_t)order[i]], ns = tns[(size_t)order[i]];
+        if (!batches.empty() && batches.back().tiles == t && batches.back().ns == ns) ++batches.back().count;
+        else batches.push_back(Batch{t, ns, (uint32_t)i, 1});
+    }
+    struct Cta { int64_t load; int32_t id; };
+    std::vector<Cta> ctas((size_t)n_ctas);      // those in use, the fullest first, equal loads by id
     std::vector<Piece> pieces_out;
     int used = 0;
     // Packs the span units under `cap`; returns false if they do not fit or leave too little room for
@@ -413,46 +441,63 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         const int64_t full = limit * 64 / policy.span_margin64;
         const int64_t cap = limit > 2 * bound ? full : std::min(full, std::max(thin, 2 * (tc.phase_ns + tc.item_ns)));
         pieces_out.clear();
-        std::fill(load.begin(), load.end(), (int64_t)0);
         used = 0;
-        int64_t least = INT64_MAX;      // lower bound of the smallest load among the span CTAs
-        bool fits = true;
-        for (int id : order) {
-            const int64_t t = tiles[(size_t)id], ns = tns[(size_t)id];
+        // moves the CTA at position `at` of `ctas` to where its new load belongs
+        auto add_load = [&](int at, int64_t more) {
+            Cta c = ctas[(size_t)at];
+            c.load += more;
+            auto fuller = [](const Cta& x, const Cta& y) { return x.load != y.load ? x.load > y.load : x.id < y.id; };
+            if (at == 0 || fuller(ctas[(size_t)at - 1], c)) {
+                ctas[(size_t)at] = c;
+                return;
+            }
+            const int to = (int)(std::upper_bound(ctas.begin(), ctas.begin() + at, c, fuller) - ctas.begin());
+            std::move_backward(ctas.begin() + to, ctas.begin() + at, ctas.begin() + at + 1);
+            ctas[(size_t)to] = c;
+        };
+        for (const Batch& batch : batches) {
+            const int64_t t = batch.tiles, ns = batch.ns;
             const int64_t fresh_room = std::max<int64_t>(1, (cap - tc.phase_ns - tc.item_ns) / ns);
             const int64_t pieces = t <= fresh_room ? 1 : (t + fresh_room - 1) / fresh_room;
-            int64_t k0 = 0;
-            for (int64_t c = 0; c < pieces; ++c) {
+            // pieces of a unit one after the other, units one after the other; whole units go to one CTA several at once
+            // as long as it stays the fullest that has room (nobody fuller has, and it only gets fuller)
+            const int64_t todo = pieces * batch.count;
+            for (int64_t k = 0; k < todo;) {
+                const int64_t c = k % pieces;
                 const int64_t take = pieces == 1 ? t : t / pieces + (c < t % pieces ? 1 : 0);
                 const int64_t need = tc.item_ns + take * ns;
-                int best = -1;
-                if (least + need <= cap)            // otherwise no span CTA has room: skip the scan
-                    for (int k = 0; k < used; ++k)
-                        if (load[(size_t)k] + need <= cap && (best < 0 || load[(size_t)k] > load[(size_t)best])) best = k;
-                if (best < 0) {
+                int at = used;
+                if (used > 0 && ctas[(size_t)used - 1].load + need <= cap)
+                    at = (int)(std::partition_point(ctas.begin(), ctas.begin() + used, [&](const Cta& x) { return x.load + need > cap; }) - ctas.begin());
+                if (at == used) {
                     if (used < n_ctas) {
-                        best = used++;
-                        load[(size_t)best] = tc.phase_ns;
+                        ctas[(size_t)used] = Cta{tc.phase_ns, (int32_t)used};
+                        ++used;
+                        if (!emit && used > span_ctas) return false;
                     } else {
-                        fits = false;
-                        best = 0;
-                        for (int k = 1; k < n_ctas; ++k) if (load[(size_t)k] < load[(size_t)best]) best = k;
+                        if (!emit) return false;
+                        --at;      // the least loaded
+                        while (at > 0 && ctas[(size_t)at - 1].load == ctas[(size_t)at].load) --at;
                     }
                 }
-                if (!fits && !emit) return false;
-                const int64_t k1 = std::min<int64_t>(units[id].n_keys, k0 + take * tc.gran);
-                if (emit) pieces_out.push_back(Piece{Item{id, (int32_t)k0, (int32_t)k1, (int32_t)c}, (int32_t)best});
-                load[(size_t)best] += need;
-                least = std::min(least, load[(size_t)best]);
-                k0 = k1;
+                const int64_t n = pieces > 1 ? 1 : std::min(todo - k, 1 + std::max<int64_t>(0, cap - need - ctas[(size_t)at].load) / need);
+                if (emit)
+                    for (int64_t j = k; j < k + n; ++j) {
+                        const int id = order[batch.at + (size_t)(j / pieces)];
+                        const int64_t k0 = c * (t / pieces) + std::min(c, t % pieces);      // tiles before piece c
+                        pieces_out.push_back(Piece{Item{id, (int32_t)(k0 * tc.gran), (int32_t)std::min<int64_t>(units[id].n_keys, (k0 + take) * tc.gran),
+                                                        (int32_t)c}, ctas[(size_t)at].id});
+                    }
+                add_load(at, n * need);
+                k += n;
             }
         }
         // room for the queue: what the span CTAs have left after restarting on the warp body, and the
         // whole limit on the others
-        int64_t room = 0;
-        for (int k = 0; k < n_ctas; ++k)
-            room += std::max<int64_t>(0, limit - load[(size_t)k] - kWarpCost.phase_ns);
-        return fits && used <= span_ctas && room >= warp_ns;
+        int64_t room = (n_ctas - used) * std::max<int64_t>(0, limit - kWarpCost.phase_ns);
+        for (int k = 0; k < used; ++k)
+            room += std::max<int64_t>(0, limit - ctas[(size_t)k].load - kWarpCost.phase_ns);
+        return used <= span_ctas && room >= warp_ns;
     };
     int64_t lo = bound;
     int64_t hi = lo + lo / 4 + tc.item_ns + tc.phase_ns + kWarpCost.phase_ns;
@@ -470,8 +515,7 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     // the CTAs' finishing times; every other unit stays whole unless it is longer than two fifths of the step (or than kBulkTiles tiles
     // and an eighth of a CTA's share), in which case it is cut into equal pieces.  The queue holds the long pieces longest first, then the short chunks.
     std::vector<int> warp_order(ids_warp);
-    std::stable_sort(warp_order.begin(), warp_order.end(),
-                     [&](int x, int y) { return units[x].n_keys > units[y].n_keys; });
+    sort_falling(warp_order, [&](int id) { return units[id].n_keys; });
     std::vector<Item> chunks, tail;
     chunks.reserve(ids_warp.size() + (size_t)n_ctas * 4);
     int64_t bulk_max = hi * 2 / 5 / kWarpCost.tile_ns;
@@ -520,9 +564,9 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     for (const UnitBuild& ub : units)
         if (ub.u.n_chunks > 1) partial_rows += (int64_t)ub.u.n_chunks * ub.u.ntok;
     if (partial_rows > max_partial_rows) return false;
-    auto longer = [](const Item& x, const Item& y) { return x.kv1 - x.kv0 > y.kv1 - y.kv0; };
-    std::stable_sort(chunks.begin(), chunks.end(), longer);
-    std::stable_sort(tail.begin(), tail.end(), longer);
+    auto length = [](const Item& x) { return (int64_t)x.kv1 - x.kv0; };
+    sort_falling(chunks, length);
+    sort_falling(tail, length);
     chunks.insert(chunks.end(), tail.begin(), tail.end());
 
     // ---- emit: warp-body items first (one start chunk for every CTA without span work, then the
@@ -530,6 +574,8 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     cta_indptr_warp.assign((size_t)n_ctas + 1, 0);
     cta_indptr_tensor.assign((size_t)n_ctas + 1, 0);
     const int n_start = (int)std::min<size_t>(chunks.size(), (size_t)(n_ctas - used));
+    items.reserve(chunks.size() + pieces_out.size());
+    item_cta.reserve(chunks.size() + pieces_out.size());
     for (size_t i = 0; i < chunks.size(); ++i) {
         items.push_back(chunks[i]);
         item_cta.push_back(i < (size_t)n_start ? used + (int32_t)i : -1);
@@ -616,10 +662,12 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
         const int64_t ql = (int64_t)q_indptr[b + 1] - q_indptr[b];
         if (ql == 0) continue;   // paused sequences are not read or written: their ids are not checked
         const int64_t need = ((int64_t)batch->kv_len_before[b] + ql + P - 1) / P;
-        for (int64_t j = 0; j < need; ++j) {
-            const int32_t pg = batch->page_indices[page_indptr[b] + j];
-            if (pg < 0 || pg >= shape->num_pages) return ASYNCLM_ERR_PAGE_TABLE;
-        }
+        // (as unsigned numbers, the negative ids are the largest; no exit inside the loop, so that it runs in vectors)
+        const int32_t* ids = batch->page_indices + page_indptr[b];
+        const uint32_t end = (uint32_t)std::min<int64_t>(shape->num_pages, (int64_t)INT32_MAX + 1);
+        uint32_t bad = 0;
+        for (int64_t j = 0; j < need; ++j) bad |= (uint32_t)((uint32_t)ids[j] >= end);
+        if (bad) return ASYNCLM_ERR_PAGE_TABLE;
     }
     if (opts && (opts->flags & ASYNCLM_PLAN_REJECT_ALIASED_WRITES)) {
         std::vector<int32_t> written;
@@ -655,6 +703,8 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     bool too_many = false;
     auto deal = [&](const CutPolicy& policy, bool tensor_on, int64_t max_partial_rows) -> int {
         units.clear(); ids_cuda.clear(); ids_tensor.clear(); items.clear(); item_cta.clear();
+        units.reserve(std::min<size_t>((size_t)std::min(B, T) * Hkv, 65536));
+        ids_cuda.reserve(units.capacity());
         split_units.clear(); merge_blocks.clear();
         n_items_cuda = queue_first = queue_count = 0;
         partial_rows = 0;
