@@ -93,7 +93,7 @@ extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const voi
         // the better first half.  (us a layer, fused | separate: 32 sequences with 8 spans of up to 64 tokens
         // 90 | 65, the same at head_dim 64 85 | 59, 24 sequences with a span each 122 | 72.  Steps without
         // span tiles keep the fused form: 4 decoding sequences 15.5 | 17.7, 16 with 8 spans of up to 7
-        // tokens 49.5 | 49.9.)
+        // tokens 49.5 | 49.9; with the append beside the first stages 12.6 a layer, from a graph, for the 4.)
         rc = cuda_status(launch_kv_append(plan->dev, k_new, v_new, kv_pool, s));
         if (rc != ASYNCLM_OK) return rc;
         rc = cuda_status(launch_attention(plan->dev, q, kv_pool, out, lse, s));
@@ -109,7 +109,7 @@ extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const voi
 // over its tile-th K tile (1-based; 0 switches it off) in the launches that follow.  The waits that depend
 // on that tile (the MMA warp's for the tile, a softmax group's for its scores, the producers' for a free
 // slot) then run out after their cycle budget (about a second); the first to do so records its code
-// (11, 12, 21, 24, 26 or 31), every role of the CTA leaves through the common exit, tensor memory is
+// (11, 12, 21, 24, 26, 28 or 31), every role of the CTA leaves through the common exit, tensor memory is
 // released and asynclm_last_device_status reports the code.  The GPU neither faults nor hangs: this is
 // the test of the bounded waits.  The CTA's output rows are undefined in such a launch.
 extern "C" int asynclm_debug_stall_span_tile(asynclm_plan_t* plan, int32_t tile) {
