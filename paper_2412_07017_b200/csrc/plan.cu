@@ -101,6 +101,20 @@ constexpr int kTailChunksPerCta = 2;
 constexpr int kMinChunkTiles = 4;
 constexpr int kShortUnitShareNum = 2, kShortUnitShareDen = 3;
 constexpr int kSaturatingCtas = 74;      // stream 6.2 TB/s of pages, 148 6.6, 37 4.4
+// That alone leaves the last wave nearly empty where the units are of about one length and not a multiple of the CTAs, so
+// an uncut queue is followed to its end (queue_ns) and cut after all if it ends later than the cut one by more than cutting
+// costs.  (us of attention a layer, cut | not | chosen: sequences of one length, 38 of 4 K keys 104 | 117 | cut, 48 135 | 124 | not,
+// 57 of 6 K 208 | 224 | cut, at head_dim 64 38 of 6 K 85.6 | 108 | cut, 74 156 | 145 | not.  Of 290 batches, half of them of one
+// length or nearly, the chosen form takes 0.2 % longer than the faster one on average and 6 % at most, the rule above
+// alone 2.1 % and 26 %.)
+struct StreamCost {
+    int64_t tile_ns, least_tile_ns;      // 128 keys on a CTA while kStreamCtas stream, and while few do
+    int64_t cut_ns;                      // what a cut sixth costs at the end: more boundaries, partial rows, merges
+};
+constexpr int kStreamCtas = 148;
+constexpr StreamCost stream_cost(int head_dim) {
+    return head_dim == 64 ? StreamCost{700, 630, 2500} : StreamCost{1390, 834, 5000};
+}
 // The other units are cut into pieces of at most kBulkTiles tiles (50-90 us) or an eighth of a CTA's share: with
 // contexts of 10^5 tokens, pieces of two fifths of the step, which used to be the only limit, left some CTAs on
 // a last piece of half a millisecond.  (8 sequences of 32-131 K tokens, two 256-token spans: 1083 us of attention
@@ -327,6 +341,54 @@ struct CutPolicy {
     bool bound_pieces = true;         // kBulkTiles
 };
 
+// Modelled time until the last CTA is through with the warp body's queue: `joins` holds when the CTAs with span work join
+// (the others are there from the start), each takes the next item as soon as it is through with one, and those that are
+// still busy when nothing is left stream faster.  Time runs in steps of 1/1024 of *mean_ns (longer ones where
+// an item or a join is very long), the CTAs' mean finish, which is what no other order of the same items ends before.
+int64_t queue_ns(const std::vector<Item>& queue, const std::vector<int64_t>& joins, int n_ctas, int head_dim, int64_t* mean_ns) {
+    const StreamCost cost = stream_cost(head_dim);
+    auto tile_ns = [&](int64_t ctas) { return std::max(cost.least_tile_ns, cost.tile_ns * ctas / kStreamCtas); };
+    const int64_t tile = tile_ns(n_ctas);
+    struct Run { int64_t ns, count; };      // items of equal cost
+    std::vector<Run> runs;
+    int64_t sum = 0, tiles_before = -1, longest = 0;
+    for (const Item& it : queue) {
+        const int64_t tiles = ((int64_t)it.kv1 - it.kv0 + kWarpCost.gran - 1) / kWarpCost.gran;
+        if (tiles != tiles_before) runs.push_back(Run{kWarpCost.item_ns + tiles * tile, 0});
+        tiles_before = tiles;
+        ++runs.back().count;
+        sum += runs.back().ns;
+        longest = std::max(longest, runs.back().ns);
+    }
+    for (int64_t at : joins) sum += at, longest = std::max(longest, at);
+    *mean_ns = sum / n_ctas;
+    const int64_t step = std::max<int64_t>(1, std::max(*mean_ns / 1024, longest / 8192));
+    std::vector<int32_t> free(2048);      // CTAs that are free from step i on
+    auto add = [&](int64_t at, int64_t ctas) {
+        if (at >= (int64_t)free.size()) free.resize((size_t)at + 1024);
+        free[(size_t)at] += (int32_t)ctas;
+    };
+    add(0, n_ctas - (int64_t)joins.size());
+    for (int64_t at : joins) add(at / step, 1);
+    size_t now = 0;
+    for (const Run& r : runs) {
+        const int64_t need = std::max<int64_t>(1, (r.ns + step / 2) / step);
+        for (int64_t left = r.count; left > 0;) {
+            while (free[now] == 0) ++now;
+            const int64_t n = std::min<int64_t>(left, free[now]);
+            free[now] -= (int32_t)n;
+            add((int64_t)now + need, n);
+            left -= n;
+        }
+    }
+    int64_t end = (int64_t)now * step;
+    for (int64_t busy = n_ctas - free[now]; busy > 0; busy -= free[now]) {
+        end += step * tile_ns(busy) / tile;
+        ++now;
+    }
+    return end;
+}
+
 // Default policy for the fused kernel.
 //   Span units (tensor-core body) are compute-heavy and predictable: they are packed whole onto as few
 // persistent CTAs as the load limit allows (largest first, each into the fullest CTA that still has
@@ -343,7 +405,7 @@ struct CutPolicy {
 //   Returns false, with only the units (their division and n_chunks) filled in, if the cuts leave more than
 // max_partial_rows partial rows.
 bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp,
-                  std::vector<UnitBuild>& units, int group, int64_t kv_bytes, int n_ctas, const CutPolicy& policy,
+                  std::vector<UnitBuild>& units, int group, int head_dim, int64_t kv_bytes, int n_ctas, const CutPolicy& policy,
                   int64_t max_partial_rows, std::vector<Item>& items,
                   std::vector<int32_t>& cta_indptr_warp, std::vector<int32_t>& cta_indptr_tensor,
                   std::vector<int32_t>& item_cta, int32_t* queue_first, int32_t* queue_count) {
@@ -523,9 +585,46 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     bulk_max = std::max<int64_t>(bulk_max, kMinChunkTiles);
     const int64_t tail_target = warp_tiles / 6;
     const int64_t tail_chunk = std::max<int64_t>(kMinChunkTiles, tail_target / ((int64_t)n_ctas * kTailChunksPerCta));
-    // which units are cut short: first those of up to four chunks (their merge is one round trip to
+    // cuts the units; which are cut short: first those of up to four chunks (their merge is one round trip to
     // L2), longest first; longer ones only if that does not give a sixth of the tiles
-    std::vector<char> to_tail(units.size(), 0);
+    std::vector<char> to_tail(units.size());
+    auto cut = [&](bool cut_tail) {
+        chunks.clear();
+        tail.clear();
+        std::fill(to_tail.begin(), to_tail.end(), 0);
+        int64_t tail_tiles = 0;
+        for (int pass = 0; pass < 2 && cut_tail && tail_tiles < tail_target; ++pass)
+            for (int id : warp_order) {
+                const int64_t t = tiles_of(units[id].n_keys, kWarpCost.gran);
+                if (tail_tiles >= tail_target) break;
+                if (to_tail[(size_t)id] || t <= tail_chunk + tail_chunk / 2 || (pass == 0 && t > 4 * tail_chunk)) continue;
+                to_tail[(size_t)id] = 1;
+                tail_tiles += t;
+            }
+        for (int id : warp_order) {
+            const int64_t t = tiles_of(units[id].n_keys, kWarpCost.gran);
+            const bool short_chunks = to_tail[(size_t)id] != 0;
+            const int64_t piece_max = short_chunks ? tail_chunk : bulk_max;
+            const int64_t pieces = t <= piece_max + piece_max / 2 ? 1 : (t + piece_max - 1) / piece_max;
+            int64_t k0 = 0;
+            for (int64_t c = 0; c < pieces; ++c) {
+                const int64_t take = t / pieces + (c < t % pieces ? 1 : 0);
+                const int64_t k1 = std::min<int64_t>(units[id].n_keys, k0 + take * kWarpCost.gran);
+                (short_chunks ? tail : chunks).push_back(Item{id, (int32_t)k0, (int32_t)k1, (int32_t)c});
+                k0 = k1;
+            }
+            units[id].u.n_chunks = (int32_t)pieces;
+        }
+    };
+    // the queue in its order: long pieces, then short chunks, the longest first
+    bool queued = false;
+    auto queue_up = [&]() {
+        auto length = [](const Item& x) { return (int64_t)x.kv1 - x.kv0; };
+        sort_falling(chunks, length);
+        sort_falling(tail, length);
+        chunks.insert(chunks.end(), tail.begin(), tail.end());
+        queued = true;
+    };
     bool cut_tail = n_ctas < kSaturatingCtas;
     int64_t shortest = 0;
     for (size_t i = warp_order.size(); i-- > 0 && shortest < tail_target && !cut_tail;) {
@@ -537,37 +636,32 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     for (int id : ids_warp)
         if (units[(size_t)id].u.ntok == 1) decode_tiles += tiles_of(units[(size_t)id].n_keys, kWarpCost.gran);
     cut_tail = cut_tail || 2 * decode_tiles < warp_tiles;      // (spans on the warp body: not measured without)
-    int64_t tail_tiles = 0;
-    for (int pass = 0; pass < 2 && cut_tail && tail_tiles < tail_target; ++pass)
-        for (int id : warp_order) {
-            const int64_t t = tiles_of(units[id].n_keys, kWarpCost.gran);
-            if (tail_tiles >= tail_target) break;
-            if (to_tail[(size_t)id] || t <= tail_chunk + tail_chunk / 2 || (pass == 0 && t > 4 * tail_chunk)) continue;
-            to_tail[(size_t)id] = 1;
-            tail_tiles += t;
+    cut(cut_tail);
+    if (!cut_tail && chunks.size() > (size_t)(n_ctas - used)) {      // (else every CTA has one to begin with and nothing is left)
+        std::vector<int64_t> joins;
+        for (int k = 0; k < used; ++k) joins.push_back(ctas[(size_t)k].load);
+        int64_t mean = 0;
+        queue_up();
+        const int64_t whole = queue_ns(chunks, joins, n_ctas, head_dim, &mean);
+        // (Span CTAs join at times of their own, which evens the waves out better than modelled: where a gain of 6 to 11 % of the
+        // mean was predicted, cutting was 1 to 7 % slower; where 20 %, 6 % faster.)
+        const int64_t cut_ns = std::max(stream_cost(head_dim).cut_ns, used > 0 ? mean / 8 : 0);
+        if (whole - mean > cut_ns) {
+            const std::vector<Item> uncut(chunks);
+            cut(true);
+            queue_up();
+            if (whole - queue_ns(chunks, joins, n_ctas, head_dim, &mean) <= cut_ns) {
+                chunks = uncut;
+                for (int id : warp_order) units[(size_t)id].u.n_chunks = 1;
+                for (const Item& it : chunks) units[(size_t)it.unit].u.n_chunks = std::max(units[(size_t)it.unit].u.n_chunks, it.chunk + 1);
+            }
         }
-    for (int id : warp_order) {
-        const int64_t t = tiles_of(units[id].n_keys, kWarpCost.gran);
-        const bool short_chunks = to_tail[(size_t)id] != 0;
-        const int64_t piece_max = short_chunks ? tail_chunk : bulk_max;
-        const int64_t pieces = t <= piece_max + piece_max / 2 ? 1 : (t + piece_max - 1) / piece_max;
-        int64_t k0 = 0;
-        for (int64_t c = 0; c < pieces; ++c) {
-            const int64_t take = t / pieces + (c < t % pieces ? 1 : 0);
-            const int64_t k1 = std::min<int64_t>(units[id].n_keys, k0 + take * kWarpCost.gran);
-            (short_chunks ? tail : chunks).push_back(Item{id, (int32_t)k0, (int32_t)k1, (int32_t)c});
-            k0 = k1;
-        }
-        units[id].u.n_chunks = (int32_t)pieces;
     }
     int64_t partial_rows = 0;
     for (const UnitBuild& ub : units)
         if (ub.u.n_chunks > 1) partial_rows += (int64_t)ub.u.n_chunks * ub.u.ntok;
     if (partial_rows > max_partial_rows) return false;
-    auto length = [](const Item& x) { return (int64_t)x.kv1 - x.kv0; };
-    sort_falling(chunks, length);
-    sort_falling(tail, length);
-    chunks.insert(chunks.end(), tail.begin(), tail.end());
+    if (!queued) queue_up();
 
     // ---- emit: warp-body items first (one start chunk for every CTA without span work, then the
     // queue), then the span items grouped by CTA
@@ -743,7 +837,7 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
         } else {
             // bytes of K and V the step has to read, each (sequence, kv head) counted once
             const int64_t kv_bytes = total_kv * Hkv * 4 * shape->head_dim;
-            too_many = !deal_dynamic(ids_tensor, ids_cuda, units, G, kv_bytes, ctas_cuda, policy, max_partial_rows, items,
+            too_many = !deal_dynamic(ids_tensor, ids_cuda, units, G, shape->head_dim, kv_bytes, ctas_cuda, policy, max_partial_rows, items,
                                      cta_indptr_cuda, cta_indptr_tensor, item_cta, &queue_first, &queue_count);
             if (too_many) return ASYNCLM_OK;
             n_items_cuda = queue_first + queue_count;

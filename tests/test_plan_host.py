@@ -398,16 +398,20 @@ def test_random_batches_stay_within_the_reported_workspaces():
         assert p.info["num_items"] <= 2 * int(ql.sum()) * hkv + 20 * sms, what
 
 
-@pytest.mark.parametrize("ctx,sms,cut", [
-    (list(range(1000, 3048, 32)), 148, False),      # the shortest units are short beside a CTA's share
-    (list(range(1000, 3048, 32)), 73, True),        # too few CTAs to saturate the memory
-    ([3050] * 19, 148, True),                       # every unit is a CTA's share
+@pytest.mark.parametrize("ctx,sms,head_dim,cut", [
+    (list(range(1000, 3048, 32)), 148, 128, False),      # the shortest units are short beside a CTA's share
+    (list(range(1000, 3048, 32)), 73, 128, True),        # too few CTAs to saturate the memory
+    ([3050] * 19, 148, 128, True),                       # every unit is a CTA's share
+    ([4096] * 38, 148, 128, True),                       # 304 equal units: two waves and a nearly empty one
+    ([4096] * 48, 148, 128, False),                      # 384: the last wave saturates the memory
+    ([6000] * 38, 148, 64, True),                        # (at head_dim 64 a CTA streams no faster when others have left)
+    ([6000] * 74, 148, 64, False),                       # 592: four full waves
 ])
-def test_short_chunks_only_where_the_shortest_units_are_long(ctx, sms, cut):
+def test_short_chunks_only_where_an_uncut_queue_would_end_later(ctx, sms, head_dim, cut):
     ctx, ql = np.array(ctx), np.ones(len(ctx), dtype=np.int64)
     need = -(-(ctx + ql) // 16)
     q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
-    p = B.plan_host(W.Shape(32, 8, 128, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
+    p = B.plan_host(W.Shape(32, 8, head_dim, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
     items = p.items()
     assert (p.info["num_split_units"] > 0) == cut
     keys = {}
