@@ -580,9 +580,12 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     sort_falling(warp_order, [&](int id) { return units[id].n_keys; });
     std::vector<Item> chunks, tail;
     chunks.reserve(ids_warp.size() + (size_t)n_ctas * 4);
-    int64_t bulk_max = hi * 2 / 5 / kWarpCost.tile_ns;
-    if (policy.bound_pieces) bulk_max = std::min(bulk_max, std::max<int64_t>(kBulkTiles, warp_tiles / (8 * (int64_t)n_ctas)));
-    bulk_max = std::max<int64_t>(bulk_max, kMinChunkTiles);
+    auto longest_piece = [&](int64_t limit) {
+        int64_t t = limit * 2 / 5 / kWarpCost.tile_ns;
+        if (policy.bound_pieces) t = std::min(t, std::max<int64_t>(kBulkTiles, warp_tiles / (8 * (int64_t)n_ctas)));
+        return std::max<int64_t>(t, kMinChunkTiles);
+    };
+    int64_t bulk_max = longest_piece(hi);
     const int64_t tail_target = warp_tiles / 6;
     const int64_t tail_chunk = std::max<int64_t>(kMinChunkTiles, tail_target / ((int64_t)n_ctas * kTailChunksPerCta));
     // cuts the units; which are cut short: first those of up to four chunks (their merge is one round trip to
@@ -637,6 +640,19 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         if (units[(size_t)id].u.ntok == 1) decode_tiles += tiles_of(units[(size_t)id].n_keys, kWarpCost.gran);
     cut_tail = cut_tail || 2 * decode_tiles < warp_tiles;      // (spans on the warp body: not measured without)
     cut(cut_tail);
+    // Two fifths of the limit were chosen when the span CTAs had a margin of 88 and the limit came out that much higher. Where
+    // pieces of that length leave no queue, they are taken: a CTA that comes from span tiles passes through the warp
+    // body's start and end (3 us) to find a queue empty.  (us of attention a layer, with a queue | without: 4 sequences of 4/2
+    // heads over 5-7 K keys, one with 75 tokens, 41 pieces on 40 CTAs 29.3 | 26.1; 23 of 4/2 heads with 2-44 tokens 30.3 | 23.2.)
+    if (used > 0 && chunks.size() + tail.size() > (size_t)(n_ctas - used) && warp_order.size() <= (size_t)(n_ctas - used)) {
+        const int64_t shorter = bulk_max;
+        bulk_max = longest_piece(hi * 88 / policy.span_margin64);
+        cut(cut_tail);
+        if (chunks.size() + tail.size() > (size_t)(n_ctas - used)) {
+            bulk_max = shorter;
+            cut(cut_tail);
+        }
+    }
     if (!cut_tail && chunks.size() > (size_t)(n_ctas - used)) {      // (else every CTA has one to begin with and nothing is left)
         std::vector<int64_t> joins;
         for (int k = 0; k < used; ++k) joins.push_back(ctas[(size_t)k].load);

@@ -421,3 +421,17 @@ def test_short_chunks_only_where_an_uncut_queue_would_end_later(ctx, sms, head_d
     for (b, _), segs in keys.items():
         segs.sort()
         assert segs[0][0] == 0 and segs[-1][1] == ctx[b] + 1 and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
+
+
+def test_long_pieces_that_fit_the_free_ctas_leave_no_queue():
+    """A span CTA that finds pieces queued passes through the warp body for nothing: where pieces of the length they had
+    under a wider span margin all start at once, none are queued."""
+    for shape, ctx, ql in ((W.Shape(4, 2, 128, 16), [6920, 7443, 6637, 4819], [1, 1, 75, 1]),
+                           (W.Shape(16, 4, 128, 16), [3669, 3455, 2559, 2078, 1756, 769], [1, 1, 42, 1, 1, 1])):
+        ctx, ql = np.array(ctx), np.array(ql)
+        need = -(-(ctx + ql) // 16)
+        q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+        p = B.plan_host(shape, int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=148)
+        items = p.items()
+        assert p.info["num_items_tensor"] > 0 and (items["path"] == 0).any()
+        assert (items["cta"] >= 0).all()
