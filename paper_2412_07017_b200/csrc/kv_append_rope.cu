@@ -34,6 +34,7 @@ __device__ __forceinline__ unsigned short f64_to_bf16(double x) {
 }
 
 constexpr int kRopeThreads = 256, kRopeTokens = 4;
+constexpr unsigned kRopeFirstCtas = 148 * 4;      // a wave (three to an SM) and a little: see angles_first
 
 // One row of one head as a thread holds it: 16-byte vectors v and v + half_vecs (values 8v .. 8v+7 and
 // their partners d/2 further), and those of the V row beside a K row.
@@ -72,6 +73,17 @@ kv_append_rope_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* _
     };
     int i = 0, h = threadIdx.x / half_vecs;
     for (; h >= heads && i < n; h -= heads) ++i;
+    // The rows and the pool belong to the kernels in front until those have completed; the angles come from the plan.  Where
+    // about all CTAs start at once, the angles overlap the tail of the kernel in front, and the rows are requested behind
+    // the wait that follows.  In a longer grid most CTAs start when that kernel has completed: they request their rows first.
+    // (us a launch, call after call, rows first | angles first: 320 tokens of 32/8 heads 4.9 | 4.3, 512 7.3 | 6.5, 2048 16.0 |
+    // 16.0, 2400 16.7 | 17.7, 3000 19.1 | 18.4, 4096 24.6 | 25.3, 8192 43.0 | 44.4.)
+    const bool angles_first = gridDim.x <= kRopeFirstCtas;
+    RopeRow cur{};
+    if (!angles_first) {
+        pdl_wait();
+        cur = load(i, h);
+    }
     for (int a = threadIdx.x; a < n * (d / 2); a += blockDim.x) {
         const int ti = a / (d / 2), j = a % (d / 2), r = r0 + ti;
         const int b = __ldg(p.row_seq + r);
@@ -84,11 +96,10 @@ kv_append_rope_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* _
             slot[ti] = page_ok(ps / kPage, p.num_pages, p.status, kStatusBadPageAppend) ? ps : -1;
         }
     }
-    // The rows and the pool belong to the kernels in front until those have completed; the angles come from the plan and
-    // overlap their tail: 32 sequences, 314 tokens, append and attention of a layer 69.6 -> 68.4 us.  (The rows used to be
-    // requested in front of the angles, behind the wait.)
-    pdl_wait();
-    RopeRow cur = load(i, h);
+    if (angles_first) {
+        pdl_wait();
+        cur = load(i, h);
+    }
     __syncthreads();
     while (i < n) {
         int ni = i, nh = h;

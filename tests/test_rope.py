@@ -66,3 +66,26 @@ def test_rotated_append_over_head_counts(Hq, Hkv, d, rotate_q):
         diff = got != ref
         assert diff.mean() < 1e-3 and ulp_diff(got[diff], ref[diff]).max(initial=0) <= 1
     assert np.array_equal(to_bits(pool_dev)[:, 1], ref_pool[:, 1])
+
+
+@pytest.mark.parametrize("q_lens", [[2000, 1, 367], [2000, 1, 368]])      # 592 CTAs of four tokens, 593
+def test_rotated_append_on_both_sides_of_a_wave(q_lens):
+    """A launch of about one wave evaluates the angles before it waits for the kernel in front, a longer one requests its rows first."""
+    import torch
+    from gpu_util import to_bits, to_dev
+    shape = W.Shape(2, 1, 64, 16)
+    wl = W.make_single_step("rope_waves", shape, [0, 900, 31], q_lens, seed=33, poison_unused=True)
+    st = wl.steps[0]
+    pool_dev, q_dev = to_dev(wl.kv_pool), to_dev(st.q)
+    plan = B.asynclm_plan(shape, wl.num_pages, st.q_indptr, st.kv_len_before, st.page_indptr, st.page_indices)
+    B.asynclm_kv_append_rope(plan, to_dev(st.k_new), to_dev(st.v_new), pool_dev, q_dev, 10000.0)
+    torch.cuda.synchronize()
+    pos = np.concatenate([np.arange(c, c + n) for c, n in zip(st.kv_len_before, st.q_len)])
+    rot = lambda bits: W.f32_to_bf16_bits(rope.rotate(W.bf16_bits_to_f64(bits), pos, 10000.0).astype(np.float32))
+    ref_pool = wl.kv_pool.copy()
+    oracle.kv_append(ref_pool, st.q_indptr, st.kv_len_before, st.page_indptr, st.page_indices, rot(st.k_new), st.v_new)
+    # (ties of the two sides' sines and cosines, as above)
+    for got, ref in ((to_bits(pool_dev)[:, 0], ref_pool[:, 0]), (to_bits(q_dev), rot(st.q))):
+        diff = got != ref
+        assert diff.mean() < 1e-3 and ulp_diff(got[diff], ref[diff]).max(initial=0) <= 1
+    assert np.array_equal(to_bits(pool_dev)[:, 1], ref_pool[:, 1])
