@@ -386,8 +386,9 @@ __device__ __forceinline__ void merge_loop(const DevPlan& p, __nv_bfloat16* __re
 }
 
 // The whole kernel body: warps 0-7 consume, warp 8 produces, warps 9 and 10 are the epilogue and the
-// merge warp, any further warps of the CTA return at once (the fused kernel has twelve).
-template <int D, int GT, bool APPEND>
+// merge warp, any further warps of the CTA return at once (the fused kernel has twelve).  With PREFETCH the first pages of a
+// CTA's first item are brought into L2 out of `pool` ahead (see the consumer warps).
+template <int D, int GT, bool APPEND, bool PREFETCH>
 __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap* kv_map, const __nv_bfloat16* pool,
                                             const __nv_bfloat16* __restrict__ q,
                                             __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
@@ -635,11 +636,11 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
     }
 
     // ---------------------------------------------------------------------- consumer warps
-    // Pages ahead of the ring, only where they pay: in steps without span tiles, and for items that are not all latency.
+    // Pages ahead of the ring, only where they pay: in the kernel of steps without span tiles, and for items that are not all latency.
     // (us a layer from a graph, without | with: 4 decoding sequences over 0.5-4 K keys 13.6 | 12.6, 64 over 1-3 K 87.3 | 85.7; with
     // span tiles, where a longer append kernel in front competes for the memory, 32 sequences with 8 spans 69.9 |
     // 70.6, and for the span tiles themselves 24 sequences with a span each 74.6 | 78.9; 4 sequences of 100-300 keys 8.4 | 8.7.)
-    if (p.num_items_tensor == 0) {
+    if constexpr (PREFETCH) {
         const int32_t* head = p.cta_heads + (size_t)blockIdx.x * kHeadWords;
         const Work* w = reinterpret_cast<const Work*>(head + kHeadWorkCuda);
         const int pages = head[2] < head[3] ? (w->kv_end - w->kv0 + kPage - 1) / kPage : 0;

@@ -34,7 +34,7 @@ attn_decode_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const 
     extern __shared__ uint8_t smem_raw[];
     pdl_trigger();      // the split-KV merge behind this kernel may start its prologue
     if (threadIdx.x == 0) { trace_mark(0); trace_set(1, 0); trace_set(5, 0); trace_set(6, 0); trace_set(7, 0); }
-    dec::decode_body<D, G, APPEND>(p, &kv_map, pool, q, out, lse, S, aligned_smem(smem_raw), app);
+    dec::decode_body<D, G, APPEND, true>(p, &kv_map, pool, q, out, lse, S, aligned_smem(smem_raw), app);
 }
 
 template <int D, int G>
@@ -67,7 +67,7 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 32) asm volatile("prefetch.tensormap [%0];" ::"l"(&kv_map));
     if (head[0] == head[1]) {
         // no span tiles for this CTA: straight to its decode rows, without the tensor-memory set-up
-        dec::decode_body<D, G, false>(p, &kv_map, pool, q, out, lse, S, smem, AppendSrc{});
+        dec::decode_body<D, G, false, false>(p, &kv_map, nullptr, q, out, lse, S, smem, AppendSrc{});
         return;
     }
     if (threadIdx.x == 0) {
@@ -77,7 +77,7 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 0) trace_mark(1);
     if (head[2] == head[3] && p.queue_count == 0) return;      // nothing left for the warp body
     __syncthreads();      // tensor memory released, shared memory free for the second phase
-    dec::decode_body<D, G, false>(p, &kv_map, pool, q, out, lse, S, smem, AppendSrc{});
+    dec::decode_body<D, G, false, false>(p, &kv_map, nullptr, q, out, lse, S, smem, AppendSrc{});
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
