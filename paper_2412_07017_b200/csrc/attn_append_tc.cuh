@@ -366,6 +366,13 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
             const int idx = first_page + lane;
             return idx < npg ? __ldg(p.page_indices + it.page0 + idx) : 0;
         };
+        auto land_copies = [&](int k0, int k1) {
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            const long long t0 = clock64();
+            for (int k = k0; k < k1; ++k)
+                while (!mbar_try_wait(bar(Geo::kRingFull0 + ring_slot(which, k, Geo::RING)), (uint32_t)ring_use(k, Geo::RING) & 1u) &&
+                       clock64() - t0 < kWaitCycles) {}
+        };
         constexpr int kPagesPerTile = kTile / kPage;          // 4
         constexpr int kGroupTiles = 32 / kPagesPerTile;       // 8
         constexpr int kChunks = D / 8, kRowsPerOp = 32 / kChunks;      // cp.async: 16-byte chunks of a row; rows a warp instruction moves
@@ -439,14 +446,9 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
             cur = nxt;
             nxt = after;
         }
-        if (!ok) {
-            // aborted: let the loads already issued land before shared memory goes away
-            asm volatile("cp.async.wait_all;" ::: "memory");
-            const long long t0 = clock64();
-            for (int k = max(0, n - Geo::RING); k < n; ++k)
-                while (!mbar_try_wait(bar(Geo::kRingFull0 + ring_slot(which, k, Geo::RING)), (uint32_t)ring_use(k, Geo::RING) & 1u) &&
-                       clock64() - t0 < kWaitCycles) {}
-        }
+        // The copies land before shared memory goes away or on to the warp body.  The MMA warps have normally waited for
+        // each of them, but another role may have given up meanwhile, whether or not this one has seen it.
+        land_copies(max(0, n - Geo::RING), n);
       } else {
         // ------------------------------------------------------------------ MMA issuers
         // One warp per softmax group, running convergently, issues the group's MMAs through an elected lane.  A

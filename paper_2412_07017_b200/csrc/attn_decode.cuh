@@ -449,6 +449,11 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             const int idx = first_page + lane;
             return idx < npg ? __ldg(p.page_indices + it.page0 + idx) : 0;
         };
+        auto land_copies = [&](int k0, int k1) {
+            const long long t0 = clock64();
+            for (int k = k0; k < k1; ++k)
+                while (!mbar_try_wait(full0 + 8 * (k % S), (uint32_t)(k / S) & 1u) && clock64() - t0 < kWaitCycles) {}
+        };
         constexpr int kPagesPerTile = kTileTok / kPage;       // 8
         constexpr int kGroupTiles = 32 / kPagesPerTile;       // 4
         bool ok = true;
@@ -544,22 +549,21 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             unappended_from = INT_MAX;
             if (ok) cur = take();
         }
+        int landing = max(0, n - S);      // the oldest stage whose copies may be in flight
         if (ok) {
             const int s = n % S;
             const uint32_t ph = (uint32_t)(n / S) & 1u;
             if (mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, p.status, 1)) {
+                landing = max(0, n - S + 1);      // stage s has been used and is given away again below
                 if (lane == 0) {
                     desc[s].flags = kFlagEnd;
                     mbar_arrive(full0 + 8 * s);
                 }
             }
-        } else {
-            // aborted: let the copies already issued land before the CTA's shared memory goes away
-            const long long t0 = clock64();
-            for (int k = max(0, n - S); k < n; ++k)
-                while (!mbar_try_wait(full0 + 8 * (k % S), (uint32_t)(k / S) & 1u) &&
-                       clock64() - t0 < kWaitCycles) {}
         }
+        // The copies land before the CTA's shared memory goes away.  The consumers have normally waited for each of them,
+        // but another role may have given up meanwhile, whether or not this one has seen it.
+        land_copies(landing, n);
         // the last CTA to leave the queue puts its counters back to zero for the next launch
         if (p.queue_count > 0 && lane == 0 && atomicAdd(p.counters + 1, 1) == (int)gridDim.x - 1) {
             atomicExch(p.counters, 0);

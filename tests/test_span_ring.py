@@ -165,3 +165,21 @@ def test_the_proxy_fence_stands_between_the_tiles_arrival_and_the_mmas_that_read
     steps = ["wait_tile(1, ", "wait_tile(0, ", "fence_async_smem();", "mma_f16_ta(", "mma_f16("]
     at = [turn.index(s) for s in steps]
     assert at == sorted(at) and turn.count("fence_async_smem();") == 1 and "cp_async16(" not in turn
+
+
+@pytest.mark.parametrize("source,role,loop", [
+    ("attn_append_tc.cuh", "producer warps\n", "for (int ii = i0; cur.kv_end > 0 && ok; ++ii) {"),
+    ("attn_decode.cuh", "producer warp\n", "while (cur.kv_end > 0 && ok) {")])
+def test_a_producer_stays_until_its_copies_have_landed(source, role, loop):
+    """A copy that lands when its CTA's shared memory belongs to somebody else overwrites that.  A producer that is
+    through cannot know that another role has given up, so the wait for the last copies depends on nothing."""
+    with open(os.path.join(lib_build.CSRC, source)) as f:
+        body = f.read().split(role, 1)[1].split(loop, 1)[1]
+    depth, at = 1, 0
+    while depth:
+        depth += {"{": 1, "}": -1}.get(body[at], 0)
+        at += 1
+    rest = body[at:]
+    drain = rest.index("land_copies(")
+    depth = rest[:drain].count("{") - rest[:drain].count("}")
+    assert depth == 0 and not rest[:drain].rstrip().endswith(("else", ")"))
