@@ -401,7 +401,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
                     // would poison P V, so the item's last V page, if it is not full, is copied row by row with zeros
                     // behind the end.  A V barrier takes 33 arrivals: one with the byte count of the TMA copies, and one
                     // of each lane's cp.async copies or all 32 at once where there are none.
-                    const bool ragged = which == 1 && (rows & (kPage - 1)) != 0;
+                    const bool ragged = which == 1 && last_page_by_rows(cur.kv_end, t == ntiles - 1, kPage);
                     const int npages_tma = npages - (ragged ? 1 : 0);
 #ifdef ASYNCLM_DEBUG
                     // checked build: a test may ask for one hand-off to be left out, to see a bounded wait run out
@@ -463,7 +463,8 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
         int cnt = 0;              // tiles of the group before this item: S buffer and phase of the hand-offs
         int item_no = 0;
         // The warps take turns, group 0 first, whether they have MMAs to issue or not: turn n of warp 1 follows turn n of
-        // warp 0, turn n of warp 0 follows turn n - 1 of warp 1.
+        // warp 0, turn n of warp 0 follows turn n - 1 of warp 1.  Not only for speed: a turn's waits for tiles stand in front of its
+        // token, and that order is what makes the parities of the ring's full barriers unambiguous (see span_ring.h).
         int turn_no = 0;
         auto take_token = [&](bool& good) {
             good = good && (b + turn_no == 0 || mbar_wait_spin(bar(Geo::kToken0 + b), (uint32_t)(turn_no + b + 1) & 1u, abort_flag, p.status, 28));
@@ -491,20 +492,15 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
             const uint64_t qd = smem_desc(sbase + Geo::OFF_Q + (dual ? (uint32_t)b * Geo::QTILE_BYTES : 0u), 16, 1024);
             const int last_pages = (it.kv_end - (it.kv0 + (ntiles - 1) * kTile) + kPage - 1) / kPage;      // of the item's last tile
             const uint32_t idesc_last = instr_desc(16u * (uint32_t)last_pages, 0);
-            const bool ragged = (it.kv_end & (kPage - 1)) != 0;
-            // where the group's next K and V tile lie: slot, and the parity of its phase
-            struct Place { int slot; uint32_t parity; };
-            Place kp{ring_slot(0, base + (dual ? 0 : b), Geo::RING), (uint32_t)ring_use(base + (dual ? 0 : b), Geo::RING) & 1u}, vp = kp;
-            auto next_place = [&](Place& x) {
-                x.slot += dual ? 1 : 2;
-                if (x.slot >= Geo::RING) { x.slot -= Geo::RING; x.parity ^= 1u; }
-            };
-            auto wait_tile = [&](int which, const Place& x, int code) {
+            // where the group's next K and V tile lie
+            RingPlace kp = ring_place(base + (dual ? 0 : b), Geo::RING), vp = kp;
+            auto next_place = [&](RingPlace& x) { x = ring_next(x, dual ? 1 : 2, Geo::RING); };
+            auto wait_tile = [&](int which, const RingPlace& x, int code) {
                 const long long tw = trace_clock();
                 ok = ok && mbar_wait_spin(bar(Geo::kRingFull0 + which * Geo::RING + x.slot), x.parity, abort_flag, p.status, code);
                 tr_kv += trace_clock() - tw;
             };
-            auto tile_addr = [&](int which, const Place& x) { return sbase + Geo::OFF_RING + (uint32_t)(which * Geo::RING + x.slot) * Geo::SLOT_BYTES; };
+            auto tile_addr = [&](int which, const RingPlace& x) { return sbase + Geo::OFF_RING + (uint32_t)(which * Geo::RING + x.slot) * Geo::SLOT_BYTES; };
             // u = -2, -1: the Q K^T of the group's first two tiles; u >= 0: the turn of its u-th tile, the P V of
             // tile j and the Q K^T of tile j + lead back to back once everything they read is there.  K/V tiles
             // are waited for first (they are normally there already), P last, so that nothing stands between
@@ -527,7 +523,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
                 // The tiles were written by TMA copies, but for the rows of an unfinished last V page: those came by cp.async,
                 // through the generic proxy, and the MMAs read through the asynchronous one.  The full barrier orders
                 // the two, the fence makes the bytes visible across.
-                if (pv && ragged && j == ntiles - 1) fence_async_smem();
+                if (pv && last_page_by_rows(it.kv_end, j == ntiles - 1, kPage)) fence_async_smem();
                 const uint32_t buf = tmem + kColS + 128u * (uint32_t)b + 64u * (uint32_t)(c & 1);      // S and P
                 const uint64_t vd = smem_desc(tile_addr(1, vp), Geo::ATOM_BYTES, Geo::GROUP_BYTES);
                 const uint64_t kd = smem_desc(tile_addr(0, kp), 16, Geo::GROUP_BYTES);

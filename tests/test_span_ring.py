@@ -2,9 +2,10 @@
 
 A barrier wait names only the parity of a phase: it tells phase k from phase k - 1, not from phase k - 2.
 The model below builds, for a CTA's sequence of items, the order that the kernel's waits and program order
-enforce among fills, tensor-core turns, softmax steps and releases, with the slots and use counts taken
+enforce among fills, arrivals, tensor-core turns, softmax steps and releases, with the slots and use counts taken
 from the kernel's own header, and checks for every wait on a ring barrier that the phase before the one it
-waits for is over whatever the warps' relative speed.
+waits for is over whatever the warps' relative speed.  Tiles arrive in any order (their copies complete by
+themselves); the MMA warps take turns, empty ones included, and those turns are part of the order.
 """
 import ctypes
 import os
@@ -20,6 +21,12 @@ using namespace asynclm::tc;
 extern "C" int slots_of(int head_dim) { return ring_slots(head_dim); }
 extern "C" int slot_of(int which, int t, int slots) { return ring_slot(which, t, slots); }
 extern "C" int use_of(int t, int slots) { return ring_use(t, slots); }
+extern "C" int carried(int t, int step, int n, int slots) {      // slot and parity of tile t + n * step, carried along from t
+    RingPlace x = ring_place(t, slots);
+    for (int k = 0; k < n; ++k) x = ring_next(x, step, slots);
+    return 2 * x.slot + (int)x.parity;
+}
+extern "C" int by_rows(int kv_end, int last_tile, int page) { return last_page_by_rows(kv_end, last_tile != 0, page); }
 """
 
 
@@ -48,8 +55,9 @@ def placed_in_one_ring(slots):
     return place
 
 
-def ambiguous_waits(items, place):
-    """items: (64-key tiles, dual) in the order a CTA runs them.  Returns the waits that could pass early."""
+def ambiguous_waits(items, place, turns=True):
+    """items: (64-key tiles, dual) in the order a CTA runs them.  Returns the waits that could pass early.  Without
+    `turns` the MMA warps issue as soon as their own waits are over."""
     before = {}          # node -> nodes known to come before it
 
     def after(node, *prev):
@@ -59,6 +67,7 @@ def ambiguous_waits(items, place):
     waits = []           # (where the warp stands when it waits, what has to be over, description)
     used = {}            # slot -> {use: (kind, tile, groups that read it)}
     last = {}            # program order of each warp: its latest node
+    turn_no = [0, 0]
     first, opened = 0, None
     for i, (n, dual) in enumerate(items):
         for t in range(first, first + n):
@@ -81,25 +90,28 @@ def ambiguous_waits(items, place):
                     w0, t0, groups = used[slot][use - 1]
                     after(fill, *[("free", w0, t0, b) for b in groups])
                 last["prod", which] = fill
-                # a lane's arrival comes after all of its earlier copies
-                after(("full", which, t), fill, ("full", which, t - 1) if t else None)
+                after(("full", which, t), fill)
         ends = []
         for b in (0, 1):
             mine = [first + j for j in range(n) if dual or j % 2 == b]
             last["mma", b] = after(("open", i, b), last.get(("mma", b)), opened)
             last["soft", b] = after(("q", i, b), last.get(("soft", b)), opened)
-            for u in range(-2, len(mine)):
-                if u >= 0:                                     # softmax of tile u: its scores came with turn u - 2
-                    s = after(("soft", i, b, u), last["soft", b], ("turn", i, b, u - 2))
+            # group 0 has a tile more where they alternate and their number is odd: warp 1 makes up for it with an empty turn
+            for u in range(-2, max(len(mine), (n + 1) // 2)):
+                number, turn_no[b] = turn_no[b], turn_no[b] + 1
+                turn = ("turn", b, number)
+                if turns:      # turn k of warp 1 follows turn k of warp 0, turn k of warp 0 follows turn k - 1 of warp 1
+                    after(turn, ("turn", 0, number) if b else ("turn", 1, number - 1) if number else None)
+                if 0 <= u < len(mine):                         # softmax of tile u: its scores came with turn u - 2
+                    s = after(("soft", i, b, u), last["soft", b], ("turn", b, number - 2))
                     after(("free", 0, mine[u], b), s)
                     if u >= 2:
                         after(("free", 1, mine[u - 2], b), s)
                     last["soft", b] = s
-                reads = ([(1, mine[u])] if u >= 0 else []) + ([(0, mine[u + 2])] if u + 2 < len(mine) else [])
-                if not reads:
-                    continue
+                    after(turn, s)
+                reads = ([(1, mine[u])] if 0 <= u < len(mine) else []) + ([(0, mine[u + 2])] if u + 2 < len(mine) else [])
                 here = last["mma", b]
-                turn = after(("turn", i, b, u), here, ("soft", i, b, u) if u >= 0 else None)
+                after(turn, here)
                 for which, t in reads:
                     slot, use = where[which, t]
                     if use >= 1:
@@ -156,15 +168,59 @@ def test_the_model_finds_the_early_wait_of_a_shared_ring():
     assert not any(kind == "empty" for kind, _, _ in ambiguous_waits([(40, True)], placed_in_one_ring(10)))
 
 
-def test_the_proxy_fence_stands_between_the_tiles_arrival_and_the_mmas_that_read_them():
-    """K and V tiles are generic-proxy writes (cp.async), tcgen05.mma reads shared memory through the asynchronous
-    proxy: without a proxy fence behind the full barriers' waits nothing says that it sees them.  A missing
-    one need not show in any result, so the order of the statements is what is checked."""
+def test_the_model_finds_the_early_waits_of_warps_that_take_no_turns(ring):
+    """With five slots and alternating tiles, the tile a slot held before is the other group's: only the turns say that
+    it has arrived."""
+    found = ambiguous_waits([(12, False)], placed_by_kernel(ring, 128), turns=False)
+    assert ("full", 0, 6) in found and ("full", 1, 6) in found
+    assert not ambiguous_waits([(12, True)], placed_by_kernel(ring, 128), turns=False)
+
+
+@pytest.mark.parametrize("head_dim", [128, 64])
+def test_positions_carried_along_are_those_of_the_tiles(ring, head_dim):
+    slots = ring.slots_of(head_dim)
+    for first in range(3 * slots):
+        for step in (1, 2):      # both groups on every tile, or alternate tiles
+            for n in range(4 * slots):
+                t = first + n * step
+                assert ring.carried(first, step, n, slots) == 2 * ring.slot_of(0, t, slots) + ring.use_of(t, slots) % 2
+
+
+def test_the_mma_warps_turns_are_as_modelled():
+    """Each warp takes and passes its token once a turn, in empty turns and in the one that makes up for an odd tile, too."""
     with open(os.path.join(lib_build.CSRC, "attn_append_tc.cuh")) as f:
-        turn = f.read().split("for (int u = -2; u < mine && ok; ++u) {", 1)[1].split("mma_commit(el, done);", 1)[0]
+        role = f.read().split("MMA issuers", 1)[1].split("softmax / epilogue groups", 1)[0]
+    turns, extra = role.split("for (int u = -2; u < mine && ok; ++u) {", 1)[1].split("if (!dual && b == 1 && (ntiles & 1) != 0) {", 1)
+    empty, full = turns.split("if (!pv && !qk) {", 1)[1].split("continue;", 1)
+    for part in (empty, extra):
+        assert part.count("take_token(ok);") == 1 and part.count("pass_token();") == 1
+    assert full.count("take_token(ok);") == 1
+    assert full.index("wait_tile(1, ") < full.index("wait_tile(0, ") < full.index("take_token(ok);") < full.index("mma_f16")
+    # passed among the MMAs of Q K^T, or behind the last MMA where there is none
+    assert full.count("pass_token();") == 2 and "if (!qk) pass_token();" in full
+
+
+def test_the_proxy_fence_stands_between_the_tiles_arrival_and_the_mmas_that_read_them(ring):
+    """TMA copies and tcgen05.mma are both of the asynchronous proxy, but an unfinished last V page comes by cp.async,
+    through the generic one: without a proxy fence behind the full barriers' waits nothing says that the MMAs see it.
+    A missing fence need not show in any result, so what is checked is the order of the statements, and that one rule
+    says which page comes that way and where the fence stands."""
+    with open(os.path.join(lib_build.CSRC, "attn_append_tc.cuh")) as f:
+        source = f.read()
+    turn = source.split("for (int u = -2; u < mine && ok; ++u) {", 1)[1].split("mma_commit(el, done);", 1)[0]
     steps = ["wait_tile(1, ", "wait_tile(0, ", "fence_async_smem();", "mma_f16_ta(", "mma_f16("]
     at = [turn.index(s) for s in steps]
     assert at == sorted(at) and turn.count("fence_async_smem();") == 1 and "cp_async16(" not in turn
+    assert "if (pv && last_page_by_rows(it.kv_end, j == ntiles - 1, kPage)) fence_async_smem();" in turn
+    producer = source.split("producer warps\n", 1)[1].split("MMA issuers", 1)[0]
+    assert "const bool ragged = which == 1 && last_page_by_rows(cur.kv_end, t == ntiles - 1, kPage);" in producer
+    assert producer.count("cp_async16(") == 1 and "if (ragged) {" in producer.split("cp_async16(", 1)[0]
+    for kv0 in (0, 64, 128, 4096):
+        for kv_end in range(kv0 + 1, kv0 + 200):
+            tiles = -(-(kv_end - kv0) // 64)
+            for t in range(tiles):
+                rows = min(64, kv_end - kv0 - 64 * t)
+                assert bool(ring.by_rows(kv_end, t == tiles - 1, 16)) == (rows % 16 != 0)
 
 
 @pytest.mark.parametrize("source,role,loop", [
