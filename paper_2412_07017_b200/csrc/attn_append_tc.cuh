@@ -172,7 +172,7 @@ __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
 }
 
 // A page's 16 K or V rows of one kv head, `block` = (2 * page + K|V) * Hkv + head, land as [2 groups of 8 rows][halves]
-// [8 rows][128 bytes], 16-byte pieces XOR-swizzled by row (see make_kv_maps).  One SM's TMA unit takes about as long
+// [8 rows][128 bytes], 16-byte pieces XOR-swizzled by row (see make_pool_map).  One SM's TMA unit takes about as long
 // for a copy of 2 KB (35 ns) as for one of 4 KB (44 ns): with a copy for each half of a page, one SM
 // streamed 57 KB/us, with one for both 92.  No multicast.
 __device__ __forceinline__ void tma_page(uint32_t dst, const CUtensorMap* map, int block, uint32_t bar) {

@@ -102,11 +102,11 @@ cudaError_t driver_function(const char* name, Fn* fn) {
 //   kv    (64 values, 16 slots, d / 64 row halves, Hkv, pages x K|V), a box is one page's K and V blocks of one kv head
 //         (dec::tma_page_kv)
 //   span  (64 values, 8 slots, d / 64 row halves, 2 groups of 8 slots, pages x K|V x Hkv), a box is one block (tc::tma_page)
-struct KvMaps { CUtensorMap kv, span; };
+enum PoolMap { kKvMap, kSpanMap };
 
 constexpr int64_t kMaxMapPages = 0x3fffffff;
 
-cudaError_t make_kv_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
+cudaError_t make_pool_map(PoolMap kind, const DevPlan& p, const void* pool, CUtensorMap* map) {
     static std::atomic<EncodeTiledFn> encode_fn{nullptr};
     EncodeTiledFn encode = encode_fn.load(std::memory_order_acquire);
     if (encode == nullptr) {
@@ -123,12 +123,11 @@ cudaError_t make_kv_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
     const cuuint64_t strides_span[4] = {d * 2, 128, 8 * d * 2, kPage * d * 2};
     const cuuint32_t box_kv[5] = {64, kPage, (cuuint32_t)(d / 64), 1, 2}, box_span[5] = {64, 8, (cuuint32_t)(d / 64), 2, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-    auto make = [&](CUtensorMap* map, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
-        return encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pool), dims, strides, box,
-                      estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                      CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-    };
-    return make(&maps->kv, dims_kv, strides_kv, box_kv) && make(&maps->span, dims_span, strides_span, box_span) ? cudaSuccess : cudaErrorInvalidValue;
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(pool), kind == kKvMap ? dims_kv : dims_span,
+                              kind == kKvMap ? strides_kv : strides_span, kind == kKvMap ? box_kv : box_span, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel and device instead of once per launch.
@@ -147,13 +146,13 @@ cudaError_t allow_smem(size_t bytes) {
     return e;
 }
 
-// A pool's tensor maps: those of its shape, of which the last few are kept per thread, with its address put in.
-// (The layers of a model have a pool each; encoding a launch's maps anew takes longer than the address.)
-cudaError_t pool_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
-    struct Entry { int64_t pages; int hkv, d; KvMaps maps; };
-    constexpr int kEntries = 4;
-    thread_local Entry cache[kEntries] = {};
-    thread_local int next = 0;
+// A pool's tensor map: that of its shape, of which the last few are kept per thread and kind, with its address put in.
+// (The layers of a model have a pool each; encoding a launch's map anew takes longer than the address.)
+cudaError_t pool_map(PoolMap kind, const DevPlan& p, const void* pool, CUtensorMap* map) {
+    struct Entry { int64_t pages; int hkv, d; CUtensorMap map; };
+    constexpr int kEntries = 8;
+    thread_local Entry cache[2][kEntries] = {};
+    thread_local int next[2] = {};
     static std::atomic<ReplaceAddressFn> replace_fn{nullptr};
     ReplaceAddressFn replace = replace_fn.load(std::memory_order_acquire);
     if (replace == nullptr) {
@@ -161,16 +160,15 @@ cudaError_t pool_maps(const DevPlan& p, const void* pool, KvMaps* maps) {
         if (e != cudaSuccess) return e;
         replace_fn.store(replace, std::memory_order_release);
     }
-    for (int i = 0; i < kEntries; ++i)
-        if (cache[i].pages == p.num_pages && cache[i].hkv == p.num_kv_heads && cache[i].d == p.head_dim) {
-            *maps = cache[i].maps;
-            void* addr = const_cast<void*>(pool);
-            return replace(&maps->kv, addr) == CUDA_SUCCESS && replace(&maps->span, addr) == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+    for (const Entry& x : cache[kind])
+        if (x.pages == p.num_pages && x.hkv == p.num_kv_heads && x.d == p.head_dim) {
+            *map = x.map;
+            return replace(map, const_cast<void*>(pool)) == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
         }
-    const cudaError_t e = make_kv_maps(p, pool, maps);
+    const cudaError_t e = make_pool_map(kind, p, pool, map);
     if (e == cudaSuccess) {
-        cache[next] = Entry{p.num_pages, p.num_kv_heads, p.head_dim, *maps};
-        next = (next + 1) % kEntries;
+        cache[kind][next[kind]] = Entry{p.num_pages, p.num_kv_heads, p.head_dim, *map};
+        next[kind] = (next[kind] + 1) % kEntries;
     }
     return e;
 }
@@ -189,11 +187,11 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
     const size_t smem = dec::smem_bytes<D>(S);
     cudaError_t e = allow_smem<attn_decode_kernel<D, G, APPEND>>(smem);
     if (e != cudaSuccess) return e;
-    KvMaps maps;
+    CUtensorMap map;
     if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
-    e = pool_maps(p, pool, &maps);
+    e = pool_map(kKvMap, p, pool, &map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, maps.kv,
+    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, map,
                       (const __nv_bfloat16*)pool, (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
@@ -202,11 +200,11 @@ cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, voi
     constexpr size_t smem = tc::Geometry<D>::SMEM_BYTES;
     cudaError_t e = allow_smem<attn_append_tc_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
-    KvMaps maps;
-    e = pool_maps(p, pool, &maps);
+    CUtensorMap map;
+    e = pool_map(kSpanMap, p, pool, &map);
     if (e != cudaSuccess) return e;
     return launch_pdl(attn_append_tc_kernel<D, G>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
-                      p, maps.span, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
+                      p, map, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
 }
 
 template <int D, int G>
@@ -216,11 +214,12 @@ cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void
     static_assert(dec::smem_bytes<D>(S) - 1024 <= tc::Geometry<D>::OFF_BAR, "the span body's barriers stay clear of the warp body");
     cudaError_t e = allow_smem<attn_fused_kernel<D, G>>(smem);
     if (e != cudaSuccess) return e;
-    KvMaps maps;
+    CUtensorMap kv_map, span_map;
     if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
-    e = pool_maps(p, pool, &maps);
+    e = pool_map(kKvMap, p, pool, &kv_map);
+    if (e == cudaSuccess) e = pool_map(kSpanMap, p, pool, &span_map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, maps.kv, maps.span,
+    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, kv_map, span_map,
                       (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S);
 }
 

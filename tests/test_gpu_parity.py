@@ -418,3 +418,12 @@ def test_span_tiles_that_end_at_any_slot(d, ql):
                             extra_pages=[i % 2 for i in range(len(ends))])
     _, _, plan = run_and_check(wl, what=f"span ends, head_dim {d}, {ql} tokens", tensor_min_rows=1)
     assert plan.info["num_items_tensor"] == plan.info["num_items"]
+
+
+def test_pools_of_many_shapes_by_turns():
+    """A thread keeps the tensor maps of the last few pool shapes: more shapes than that, in launches of every kind (both
+    bodies, spans only, decode rows only), twice round."""
+    wls = [W.make_single_step("turns", W.Shape(8, 2, d, 16), [200, 90], ql, seed=60 + k, extra_pages=[k, 0], poison_unused=True)
+           for k, (d, ql) in enumerate([(d, ql) for d in (128, 64) for ql in ([1, 40], [40, 33], [1, 1])] * 4)]
+    for wl in wls + wls:
+        run_and_check(wl, what=f"{wl.num_pages} pages, {wl.steps[0].q_len}")
