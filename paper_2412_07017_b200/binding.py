@@ -268,8 +268,9 @@ def _stream_ptr(stream):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    # (the raw handle of the current stream, without a Stream object around it)
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    # the raw handle without a Stream object around it, where this torch has that function
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
 
 
 def asynclm_kv_append(plan: Plan, k_new, v_new, kv_pool, stream=None) -> None:

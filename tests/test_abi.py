@@ -37,3 +37,17 @@ def test_struct_sizes_match_header_layout():
     assert ctypes.sizeof(B.CPlanOptions) == 16
     assert ctypes.sizeof(B.CPlanInfo) == 12 * 4 + 3 * 8
     assert B.ITEM_DTYPE.itemsize == 32
+
+
+def test_stream_handles_do_not_depend_on_a_private_function_of_torch(monkeypatch):
+    import types
+
+    import torch
+    stream = types.SimpleNamespace(cuda_stream=0x5550)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: stream)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda device: 0x7000 + device, raising=False)
+    assert B._stream_ptr(None) == 0x7003
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert B._stream_ptr(None) == 0x5550
+    assert B._stream_ptr(types.SimpleNamespace(cuda_stream=7)) == 7
