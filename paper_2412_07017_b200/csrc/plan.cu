@@ -305,8 +305,9 @@ constexpr int64_t kDramBytesPerUs = 6000000;
 // 463 at best: power); at head_dim 64, 64 | 72 | 76 | 88: 32 with 8 50.0 | 49.8 | 49.4 | 55.4, 64 with 16 83.3 | 81.1 | 80.7 |
 // 80.2, 64 of 8/8 heads with 8 103 | 103 | 104 | 106, 100 of 8/2 heads with 20 48.1 | 50.4 | 50.7 | 55.1.
 constexpr int64_t span_margin64(int head_dim) { return head_dim == 64 ? 72 : 66; }
-// The same, for the decision to divide a unit by rows: a unit just above the span CTAs' share is better cut by
-// the packing than divided, its halves would stream the keys twice.
+// The same, for the decision to divide a unit by rows.  At head_dim 128 it lies above the span CTAs' margin, so that a unit
+// between the two limits is divided although it would fit a CTA whole.  Both ways measured: with 66 here 28 of 1632 random
+// batches come out otherwise, attention of a layer 0.80 to 1.18 of the time with 72, 1.002 on average.
 constexpr int64_t kDivideMargin64 = 72;
 // Share (in 1/64) of the queue that the CTAs without span work must be able to stream by themselves.
 constexpr int64_t kStreamShare64 = 58;
@@ -336,7 +337,6 @@ void sort_falling(std::vector<T>& v, Key key) {
 // How span units and long decode units are cut.  The default is the fastest; asynclm_plan asks for fewer cuts
 // where the partial results would outgrow the fixed array of asynclm_attn_mixed_static.
 struct CutPolicy {
-    int64_t span_margin64;
     int units_by_keys = INT_MAX;      // long span units (kLongPieceTiles) that may be cut by keys, the longest first
     bool bound_pieces = true;         // kBulkTiles
 };
@@ -500,7 +500,7 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
         const int64_t thin = order.empty() ? 0 : span_work / span_ctas * 5 / 4 + tc.phase_ns + tc.item_ns + dual_tile_ns;
         // (Past twice the lower bound the spread is given up: items of more than half of `thin` take a CTA each,
         // and there may be more of them than CTAs.)
-        const int64_t full = limit * 64 / policy.span_margin64;
+        const int64_t full = limit * 64 / span_margin64(head_dim);
         const int64_t cap = limit > 2 * bound ? full : std::min(full, std::max(thin, 2 * (tc.phase_ns + tc.item_ns)));
         pieces_out.clear();
         used = 0;
@@ -646,7 +646,7 @@ bool deal_dynamic(std::vector<int>& ids_tensor, const std::vector<int>& ids_warp
     // heads over 5-7 K keys, one with 75 tokens, 41 pieces on 40 CTAs 29.3 | 26.1; 23 of 4/2 heads with 2-44 tokens 30.3 | 23.2.)
     if (used > 0 && chunks.size() + tail.size() > (size_t)(n_ctas - used) && warp_order.size() <= (size_t)(n_ctas - used)) {
         const int64_t shorter = bulk_max;
-        bulk_max = longest_piece(hi * 88 / policy.span_margin64);
+        bulk_max = longest_piece(hi * 88 / span_margin64(head_dim));
         cut(cut_tail);
         if (chunks.size() + tail.size() > (size_t)(n_ctas - used)) {
             bulk_max = shorter;
@@ -883,8 +883,7 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     int64_t static_rows = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float)));
     while (partial_bytes(static_rows, G, shape->head_dim) > ASYNCLM_STATIC_SCRATCH_BYTES) --static_rows;
     auto fits_static = [&]() { return !too_many && partial_rows <= static_rows; };
-    const int64_t margin = span_margin64(shape->head_dim), fuller = std::min(margin, kDivideMargin64);
-    const CutPolicy fastest{margin};
+    const CutPolicy fastest;
     rc = deal(fastest, tensor_wanted, static_rows);
     if (rc == ASYNCLM_OK && !fits_static()) {
         if (fixed_chunk == 0) {
@@ -895,14 +894,14 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
                 else if (rows > 0) span_rows += rows, ++span_units;
             }
             const int64_t room = (int64_t)(ASYNCLM_STATIC_SCRATCH_BYTES / ((size_t)G * (shape->head_dim + 1) * sizeof(float))) - warp_rows;
-            CutPolicy fewer{margin};
+            CutPolicy fewer;
             fewer.units_by_keys = room <= 0 ? 0 : (int)(span_units * room / std::max<int64_t>(1, span_rows) * 15 / 16);
             if (fewer.units_by_keys > 0) rc = deal(fewer, tensor_wanted, static_rows);
-            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{fuller, 0, true}, tensor_wanted, static_rows);
-            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{fuller, 0, false}, tensor_wanted, static_rows);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{0, true}, tensor_wanted, static_rows);
+            if (rc == ASYNCLM_OK && !fits_static()) rc = deal(CutPolicy{0, false}, tensor_wanted, static_rows);
         }
         if (rc == ASYNCLM_OK && !fits_static() && tensor_wanted && shape->head_dim == 64)
-            rc = deal(CutPolicy{fuller, 0, false}, false, static_rows);
+            rc = deal(CutPolicy{0, false}, false, static_rows);
         if (rc == ASYNCLM_OK && !fits_static()) rc = deal(fastest, tensor_wanted, INT64_MAX);
     }
     if (rc != ASYNCLM_OK) return rc;
