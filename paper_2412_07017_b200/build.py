@@ -15,7 +15,8 @@ LIB = os.path.join(CSRC, "libasynclm.so")
 # performance work only; the binding loads it when ASYNCLM_LIBRARY points at it.
 TRACE_LIB = os.path.join(CSRC, "libasynclm_trace.so")
 # A third build with device-side checks of every page id a kernel turns into an address (-DASYNCLM_DEBUG):
-# a bad id sets the plan's status word and the access is left out.  For bringing up a new caller.
+# a bad id sets the plan's status word and is not used (an append leaves the row out, a read takes page 0).  For
+# bringing up a new caller.
 DEBUG_LIB = os.path.join(CSRC, "libasynclm_debug.so")
 
 NVCC_FLAGS = [

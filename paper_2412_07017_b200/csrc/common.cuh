@@ -93,7 +93,7 @@ __device__ __forceinline__ void trace_set(int, unsigned long long) {}
 
 // Checked build (-DASYNCLM_DEBUG, see build.py): every page id a kernel is about to turn into an address is
 // compared with the pool's size first; a bad one puts `code` into the status word (the first one wins)
-// and the caller leaves the access out.  The ordinary build relies on the planner, which validates every
+// and the caller leaves a store out, or reads page 0 instead (the barriers count its bytes).  The ordinary build relies on the planner, which validates every
 // id on the host, and compiles the check away.
 #ifdef ASYNCLM_DEBUG
 __device__ __forceinline__ bool page_ok(int64_t page, int64_t num_pages, int32_t* status, int code) {

@@ -69,7 +69,7 @@ def main():
     # the rows of the other sequences do not depend on it
     rows = np.arange(int(st.q_indptr[1]), st.total_q)
     assert_close(out[rows], lse[rows], ref_out[rows], ref_lse[rows], what="checked build, other sequences")
-    # the same in the span's table: the span body reports it and takes zeros for the page
+    # the same in the span's table: the span body reports it and reads page 0 instead
     status, out, lse, _ = run(1)
     result["bad_id_span_body"] = status
     keep = np.r_[0, np.arange(int(st.q_indptr[2]), st.total_q)]

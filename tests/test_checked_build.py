@@ -1,6 +1,6 @@
 """The checked build of the library (-DASYNCLM_DEBUG): every page id a kernel turns into an address is
-compared with the pool's size on the device; a bad one sets the plan's status word and the access is
-left out, so nothing faults.  The planner already rejects bad ids on the host, so the test overwrites
+compared with the pool's size on the device; a bad one sets the plan's status word and is not used (an
+append leaves the row out, a read takes page 0), so nothing faults.  The planner already rejects bad ids on the host, so the test overwrites
 one id in the plan's device copy after planning, in a child process that has loaded the checked build
 only (the ordinary build has no such check and must never see that plan)."""
 import json
@@ -41,6 +41,6 @@ def test_a_bounded_wait_that_runs_out_is_reported_and_the_next_step_is_correct()
     the kernel returns, the status word names the wait, and the next step on the same context matches
     the oracle.  No trap, no fault, no endless loop is involved."""
     res = run_child("wait")
-    assert res["stalled_status"] in (11, 12, 21, 24, 26, 31), res
+    assert res["stalled_status"] in (11, 12, 21, 24, 26, 28, 31), res
     assert 500.0 < res["stalled_ms"] < 5000.0, res      # the budget is 2e9 cycles
     assert res["next_status"] == 0 and res["next_ms"] < 50.0, res
