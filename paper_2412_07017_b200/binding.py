@@ -268,9 +268,11 @@ def _stream_ptr(stream):
     if stream is not None:
         return stream.cuda_stream
     import torch
-    # the raw handle without a Stream object around it, where this torch has that function
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    return torch.cuda.current_stream().cuda_stream if raw is None else raw(torch.cuda.current_device())
+    try:      # the raw handle without a Stream object around it, where this torch has that function
+        raw = torch._C._cuda_getCurrentRawStream
+    except AttributeError:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def asynclm_kv_append(plan: Plan, k_new, v_new, kv_pool, stream=None) -> None:
