@@ -343,8 +343,8 @@ struct CutPolicy {
 
 // Modelled time until the last CTA is through with the warp body's queue: `joins` holds when the CTAs with span work join
 // (the others are there from the start), each takes the next item as soon as it is through with one, and those that are
-// still busy when nothing is left stream faster.  Time runs in steps of 1/1024 of *mean_ns (longer ones where
-// an item or a join is very long), the CTAs' mean finish, which is what no other order of the same items ends before.
+// still busy when nothing is left stream faster.  Time runs in steps of 1/1024 of the mean (longer ones where
+// an item or a join is very long); *mean_ns, the mean finish, is what no other order of the same items ends before.
 int64_t queue_ns(const std::vector<Item>& queue, const std::vector<int64_t>& joins, int n_ctas, int head_dim, int64_t* mean_ns) {
     const StreamCost cost = stream_cost(head_dim);
     auto tile_ns = [&](int64_t ctas) { return std::max(cost.least_tile_ns, cost.tile_ns * ctas / kStreamCtas); };
@@ -361,8 +361,7 @@ int64_t queue_ns(const std::vector<Item>& queue, const std::vector<int64_t>& joi
         longest = std::max(longest, runs.back().ns);
     }
     for (int64_t at : joins) sum += at, longest = std::max(longest, at);
-    *mean_ns = sum / n_ctas;
-    const int64_t step = std::max<int64_t>(1, std::max(*mean_ns / 1024, longest / 8192));
+    const int64_t step = std::max<int64_t>(16, std::max(sum / n_ctas / 1024, longest / 4096));
     std::vector<int32_t> free(2048);      // CTAs that are free from step i on
     auto add = [&](int64_t at, int64_t ctas) {
         if (at >= (int64_t)free.size()) free.resize((size_t)at + 1024);
@@ -381,10 +380,17 @@ int64_t queue_ns(const std::vector<Item>& queue, const std::vector<int64_t>& joi
             left -= n;
         }
     }
-    int64_t end = (int64_t)now * step;
-    for (int64_t busy = n_ctas - free[now]; busy > 0; busy -= free[now]) {
-        end += step * tile_ns(busy) / tile;
-        ++now;
+    // (CTAs that join when nothing is left have no part in it)
+    int64_t late = 0;
+    for (int64_t at : joins)
+        if (at / step > (int64_t)now) --free[(size_t)(at / step)], ++late, sum -= at;
+    *mean_ns = sum / (n_ctas - late);
+    int64_t end = (int64_t)now * step, busy = n_ctas - late - free[now];
+    for (size_t at = now + 1; busy > 0; ++at) {
+        if (free[at] == 0) continue;
+        end += (int64_t)(at - now) * step * tile_ns(busy) / tile;
+        now = at;
+        busy -= free[at];
     }
     return end;
 }
