@@ -37,7 +37,7 @@
 // front of its first MMA counts, too: positions in the rings are carried along instead of divided out.
 // A tile pair takes 1500-1640 cycles on a CTA alone (2050 with both warps issuing at once and cp.async copies), a
 // tile of one row tile 890 (1250; with a copy for each half of a page 1150: see tma_page); at head_dim 64 1520
-// (1700) and 900-940 (1070).  When all CTAs stream, power holds the clock at about 1.5 GHz: attention of 8192 tokens
+// (1700) and 900-940 (1070).  When all CTAs stream, the power limit leaves a clock of 1.5-1.7 GHz: attention of 8192 tokens
 // of one sequence (32 / 8 heads, head_dim 128) 530-570 -> 490-520 us, 24 sequences with spans of 33-96 tokens over 1-3 K keys
 // 82 -> 71-74 us a layer.
 // All hand-offs are mbarriers with bounded waits; a wait that runs out sets the plan's status word
