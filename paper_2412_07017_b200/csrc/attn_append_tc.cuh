@@ -304,7 +304,14 @@ __device__ __forceinline__ TItem load_titem(const Work* rec, bool valid) {
 }
 
 // The whole kernel body, called by all twelve warps with `smem` 1024-byte aligned.
-template <int D, int G>
+// ALONE: in the kernel of steps that have span tiles only.  A launch starts on cold instruction caches, and there every line
+// of code that is fetched for the first time stands in the way: the P V of an unfinished last tile is a loop, and the output rows
+// go out in two passes of four at head_dim 128 (at 64, where a warp has one or two slices, two passes are slower).  us of
+// attention, unrolled | so, before the tiles came by TMA in brackets: 4 sequences of 100-300 keys with spans of 20-60 tokens
+// 14.04 | 13.68 (14.04), one span over 2000 keys 15.6 | 15.1 (15.2), head_dim 64 9.57 | 9.47 (9.18), 24 sequences with spans of 33-96
+// tokens 70.3 | 69.1, 8192 tokens 545 | 528.  Beside the warp body's code it is a loss: 8 sequences of 32-131 K keys with two
+// 256-token spans 917 | 925.
+template <int D, int G, bool ALONE>
 __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* span_map, const __nv_bfloat16* __restrict__ q,
                                         const __nv_bfloat16* pool,
                                         __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
@@ -543,6 +550,10 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
                     if (j < ntiles - 1 || last_pages == kTile / kPage) {
 #pragma unroll
                         for (int ks = 0; ks < kTile / kPage; ++ks)
+                            mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)ks * (Geo::PAGE_BYTES >> 4), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
+                    } else if constexpr (ALONE) {
+#pragma unroll 1
+                        for (int ks = 0; ks < last_pages; ++ks)
                             mma_f16_ta(el, ocol, buf + 8u * (uint32_t)ks, vd + (uint64_t)ks * (Geo::PAGE_BYTES >> 4), idesc_pv, (u > 0 || ks > 0) ? 1u : 0u);
                     } else {
                         for (int ks = 0; ks < last_pages; ++ks)
@@ -815,7 +826,7 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
             const bool final_out = it.partial_row0 < 0;
             auto flush = [&](int byte0) {      // byte0: offset of the slice inside an output row
                 __syncwarp();
-#pragma unroll
+#pragma unroll (ALONE && D == 128 ? 4 : 8)
                 for (int i = 0; i < 8; ++i) {
                     const int row = 4 * i + (lane >> 3), pc = lane & 7;
                     const uint4 v = *reinterpret_cast<const uint4*>(stage + row * 128 + ((pc ^ (row & 7)) << 4));

@@ -47,7 +47,7 @@ attn_append_tc_kernel(DevPlan p, const __grid_constant__ CUtensorMap span_map, c
         trace_mark(0);
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<D, G>(p, &span_map, q, pool, out, lse, aligned_smem(smem_raw));
+    tc::tc_body<D, G, true>(p, &span_map, q, pool, out, lse, aligned_smem(smem_raw));
     if (threadIdx.x == 0) trace_mark(1);
 }
 
@@ -73,7 +73,7 @@ attn_fused_kernel(DevPlan p, const __grid_constant__ CUtensorMap kv_map, const _
     if (threadIdx.x == 0) {
         for (int s = 8; s < 16; ++s) trace_set(s, 0);
     }
-    tc::tc_body<D, G>(p, &span_map, q, pool, out, lse, smem);
+    tc::tc_body<D, G, false>(p, &span_map, q, pool, out, lse, smem);
     if (threadIdx.x == 0) trace_mark(1);
     if (head[2] == head[3] && p.queue_count == 0) return;      // nothing left for the warp body
     __syncthreads();      // tensor memory released, shared memory free for the second phase
