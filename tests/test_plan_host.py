@@ -398,20 +398,16 @@ def test_random_batches_stay_within_the_reported_workspaces():
         assert p.info["num_items"] <= 2 * int(ql.sum()) * hkv + 20 * sms, what
 
 
-@pytest.mark.parametrize("ctx,sms,head_dim,cut", [
-    (list(range(1000, 3048, 32)), 148, 128, False),      # the shortest units are short beside a CTA's share
-    (list(range(1000, 3048, 32)), 73, 128, True),        # too few CTAs to saturate the memory
-    ([3050] * 19, 148, 128, True),                       # every unit is a CTA's share
-    ([4096] * 38, 148, 128, True),                       # 304 equal units: two waves and a nearly empty one
-    ([4096] * 48, 148, 128, False),                      # 384: the last wave saturates the memory
-    ([6000] * 38, 148, 64, True),                        # (at head_dim 64 a CTA streams no faster when others have left)
-    ([6000] * 74, 148, 64, False),                       # 592: four full waves
+@pytest.mark.parametrize("ctx,sms,cut", [
+    (list(range(1000, 3048, 32)), 148, False),      # the shortest units are short beside a CTA's share
+    (list(range(1000, 3048, 32)), 73, True),        # too few CTAs to saturate the memory
+    ([3050] * 19, 148, True),                       # every unit is a CTA's share
 ])
-def test_short_chunks_only_where_an_uncut_queue_would_end_later(ctx, sms, head_dim, cut):
+def test_short_chunks_only_where_the_shortest_units_are_long(ctx, sms, cut):
     ctx, ql = np.array(ctx), np.ones(len(ctx), dtype=np.int64)
     need = -(-(ctx + ql) // 16)
     q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
-    p = B.plan_host(W.Shape(32, 8, head_dim, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
+    p = B.plan_host(W.Shape(32, 8, 128, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=sms)
     items = p.items()
     assert (p.info["num_split_units"] > 0) == cut
     keys = {}
@@ -421,6 +417,27 @@ def test_short_chunks_only_where_an_uncut_queue_would_end_later(ctx, sms, head_d
     for (b, _), segs in keys.items():
         segs.sort()
         assert segs[0][0] == 0 and segs[-1][1] == ctx[b] + 1 and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
+
+
+@pytest.mark.parametrize("n,keys,head_dim,cut", [
+    (38, 4096, 128, True),       # 304 equal units on 148 CTAs: two waves and a nearly empty one
+    (48, 4096, 128, False),      # 384: the last wave saturates the memory
+    (38, 6000, 64, True),        # (at head_dim 64 a CTA streams no faster when others have left)
+    (74, 6000, 64, False),       # 592: four full waves
+])
+def test_short_chunks_where_an_uncut_queue_would_end_unevenly(n, keys, head_dim, cut):
+    ctx, ql = np.full(n, keys), np.ones(n, dtype=np.int64)
+    need = -(-(ctx + ql) // 16)
+    q_indptr, page_indptr, page_indices, _ = W.build_step_tables(ctx, ql, 16, np.arange(need.sum()))
+    p = B.plan_host(W.Shape(32, 8, head_dim, 16), int(need.sum()), q_indptr, ctx, page_indptr, page_indices, num_sms=148)
+    assert (p.info["num_split_units"] > 0) == cut
+    keys_of = {}
+    for it in p.items():
+        keys_of.setdefault((it["seq"], it["kv_head"]), []).append((it["kv0"], it["kv1"]))
+    assert len(keys_of) == 8 * n
+    for segs in keys_of.values():
+        segs.sort()
+        assert segs[0][0] == 0 and segs[-1][1] == keys + 1 and all(x[1] == y[0] for x, y in zip(segs, segs[1:]))
 
 
 def test_long_pieces_that_fit_the_free_ctas_leave_no_queue():
