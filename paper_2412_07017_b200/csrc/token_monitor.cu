@@ -50,8 +50,9 @@ __device__ __forceinline__ unsigned long long pack_key(float v, int i) {
     const unsigned ord = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
     return ((unsigned long long)ord << 32) | (unsigned)(0x7fffffff - i);
 }
+constexpr unsigned long long kNoCandidate = 1ull;      // below every candidate's key, too
 __device__ __forceinline__ Best unpack_key(unsigned long long k) {
-    if (k == 0) return Best{-INFINITY, INT_MAX};
+    if (k <= kNoCandidate) return Best{-INFINITY, INT_MAX};
     const unsigned ord = (unsigned)(k >> 32);
     const unsigned u = (ord & 0x80000000u) ? (ord & 0x7fffffffu) : ~ord;
     return Best{__uint_as_float(u), 0x7fffffff - (int)(unsigned)(k & 0xffffffffu)};
@@ -60,13 +61,15 @@ __device__ __forceinline__ Best unpack_key(unsigned long long k) {
 template <typename T> struct Vec;
 template <> struct Vec<__nv_bfloat16> {
     static constexpr int N = 8;
+    static __device__ __forceinline__ unsigned max2(unsigned a, unsigned b) {
+        unsigned r;
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+        return r;
+    }
     // largest of the 8 values of a 16-byte vector (NaN drops out of max)
     static __device__ __forceinline__ float vmax(const uint4& w) {
-        const unsigned u[4] = {w.x, w.y, w.z, w.w};
-        float m = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) m = fmaxf(m, fmaxf(bf16_lo(u[k]), bf16_hi(u[k])));
-        return m;
+        const unsigned m = max2(max2(w.x, w.y), max2(w.z, w.w));
+        return fmaxf(fmaxf(bf16_lo(m), bf16_hi(m)), -INFINITY);      // (-inf where all are NaN)
     }
     static __device__ __forceinline__ float at(const uint4& w, int k) {
         const unsigned u[4] = {w.x, w.y, w.z, w.w};
@@ -86,53 +89,66 @@ template <> struct Vec<float> {
 
 // Largest ordinary element (no CML token) of vectors [j_begin, j_end) of a row (stride of the CTA's
 // threads), lowest id among equals.  Per vector only its maximum is computed; the position inside the
-// best vector is found at the end by looking at that one vector again.  Only the vectors that hold a CML token
+// best vector is found at the end in the thread's copy of that one vector.  Only the vectors that hold a CML token
 // have their elements looked at: when all vectors of a stretch with one were, the CTA that had it finished
-// last (bf16 rows of 128 256 without a forbidden winner, 256 | 32 | 8 | 1 of them, us a call from a graph:
-// 20.5 | 9.0 | 6.9 | 5.8, 15.8 | 7.1 | 6.0 | 4.9 now).
+// last (15.8 us a call instead of 20.5 for 256 bf16 rows of 128 256).
+// The first vectors are requested before the row's state is known, and the best vector stays in registers instead of being
+// read again at the end, because both stood as a round trip to memory of their own in every CTA (us a call from a graph,
+// before | now, with the two slices' trade below: bf16 rows of 128 256, 256 | 148 | 64 | 8 | 1 of them: 14.1 | 10.7 | 8.3 | 5.3 | 4.7
+// before, 12.7 | 9.5 | 7.8 | 5.0 | 4.4 now; 256 rows of 32 000 6.7 and 6.4, fp32 9.3 and 7.9).
 template <typename T>
-__device__ __forceinline__ Best scan_row(const T* row, int j_begin, int j_end, const asynclm_cml_tokens& tok) {
-    constexpr int VEC = Vec<T>::N;
-    const uint4* v4 = reinterpret_cast<const uint4*>(row);
-    const int sv[5] = {tok.call / VEC, tok.intr / VEC, tok.trap / VEC, tok.end / VEC, tok.head / VEC};
-    auto holds_special = [&](int j) { return j == sv[0] || j == sv[1] || j == sv[2] || j == sv[3] || j == sv[4]; };
-    float bv = -INFINITY;
-    int bj = -1;
-    for (int b0 = j_begin; b0 < j_end; b0 += kMonVecs * kMonThreads) {
-        const int j0 = b0 + threadIdx.x;
-        uint4 w[kMonVecs];
+struct Scan {
+    static constexpr int VEC = Vec<T>::N;
+    const uint4* v4;
+    int j_begin, j_end;
+    uint4 w[kMonVecs];      // the vectors requested last
+
+    __device__ __forceinline__ void request(int b0) {
 #pragma unroll
         for (int u = 0; u < kMonVecs; ++u) {
-            const int j = j0 + u * kMonThreads;
+            const int j = b0 + threadIdx.x + u * kMonThreads;
             w[u] = make_uint4(0, 0, 0, 0);
             if (j < j_end) w[u] = ldg_nc_v4(v4 + j);
         }
-        bool special = false;      // does this stretch of vectors hold a CML token? (the same for all threads)
+    }
+    // Requests the first vectors; nothing is waited for.
+    __device__ __forceinline__ Scan(const T* row, int begin, int end) : v4(reinterpret_cast<const uint4*>(row)), j_begin(begin), j_end(end) { request(begin); }
+
+    __device__ __forceinline__ Best run(const asynclm_cml_tokens& tok) {
+        const int sv[5] = {tok.call / VEC, tok.intr / VEC, tok.trap / VEC, tok.end / VEC, tok.head / VEC};
+        auto holds_special = [&](int j) { return j == sv[0] || j == sv[1] || j == sv[2] || j == sv[3] || j == sv[4]; };
+        float bv = -INFINITY;
+        int bj = -1;
+        uint4 bw = make_uint4(0, 0, 0, 0);      // the vector that holds the best value
+        for (int b0 = j_begin; b0 < j_end; b0 += kMonVecs * kMonThreads) {
+            if (b0 != j_begin) request(b0);
+            const int j0 = b0 + threadIdx.x;
+            bool special = false;      // does this stretch of vectors hold a CML token? (the same for all threads)
 #pragma unroll
-        for (int a = 0; a < 5; ++a) special |= (unsigned)(sv[a] - b0) < (unsigned)(kMonVecs * kMonThreads);
+            for (int a = 0; a < 5; ++a) special |= (unsigned)(sv[a] - b0) < (unsigned)(kMonVecs * kMonThreads);
 #pragma unroll
-        for (int u = 0; u < kMonVecs; ++u) {
-            const int j = j0 + u * kMonThreads;
-            float m = Vec<T>::vmax(w[u]);
-            if (special && holds_special(j)) {
-                m = -INFINITY;
+            for (int u = 0; u < kMonVecs; ++u) {
+                const int j = j0 + u * kMonThreads;
+                float m = Vec<T>::vmax(w[u]);
+                if (special && holds_special(j)) {
+                    m = -INFINITY;
 #pragma unroll
-                for (int k = 0; k < VEC; ++k)
-                    if (!is_special(j * VEC + k, tok)) m = fmaxf(m, Vec<T>::at(w[u], k));
+                    for (int k = 0; k < VEC; ++k)
+                        if (!is_special(j * VEC + k, tok)) m = fmaxf(m, Vec<T>::at(w[u], k));
+                }
+                if (j < j_end && m > bv) { bv = m; bj = j; bw = w[u]; }      // a thread's vectors come in increasing order: the first one wins a tie
             }
-            if (j < j_end && m > bv) { bv = m; bj = j; }      // a thread's vectors come in increasing order: the first one wins a tie
         }
-    }
-    Best best{-INFINITY, INT_MAX};
-    if (bj >= 0) {
-        const uint4 w = ldg_nc_v4(v4 + bj);
-        const bool mixed = holds_special(bj);
+        Best best{-INFINITY, INT_MAX};
+        if (bj >= 0) {
+            const bool mixed = holds_special(bj);
 #pragma unroll
-        for (int k = VEC - 1; k >= 0; --k)
-            if (Vec<T>::at(w, k) == bv && !(mixed && is_special(bj * VEC + k, tok))) best = Best{bv, bj * VEC + k};
+            for (int k = VEC - 1; k >= 0; --k)
+                if (Vec<T>::at(bw, k) == bv && !(mixed && is_special(bj * VEC + k, tok))) best = Best{bv, bj * VEC + k};
+        }
+        return best;
     }
-    return best;
-}
+};
 
 // CTA-wide best in thread 0 (shuffles inside a warp, shared memory across warps).
 __device__ __forceinline__ Best block_best(Best best, float* sv, int* si) {
@@ -153,7 +169,7 @@ __device__ __forceinline__ Best block_best(Best best, float* sv, int* si) {
 // Grid: (slices, batch).  Every CTA scans one slice of a sequence's row and folds its best ordinary token
 // into the row's key with one atomic max; the CTA that arrives last (per-row counter) lets the CML tokens
 // that the state allows compete, advances the state machine and puts the two workspace words back to zero.
-// The CTAs of a row in the TRAP state read no logits but arrive all the same: state_out may be state_in, so
+// The CTAs of a row in the TRAP state read no logits beyond their first request but arrive all the same: state_out may be state_in, so
 // nothing is written before every slice of the row has read the state (a CTA arrives behind a block-wide
 // barrier, and the two state pointers are not __restrict__).
 // The result does not depend on arrival order.  (Scanning all tokens alike and looking at a row a second
@@ -172,7 +188,10 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
     const T* row = logits + (int64_t)seq * row_stride;
     pdl_trigger();      // a kernel behind this one that waits for it may start its prologue
     pdl_wait();         // logits, states and the workspace belong to the kernels in front until those have completed
+    const int nvec = vocab / VEC;
+    const int per = (nvec + gridDim.x - 1) / gridDim.x;
     const int state = state_in[seq];
+    Scan<T> scan(row, blockIdx.x * per, min(nvec, (int)(blockIdx.x + 1) * per));      // on its way beside the state
     // the CML tokens this state allows (INT_MAX: none) and their logits, for the thread that may finish the row
     const int spec0 = state == kText ? tok.call : state == kCall || state == kBody ? tok.end : INT_MAX;
     const int spec1 = state == kText ? tok.trap : state == kCall ? tok.head : INT_MAX;
@@ -183,9 +202,7 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
             if (spec0 != INT_MAX) spec_v0 = to_f32<T>(row[spec0]);
             if (spec1 != INT_MAX) spec_v1 = to_f32<T>(row[spec1]);
         }
-        const int nvec = vocab / VEC;
-        const int per = (nvec + gridDim.x - 1) / gridDim.x;
-        best = scan_row<T>(row, blockIdx.x * per, min(nvec, (int)(blockIdx.x + 1) * per), tok);
+        best = scan.run(tok);
         if (blockIdx.x == gridDim.x - 1)      // the row's ragged end, element by element
             for (int i = nvec * VEC + threadIdx.x; i < vocab; i += kMonThreads) {
                 const float v = to_f32<T>(row[i]);
@@ -199,12 +216,22 @@ token_monitor_kernel(const T* __restrict__ logits, int vocab, int64_t row_stride
     if (gridDim.x > 1) {
         unsigned long long* key = ws + 2 * (size_t)seq;
         unsigned* arrived = reinterpret_cast<unsigned*>(key + 1);
-        if (best.i != INT_MAX) atomicMax(key, pack_key(best.v, best.i));
-        __threadfence();
-        if (atomicAdd(arrived, 1u) != gridDim.x - 1) return;      // not the last CTA of its row
-        __threadfence();
-        best = unpack_key(atomicExch(key, 0ull));
-        *arrived = 0;
+        if (gridDim.x == 2) {
+            // Two slices trade their keys in one atomic, without a counter and the fence in front of it (a round trip each):
+            // whoever finds the other's key is the last one.  Its branch on the state is behind it by then, as
+            // the other's is behind the trade.
+            const unsigned long long mine = best.i != INT_MAX ? pack_key(best.v, best.i) : kNoCandidate, other = atomicExch(key, mine);
+            if (other == 0ull) return;
+            *key = 0ull;
+            best = unpack_key(mine > other ? mine : other);
+        } else {
+            if (best.i != INT_MAX) atomicMax(key, pack_key(best.v, best.i));
+            __threadfence();
+            if (atomicAdd(arrived, 1u) != gridDim.x - 1) return;      // not the last CTA of its row
+            __threadfence();
+            best = unpack_key(atomicExch(key, 0ull));
+            *arrived = 0;
+        }
     }
     if (state == kTrap) {
         // [TRAP] is followed by [END] whatever the logits say
@@ -268,7 +295,7 @@ extern "C" int asynclm_token_monitor_step(const void* logits, int32_t dtype, int
     const int slices = std::max(1, std::min(max_slices, (148 * 2 + batch - 1) / batch));
     const dim3 grid((unsigned)slices, (unsigned)batch);
     // Launched with programmatic serialization: the launch overlaps the tail of the kernel in front
-    // (256 rows of 128 256 bf16, call after call: 16.0 -> 14.6 us).
+    // (256 rows of 128 256 bf16, call after call: 16.0 -> 14.6 us, 13.3 with the shorter chain of round trips in each CTA).
     unsigned long long* ws = (unsigned long long*)workspace;
     if (dtype == ASYNCLM_DTYPE_BF16)
         return cuda_status(launch_pdl(token_monitor_kernel<__nv_bfloat16>, grid, dim3(kMonThreads), 0, s, (const __nv_bfloat16*)logits,

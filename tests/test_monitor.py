@@ -159,3 +159,38 @@ def test_a_state_outside_the_grammar_allows_ordinary_tokens_only():
     tok, nxt, fl = run(vals, states, special, False)
     rt, rn, rf = M.step(vals.astype(np.float64), states, special)
     assert np.array_equal(tok, rt) and np.array_equal(nxt, rn) and np.array_equal(fl, rf)
+
+
+@pytest.mark.parametrize("Bsz,vocab,bf16", [(148, 16384, False), (150, 16411, False), (295, 32776, True)])
+def test_rows_of_two_slices(Bsz, vocab, bf16):
+    """The two slices of a row trade their candidates: either may hold the best one, both the same value (the lower id wins), or
+    one or both none at all (NaN or -inf), in every state; states advance in place and the workspace comes back zero."""
+    import torch
+    half = (vocab // (8 if bf16 else 4) + 1) // 2 * (8 if bf16 else 4)      # first element of the second slice
+    special = {"CALL": 5, "INTR": half - 1, "TRAP": half, "END": vocab - 1, "HEAD": half + 9}
+    g = np.random.default_rng(Bsz + vocab)
+    vals32 = g.normal(size=(Bsz, vocab)).astype(np.float32)
+    for b in range(Bsz):
+        kind = b % 9
+        if kind == 1: vals32[b, 3] = 20.0
+        if kind == 2: vals32[b, vocab - 2] = 20.0
+        if kind == 3: vals32[b, [half - 2, half + 1]] = 20.0
+        if kind == 4: vals32[b, :half] = np.nan
+        if kind == 5: vals32[b, half:] = -np.inf
+        if kind == 6: vals32[b, :] = -np.inf
+        if kind == 7: vals32[b, special["END"]] = 30.0
+        if kind == 8: vals32[b, special["TRAP"]] = 30.0
+    stride = -(-vocab // 8) * 8
+    full = torch.zeros((Bsz, stride), dtype=torch.bfloat16 if bf16 else torch.float32, device="cuda")
+    full[:, :vocab] = torch.from_numpy(vals32).cuda().to(full.dtype)
+    vals = full[:, :vocab].float().cpu().numpy().astype(np.float64)
+    states = (np.arange(Bsz) // 9 % 4).astype(np.int32)
+    st = torch.from_numpy(states).cuda()
+    tok, fl = torch.full_like(st, -7), torch.full_like(st, -7)
+    ws = torch.zeros(B.token_monitor_workspace_bytes(Bsz), dtype=torch.uint8, device="cuda")
+    for _ in range(4):
+        B.asynclm_token_monitor_step(full[:, :vocab], special, st, tok, st, fl, ws)
+        torch.cuda.synchronize()
+        rt, states, rf = M.step(vals, states, special)
+        assert int(ws.max()) == 0
+        assert np.array_equal(tok.cpu().numpy(), rt) and np.array_equal(st.cpu().numpy(), states) and np.array_equal(fl.cpu().numpy(), rf)
