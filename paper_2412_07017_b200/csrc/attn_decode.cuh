@@ -222,44 +222,60 @@ __device__ __forceinline__ void epilogue_loop(const DevPlan& p, __nv_bfloat16* _
         }
         const uint8_t* stage = stage_base + (size_t)d.stage * Geo::STAGE_BYTES;
         const int ncols = d.ntok * G;
+        // The weights first, a (column, warp) pair to a lane (four columns at once, the other four of a unit with more behind
+        // them); the passes over the values get them by shuffle.  With weights worked out in every lane and pass, this stood between an
+        // item's last page and its result for 1.95 us at 4 columns of 128, 1.15 now (us a layer from a graph: 4 decoding sequences
+        // 12.66 -> 11.83, 64 over 1-3 K keys 82.6 -> 80.9, 32 with 8 spans 58.6 -> 57.0).  Unrolled passes are slower (12.02): a CTA
+        // of a short step fetches this code once.
+        auto state = [&](int w) { return reinterpret_cast<const float*>(stage + (size_t)w * Geo::PAGE_BYTES); };
+        float wgt[2] = {0.f, 0.f}, inv[2] = {0.f, 0.f}, lse2[2] = {0.f, 0.f};
+#pragma unroll
+        for (int q4 = 0; q4 < 2; ++q4) {
+            if (4 * q4 >= ncols) break;      // (the same for all lanes)
+            const float* ms = state(lane & 7) + kCols * Geo::O_STRIDE + 4 * q4 + (lane >> 3);
+            const float m = ms[0], l = ms[kCols];
+            float M = m;
+#pragma unroll
+            for (int off = 1; off < kWarps; off <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
+            wgt[q4] = m == -INFINITY ? 0.f : fast_exp2(m - M);
+            float L = wgt[q4] != 0.f ? l * wgt[q4] : 0.f;
+#pragma unroll
+            for (int off = 1; off < kWarps; off <<= 1) L += __shfl_xor_sync(0xffffffffu, L, off);
+            inv[q4] = L > 0.f ? 1.f / L : 0.f;
+            lse2[q4] = L > 0.f ? M + log2f(L) : -INFINITY;
+        }
         // four consecutive values of one column per lane and pass; the eight warps' copies are read
         // with independent loads
-        for (int e = 4 * lane; e < ncols * D; e += 128) {
-            const int col = e / D, dd = e % D;
-            float mw[kWarps], lw[kWarps];
-            float4 ov[kWarps];
-            float M = -INFINITY;
+#pragma unroll 1
+        for (int e0 = 0; e0 < ncols * D; e0 += 128) {
+            const int e = e0 + 4 * lane, col = e / D, dd = e % D;
+            const bool on = col < ncols;      // (head_dim 64: a pass covers two columns)
+            const int from = (col & 3) * kWarps, q4 = e0 >= 4 * D;
+            float4 ov[kWarps], a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) ov[w] = *reinterpret_cast<const float4*>(state(w) + (size_t)col * Geo::O_STRIDE + dd);
+            const float my_wgt = q4 ? wgt[1] : wgt[0];
 #pragma unroll
             for (int w = 0; w < kWarps; ++w) {
-                const float* sw = reinterpret_cast<const float*>(stage + (size_t)w * Geo::PAGE_BYTES);
-                mw[w] = sw[kCols * Geo::O_STRIDE + col];
-                lw[w] = sw[kCols * Geo::O_STRIDE + kCols + col];
-                ov[w] = *reinterpret_cast<const float4*>(sw + (size_t)col * Geo::O_STRIDE + dd);
-                M = fmaxf(M, mw[w]);
+                const float g = __shfl_sync(0xffffffffu, my_wgt, from + w);
+                const bool any = g != 0.f;      // a warp without a visible key left nothing meaningful behind
+                a.x = any ? fmaf(ov[w].x, g, a.x) : a.x;
+                a.y = any ? fmaf(ov[w].y, g, a.y) : a.y;
+                a.z = any ? fmaf(ov[w].z, g, a.z) : a.z;
+                a.w = any ? fmaf(ov[w].w, g, a.w) : a.w;
             }
-            float L = 0.f;
-            float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) {
-                const float wgt = mw[w] == -INFINITY ? 0.f : fast_exp2(mw[w] - M);
-                if (wgt != 0.f) {      // a warp without a visible key left nothing meaningful behind
-                    L = fmaf(lw[w], wgt, L);
-                    a.x = fmaf(ov[w].x, wgt, a.x); a.y = fmaf(ov[w].y, wgt, a.y);
-                    a.z = fmaf(ov[w].z, wgt, a.z); a.w = fmaf(ov[w].w, wgt, a.w);
-                }
-            }
-            const float inv = L > 0.f ? 1.f / L : 0.f;
-            const float lse2 = L > 0.f ? M + log2f(L) : -INFINITY;
+            const float r = __shfl_sync(0xffffffffu, q4 ? inv[1] : inv[0], from), ls = __shfl_sync(0xffffffffu, q4 ? lse2[1] : lse2[0], from);
+            if (!on) continue;
             const int tok = col / G, hh = col % G;
             const size_t hq = (size_t)d.kv_head * G + hh;
             if (d.partial_row < 0) {
                 *reinterpret_cast<uint2*>(out + ((size_t)(d.out_row + tok) * Hq + hq) * D + dd) =
-                    make_uint2(pack_bf16x2(a.x * inv, a.y * inv), pack_bf16x2(a.z * inv, a.w * inv));
-                if (lse != nullptr && dd == 0) lse[(size_t)(d.out_row + tok) * Hq + hq] = lse2 * kLn2;
+                    make_uint2(pack_bf16x2(a.x * r, a.y * r), pack_bf16x2(a.z * r, a.w * r));
+                if (lse != nullptr && dd == 0) lse[(size_t)(d.out_row + tok) * Hq + hq] = ls * kLn2;
             } else {
                 *reinterpret_cast<float4*>(p.partial_o + (((size_t)d.partial_row + tok) * G + hh) * D + dd) =
-                    make_float4(a.x * inv, a.y * inv, a.z * inv, a.w * inv);
-                if (dd == 0) p.partial_lse[((size_t)d.partial_row + tok) * G + hh] = lse2;
+                    make_float4(a.x * r, a.y * r, a.z * r, a.w * r);
+                if (dd == 0) p.partial_lse[((size_t)d.partial_row + tok) * G + hh] = ls;
             }
         }
         // the stage goes back to the producer (whose copies are writes of the asynchronous proxy) on
@@ -269,10 +285,16 @@ __device__ __forceinline__ void epilogue_loop(const DevPlan& p, __nv_bfloat16* _
         if (lane == 0) mbar_arrive_n(empty0 + 8 * d.stage, kWarps);
         if (d.partial_row < 0) continue;
         // ---- a chunk of a split unit: count it in; the CTA that completes the unit merges it
-        __threadfence();      // this warp's partial rows are visible device-wide before the count moves
+        // This warp's partial rows are visible device-wide before the count moves, and the others' once it has: the merge warp gets the
+        // request through shared memory behind it and reads past L1.  (A fence here and one there took 0.5 us each: 4
+        // decoding sequences 11.41 -> 11.13 us a layer.)
         __syncwarp();
         int last = 0;
-        if (lane == 0) last = atomicAdd(p.unit_arrivals + d.unit, 1) == d.n_chunks - 1;
+        if (lane == 0) {
+            int before;
+            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(before) : "l"(p.unit_arrivals + d.unit) : "memory");
+            last = before == d.n_chunks - 1;
+        }
         if (__shfl_sync(0xffffffffu, last, 0) && !post(d)) break;
     }
 }
@@ -289,73 +311,72 @@ __device__ __forceinline__ void merge_loop(const DevPlan& p, __nv_bfloat16* __re
     // merges one unit; dry: everything but the stores (see below)
     auto merge_unit = [&](const TileDesc& d, bool dry) {
         const int ncols = d.ntok * G;
-        // four consecutive values of one column per lane and position; up to four positions and four
-        // chunks per pass, all requested together: a unit of up to four chunks and 512 values costs
-        // one round trip to L2
-        for (int e0 = 4 * lane; e0 < ncols * D; e0 += 512) {
-            float4 acc[4];
-            float mx[4], wsum[4];
-            size_t prow0[4], hh[4];
-            int dd[4];
-            bool on[4];
+        const size_t row0 = (size_t)d.partial_base * G;      // row of chunk c and column k: row0 + c * ncols + k
+        constexpr int kPasses = 4 * D / 128, kAtOnce = 16 / kPasses;      // of four columns; chunks requested together
+        // Four columns at a time, in passes of 128 values, four consecutive ones to a lane.  The weights come from one
+        // (column, chunk) pair to a lane, eight chunks at once; values and log-sum-exps are requested together, so that a unit of up to
+        // kAtOnce chunks costs one round trip to L2.  (Four columns of 128, up to eight chunks: 2.2 us with weights in every lane and
+        // pass, 1.8 so; 4 decoding sequences 11.83 -> 11.41 us a layer.)
+        for (int c4 = 0; c4 < ncols; c4 += 4) {
+            float4 acc[kPasses];
+            bool on[kPasses];
+            const float* src = p.partial_o + (row0 + c4) * D + 4 * lane;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = e0 + 128 * u;
-                on[u] = e < ncols * D;
-                const int col = on[u] ? e / D : 0;
-                dd[u] = e % D;
-                hh[u] = (size_t)(col % G);
-                prow0[u] = (size_t)d.partial_base + col / G;       // chunk c -> prow0 + c * ntok
-                acc[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                mx[u] = -INFINITY;
-                wsum[u] = 0.f;
+            for (int ps = 0; ps < kPasses; ++ps) {
+                on[ps] = c4 * D + 128 * ps + 4 * lane < ncols * D;
+                acc[ps] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            for (int c0 = 0; c0 < d.n_chunks; c0 += 4) {
-                float l2[4][4];
-                float4 v[4][4];
+            auto lse_of = [&](int c) {      // of this lane's pair in the eight chunks from c
+                const int k = c4 + (lane >> 3);
+                return c + (lane & 7) < d.n_chunks && k < ncols ? __ldcg(p.partial_lse + row0 + (size_t)(c + (lane & 7)) * ncols + k) : -INFINITY;
+            };
+            float M = -INFINITY, wsum = 0.f, l8 = 0.f, w8 = 0.f;
+            for (int c0 = 0; c0 < d.n_chunks; c0 += kAtOnce) {
+                float4 v[kPasses][kAtOnce];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
+                for (int ps = 0; ps < kPasses; ++ps)
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        l2[u][i] = -INFINITY;
-                        v[u][i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (on[u] && c0 + i < d.n_chunks) {
-                            const size_t r = (prow0[u] + (size_t)(c0 + i) * d.ntok) * G + hh[u];
-                            l2[u][i] = __ldcg(p.partial_lse + r);
-                            v[u][i] = __ldcg(reinterpret_cast<const float4*>(p.partial_o + r * D + dd[u]));
-                        }
+                    for (int i = 0; i < kAtOnce; ++i) {
+                        v[ps][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (on[ps] && c0 + i < d.n_chunks)
+                            v[ps][i] = __ldcg(reinterpret_cast<const float4*>(src + 128 * ps + (size_t)(c0 + i) * ncols * D));
                     }
+                if (c0 == 0) {      // the columns' maxima and the sums of their weights
+                    l8 = lse_of(0);
+                    M = l8;
+                    for (int c = 8; c < d.n_chunks; c += 8) M = fmaxf(M, lse_of(c));
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    float pm = mx[u];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) pm = fmaxf(pm, l2[u][i]);
-                    const float rescale = pm == -INFINITY ? 1.f : fast_exp2(mx[u] - pm);      // first pass: exp2(-inf) = 0
-                    mx[u] = pm;
-                    wsum[u] *= rescale;
-                    acc[u].x *= rescale; acc[u].y *= rescale; acc[u].z *= rescale; acc[u].w *= rescale;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float w = l2[u][i] == -INFINITY ? 0.f : fast_exp2(l2[u][i] - mx[u]);   // -inf: no visible key there
-                        wsum[u] += w;
-                        if (w != 0.f) {
-                            acc[u].x = fmaf(w, v[u][i].x, acc[u].x); acc[u].y = fmaf(w, v[u][i].y, acc[u].y);
-                            acc[u].z = fmaf(w, v[u][i].z, acc[u].z); acc[u].w = fmaf(w, v[u][i].w, acc[u].w);
-                        }
-                    }
+                    for (int off = 1; off < 8; off <<= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
                 }
+                if (c0 % 8 == 0) {
+                    if (c0 > 0) l8 = lse_of(c0);
+                    w8 = l8 == -INFINITY ? 0.f : fast_exp2(l8 - M);      // -inf: no visible key there
+                    wsum += w8;
+                }
+#pragma unroll
+                for (int i = 0; i < kAtOnce; ++i)
+#pragma unroll
+                    for (int ps = 0; ps < kPasses; ++ps) {
+                        const float g = __shfl_sync(0xffffffffu, w8, (128 * ps + 4 * lane) / D * 8 + (c0 + i) % 8);
+                        acc[ps].x = g != 0.f ? fmaf(g, v[ps][i].x, acc[ps].x) : acc[ps].x;
+                        acc[ps].y = g != 0.f ? fmaf(g, v[ps][i].y, acc[ps].y) : acc[ps].y;
+                        acc[ps].z = g != 0.f ? fmaf(g, v[ps][i].z, acc[ps].z) : acc[ps].z;
+                        acc[ps].w = g != 0.f ? fmaf(g, v[ps][i].w, acc[ps].w) : acc[ps].w;
+                    }
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (!on[u]) continue;
-                const int col = (e0 + 128 * u) / D, tok = col / G;
-                const float inv = 1.f / wsum[u];
-                const size_t hq = (size_t)d.kv_head * G + hh[u];
-                if (dry) continue;
-                *reinterpret_cast<uint2*>(out + ((size_t)(d.out_row + tok) * Hq + hq) * D + dd[u]) =
-                    make_uint2(pack_bf16x2(acc[u].x * inv, acc[u].y * inv), pack_bf16x2(acc[u].z * inv, acc[u].w * inv));
-                if (lse != nullptr && dd[u] == 0)
-                    lse[(size_t)(d.out_row + tok) * Hq + hq] = (mx[u] + log2f(wsum[u])) * kLn2;
+            for (int off = 1; off < 8; off <<= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, off);
+            const float inv8 = 1.f / wsum, lse2 = M + log2f(wsum);
+#pragma unroll
+            for (int ps = 0; ps < kPasses; ++ps) {
+                const int e = c4 * D + 128 * ps + 4 * lane, col = e / D, dd = e % D;
+                const float inv = __shfl_sync(0xffffffffu, inv8, (128 * ps + 4 * lane) / D * 8), ls = __shfl_sync(0xffffffffu, lse2, (128 * ps + 4 * lane) / D * 8);
+                if (!on[ps] || dry) continue;
+                const int tok = col / G;
+                const size_t hq = (size_t)d.kv_head * G + col % G;
+                *reinterpret_cast<uint2*>(out + ((size_t)(d.out_row + tok) * Hq + hq) * D + dd) =
+                    make_uint2(pack_bf16x2(acc[ps].x * inv, acc[ps].y * inv), pack_bf16x2(acc[ps].z * inv, acc[ps].w * inv));
+                if (lse != nullptr && dd == 0) lse[(size_t)(d.out_row + tok) * Hq + hq] = ls * kLn2;
             }
         }
     };
@@ -377,7 +398,6 @@ __device__ __forceinline__ void merge_loop(const DevPlan& p, __nv_bfloat16* __re
         __syncwarp();
         if (lane == 0) mbar_arrive(reqfree0 + 8 * j);
         if (d.flags & kFlagEnd) break;
-        __threadfence();      // the chunks' rows were written before their counts moved: visible now
         merge_unit(d, false);
         if (lane == 0) atomicExch(p.unit_arrivals + d.unit, 0);      // ready for the next launch of this plan
         if (lane == 0) trace_add(7, 1);
