@@ -1,4 +1,4 @@
-"""ctypes binding of libasynclm.so: argument marshalling only.
+"""Binding of libasynclm.so (ctypes, and a CPython extension for the per-layer calls): argument marshalling only.
 
 Every step of the path (planning, append, attention, merge) runs inside the shared library; this
 module converts Python objects to the C structs of include/asynclm.h and owns the two workspaces a
@@ -143,6 +143,32 @@ def load(rebuild_if_stale: bool = True):
     return lib
 
 
+_call_ext = None          # the extension of csrc/call_ext.c, False where it cannot be had
+
+
+def _calls():
+    """The extension that marshals the per-layer calls, bound to the loaded library; False: they go through ctypes."""
+    global _call_ext
+    if _call_ext is None:
+        lib = load()
+        try:
+            import importlib.util
+
+            import torch
+            path = _build.build_call_ext()
+            spec = importlib.util.spec_from_file_location("call_ext", path)
+            ext = importlib.util.module_from_spec(spec)
+            spec.loader.exec_module(ext)
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
+            ext.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.asynclm_plan, lib.asynclm_kv_append, lib.asynclm_kv_append_rope,
+                                                                        lib.asynclm_attn_mixed, lib.asynclm_step)),
+                     torch.cuda.current_device, raw)
+            _call_ext = ext
+        except (ImportError, OSError, RuntimeError, AttributeError, TypeError):
+            _call_ext = False
+    return _call_ext
+
+
 def strerror(status: int) -> str:
     return load().asynclm_strerror(int(status)).decode()
 
@@ -241,6 +267,12 @@ def asynclm_plan(shape, num_pages, q_indptr, kv_len_before, page_indptr, page_in
     host_ws (pinned uint8 tensor) and dev_ws (cuda uint8 tensor) may be supplied for reuse;
     otherwise they are sized exactly by a host-only dry run and allocated here.
     """
+    if host_ws is not None and dev_ws is not None and not opts and (ext := _calls()):
+        got = ext.plan(shape, int(num_pages), q_indptr, kv_len_before, page_indptr, page_indices, stream, float(sm_scale), host_ws, dev_ws)
+        if got is not None:
+            if got[0] != 0:
+                _check(got[0], "asynclm_plan")
+            return Plan(got[1], host_ws, dev_ws, None)
     import torch
     lib = load()
     cs, co = _cshape(shape, num_pages, sm_scale), _copts(**opts)
@@ -277,30 +309,40 @@ def _stream_ptr(stream):
 
 def asynclm_kv_append(plan: Plan, k_new, v_new, kv_pool, stream=None) -> None:
     """Scatter the step's new K/V rows (device tensors) into kv_pool through the page table."""
-    _check(load().asynclm_kv_append(plan.handle, k_new.data_ptr(), v_new.data_ptr(),
-                                    kv_pool.data_ptr(), _stream_ptr(stream)), "asynclm_kv_append")
+    ext = _calls()
+    rc = ext.append(plan.handle, k_new, v_new, kv_pool, stream) if ext else load().asynclm_kv_append(
+        plan.handle, k_new.data_ptr(), v_new.data_ptr(), kv_pool.data_ptr(), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "asynclm_kv_append")
 
 
 def asynclm_kv_append_rope(plan: Plan, k_new, v_new, kv_pool, q_inout=None, rope_theta=500000.0, stream=None) -> None:
     """asynclm_kv_append with the keys (and, if given, the queries, in place) rotated by their positions."""
-    _check(load().asynclm_kv_append_rope(plan.handle, k_new.data_ptr(), v_new.data_ptr(), kv_pool.data_ptr(),
-                                         None if q_inout is None else q_inout.data_ptr(), float(rope_theta),
-                                         _stream_ptr(stream)), "asynclm_kv_append_rope")
+    ext = _calls()
+    rc = ext.append_rope(plan.handle, k_new, v_new, kv_pool, q_inout, float(rope_theta), stream) if ext else load().asynclm_kv_append_rope(
+        plan.handle, k_new.data_ptr(), v_new.data_ptr(), kv_pool.data_ptr(), None if q_inout is None else q_inout.data_ptr(),
+        float(rope_theta), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "asynclm_kv_append_rope")
 
 
 def asynclm_attn_mixed(plan: Plan, q, kv_pool, out, lse=None, stream=None) -> None:
     """Attention of every new row over its sequence's pages; writes `out` (bf16) and `lse` (fp32)."""
-    _check(load().asynclm_attn_mixed(plan.handle, q.data_ptr(), kv_pool.data_ptr(), out.data_ptr(),
-                                     None if lse is None else lse.data_ptr(), _stream_ptr(stream)),
-           "asynclm_attn_mixed")
+    ext = _calls()
+    rc = ext.attn(plan.handle, q, kv_pool, out, lse, stream) if ext else load().asynclm_attn_mixed(
+        plan.handle, q.data_ptr(), kv_pool.data_ptr(), out.data_ptr(), None if lse is None else lse.data_ptr(), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "asynclm_attn_mixed")
 
 
 def asynclm_step(plan: Plan, q, k_new, v_new, kv_pool, out, lse=None, stream=None) -> None:
     """Append and attention in one launch (asynclm_kv_append + asynclm_attn_mixed)."""
-    _check(load().asynclm_step(plan.handle, q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(),
-                               kv_pool.data_ptr(), out.data_ptr(),
-                               None if lse is None else lse.data_ptr(), _stream_ptr(stream)),
-           "asynclm_step")
+    ext = _calls()
+    rc = ext.step(plan.handle, q, k_new, v_new, kv_pool, out, lse, stream) if ext else load().asynclm_step(
+        plan.handle, q.data_ptr(), k_new.data_ptr(), v_new.data_ptr(), kv_pool.data_ptr(), out.data_ptr(),
+        None if lse is None else lse.data_ptr(), _stream_ptr(stream))
+    if rc != 0:
+        _check(rc, "asynclm_step")
 
 
 def kv_swap_staging_bytes(shape, num_pages: int, n_pages: int) -> int:

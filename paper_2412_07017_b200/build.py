@@ -6,6 +6,7 @@ import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
@@ -18,6 +19,9 @@ TRACE_LIB = os.path.join(CSRC, "libasynclm_trace.so")
 # a bad id sets the plan's status word and is not used (an append leaves the row out, a read takes page 0).  For
 # bringing up a new caller.
 DEBUG_LIB = os.path.join(CSRC, "libasynclm_debug.so")
+# Argument marshalling of the per-layer calls, a CPython extension (see csrc/call_ext.c); the binding does without it where it
+# cannot be built.
+CALL_EXT = os.path.join(HERE, "call_ext" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -41,6 +45,24 @@ def is_stale() -> bool:
     return any(os.path.getmtime(f) > t for f in _inputs())
 
 
+def build_call_ext(force: bool = False) -> str | None:
+    """The path of the built extension, or None where there is no compiler or no Python header for it."""
+    src = os.path.join(CSRC, "call_ext.c")
+    inputs = [src, os.path.join(INCLUDE, "asynclm.h"), os.path.abspath(__file__)]
+    if not force and os.path.exists(CALL_EXT) and all(os.path.getmtime(f) <= os.path.getmtime(CALL_EXT) for f in inputs):
+        return CALL_EXT
+    cc = shutil.which("gcc") or shutil.which("cc")
+    header = sysconfig.get_paths()["include"]
+    if cc is None or not os.path.exists(os.path.join(header, "Python.h")):
+        return CALL_EXT if os.path.exists(CALL_EXT) else None
+    tmp = CALL_EXT + f".tmp{os.getpid()}"
+    proc = subprocess.run([cc, "-O2", "-Wall", "-shared", "-fPIC", "-I", header, "-I", INCLUDE, "-o", tmp, src], capture_output=True, text=True)
+    if proc.returncode != 0:
+        raise RuntimeError("cc failed:\n" + proc.stdout + proc.stderr)
+    os.replace(tmp, CALL_EXT)
+    return CALL_EXT
+
+
 def find_nvcc():
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     return nvcc if os.path.exists(nvcc) else None
@@ -48,6 +70,11 @@ def find_nvcc():
 
 def build(force: bool = False, verbose: bool = False, trace: bool = False, debug: bool = False) -> str:
     lib = TRACE_LIB if trace else DEBUG_LIB if debug else LIB
+    try:
+        build_call_ext(force)
+    except RuntimeError:      # (the binding does without it)
+        if force:
+            raise
     if not force and not trace and not debug and not is_stale():
         return lib
     nvcc = find_nvcc()

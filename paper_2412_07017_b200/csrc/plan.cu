@@ -915,9 +915,18 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
 
     const int n_split = (int)split_units.size();
 
+    // CTAs without an item, which stand at the end, have something to do only where there is a queue: else they are not
+    // launched, and their headers (384 bytes each, of which a small plan mostly consists) are neither cleared nor uploaded.
+    int grid_cuda = ctas_cuda, grid_tensor = ctas_tensor;
+    if (queue_count == 0 && ctas_cuda == ctas_tensor) {
+        auto idle = [&](int c) { return cta_indptr_cuda[(size_t)c] == cta_indptr_cuda[(size_t)c + 1] && cta_indptr_tensor[(size_t)c] == cta_indptr_tensor[(size_t)c + 1]; };
+        while (grid_cuda > 1 && idle(grid_cuda - 1)) --grid_cuda;
+        grid_tensor = grid_cuda;
+    }
+
     // ---- pack ---------------------------------------------------------------------------------
-    BlobLayout L = layout_blob(B, T, total_pages, (int64_t)units.size(), n_items, ctas_cuda,
-                               ctas_tensor, (int64_t)n_split, (int64_t)merge_blocks.size());
+    BlobLayout L = layout_blob(B, T, total_pages, (int64_t)units.size(), n_items, grid_cuda,
+                               grid_tensor, (int64_t)n_split, (int64_t)merge_blocks.size());
     const size_t plan_bytes = align_up(sizeof(asynclm_plan_s), 256);
     const size_t item_cta_bytes = align_up(sizeof(int32_t) * (size_t)std::max(n_items, 1), 256);
     const size_t host_need = plan_bytes + L.blob_bytes + item_cta_bytes;
@@ -950,7 +959,7 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     for (size_t i = 0; i < units.size(); ++i) h_units[i] = units[i].u;
     if (n_items > 0) std::memcpy(hb + L.off_items, items.data(), sizeof(Item) * (size_t)n_items);
     int32_t* h_heads = (int32_t*)(hb + L.off_heads);
-    std::memset(h_heads, 0, sizeof(int32_t) * kHeadWords * (size_t)std::max(ctas_cuda, ctas_tensor));
+    std::memset(h_heads, 0, sizeof(int32_t) * kHeadWords * (size_t)std::max(grid_cuda, grid_tensor));
     Work* h_works = (Work*)(hb + L.off_works);
     for (int i = 0; i < n_items; ++i) {
         const Item& it = items[(size_t)i];
@@ -970,12 +979,12 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
         w.q_seq0 = q_indptr[u.seq];
         h_works[i] = w;
     }
-    for (int c = 0; c < std::max(ctas_cuda, ctas_tensor); ++c) {
+    for (int c = 0; c < std::max(grid_cuda, grid_tensor); ++c) {
         int32_t* h = h_heads + (size_t)c * kHeadWords;
-        const int32_t range[4] = {c < ctas_tensor ? cta_indptr_tensor[(size_t)c] : 0,
-                                  c < ctas_tensor ? cta_indptr_tensor[(size_t)c + 1] : 0,
-                                  c < ctas_cuda ? cta_indptr_cuda[(size_t)c] : 0,
-                                  c < ctas_cuda ? cta_indptr_cuda[(size_t)c + 1] : 0};
+        const int32_t range[4] = {c < grid_tensor ? cta_indptr_tensor[(size_t)c] : 0,
+                                  c < grid_tensor ? cta_indptr_tensor[(size_t)c + 1] : 0,
+                                  c < grid_cuda ? cta_indptr_cuda[(size_t)c] : 0,
+                                  c < grid_cuda ? cta_indptr_cuda[(size_t)c + 1] : 0};
         std::memcpy(h, range, sizeof(range));
         for (int path = 0; path < 2; ++path) {
             const int first = range[2 * path], last = range[2 * path + 1];
@@ -987,9 +996,9 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
                 h[(path == 0 ? kHeadPagesTensor : kHeadPagesCuda) + k] = batch->page_indices[w.page0 + k];
         }
     }
-    std::memcpy(hb + L.off_cta_cuda, cta_indptr_cuda.data(), sizeof(int32_t) * (size_t)(ctas_cuda + 1));
+    std::memcpy(hb + L.off_cta_cuda, cta_indptr_cuda.data(), sizeof(int32_t) * (size_t)(grid_cuda + 1));
     std::memcpy(hb + L.off_cta_tensor, cta_indptr_tensor.data(),
-                sizeof(int32_t) * (size_t)(ctas_tensor + 1));
+                sizeof(int32_t) * (size_t)(grid_tensor + 1));
     if (n_split > 0) std::memcpy(hb + L.off_split, split_units.data(), sizeof(int32_t) * split_units.size());
     if (!merge_blocks.empty())
         std::memcpy(hb + L.off_merge, merge_blocks.data(), sizeof(int32_t) * merge_blocks.size());
@@ -1042,8 +1051,8 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     d.num_items_tensor = n_items - n_items_cuda;
     d.num_split_units = n_split;
     d.num_merge_blocks = (int32_t)merge_blocks.size();
-    d.num_ctas_cuda = ctas_cuda;
-    d.num_ctas_tensor = ctas_tensor;
+    d.num_ctas_cuda = grid_cuda;
+    d.num_ctas_tensor = grid_tensor;
     d.num_q_heads = shape->num_q_heads;
     d.num_kv_heads = Hkv;
     d.head_dim = shape->head_dim;
