@@ -14,10 +14,10 @@
 // of the kv head; unused columns carry zeros.  About 70 warp instructions per page instead of 700.
 //
 // Structure: one persistent CTA per SM walks the item list the planner gave it.  A producer warp
-// streams the items' pages into a shared-memory ring of 128-key stages, one tiled TMA copy per
+// streams the items' pages into a shared-memory ring of 64 KiB stages (128 keys, 256 at head_dim 64), one tiled TMA copy per
 // (page, kv head) that brings the K block and the V block together and lands them with the
 // 128-byte swizzle that makes ldmatrix conflict-free; a small descriptor and the unit's query rows
-// travel with each stage.  Eight consumer warps take one page of a stage each: ldmatrix, the two
+// travel with each stage.  Eight consumer warps take one page of a stage each (two at head_dim 64): ldmatrix, the two
 // contractions, softmax against a lazily moved reference maximum on the accumulator fragment
 // (4 values per thread), P transposed in registers (movmatrix) into the B operand.  At the end of
 // an item each consumer warp drops its state into its own page slot of the item's last stage and
@@ -42,7 +42,7 @@ namespace asynclm {
 
 namespace dec {
 
-constexpr int kWarps = 8;                    // consumer warps: one page of a 128-key stage each
+constexpr int kWarps = 8;                    // consumer warps: a page of a stage each, or two (Geometry::WARP_PAGES)
 constexpr int kProducerWarp = kWarps;        // the warp behind them streams the pages
 constexpr int kEpilogueWarp = kWarps + 1;    // combines the consumers' states at the end of an item
 constexpr int kMergeWarp = kWarps + 2;       // merges the chunks of a split unit once all have arrived
@@ -52,7 +52,6 @@ constexpr int kMergeReqs = 4;                // merge requests in flight between
 constexpr int kMaxStages = 6;
 constexpr int kHandoffs = kMaxStages + 2;    // item hand-offs in flight: a stage each, so at most kMaxStages
 constexpr int kCols = 8;                     // (token, head) columns of a unit: the N of the MMAs
-constexpr int kTileTok = kWarps * kPage;     // keys per ring stage
 constexpr int kPrefetchMinPages = 24;        // of a first item that is brought into L2 ahead
 constexpr float kRescaleThreshold = 8.f;     // log2 units a score may exceed the reference max by
 constexpr long long kWaitCycles = 2000000000ll;
@@ -171,7 +170,10 @@ struct Geometry {
     static constexpr int HALVES = D / 64;                       // 128-byte pieces of a K or V row
     static constexpr int BLOCK_BYTES = kPage * D * 2;           // one (page, K|V, head) block
     static constexpr int PAGE_BYTES = 2 * BLOCK_BYTES;          // K block + V block: one TMA copy
-    static constexpr int STAGE_BYTES = kWarps * PAGE_BYTES;     // 64 KiB at d = 128
+    static constexpr int WARP_PAGES = 128 / D;                  // pages of a stage that a consumer warp takes, kWarps apart
+    static constexpr int STAGE_PAGES = kWarps * WARP_PAGES;
+    static constexpr int STAGE_TOK = STAGE_PAGES * kPage;       // keys per ring stage: 128 or 256
+    static constexpr int STAGE_BYTES = STAGE_PAGES * PAGE_BYTES;      // 64 KiB
     static constexpr int Q_BYTES = kCols * D * 2;               // the unit's query rows, [column][d]
     static constexpr int KSTEPS = D / 16;
     // merge area of a warp inside its page slot: O^T as [column][d + 4] fp32 (the pad keeps the
@@ -474,8 +476,8 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             for (int k = k0; k < k1; ++k)
                 while (!mbar_try_wait(full0 + 8 * (k % S), (uint32_t)(k / S) & 1u) && clock64() - t0 < kWaitCycles) {}
         };
-        constexpr int kPagesPerTile = kTileTok / kPage;       // 8
-        constexpr int kGroupTiles = 32 / kPagesPerTile;       // 4
+        constexpr int kTileTok = Geo::STAGE_TOK, kPagesPerTile = Geo::STAGE_PAGES;
+        constexpr int kGroupTiles = 32 / kPagesPerTile;       // 4 or 2
         bool ok = true;
         int taken = 0;
         int pages_cur = 0;
@@ -713,44 +715,71 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             m0 = m1 = -INFINITY;
             l0 = l1 = 0.f;
         }
-        const int key0 = warp * kPage;                    // this warp's page inside the stage
-        if (key0 < d.rows) {
-            const uint32_t page_smem = smem_u32(stage) + (uint32_t)warp * Geo::PAGE_BYTES;
-            const int valid = d.rows - key0;              // slots of the page that hold keys of the sequence
-            if (valid < kPage) {
-                // Slots past the sequence's end hold whatever was in the page before: their scores are
-                // masked below, but 0 * NaN would still poison P V, so their V rows are cleared.
-                for (int r = valid + (lane >> 4); r < kPage; r += 2)
+        // This warp's pages inside the stage: `warp` and, at head_dim 64, the one kWarps behind it.  Two pages at once are two
+        // independent chains of loads, MMAs and exponentials: with one, a warp took as long for a page as at head_dim 128, for half the
+        // bytes, and that time bound a CTA.  (ns for 128 keys of head_dim 64, one page | two: one CTA alone 710 | 528, 56 of them 730 |
+        // 577, 148, which memory bounds, 768 | 644; us of attention a layer: 64 decoding sequences of 32/8 heads over 1-3 K keys
+        // 47.8 -> 44.6, 256 of 8/2 heads 29.9 -> 27.8, 32 with 8 spans 49.1 -> 46.3, 100 of 8/2 heads with 20 spans 49.2 -> 42.0.)
+        constexpr int WP = Geo::WARP_PAGES;
+        if (warp * kPage < d.rows) {
+            bool on[WP];
+            float sc[WP][4];
 #pragma unroll
-                    for (int h = 0; h < Geo::HALVES; ++h)
-                        if ((lane & 15) < 8)
-                            *reinterpret_cast<uint4*>(stage + (size_t)warp * Geo::PAGE_BYTES + Geo::BLOCK_BYTES + h * 2048 +
-                                                      r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
-                __syncwarp();
+            for (int pp = 0; pp < WP; ++pp) {
+                const int key0 = (pp * kWarps + warp) * kPage;
+                on[pp] = pp == 0 || key0 < d.rows;
+                const int valid = d.rows - key0;              // slots of the page that hold keys of the sequence
+                if (on[pp] && valid < kPage) {
+                    // Slots past the sequence's end hold whatever was in the page before: their scores are
+                    // masked below, but 0 * NaN would still poison P V, so their V rows are cleared.
+                    for (int r = valid + (lane >> 4); r < kPage; r += 2)
+#pragma unroll
+                        for (int h = 0; h < Geo::HALVES; ++h)
+                            if ((lane & 15) < 8)
+                                *reinterpret_cast<uint4*>(stage + (size_t)(pp * kWarps + warp) * Geo::PAGE_BYTES + Geo::BLOCK_BYTES + h * 2048 +
+                                                          r * 128 + (lane & 7) * 16) = make_uint4(0, 0, 0, 0);
+                    __syncwarp();
+                }
             }
+            auto page_smem = [&](int pp) { return smem_u32(stage) + (uint32_t)(pp * kWarps + warp) * Geo::PAGE_BYTES; };
             // ---- S^T = K Q^T, two accumulators so that the MMAs are not one dependent chain
-            float sa[4] = {0.f, 0.f, 0.f, 0.f}, sb[4] = {0.f, 0.f, 0.f, 0.f};
+            float sa[WP][4], sb[WP][4];
+#pragma unroll
+            for (int pp = 0; pp < WP; ++pp)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sa[pp][e] = sb[pp][e] = 0.f;
 #pragma unroll
             for (int ks = 0; ks < Geo::KSTEPS; ++ks) {
                 const int piece = 2 * ks + k_piece;       // 16-byte piece of the row: half piece / 8
-                uint32_t a[4];
-                ldsm_x4(page_smem + (uint32_t)(piece >> 3) * 2048u + k_row + ((((uint32_t)piece & 7u) ^ k_swz) << 4), a);
-                if (ks & 1) mma_bf16(sb, a, qb[ks][0], qb[ks][1]);
-                else mma_bf16(sa, a, qb[ks][0], qb[ks][1]);
-            }
-            float sc[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) sc[e] = (sa[e] + sb[e]) * qscale;      // log2 domain
-            // ---- mask: key key0 + g (+8) is visible to column c iff it lies below lim0 + token(c)
-            if (d.lim0 < key0 + kPage) {
-                const int lim_a = d.lim0 + (2 * t4) / G - key0, lim_b = d.lim0 + (2 * t4 + 1) / G - key0;
-                if (g >= lim_a) sc[0] = -INFINITY;
-                if (g >= lim_b) sc[1] = -INFINITY;
-                if (g + 8 >= lim_a) sc[2] = -INFINITY;
-                if (g + 8 >= lim_b) sc[3] = -INFINITY;
+                for (int pp = 0; pp < WP; ++pp) {
+                    if (!on[pp]) continue;
+                    uint32_t a[4];
+                    ldsm_x4(page_smem(pp) + (uint32_t)(piece >> 3) * 2048u + k_row + ((((uint32_t)piece & 7u) ^ k_swz) << 4), a);
+                    if (ks & 1) mma_bf16(sb[pp], a, qb[ks][0], qb[ks][1]);
+                    else mma_bf16(sa[pp], a, qb[ks][0], qb[ks][1]);
+                }
+            }
+#pragma unroll
+            for (int pp = 0; pp < WP; ++pp) {
+                const int key0 = (pp * kWarps + warp) * kPage;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sc[pp][e] = on[pp] ? (sa[pp][e] + sb[pp][e]) * qscale : -INFINITY;      // log2 domain
+                // ---- mask: key key0 + g (+8) is visible to column c iff it lies below lim0 + token(c)
+                if (d.lim0 < key0 + kPage) {
+                    const int lim_a = d.lim0 + (2 * t4) / G - key0, lim_b = d.lim0 + (2 * t4 + 1) / G - key0;
+                    if (g >= lim_a) sc[pp][0] = -INFINITY;
+                    if (g >= lim_b) sc[pp][1] = -INFINITY;
+                    if (g + 8 >= lim_a) sc[pp][2] = -INFINITY;
+                    if (g + 8 >= lim_b) sc[pp][3] = -INFINITY;
+                }
             }
             // ---- softmax against the lazily moved reference maxima of this thread's two columns
-            float c0 = fmaxf(sc[0], sc[2]), c1 = fmaxf(sc[1], sc[3]);
+            float c0 = fmaxf(sc[0][0], sc[0][2]), c1 = fmaxf(sc[0][1], sc[0][3]);
+            if constexpr (WP == 2) {
+                c0 = fmaxf(c0, fmaxf(sc[1][0], sc[1][2]));
+                c1 = fmaxf(c1, fmaxf(sc[1][1], sc[1][3]));
+            }
             if (__any_sync(0xffffffffu, c0 > m0 + kRescaleThreshold || c1 > m1 + kRescaleThreshold)) {
 #pragma unroll
                 for (int off = 4; off < 32; off <<= 1) {
@@ -768,20 +797,28 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
                 }
             }
             const float u0 = m0 == -INFINITY ? 0.f : m0, u1 = m1 == -INFINITY ? 0.f : m1;
-            const float p0 = fast_exp2(sc[0] - u0), p1 = fast_exp2(sc[1] - u1);
-            const float p2 = fast_exp2(sc[2] - u0), p3 = fast_exp2(sc[3] - u1);
-            l0 += p0 + p2;
-            l1 += p1 + p3;
-            // P (keys x columns, bf16) -> P^T as the B operand: two 8x8 transposes in registers
-            const uint32_t b0 = movmatrix_t(pack_bf16x2(p0, p1));
-            const uint32_t b1 = movmatrix_t(pack_bf16x2(p2, p3));
+            uint32_t b0[WP], b1[WP];
+#pragma unroll
+            for (int pp = 0; pp < WP; ++pp) {
+                const float p0 = fast_exp2(sc[pp][0] - u0), p1 = fast_exp2(sc[pp][1] - u1);
+                const float p2 = fast_exp2(sc[pp][2] - u0), p3 = fast_exp2(sc[pp][3] - u1);
+                l0 += p0 + p2;
+                l1 += p1 + p3;
+                // P (keys x columns, bf16) -> P^T as the B operand: two 8x8 transposes in registers
+                b0[pp] = movmatrix_t(pack_bf16x2(p0, p1));
+                b1[pp] = movmatrix_t(pack_bf16x2(p2, p3));
+            }
             // ---- O^T += V^T P^T
 #pragma unroll
-            for (int i = 0; i < Geo::KSTEPS; ++i) {
-                const int piece = 2 * i + v_piece;
-                uint32_t a[4];
-                ldsm_x4_t(page_smem + (uint32_t)(piece >> 3) * 2048u + v_row + ((((uint32_t)piece & 7u) ^ v_swz) << 4), a);
-                mma_bf16(o[i], a, b0, b1);
+            for (int pp = 0; pp < WP; ++pp) {
+                if (!on[pp]) continue;
+#pragma unroll
+                for (int i = 0; i < Geo::KSTEPS; ++i) {
+                    const int piece = 2 * i + v_piece;
+                    uint32_t a[4];
+                    ldsm_x4_t(page_smem(pp) + (uint32_t)(piece >> 3) * 2048u + v_row + ((((uint32_t)piece & 7u) ^ v_swz) << 4), a);
+                    mma_bf16(o[i], a, b0[pp], b1[pp]);
+                }
             }
         }
 

@@ -111,6 +111,8 @@ struct StreamCost {
     int64_t tile_ns, least_tile_ns;      // 128 keys on a CTA while kStreamCtas stream, and while few do
     int64_t cut_ns;                      // what a cut sixth costs at the end: more boundaries, partial rows, merges
 };
+// (Those of head_dim 64 were taken with a warp body that had one page of a stage for each warp; 640 and 570 are what it takes with two.
+// 11 batches of one length and 11 others come out the same with either.)
 constexpr int kStreamCtas = 148;
 constexpr StreamCost stream_cost(int head_dim) {
     return head_dim == 64 ? StreamCost{700, 630, 2500} : StreamCost{1390, 834, 5000};
@@ -288,8 +290,9 @@ constexpr PathCost kTensorOnlyCost{128, 1543, 8000, 2400};
 constexpr int64_t kTensorOnlyDualTileNs = 3126;
 // Warp body: 64 KB per 128-key tile (32 KB at head_dim 64).  It is bound by memory, so its tile time depends on
 // how many SMs stream at once: 1.39 us when all 148 do, 1.05 us (62 KB/us) when half of them run span tiles,
-// which draw some bandwidth too, 0.77 us for 74 and 0.68 for one by themselves; at head_dim 64 0.77, 0.75 and
-// 0.67.  The model takes the second figure.
+// which draw some bandwidth too, 0.79 us for 74 and 0.73 for one by themselves; at head_dim 64 0.64, 0.58 for 37 to
+// 100 and 0.53 for one.  The model takes the second figure for both.  (At head_dim 64 900 here gives layers of 0.88 to 1.08 of the time
+// with 1050, 750 of 0.90 to 1.11, without a rule to tell which batch gains.)
 constexpr PathCost kWarpCost{128, 1050, 400, 2000};
 // No step ends before its bytes have crossed the memory bus: K/V pages stream at about 6 bytes per
 // nanosecond on this access pattern (4 KB runs through a shuffled page table), after about 3 us in

@@ -427,3 +427,19 @@ def test_pools_of_many_shapes_by_turns():
            for k, (d, ql) in enumerate([(d, ql) for d in (128, 64) for ql in ([1, 40], [40, 33], [1, 1])] * 4)]
     for wl in wls + wls:
         run_and_check(wl, what=f"{wl.num_pages} pages, {wl.steps[0].q_len}")
+
+
+@pytest.mark.parametrize("Hq,Hkv", [(8, 1), (8, 2), (4, 2), (4, 4)])
+def test_stages_of_two_pages_a_warp(Hq, Hkv):
+    """head_dim 64: a stage is 256 keys and a consumer warp has two of its pages.  Contexts that end in either of them, on and beside
+    the edges of pages, half stages and stages; causal limits of short spans that fall into the second page; chunks of half a stage."""
+    shape = W.Shape(Hq, Hkv, 64, 16)
+    ctx = [0, 14, 15, 16, 126, 127, 128, 143, 200, 239, 254, 255, 256, 271, 383, 384, 511, 512, 700]
+    wl = W.make_single_step("two pages", shape, ctx, [1] * len(ctx), seed=6400 + Hkv, interleave_pages=True, poison_unused=True)
+    for opts in ({}, {"kv_chunk_tokens": 128}, {"kv_chunk_tokens": 64}, {"num_sms": 2}):
+        _, _, plan = run_and_check(wl, what=f"decode {Hq}/{Hkv} {opts}", **opts)
+        assert plan.info["num_items_tensor"] == 0
+    ctx, ql = [120, 121, 127, 128, 250, 251, 256, 380], [9, 7, 16, 5, 7, 6, 3, 8]
+    wl = W.make_single_step("two pages", shape, ctx, ql, seed=6500 + Hkv, interleave_pages=True, poison_unused=True)
+    for opts in ({}, {"kv_chunk_tokens": 64}):
+        run_and_check(wl, what=f"spans {Hq}/{Hkv} {opts}", flags=B.PLAN_NO_TENSOR_PATH, **opts)
