@@ -60,7 +60,8 @@ extern "C" int asynclm_kv_append(const asynclm_plan_t* plan, const void* k_new, 
     if (!k_new || !v_new || !kv_pool || !aligned16(k_new) || !aligned16(v_new) || !aligned16(kv_pool))
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
-    return cuda_status(launch_kv_append(plan->dev, k_new, v_new, kv_pool, (cudaStream_t)stream));
+    const PlanUse use(plan, (cudaStream_t)stream);
+    return cuda_status(launch_kv_append(use.dev, k_new, v_new, kv_pool, (cudaStream_t)stream));
 }
 
 extern "C" int asynclm_attn_mixed(const asynclm_plan_t* plan, const void* q, const void* kv_pool,
@@ -71,9 +72,10 @@ extern "C" int asynclm_attn_mixed(const asynclm_plan_t* plan, const void* q, con
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = cuda_status(launch_attention(plan->dev, q, kv_pool, out, lse, s));
+    const PlanUse use(plan, s);
+    int rc = cuda_status(launch_attention(use.dev, q, kv_pool, out, lse, s));
     if (rc != ASYNCLM_OK) return rc;
-    return cuda_status(launch_lse_merge(plan->dev, out, lse, s));
+    return cuda_status(launch_lse_merge(use.dev, out, lse, s));
 }
 
 extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const void* k_new, const void* v_new,
@@ -85,6 +87,7 @@ extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const voi
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
+    PlanUse use(plan, s);
     int rc;
     if (plan->dev.num_items_tensor > 0 || plan->max_q_len > kStepFusedMaxSpan) {
         // With the append fused in, every item copies the new rows it reads, so the units of one long span
@@ -94,14 +97,15 @@ extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const voi
         // 90 | 65, the same at head_dim 64 85 | 59, 24 sequences with a span each 122 | 72.  Steps without
         // span tiles keep the fused form: 4 decoding sequences 15.5 | 17.7, 16 with 8 spans of up to 7
         // tokens 49.5 | 49.9; with the append beside the first stages 12.6 a layer, from a graph, for the 4.)
-        rc = cuda_status(launch_kv_append(plan->dev, k_new, v_new, kv_pool, s));
+        rc = cuda_status(launch_kv_append(use.dev, k_new, v_new, kv_pool, s));
         if (rc != ASYNCLM_OK) return rc;
-        rc = cuda_status(launch_attention(plan->dev, q, kv_pool, out, lse, s));
+        use.dev.full_launch = 0;
+        rc = cuda_status(launch_attention(use.dev, q, kv_pool, out, lse, s));
     } else {
-        rc = cuda_status(launch_attention(plan->dev, q, kv_pool, out, lse, s, AppendSrc{k_new, v_new, kv_pool}));
+        rc = cuda_status(launch_attention(use.dev, q, kv_pool, out, lse, s, AppendSrc{k_new, v_new, kv_pool}));
     }
     if (rc != ASYNCLM_OK) return rc;
-    return cuda_status(launch_lse_merge(plan->dev, out, lse, s));
+    return cuda_status(launch_lse_merge(use.dev, out, lse, s));
 }
 
 #ifdef ASYNCLM_DEBUG

@@ -191,7 +191,7 @@ cudaError_t launch_decode(const DevPlan& p, const void* q, const void* pool, voi
     if (p.num_pages > kMaxMapPages) return cudaErrorInvalidValue;
     e = pool_map(kKvMap, p, pool, &map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, map,
+    return launch_when(!p.full_launch, attn_decode_kernel<D, G, APPEND>, dim3(p.num_ctas_cuda), dim3(dec::kThreads), smem, stream, p, map,
                       (const __nv_bfloat16*)pool, (const __nv_bfloat16*)q, (__nv_bfloat16*)out, lse, S, app);
 }
 
@@ -203,7 +203,7 @@ cudaError_t launch_tensor(const DevPlan& p, const void* q, const void* pool, voi
     CUtensorMap map;
     e = pool_map(kSpanMap, p, pool, &map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_append_tc_kernel<D, G>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
+    return launch_when(!p.full_launch, attn_append_tc_kernel<D, G>, dim3(p.num_ctas_tensor), dim3(tc::kThreads), smem, stream,
                       p, map, (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse);
 }
 
@@ -219,7 +219,7 @@ cudaError_t launch_fused(const DevPlan& p, const void* q, const void* pool, void
     e = pool_map(kKvMap, p, pool, &kv_map);
     if (e == cudaSuccess) e = pool_map(kSpanMap, p, pool, &span_map);
     if (e != cudaSuccess) return e;
-    return launch_pdl(attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, kv_map, span_map,
+    return launch_when(!p.full_launch, attn_fused_kernel<D, G>, dim3(p.num_ctas_cuda), dim3(tc::kThreads), smem, stream, p, kv_map, span_map,
                       (const __nv_bfloat16*)q, (const __nv_bfloat16*)pool, (__nv_bfloat16*)out, lse, S);
 }
 

@@ -69,10 +69,11 @@ extern "C" int asynclm_attn_mixed_static(const asynclm_plan_t* plan, const void*
     if (int rc = check_plan_device(plan->device)) return rc;
     void* base = nullptr;
     if (int rc = cuda_status(scratch_address(&base))) return rc;
-    DevPlan d = plan->dev;                       // same plan, partial results redirected
+    cudaStream_t s = (cudaStream_t)stream;
+    PlanUse use(plan, s);
+    DevPlan& d = use.dev;                        // same plan, partial results redirected
     d.partial_o = (float*)base;
     d.partial_lse = (float*)((unsigned char*)base + o_bytes);
-    cudaStream_t s = (cudaStream_t)stream;
     if (int rc = cuda_status(launch_attention(d, q, kv_pool, out, lse, s))) return rc;
     return cuda_status(launch_lse_merge(d, out, lse, s));
 }

@@ -6,6 +6,9 @@
 
 namespace asynclm {
 
+// The packed plan from page-locked host memory into the device workspace, by a kernel.
+cudaError_t upload_plan(void* dev, const void* host, size_t bytes, cudaStream_t stream);
+
 cudaError_t launch_kv_append(const DevPlan& p, const void* k_new, const void* v_new, void* kv_pool,
                              cudaStream_t stream);
 

@@ -45,7 +45,7 @@ cudaError_t launch_kv_append(const DevPlan& p, const void* k_new, const void* v_
     if (p.total_q == 0) return cudaSuccess;
     const int64_t total = (int64_t)p.total_q * p.num_kv_heads * 2 * (p.head_dim / 8);
     const int blocks = (int)((total + 255) / 256 < 148 * 8 ? (total + 255) / 256 : 148 * 8);
-    return launch_pdl(kv_append_kernel, dim3(blocks), dim3(256), 0, stream, p, (const uint4*)k_new, (const uint4*)v_new,
+    return launch_when(!p.full_launch, kv_append_kernel, dim3(blocks), dim3(256), 0, stream, p, (const uint4*)k_new, (const uint4*)v_new,
                       (uint4*)kv_pool);
 }
 

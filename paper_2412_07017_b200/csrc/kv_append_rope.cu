@@ -151,12 +151,13 @@ extern "C" int asynclm_kv_append_rope(const asynclm_plan_t* plan, const void* k_
     if (!k_new || !v_new || !kv_pool || (((uintptr_t)k_new | (uintptr_t)v_new | (uintptr_t)kv_pool | (uintptr_t)q_inout) & 15) != 0)
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
-    const DevPlan& p = plan->dev;
+    const PlanUse use(plan, (cudaStream_t)stream);
+    const DevPlan& p = use.dev;
     // One token per CTA while that leaves SMs idle (a step of single tokens is all latency), up to four
     // when there are enough tokens: then every thread of the CTA has an angle to evaluate.
     const int tokens = std::max(1, std::min(p.total_q / (148 * 2), kRopeTokens));
     const int work = tokens * (p.num_kv_heads + (q_inout ? p.num_q_heads : 0)) * (p.head_dim / 16);      // threads' worth of a CTA
     const int threads = std::min((work + 31) / 32 * 32, kRopeThreads);
-    return cuda_status(launch_pdl(kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), 0, (cudaStream_t)stream,
+    return cuda_status(launch_when(!p.full_launch, kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), 0, (cudaStream_t)stream,
                                   p, (const uint4*)k_new, (const uint4*)v_new, (uint4*)kv_pool, (uint4*)q_inout, log2(rope_theta), tokens));
 }

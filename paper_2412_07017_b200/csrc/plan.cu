@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "asynclm.h"
+#include "kernels.h"
 #include "plan_internal.h"
 
 namespace asynclm {
@@ -269,6 +270,11 @@ void cut_and_deal(const std::vector<int>& unit_ids, std::vector<UnitBuild>& unit
     cta_indptr[(size_t)n_ctas] = at;
 }
 
+
+// Plans of these sizes are uploaded by a kernel (see plan_upload.cu).  Smaller ones belong to steps that the host bounds, where the question
+// whether the workspace is page-locked costs more than the copy does; of larger ones the bus takes most of the time either way
+// (none was measured: 2 MB are pages of 7 million tokens).
+constexpr size_t kUploadMinBytes = 32 << 10, kUploadMaxBytes = 2 << 20;
 
 // Costs of the attention kernels on B200 as the packing sees them, in nanoseconds, used only to size the span
 // CTAs.  At head_dim 128 they are those of an earlier form of the span body with 128-key tiles, which the margins
@@ -1086,9 +1092,15 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     info.host_bytes_used = host_need;
 
     if (!host_only) {
-        cudaError_t e = cudaMemcpyAsync(db, hb, L.blob_bytes, cudaMemcpyHostToDevice,
-                                        (cudaStream_t)stream);
+        // By kernel where the workspace is page-locked, so that kernels can read it, and the plan neither so small that the
+        // copy engine is as fast nor so large that the bus is what takes the time.
+        cudaPointerAttributes at{};
+        const bool by_kernel = L.blob_bytes >= kUploadMinBytes && L.blob_bytes <= kUploadMaxBytes &&
+                               cudaPointerGetAttributes(&at, hb) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr;
+        cudaError_t e = by_kernel ? upload_plan(db, at.devicePointer, L.blob_bytes, (cudaStream_t)stream)
+                                  : cudaMemcpyAsync(db, hb, L.blob_bytes, cudaMemcpyHostToDevice, (cudaStream_t)stream);
         if (e != cudaSuccess) return ASYNCLM_ERR_CUDA;
+        plan->fresh = by_kernel ? 1 : 0;
     }
     *out_plan = plan;
     return ASYNCLM_OK;

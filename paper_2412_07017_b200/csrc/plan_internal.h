@@ -1,5 +1,6 @@
 // Host-side plan object and planner constants (internal).
 #pragma once
+#include <cuda_runtime.h>
 #include <math.h>
 
 #include "asynclm.h"
@@ -32,4 +33,31 @@ struct asynclm_plan_s {
     int32_t device;
     int32_t host_only;
     int32_t max_q_len;            // longest span of the step
+    mutable int32_t fresh;        // the upload was a kernel, and no launch has been ordered behind it yet (see PlanUse)
+    mutable unsigned long long captured_in;      // the last stream capture that a launch of a fresh plan went into
 };
+
+namespace asynclm {
+
+// The device plan for one call.  The kernels read the plan ahead of their wait for the kernel in front, which may only be as far as its
+// trigger then: what a copy in the stream wrote is complete and in no cache by that time, what a kernel in front is
+// writing need not be.  So the first launch behind an upload by kernel starts when that has completed, as behind a copy, and the others, which
+// come behind that one, early again.  (A captured launch orders nothing now: each capture has a first launch of its own, and the plan
+// stays fresh for launches outside.)
+struct PlanUse {
+    DevPlan dev;
+    PlanUse(const asynclm_plan_s* plan, cudaStream_t stream) : dev(plan->dev) {
+        dev.full_launch = 0;
+        if (__atomic_load_n(&plan->fresh, __ATOMIC_ACQUIRE) == 0) return;
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        unsigned long long id = 0;
+        if (cudaStreamGetCaptureInfo(stream, &status, &id) == cudaSuccess && status == cudaStreamCaptureStatusActive) {
+            dev.full_launch = __atomic_exchange_n(&plan->captured_in, id, __ATOMIC_ACQ_REL) != id;
+        } else {
+            dev.full_launch = 1;
+            __atomic_store_n(&plan->fresh, 0, __ATOMIC_RELEASE);
+        }
+    }
+};
+
+}  // namespace asynclm

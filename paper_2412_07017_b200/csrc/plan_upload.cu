@@ -1,0 +1,49 @@
+// A plan's way to the GPU as a kernel that reads it out of page-locked host memory.
+//
+// A copy in the stream stands between two steps' kernels for 12-17 us, whatever its 100-300 KB take on the bus: the copy engine
+// starts when the kernel in front has been flushed, and the kernel behind when the copy has.  This kernel is resident
+// while the kernel in front runs out, has requested its share from the host by then and only stores it behind the wait.
+// (Whole passes, copy | kernel: four steps of 256 sequences, planned anew each, 816 | 777 us; 64 decoding sequences in 8 layers 669 |
+// 660, 24 spans in 4 layers 344 | 337, 4 decoding sequences in 32 layers 386 | 377, 32 of head_dim 64 in 16 layers 781 | 771.)
+#include <algorithm>
+
+#include "common.cuh"
+#include "kernels.h"
+
+namespace asynclm {
+
+namespace {
+
+constexpr int kUploadThreads = 256, kUploadAhead = 8;      // 16-byte vectors that a thread requests ahead of the wait
+
+__device__ __forceinline__ uint4 ld_host(const uint4* p) {      // never from a cache: the host rewrites its workspace
+    uint4 v;
+    asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+__global__ void __launch_bounds__(kUploadThreads)
+plan_upload_kernel(uint4* __restrict__ dev, const uint4* host, int n) {
+    const int step = gridDim.x * kUploadThreads;
+    int i = blockIdx.x * kUploadThreads + threadIdx.x;
+    uint4 v[kUploadAhead];
+#pragma unroll
+    for (int k = 0; k < kUploadAhead; ++k)
+        if (i + k * step < n) v[k] = ld_host(host + i + k * step);
+    pdl_wait();      // the workspace belongs to the kernels in front until those have completed
+#pragma unroll
+    for (int k = 0; k < kUploadAhead; ++k)
+        if (i + k * step < n) dev[i + k * step] = v[k];
+    for (i += kUploadAhead * step; i < n; i += step) dev[i] = ld_host(host + i);
+    // No early trigger: the kernels behind read the plan ahead of their own wait (see PlanUse).
+}
+
+}  // namespace
+
+cudaError_t upload_plan(void* dev, const void* host, size_t bytes, cudaStream_t stream) {
+    const int n = (int)(bytes / 16);      // (the sections of a plan are multiples of 256 bytes)
+    const int blocks = std::min(148, (n + kUploadThreads - 1) / kUploadThreads);
+    return launch_pdl(plan_upload_kernel, dim3(blocks), dim3(kUploadThreads), 0, stream, (uint4*)dev, (const uint4*)host, n);
+}
+
+}  // namespace asynclm

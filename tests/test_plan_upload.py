@@ -1,0 +1,149 @@
+"""Plans of middling size are uploaded by a kernel out of a page-locked workspace, and the kernels behind read them ahead of
+their wait for the one in front: whatever comes first behind an upload sees that plan and no older one."""
+import numpy as np
+import pytest
+
+from paper_2412_07017_b200 import binding as B
+from paper_2412_07017_b200 import workload as W
+
+pytestmark = pytest.mark.gpu
+SHAPE = W.Shape(32, 8, 64, 16)
+
+
+class Batch:
+    """24 sequences in one pool; the same lengths with another page table each time, so that plans differ in page ids only."""
+
+    def __init__(self):
+        import torch
+        g = np.random.default_rng(5)
+        self.ctx = g.integers(200, 900, 24).astype(np.int32)
+        self.qi = np.arange(25, dtype=np.int32)
+        need = -(-(self.ctx + 1) // 16)
+        self.pi = np.zeros(25, np.int32)
+        self.pi[1:] = np.cumsum(need)
+        self.pages = int(self.pi[-1]) + 300
+        torch.manual_seed(1)
+        self.pool = torch.randn(self.pages, 2, 8, 16, 64, device="cuda").bfloat16()
+        self.q = torch.randn(24, 32, 64, device="cuda").bfloat16()
+        self.k, self.v = (torch.randn(24, 8, 64, device="cuda").bfloat16() for _ in range(2))
+        host, dev = B.workspace_size(SHAPE, self.pages, 24, 24, int(self.pi[-1]))
+        self.dev_ws = torch.empty(dev, dtype=torch.uint8, device="cuda")
+        self.host_bytes = host
+        torch.cuda.synchronize()
+
+    def ids(self, k):
+        return np.random.default_rng(100 + k).permutation(self.pages)[:self.pi[-1]].astype(np.int32)
+
+    def plan(self, ids, host_ws):
+        return B.asynclm_plan(SHAPE, self.pages, self.qi, self.ctx, self.pi, ids, host_ws=host_ws, dev_ws=self.dev_ws)
+
+    def pinned(self):
+        import torch
+        return torch.empty(self.host_bytes, dtype=torch.uint8).pin_memory()
+
+    def call(self, plan, kind, pool, out):
+        if kind == "step":
+            B.asynclm_step(plan, self.q, self.k, self.v, pool, out, None)
+        else:
+            if kind == "rope":
+                B.asynclm_kv_append_rope(plan, self.k, self.v, pool, None, 1e4)
+            elif kind == "calls":
+                B.asynclm_kv_append(plan, self.k, self.v, pool)
+            (B.asynclm_attn_mixed_static if kind == "static" else B.asynclm_attn_mixed)(plan, self.q, pool, out, None)
+
+
+def bits(x):
+    import torch
+    return x.view(torch.int16).cpu()
+
+
+@pytest.mark.parametrize("kind", ["calls", "step", "rope", "attention", "static"])
+def test_steps_in_a_row_see_their_own_plan(kind):
+    """One device workspace, planned anew ahead of every step without waiting for anything, page-locked against pageable memory
+    (a copy in the stream) with a synchronisation around every call."""
+    import torch
+    t = Batch()
+    want = []
+    for k in range(6):
+        pool, out = t.pool.clone(), torch.empty_like(t.q)
+        plan = t.plan(t.ids(k), torch.empty(t.host_bytes, dtype=torch.uint8))
+        assert plan.info["device_bytes_used"] > 40000
+        torch.cuda.synchronize()
+        t.call(plan, kind, pool, out)
+        torch.cuda.synchronize()
+        want.append((bits(pool), bits(out)))
+    pools, outs = [t.pool.clone() for _ in range(6)], [torch.empty_like(t.q) for _ in range(6)]
+    slots, ids = [t.pinned() for _ in range(6)], [t.ids(k) for k in range(6)]
+    torch.cuda.synchronize()
+    for k in range(6):
+        plan = t.plan(ids[k], slots[k])
+        for _ in range(2):
+            t.call(plan, kind, pools[k], outs[k])
+    torch.cuda.synchronize()
+    assert B.last_device_status(plan) == 0
+    for k in range(6):
+        assert torch.equal(bits(pools[k]), want[k][0]) and torch.equal(bits(outs[k]), want[k][1]), k
+
+
+def test_captured_launches_and_launches_behind_a_capture():
+    """A capture between the upload and the first launch leaves that launch the first; the graph, replayed behind later uploads into the
+    same workspace, sees the plan that is there."""
+    import torch
+    t = Batch()
+    ws = [t.pinned() for _ in range(3)]
+    out = torch.empty_like(t.q)
+    warm = t.plan(t.ids(0), ws[0])
+    t.call(warm, "calls", t.pool.clone(), out)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    pool, pool2 = t.pool.clone(), t.pool.clone()
+    out2 = torch.empty_like(t.q)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        plan = t.plan(t.ids(1), ws[1])
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            t.call(plan, "calls", pool, out)
+            t.call(plan, "calls", pool, out)
+        t.call(plan, "calls", pool2, out2)
+        g.replay()
+        s.synchronize()
+        assert torch.equal(bits(out), bits(out2)) and torch.equal(bits(pool), bits(pool2))
+        first = bits(out)
+        t.plan(t.ids(2), ws[2])
+        g.replay()
+        s.synchronize()
+        again, ref = bits(out), torch.empty_like(t.q)
+        plan = t.plan(t.ids(2), torch.empty(t.host_bytes, dtype=torch.uint8))
+        s.synchronize()
+        t.call(plan, "attention", pool, ref)
+        s.synchronize()
+    assert torch.equal(again, bits(ref)) and not torch.equal(again, first)
+
+
+def test_a_captured_upload():
+    """The upload itself in a graph reads what the host workspace holds when the graph is launched."""
+    import torch
+    t = Batch()
+    ws, out, ref = t.pinned(), torch.empty_like(t.q), torch.empty_like(t.q)
+    pool = t.pool.clone()
+    t.call(t.plan(t.ids(0), ws), "calls", pool, out)
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s):
+        with torch.cuda.graph(g, stream=s):
+            plan = t.plan(t.ids(1), ws)
+            t.call(plan, "calls", pool, out)
+            t.call(plan, "attention", pool, out)
+        for k in (1, 2):
+            if k == 2:      # another plan of the same lengths, written by the planner on the host only
+                keep = ws.clone()
+                t.plan(t.ids(2), ws)
+                s.synchronize()
+                assert not torch.equal(keep, ws)
+                t.dev_ws.zero_()
+            g.replay()
+            s.synchronize()
+            t.call(t.plan(t.ids(k), torch.empty(t.host_bytes, dtype=torch.uint8)), "attention", pool, ref)
+            s.synchronize()
+            assert torch.equal(bits(out), bits(ref)), k
