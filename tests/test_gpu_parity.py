@@ -443,3 +443,15 @@ def test_stages_of_two_pages_a_warp(Hq, Hkv):
     wl = W.make_single_step("two pages", shape, ctx, ql, seed=6500 + Hkv, interleave_pages=True, poison_unused=True)
     for opts in ({}, {"kv_chunk_tokens": 64}):
         run_and_check(wl, what=f"spans {Hq}/{Hkv} {opts}", flags=B.PLAN_NO_TENSOR_PATH, **opts)
+
+
+@pytest.mark.parametrize("Hq,Hkv,d", [(8, 2, 128), (8, 1, 128), (2, 1, 128), (1, 1, 128), (8, 2, 64), (8, 1, 64), (2, 2, 64)])
+def test_units_merged_by_two_warps(Hq, Hkv, d):
+    """Nothing queued and an item at most for each CTA: two warps merge a unit, half of its values each.  Units of 2 to 24 chunks (rounds of
+    8 and 16 at once and their remainders), of one and of several tokens."""
+    shape = W.Shape(Hq, Hkv, d, 16)
+    for ctx, ql in (([3071], [1]), ([2200], [1]), ([1024, 300, 129], [1, 1, 1]), ([1150], [5]), ([1000, 130], [3, 2])):
+        wl = W.make_single_step("two mergers", shape, ctx, ql, seed=6600 + ctx[0], interleave_pages=True, poison_unused=True)
+        _, _, plan = run_and_check(wl, what=f"{ctx}", kv_chunk_tokens=128, flags=B.PLAN_NO_TENSOR_PATH)
+        items = plan.items()
+        assert plan.info["num_split_units"] > 0 and np.bincount(items["cta"]).max() == 1
