@@ -10,13 +10,14 @@
 // An fp64 sincos and exp2 cost a few hundred instructions, and an angle depends on the token and the
 // pair only, so a CTA takes whole tokens: their d / 2 angles are evaluated once, a thread each, kept in
 // shared memory and used by all heads.  (One thread per (head, 8 pairs) that evaluated its own eight
-// angles, one after the other, was bound by that arithmetic: 10.1 us against 6.2 now for 314 tokens of
-// 32 + 8 heads, d = 128, and 142 us against 41 for 8192 tokens, whose rows take 36 us at the copy rate.)
+// angles, one after the other, was bound by that arithmetic: 10.1 us against 6.2 so for 314 tokens of
+// 32 + 8 heads, d = 128, and 142 us against 41 for 8192 tokens, whose rows take 31 us at the copy rate.)
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
 #include <algorithm>
+#include <cstdint>
 
 #include "asynclm.h"
 #include "common.cuh"
@@ -33,8 +34,9 @@ __device__ __forceinline__ unsigned short f64_to_bf16(double x) {
     return *reinterpret_cast<const unsigned short*>(&h);
 }
 
-constexpr int kRopeThreads = 256, kRopeTokens = 4;
-constexpr unsigned kRopeFirstCtas = 148 * 4;      // a wave (three to an SM) and a little: see angles_first
+constexpr int kRopeThreads = 256, kRopeTokens = 20;      // of a CTA, at most
+constexpr int kRopeWave = 148 * 3;                // CTAs of that many threads that run at once
+constexpr unsigned kRopeFirstCtas = 148 * 4;      // a wave and a little: see angles_first
 
 // One row of one head as a thread holds it: 16-byte vectors v and v + half_vecs (values 8v .. 8v+7 and
 // their partners d/2 further), and those of the V row beside a K row.
@@ -77,7 +79,7 @@ kv_append_rope_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* _
     // about all CTAs start at once, the angles overlap the tail of the kernel in front, and the rows are requested behind
     // the wait that follows.  In a longer grid most CTAs start when that kernel has completed: they request their rows first.
     // (us a launch, call after call, rows first | angles first: 320 tokens of 32/8 heads 4.9 | 4.3, 512 7.3 | 6.5, 2048 16.0 |
-    // 16.0, 2400 16.7 | 17.7, 3000 19.1 | 18.4, 4096 24.6 | 25.3, 8192 43.0 | 44.4.)
+    // 16.0, 2400 16.7 | 17.7, 3000 19.1 | 18.4, 4096 24.6 | 25.3, 8192 43.0 | 44.4, with at most four tokens to a CTA.)
     const bool angles_first = gridDim.x <= kRopeFirstCtas;
     RopeRow cur{};
     if (!angles_first) {
@@ -153,9 +155,16 @@ extern "C" int asynclm_kv_append_rope(const asynclm_plan_t* plan, const void* k_
     if (int rc = check_plan_device(plan->device)) return rc;
     const PlanUse use(plan, (cudaStream_t)stream);
     const DevPlan& p = use.dev;
-    // One token per CTA while that leaves SMs idle (a step of single tokens is all latency), up to four
-    // when there are enough tokens: then every thread of the CTA has an angle to evaluate.
-    const int tokens = std::max(1, std::min(p.total_q / (148 * 2), kRopeTokens));
+    // As many tokens to a CTA as fill the fewest waves: a wave takes as long as its CTAs, about one token more than they
+    // have.  (us a launch from a graph, with one token for each 296 and at most four | so: 320 tokens of 32/8 heads 3.4 | 3.4, 512 5.7 |
+    // 4.9, 1200 8.8 | 7.8, 2048 15.1 | 12.0, 4096 23.7 | 21.1, 8192 41.9 | 38.7, at head_dim 64 6000 20.1 | 16.3; 6000 of 8/1
+    // heads 8.3 | 6.2.  With 16 at most 8192 take 43.2.)
+    int tokens = 1;
+    int64_t least = INT64_MAX;
+    for (int t = 1; t <= kRopeTokens; ++t) {
+        const int64_t ctas = ((int64_t)p.total_q + t - 1) / t, cost = (ctas + kRopeWave - 1) / kRopeWave * (t + 1);
+        if (cost < least) least = cost, tokens = t;
+    }
     const int work = tokens * (p.num_kv_heads + (q_inout ? p.num_q_heads : 0)) * (p.head_dim / 16);      // threads' worth of a CTA
     const int threads = std::min((work + 31) / 32 * 32, kRopeThreads);
     return cuda_status(launch_when(!p.full_launch, kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), 0, (cudaStream_t)stream,

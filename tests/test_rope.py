@@ -89,3 +89,26 @@ def test_rotated_append_on_both_sides_of_a_wave(q_lens):
         diff = got != ref
         assert diff.mean() < 1e-3 and ulp_diff(got[diff], ref[diff]).max(initial=0) <= 1
     assert np.array_equal(to_bits(pool_dev)[:, 1], ref_pool[:, 1])
+
+
+@pytest.mark.parametrize("tokens", [444, 445, 3001, 8437, 8881, 9001])      # of a CTA: 1, 2, 7, 20, and 11 in two waves
+def test_rotated_append_over_tokens_of_a_cta(tokens):
+    """The tokens of a CTA follow from the waves that they make: one, a few, the most, with a remainder in the last CTA, and grids of more than
+    one wave."""
+    import torch
+    from gpu_util import to_bits, to_dev
+    shape = W.Shape(2, 1, 64, 16)
+    wl = W.make_single_step("rope_tokens", shape, [3, 900, 31], [tokens - 40, 1, 39], seed=34, poison_unused=True)
+    st = wl.steps[0]
+    pool_dev, q_dev = to_dev(wl.kv_pool), to_dev(st.q)
+    plan = B.asynclm_plan(shape, wl.num_pages, st.q_indptr, st.kv_len_before, st.page_indptr, st.page_indices)
+    B.asynclm_kv_append_rope(plan, to_dev(st.k_new), to_dev(st.v_new), pool_dev, q_dev, 10000.0)
+    torch.cuda.synchronize()
+    pos = np.concatenate([np.arange(c, c + n) for c, n in zip(st.kv_len_before, st.q_len)])
+    rot = lambda bits: W.f32_to_bf16_bits(rope.rotate(W.bf16_bits_to_f64(bits), pos, 10000.0).astype(np.float32))
+    ref_pool = wl.kv_pool.copy()
+    oracle.kv_append(ref_pool, st.q_indptr, st.kv_len_before, st.page_indptr, st.page_indices, rot(st.k_new), st.v_new)
+    for got, ref in ((to_bits(pool_dev)[:, 0], ref_pool[:, 0]), (to_bits(q_dev), rot(st.q))):
+        diff = got != ref
+        assert diff.mean() < 1e-3 and ulp_diff(got[diff], ref[diff]).max(initial=0) <= 1
+    assert np.array_equal(to_bits(pool_dev)[:, 1], ref_pool[:, 1])
