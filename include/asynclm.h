@@ -161,8 +161,8 @@ int asynclm_plan_workspace_size(const asynclm_shape* shape, const asynclm_plan_o
  * spans are cut into chunks (long pieces first, short ones from a few units at the end) that the CTAs
  * take from a queue at run time, one atomic add per chunk, so that no cost model has to predict how
  * fast each SM streams.  Results do not depend on which CTA ran which chunk: partial results are
- * indexed by chunk and merged in chunk order.  Then ONE host->device copy of the packed plan is
- * enqueued on `stream`.
+ * indexed by chunk and merged in chunk order.  Then ONE upload of the packed plan is enqueued on `stream`: a
+ * copy, or, from page-locked memory and for all but small and very large plans, a kernel that reads it from there.
  *
  * Where the cuts would leave more partial results than asynclm_attn_mixed_static has room for, fewer of
  * the long spans are cut by keys, so that the plan serves that call too (a span divided by rows instead
@@ -175,7 +175,7 @@ int asynclm_plan_workspace_size(const asynclm_shape* shape, const asynclm_plan_o
  * the GPU (use one stream, as the layers of a model do, or order them with events).
  *
  *   host_ws / host_bytes  host memory (16-byte aligned; pinned recommended) that must stay
- *                         untouched until the copy has completed and for as long as the plan is
+ *                         untouched until the upload has completed and for as long as the plan is
  *                         used.
  *   dev_ws / dev_bytes    device memory (256-byte aligned) owned by the caller.  dev_ws == NULL
  *                         builds the plan on the host only (no CUDA call is made; opts->num_sms
