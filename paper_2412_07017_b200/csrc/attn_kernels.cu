@@ -86,18 +86,6 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 
 typedef CUresult (*ReplaceAddressFn)(CUtensorMap*, void*);
 
-// The driver's entry points are looked up once per process.
-template <typename Fn>
-cudaError_t driver_function(const char* name, Fn* fn) {
-    void* sym = nullptr;
-    cudaDriverEntryPointQueryResult qres;
-    cudaError_t e = cudaGetDriverEntryPoint(name, &sym, cudaEnableDefault, &qres);
-    if (e != cudaSuccess) return e;
-    if (qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-    *fn = (Fn)sym;
-    return cudaSuccess;
-}
-
 // The pool as the two bodies read it, landed with the 128-byte swizzle:
 //   kv    (64 values, 16 slots, d / 64 row halves, Hkv, pages x K|V), a box is one page's K and V blocks of one kv head
 //         (dec::tma_page_kv)

@@ -35,6 +35,13 @@ __device__ __forceinline__ uint4 ldg_nc_v4(const void* p) {
     return v;
 }
 
+// From page-locked host memory, never from a cache: the host rewrites it between launches.
+__device__ __forceinline__ uint4 ld_host_v4(const uint4* p) {
+    uint4 v;
+    asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
 // Programmatic dependent launch: a kernel launched with the programmatic-serialization attribute may
 // start while the kernel before it in the stream is still running; pdl_wait() blocks until that
 // kernel has completed and its writes are visible, pdl_trigger() lets the next kernel start early.

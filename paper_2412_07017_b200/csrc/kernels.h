@@ -6,6 +6,22 @@
 
 namespace asynclm {
 
+// The driver's entry points are looked up once per process.
+template <typename Fn>
+cudaError_t driver_function(const char* name, Fn* fn) {
+    void* sym = nullptr;
+    cudaDriverEntryPointQueryResult qres;
+    cudaError_t e = cudaGetDriverEntryPoint(name, &sym, cudaEnableDefault, &qres);
+    if (e != cudaSuccess) return e;
+    if (qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+    *fn = (Fn)sym;
+    return cudaSuccess;
+}
+
+// Page-locked host memory as kernels of the current device see it, or null: pageable or managed memory, and memory that is not
+// all in one allocation or one registration.
+void* page_locked_on_device(const void* host, size_t bytes);
+
 // The packed plan from page-locked host memory into the device workspace, by a kernel.
 cudaError_t upload_plan(void* dev, const void* host, size_t bytes, cudaStream_t stream);
 

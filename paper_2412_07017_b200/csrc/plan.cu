@@ -1094,12 +1094,10 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     if (!host_only) {
         // By kernel where the workspace is page-locked, so that kernels can read it, and the plan neither so small that the
         // copy engine is as fast nor so large that the bus is what takes the time.
-        cudaPointerAttributes at{};
-        const bool by_kernel = L.blob_bytes >= kUploadMinBytes && L.blob_bytes <= kUploadMaxBytes &&
-                               cudaPointerGetAttributes(&at, hb) == cudaSuccess && at.type == cudaMemoryTypeHost && at.devicePointer != nullptr;
-        cudaError_t e = by_kernel ? upload_plan(db, at.devicePointer, L.blob_bytes, (cudaStream_t)stream)
+        const void* by_kernel = L.blob_bytes >= kUploadMinBytes && L.blob_bytes <= kUploadMaxBytes ? page_locked_on_device(hb, L.blob_bytes) : nullptr;
+        cudaError_t e = by_kernel ? upload_plan(db, by_kernel, L.blob_bytes, (cudaStream_t)stream)
                                   : cudaMemcpyAsync(db, hb, L.blob_bytes, cudaMemcpyHostToDevice, (cudaStream_t)stream);
-        if (e != cudaSuccess) return ASYNCLM_ERR_CUDA;
+        if (int rc = cuda_status(e)) return rc;
         plan->fresh = by_kernel ? 1 : 0;
     }
     *out_plan = plan;

@@ -5,7 +5,10 @@
 // while the kernel in front runs out, has requested its share from the host by then and only stores it behind the wait.
 // (Whole passes, copy | kernel: four steps of 256 sequences, planned anew each, 816 | 777 us; 64 decoding sequences in 8 layers 669 |
 // 660, 24 spans in 4 layers 344 | 337, 4 decoding sequences in 32 layers 386 | 377, 32 of head_dim 64 in 16 layers 781 | 771.)
+#include <cuda.h>
+
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -16,12 +19,6 @@ namespace {
 
 constexpr int kUploadThreads = 256, kUploadAhead = 8;      // 16-byte vectors that a thread requests ahead of the wait
 
-__device__ __forceinline__ uint4 ld_host(const uint4* p) {      // never from a cache: the host rewrites its workspace
-    uint4 v;
-    asm volatile("ld.volatile.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-    return v;
-}
-
 __global__ void __launch_bounds__(kUploadThreads)
 plan_upload_kernel(uint4* __restrict__ dev, const uint4* host, int n) {
     const int step = gridDim.x * kUploadThreads;
@@ -29,16 +26,39 @@ plan_upload_kernel(uint4* __restrict__ dev, const uint4* host, int n) {
     uint4 v[kUploadAhead];
 #pragma unroll
     for (int k = 0; k < kUploadAhead; ++k)
-        if (i + k * step < n) v[k] = ld_host(host + i + k * step);
+        if (i + k * step < n) v[k] = ld_host_v4(host + i + k * step);
     pdl_wait();      // the workspace belongs to the kernels in front until those have completed
 #pragma unroll
     for (int k = 0; k < kUploadAhead; ++k)
         if (i + k * step < n) dev[i + k * step] = v[k];
-    for (i += kUploadAhead * step; i < n; i += step) dev[i] = ld_host(host + i);
+    for (i += kUploadAhead * step; i < n; i += step) dev[i] = ld_host_v4(host + i);
     // No early trigger: the kernels behind read the plan ahead of their own wait (see PlanUse).
 }
 
+typedef CUresult (*PointerAttributesFn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+
 }  // namespace
+
+void* page_locked_on_device(const void* host, size_t bytes) {
+    static std::atomic<PointerAttributesFn> attributes_fn{nullptr};
+    PointerAttributesFn attributes = attributes_fn.load(std::memory_order_acquire);
+    if (attributes == nullptr) {
+        if (driver_function("cuPointerGetAttributes", &attributes) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        attributes_fn.store(attributes, std::memory_order_release);
+    }
+    unsigned type = 0, managed = 0;
+    CUdeviceptr dev = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute which[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                    CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* to[5] = {&type, &managed, &dev, &start, &size};
+    if (attributes(5, which, to, (CUdeviceptr)(uintptr_t)host) != CUDA_SUCCESS) return nullptr;
+    if (type != CU_MEMORYTYPE_HOST || managed != 0 || dev == 0 || dev < start || dev - start > size || size - (dev - start) < bytes) return nullptr;
+    return (void*)(uintptr_t)dev;
+}
 
 cudaError_t upload_plan(void* dev, const void* host, size_t bytes, cudaStream_t stream) {
     const int n = (int)(bytes / 16);      // (the sections of a plan are multiples of 256 bytes)

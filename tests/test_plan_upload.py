@@ -121,6 +121,26 @@ def test_captured_launches_and_launches_behind_a_capture():
     assert torch.equal(again, bits(ref)) and not torch.equal(again, first)
 
 
+def test_a_workspace_of_two_registrations_is_refused():
+    """Page-locked in two parts that no single range covers: the copy refuses it, and no kernel reads it."""
+    import torch
+    t = Batch()
+    cut, base = 32768, torch.empty(t.host_bytes + 8192, dtype=torch.uint8)
+    base, rt = base[-base.data_ptr() % 4096:], torch.cuda.cudart()
+    parts = [(base.data_ptr(), cut), (base.data_ptr() + cut, -(-(t.host_bytes - cut) // 4096) * 4096)]
+    t.dev_ws.zero_()
+    for p, n in parts:
+        assert int(rt.cudaHostRegister(p, n, 0)) == 0
+    try:
+        with pytest.raises(B.AsynclmError, match="CUDA"):
+            t.plan(t.ids(1), base[:t.host_bytes])
+        torch.cuda.synchronize()
+    finally:
+        for p, n in parts:
+            rt.cudaHostUnregister(p)
+    assert not t.dev_ws.any()
+
+
 def test_a_captured_upload():
     """The upload itself in a graph reads what the host workspace holds when the graph is launched."""
     import torch
