@@ -282,12 +282,14 @@ int asynclm_last_device_status(const asynclm_plan_t* plan, void* stream, int32_t
  * asynclm_kv_swap_out copies page page_ids[j] of the pool to page j of the image: one gather kernel
  * into `staging`, then ONE device->host copy of the whole image.  asynclm_kv_swap_in is the reverse,
  * into whatever pages the sequence is given then (page_ids must be distinct): one host->device copy,
- * one scatter kernel.  Both are bit copies and asynchronous on `stream`; no other byte of the pool or
+ * one scatter kernel.  An image of at most 2 MB in page-locked memory is written and read by that kernel
+ * itself.  Both are bit copies and asynchronous on `stream`; no other byte of the pool or
  * of the image is written.  A model with several layers calls them once per layer's pool.
  *
  *   shape        head shape and pool capacity (page ids are checked against num_pages)
  *   page_ids     host, int32 [n_pages]; may be reused as soon as the call returns if it is pageable
- *                memory, and must stay untouched until the stream reaches the copy if it is pinned
+ *                memory, and must stay untouched until the stream reaches the copy if it is pinned (up to 960
+ *                ids outside a capture are taken at the call)
  *   kv_pool      device, layout above
  *   staging      device, 256-byte aligned, asynclm_kv_swap_staging_bytes(shape, n_pages) bytes, owned
  *                by the caller (the library allocates nothing)

@@ -67,3 +67,49 @@ def test_swap_out_and_in_are_bit_copies(Hq, Hkv, d):
     torch.cuda.synchronize()
     trap.swap_in(ref_pool, new, ref_image)
     assert np.array_equal(to_bits(pool_dev), ref_pool)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("hk,pages,memory", [(1, 1, "pinned"), (1, 511, "pinned"), (1, 512, "pinned"), (1, 513, "pinned"),
+                                             (1, 960, "pinned"), (1, 961, "pinned"), (3, 170, "pinned"), (3, 171, "pinned"),
+                                             (1, 512, "pageable"), (1, 961, "pageable"), (1, 300, "part of a larger one"), (1, 300, "captured")])
+def test_swaps_in_place_and_through_staging(hk, pages, memory):
+    """Images up to and beyond 2 MB (4096 bytes a page and head) and page ids up to and beyond those that parameters hold, behind
+    one another in one stream."""
+    import torch
+    shape, num = W.Shape(8, hk, 64, 16), 1200
+    g = np.random.default_rng(pages)
+    pool = g.integers(0, 1 << 16, (num, 2, hk, 16, 64)).astype(np.uint16)
+    old, new = (g.permutation(num)[:pages].astype(np.int32) for _ in range(2))
+    want_image = trap.swap_out(pool, old)
+    want = np.zeros_like(pool)
+    trap.swap_in(want, new, want_image)
+    src, dst = torch.from_numpy(pool.view(np.int16)).cuda(), torch.zeros(pool.shape, dtype=torch.int16, device="cuda")
+    staging = torch.empty(B.kv_swap_staging_bytes(shape, num, pages), dtype=torch.uint8, device="cuda")
+    whole = torch.full((pages + 2,) + pool.shape[1:], 77, dtype=torch.int16)
+    whole = whole if memory == "pageable" else whole.pin_memory()
+    image = whole[1:-1]
+    out = lambda ids: B.asynclm_kv_swap_out(shape, num, ids, src, staging, image)
+    back = lambda ids: B.asynclm_kv_swap_in(shape, num, ids, dst, staging, image)
+    torch.cuda.synchronize()
+    if memory == "captured":      # the graph reads ids and image when it runs
+        ids = torch.empty((2, pages), dtype=torch.int32).pin_memory()
+        ids[:] = torch.arange(pages, dtype=torch.int32)
+        graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph, stream=s):
+            out(ids[0].numpy()), back(ids[1].numpy())
+        ids[0], ids[1] = torch.from_numpy(old), torch.from_numpy(new)
+        graph.replay()
+    else:
+        for k in range(3):
+            ids = old.copy()
+            out(ids)
+            ids[:] = 0
+            if memory == "pageable":
+                torch.cuda.synchronize()
+            ids = new.copy()
+            back(ids)
+            ids[:] = 0
+    torch.cuda.synchronize()
+    assert np.array_equal(image.numpy().view(np.uint16), want_image) and (whole[0] == 77).all() and (whole[-1] == 77).all()
+    assert np.array_equal(dst.cpu().numpy().view(np.uint16), want) and np.array_equal(src.cpu().numpy().view(np.uint16), pool)
