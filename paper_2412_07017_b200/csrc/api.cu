@@ -60,8 +60,8 @@ extern "C" int asynclm_kv_append(const asynclm_plan_t* plan, const void* k_new, 
     if (!k_new || !v_new || !kv_pool || !aligned16(k_new) || !aligned16(v_new) || !aligned16(kv_pool))
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
-    const PlanUse use(plan, (cudaStream_t)stream);
-    return cuda_status(launch_kv_append(use.dev, k_new, v_new, kv_pool, (cudaStream_t)stream));
+    PlanUse use(plan, (cudaStream_t)stream);
+    return cuda_status(use.launched(launch_kv_append(use.dev, k_new, v_new, kv_pool, (cudaStream_t)stream)));
 }
 
 extern "C" int asynclm_attn_mixed(const asynclm_plan_t* plan, const void* q, const void* kv_pool,
@@ -72,8 +72,8 @@ extern "C" int asynclm_attn_mixed(const asynclm_plan_t* plan, const void* q, con
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    const PlanUse use(plan, s);
-    int rc = cuda_status(launch_attention(use.dev, q, kv_pool, out, lse, s));
+    PlanUse use(plan, s);
+    int rc = cuda_status(use.launched(launch_attention(use.dev, q, kv_pool, out, lse, s)));
     if (rc != ASYNCLM_OK) return rc;
     return cuda_status(launch_lse_merge(use.dev, out, lse, s));
 }
@@ -97,12 +97,11 @@ extern "C" int asynclm_step(const asynclm_plan_t* plan, const void* q, const voi
         // 90 | 65, the same at head_dim 64 85 | 59, 24 sequences with a span each 122 | 72.  Steps without
         // span tiles keep the fused form: 4 decoding sequences 15.5 | 17.7, 16 with 8 spans of up to 7
         // tokens 49.5 | 49.9; with the append beside the first stages 12.6 a layer, from a graph, for the 4.)
-        rc = cuda_status(launch_kv_append(use.dev, k_new, v_new, kv_pool, s));
+        rc = cuda_status(use.launched(launch_kv_append(use.dev, k_new, v_new, kv_pool, s)));
         if (rc != ASYNCLM_OK) return rc;
-        use.dev.full_launch = 0;
         rc = cuda_status(launch_attention(use.dev, q, kv_pool, out, lse, s));
     } else {
-        rc = cuda_status(launch_attention(use.dev, q, kv_pool, out, lse, s, AppendSrc{k_new, v_new, kv_pool}));
+        rc = cuda_status(use.launched(launch_attention(use.dev, q, kv_pool, out, lse, s, AppendSrc{k_new, v_new, kv_pool})));
     }
     if (rc != ASYNCLM_OK) return rc;
     return cuda_status(launch_lse_merge(use.dev, out, lse, s));

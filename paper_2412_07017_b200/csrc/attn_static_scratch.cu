@@ -74,7 +74,7 @@ extern "C" int asynclm_attn_mixed_static(const asynclm_plan_t* plan, const void*
     DevPlan& d = use.dev;                        // same plan, partial results redirected
     d.partial_o = (float*)base;
     d.partial_lse = (float*)((unsigned char*)base + o_bytes);
-    if (int rc = cuda_status(launch_attention(d, q, kv_pool, out, lse, s))) return rc;
+    if (int rc = cuda_status(use.launched(launch_attention(d, q, kv_pool, out, lse, s)))) return rc;
     return cuda_status(launch_lse_merge(d, out, lse, s));
 }
 

@@ -153,7 +153,7 @@ extern "C" int asynclm_kv_append_rope(const asynclm_plan_t* plan, const void* k_
     if (!k_new || !v_new || !kv_pool || (((uintptr_t)k_new | (uintptr_t)v_new | (uintptr_t)kv_pool | (uintptr_t)q_inout) & 15) != 0)
         return ASYNCLM_ERR_INVALID_ARG;
     if (int rc = check_plan_device(plan->device)) return rc;
-    const PlanUse use(plan, (cudaStream_t)stream);
+    PlanUse use(plan, (cudaStream_t)stream);
     const DevPlan& p = use.dev;
     // As many tokens to a CTA as fill the fewest waves: a wave takes as long as its CTAs, about one token more than they
     // have.  (us a launch from a graph, with one token for each 296 and at most four | so: 320 tokens of 32/8 heads 3.4 | 3.4, 512 5.7 |
@@ -167,6 +167,7 @@ extern "C" int asynclm_kv_append_rope(const asynclm_plan_t* plan, const void* k_
     }
     const int work = tokens * (p.num_kv_heads + (q_inout ? p.num_q_heads : 0)) * (p.head_dim / 16);      // threads' worth of a CTA
     const int threads = std::min((work + 31) / 32 * 32, kRopeThreads);
-    return cuda_status(launch_when(!p.full_launch, kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), 0, (cudaStream_t)stream,
-                                  p, (const uint4*)k_new, (const uint4*)v_new, (uint4*)kv_pool, (uint4*)q_inout, log2(rope_theta), tokens));
+    return cuda_status(use.launched(launch_when(!p.full_launch, kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), 0,
+                                                (cudaStream_t)stream, p, (const uint4*)k_new, (const uint4*)v_new, (uint4*)kv_pool,
+                                                (uint4*)q_inout, log2(rope_theta), tokens)));
 }

@@ -34,7 +34,7 @@ struct asynclm_plan_s {
     int32_t host_only;
     int32_t max_q_len;            // longest span of the step
     mutable int32_t fresh;        // the upload was a kernel, and no launch has been ordered behind it yet (see PlanUse)
-    mutable unsigned long long captured_in;      // the last stream capture that a launch of a fresh plan went into
+    mutable unsigned long long captured_in;      // 1 + the id of the last stream capture that a launch of a fresh plan went into, or 0
 };
 
 namespace asynclm {
@@ -42,21 +42,34 @@ namespace asynclm {
 // The device plan for one call.  The kernels read the plan ahead of their wait for the kernel in front, which may only be as far as its
 // trigger then: what a copy in the stream wrote is complete and in no cache by that time, what a kernel in front is
 // writing need not be.  So the first launch behind an upload by kernel starts when that has completed, as behind a copy, and the others, which
-// come behind that one, early again.  (A captured launch orders nothing now: each capture has a first launch of its own, and the plan
-// stays fresh for launches outside.)
-struct PlanUse {
+// come behind that one, early again.  A launch counts as the first when it has been accepted: behind a refused call the next one is
+// the first again.  (A captured launch orders nothing now: each capture has a first launch of its own, and the plan
+// stays fresh for launches outside.  So does a launch whose stream does not say whether it is being captured.)
+class PlanUse {
+    const asynclm_plan_s* plan;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusInvalidated;
+    unsigned long long id = 0;
+
+  public:
     DevPlan dev;
-    PlanUse(const asynclm_plan_s* plan, cudaStream_t stream) : dev(plan->dev) {
+
+    PlanUse(const asynclm_plan_s* p, cudaStream_t stream) : plan(p), dev(p->dev) {
         dev.full_launch = 0;
         if (__atomic_load_n(&plan->fresh, __ATOMIC_ACQUIRE) == 0) return;
-        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
-        unsigned long long id = 0;
-        if (cudaStreamGetCaptureInfo(stream, &status, &id) == cudaSuccess && status == cudaStreamCaptureStatusActive) {
-            dev.full_launch = __atomic_exchange_n(&plan->captured_in, id, __ATOMIC_ACQ_REL) != id;
-        } else {
-            dev.full_launch = 1;
-            __atomic_store_n(&plan->fresh, 0, __ATOMIC_RELEASE);
+        if (cudaStreamGetCaptureInfo(stream, &status, &id) != cudaSuccess) {
+            (void)cudaGetLastError();
+            status = cudaStreamCaptureStatusInvalidated;
         }
+        dev.full_launch = status != cudaStreamCaptureStatusActive || __atomic_load_n(&plan->captured_in, __ATOMIC_ACQUIRE) != id + 1;
+    }
+
+    // Takes and returns the outcome of the call's first launch with `dev`; what the call launches behind it starts early.
+    cudaError_t launched(cudaError_t e) {
+        if (e != cudaSuccess || dev.full_launch == 0) return e;
+        if (status == cudaStreamCaptureStatusActive) __atomic_store_n(&plan->captured_in, id + 1, __ATOMIC_RELEASE);
+        if (status == cudaStreamCaptureStatusNone) __atomic_store_n(&plan->fresh, 0, __ATOMIC_RELEASE);
+        dev.full_launch = 0;
+        return e;
     }
 };
 
