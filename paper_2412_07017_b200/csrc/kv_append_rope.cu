@@ -16,13 +16,11 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
-#include <algorithm>
-#include <cstdint>
-
 #include "asynclm.h"
 #include "common.cuh"
 #include "kernels.h"
 #include "plan_internal.h"
+#include "rope_grid.h"
 
 namespace asynclm {
 
@@ -33,10 +31,6 @@ __device__ __forceinline__ unsigned short f64_to_bf16(double x) {
     const __nv_bfloat16 h = __float2bfloat16_rn(__double2float_rn(x));
     return *reinterpret_cast<const unsigned short*>(&h);
 }
-
-constexpr int kRopeThreads = 256, kRopeTokens = 20;      // of a CTA, at most
-constexpr int kRopeWave = 148 * 3;                // CTAs of that many threads that run at once
-constexpr unsigned kRopeFirstCtas = 148 * 4;      // a wave and a little: see angles_first
 
 // One row of one head as a thread holds it: 16-byte vectors v and v + half_vecs (values 8v .. 8v+7 and
 // their partners d/2 further), and those of the V row beside a K row.
@@ -50,8 +44,8 @@ __global__ void __launch_bounds__(kRopeThreads)
 kv_append_rope_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* __restrict__ v_new,
                       uint4* __restrict__ pool, uint4* __restrict__ q, double log2_theta, int tokens) {
     // (cos, sin) of pair 8 v + k of token i at [i][k][v]: the threads of a warp read consecutive entries
-    __shared__ double2 rot[kRopeTokens * 64];
-    __shared__ int64_t slot[kRopeTokens];
+    extern __shared__ double2 rot[];      // [tokens][64]
+    int64_t* slot = reinterpret_cast<int64_t*>(rot + tokens * 64);
     pdl_trigger();   // the attention kernel may start its prologue; it waits for this grid before reading the pool
     const int d = p.head_dim, half_vecs = d / 16;                 // vectors in half a row: 8 or 4
     const int heads_k = p.num_kv_heads, heads_q = q != nullptr ? p.num_q_heads : 0, heads = heads_k + heads_q;
@@ -80,7 +74,7 @@ kv_append_rope_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* _
     // the wait that follows.  In a longer grid most CTAs start when that kernel has completed: they request their rows first.
     // (us a launch, call after call, rows first | angles first: 320 tokens of 32/8 heads 4.9 | 4.3, 512 7.3 | 6.5, 2048 16.0 |
     // 16.0, 2400 16.7 | 17.7, 3000 19.1 | 18.4, 4096 24.6 | 25.3, 8192 43.0 | 44.4, with at most four tokens to a CTA.)
-    const bool angles_first = gridDim.x <= kRopeFirstCtas;
+    const bool angles_first = gridDim.x <= (unsigned)kRopeFirstCtas;
     RopeRow cur{};
     if (!angles_first) {
         pdl_wait();
@@ -155,19 +149,9 @@ extern "C" int asynclm_kv_append_rope(const asynclm_plan_t* plan, const void* k_
     if (int rc = check_plan_device(plan->device)) return rc;
     PlanUse use(plan, (cudaStream_t)stream);
     const DevPlan& p = use.dev;
-    // As many tokens to a CTA as fill the fewest waves: a wave takes as long as its CTAs, about one token more than they
-    // have.  (us a launch from a graph, with one token for each 296 and at most four | so: 320 tokens of 32/8 heads 3.4 | 3.4, 512 5.7 |
-    // 4.9, 1200 8.8 | 7.8, 2048 15.1 | 12.0, 4096 23.7 | 21.1, 8192 41.9 | 38.7, at head_dim 64 6000 20.1 | 16.3; 6000 of 8/1
-    // heads 8.3 | 6.2.  With 16 at most 8192 take 43.2.)
-    int tokens = 1;
-    int64_t least = INT64_MAX;
-    for (int t = 1; t <= kRopeTokens; ++t) {
-        const int64_t ctas = ((int64_t)p.total_q + t - 1) / t, cost = (ctas + kRopeWave - 1) / kRopeWave * (t + 1);
-        if (cost < least) least = cost, tokens = t;
-    }
-    const int work = tokens * (p.num_kv_heads + (q_inout ? p.num_q_heads : 0)) * (p.head_dim / 16);      // threads' worth of a CTA
-    const int threads = std::min((work + 31) / 32 * 32, kRopeThreads);
-    return cuda_status(use.launched(launch_when(!p.full_launch, kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), 0,
+    const int heads = p.num_kv_heads + (q_inout ? p.num_q_heads : 0);
+    const int tokens = rope_tokens(p.total_q, heads, p.head_dim), threads = rope_threads(tokens, heads, p.head_dim);
+    return cuda_status(use.launched(launch_when(!p.full_launch, kv_append_rope_kernel, dim3((p.total_q + tokens - 1) / tokens), dim3(threads), rope_smem(tokens),
                                                 (cudaStream_t)stream, p, (const uint4*)k_new, (const uint4*)v_new, (uint4*)kv_pool,
                                                 (uint4*)q_inout, log2(rope_theta), tokens)));
 }

@@ -91,13 +91,15 @@ def test_rotated_append_on_both_sides_of_a_wave(q_lens):
     assert np.array_equal(to_bits(pool_dev)[:, 1], ref_pool[:, 1])
 
 
-@pytest.mark.parametrize("tokens", [444, 445, 3001, 8437, 8881, 9001])      # of a CTA: 1, 2, 7, 20, and 11 in two waves
-def test_rotated_append_over_tokens_of_a_cta(tokens):
-    """The tokens of a CTA follow from the waves that they make: one, a few, the most, with a remainder in the last CTA, and grids of more than
-    one wave."""
+# tokens of a CTA: 1, 1, 2, 7, 20, and 4 in several waves; with more heads 2, 4, and 8 in several waves
+@pytest.mark.parametrize("tokens,Hq,Hkv", [(444, 2, 1), (445, 2, 1), (593, 2, 1), (3001, 2, 1), (8437, 2, 1), (8881, 2, 1), (9001, 2, 1),
+                                           (445, 64, 8), (1775, 64, 8), (8881, 8, 8)])
+def test_rotated_append_over_tokens_of_a_cta(tokens, Hq, Hkv):
+    """The tokens of a CTA follow from the waves that they make (see test_rope_grid.py): one, a few, the most, with a remainder in the last CTA,
+    and grids of more than one wave."""
     import torch
     from gpu_util import to_bits, to_dev
-    shape = W.Shape(2, 1, 64, 16)
+    shape = W.Shape(Hq, Hkv, 64, 16)
     wl = W.make_single_step("rope_tokens", shape, [3, 900, 31], [tokens - 40, 1, 39], seed=34, poison_unused=True)
     st = wl.steps[0]
     pool_dev, q_dev = to_dev(wl.kv_pool), to_dev(st.q)
