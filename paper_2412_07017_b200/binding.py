@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 from dataclasses import dataclass
 from typing import Optional
 
@@ -147,25 +148,29 @@ _call_ext = None          # the extension of csrc/call_ext.c, False where it can
 
 
 def _calls():
-    """The extension that marshals the per-layer calls, bound to the loaded library; False: they go through ctypes."""
+    """The extension that marshals the per-layer calls, bound to the loaded library; False: they go through ctypes.  That is so without
+    a word only where there is nothing to build it with."""
     global _call_ext
     if _call_ext is None:
         lib = load()
+        ext = False
         try:
             import importlib.util
 
             import torch
             path = _build.build_call_ext()
-            spec = importlib.util.spec_from_file_location("call_ext", path)
-            ext = importlib.util.module_from_spec(spec)
-            spec.loader.exec_module(ext)
-            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
-            ext.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.asynclm_plan, lib.asynclm_kv_append, lib.asynclm_kv_append_rope,
-                                                                        lib.asynclm_attn_mixed, lib.asynclm_step)),
-                     torch.cuda.current_device, raw)
-            _call_ext = ext
-        except (ImportError, OSError, RuntimeError, AttributeError, TypeError):
-            _call_ext = False
+            if path is not None:
+                spec = importlib.util.spec_from_file_location("call_ext", path)
+                ext = importlib.util.module_from_spec(spec)
+                spec.loader.exec_module(ext)
+                raw = getattr(torch._C, "_cuda_getCurrentRawStream", None) or (lambda device: torch.cuda.current_stream(device).cuda_stream)
+                ext.bind(*(ctypes.cast(f, ctypes.c_void_p).value for f in (lib.asynclm_plan, lib.asynclm_kv_append, lib.asynclm_kv_append_rope,
+                                                                            lib.asynclm_attn_mixed, lib.asynclm_step)),
+                         torch.cuda.current_device, raw)
+        except (ImportError, OSError, RuntimeError, AttributeError, TypeError) as e:
+            ext = False
+            warnings.warn(f"the per-layer calls go through ctypes, because their extension cannot be built or loaded: {e}", RuntimeWarning, stacklevel=3)
+        _call_ext = ext
     return _call_ext
 
 

@@ -46,7 +46,8 @@ def is_stale() -> bool:
 
 
 def build_call_ext(force: bool = False) -> str | None:
-    """The path of the built extension, or None where there is no compiler or no Python header for it."""
+    """The path of the extension built from the present sources, or None where there is neither such a one nor a compiler and a Python
+    header to build it (one of other sources is not used: it may know other structs)."""
     src = os.path.join(CSRC, "call_ext.c")
     inputs = [src, os.path.join(INCLUDE, "asynclm.h"), os.path.abspath(__file__)]
     if not force and os.path.exists(CALL_EXT) and all(os.path.getmtime(f) <= os.path.getmtime(CALL_EXT) for f in inputs):
@@ -54,7 +55,7 @@ def build_call_ext(force: bool = False) -> str | None:
     cc = shutil.which("gcc") or shutil.which("cc")
     header = sysconfig.get_paths()["include"]
     if cc is None or not os.path.exists(os.path.join(header, "Python.h")):
-        return CALL_EXT if os.path.exists(CALL_EXT) else None
+        return None
     tmp = CALL_EXT + f".tmp{os.getpid()}"
     proc = subprocess.run([cc, "-O2", "-Wall", "-shared", "-fPIC", "-I", header, "-I", INCLUDE, "-o", tmp, src], capture_output=True, text=True)
     if proc.returncode != 0:
@@ -72,7 +73,7 @@ def build(force: bool = False, verbose: bool = False, trace: bool = False, debug
     lib = TRACE_LIB if trace else DEBUG_LIB if debug else LIB
     try:
         build_call_ext(force)
-    except RuntimeError:      # (the binding does without it)
+    except RuntimeError:      # (the binding tries again, says why and does without it)
         if force:
             raise
     if not force and not trace and not debug and not is_stale():

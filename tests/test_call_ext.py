@@ -1,12 +1,15 @@
 """The extension that marshals the per-layer calls takes what needs no conversion and leaves the rest to ctypes; both ways
 lead to the same call."""
 import array
+import os
 import types
+import warnings
 
 import numpy as np
 import pytest
 
 from paper_2412_07017_b200 import binding as B
+from paper_2412_07017_b200 import build as lib_build
 from paper_2412_07017_b200 import workload as W
 
 
@@ -15,9 +18,10 @@ def fake(ptr, n=0):
 
 
 def ext():
-    e = B._calls()
-    if not e:
+    if lib_build.build_call_ext() is None:
         pytest.skip("no C compiler or Python header here: the calls go through ctypes")
+    e = B._calls()
+    assert e, "it was built, but cannot be loaded or bound"
     return e
 
 
@@ -52,6 +56,29 @@ def test_what_is_refused_is_refused_with_the_same_exceptions():
     for rc in (e.append(0, fake(16), fake(16), fake(16), STREAM), e.append_rope(0, fake(16), fake(16), fake(16), None, 1e4, STREAM),
                e.attn(0, fake(16), fake(16), fake(16), None, STREAM), e.step(0, *[fake(16)] * 5, None, STREAM)):
         assert rc == -1      # no plan
+
+
+def test_an_extension_that_fails_is_named_and_an_old_one_is_not_used(monkeypatch, tmp_path):
+    def broken(force=False):
+        raise RuntimeError("cc failed: no such struct")
+    with monkeypatch.context() as m:
+        m.setattr(B, "_call_ext", None)
+        m.setattr(lib_build, "build_call_ext", broken)
+        with pytest.warns(RuntimeWarning, match="no such struct"):
+            assert B._calls() is False
+        assert B._calls() is False      # once is enough
+    with monkeypatch.context() as m:      # nothing to build it with, and none or an old one there
+        old = tmp_path / "call_ext.so"
+        m.setattr(lib_build, "CALL_EXT", str(old))
+        m.setattr(lib_build.shutil, "which", lambda name: None)
+        m.setattr(B, "_call_ext", None)
+        assert lib_build.build_call_ext() is None
+        old.write_bytes(b"")
+        os.utime(old, (1, 1))
+        assert lib_build.build_call_ext() is None
+        with warnings.catch_warnings():
+            warnings.simplefilter("error")
+            assert B._calls() is False
 
 
 def test_a_small_plan_holds_headers_of_the_ctas_it_uses_only():
