@@ -111,8 +111,8 @@ typedef struct asynclm_plan_info {
     int32_t num_split_units;  /* units whose keys were split into > 1 chunk */
     int32_t partial_rows;     /* rows of fp32 partial output held in the device workspace */
     int32_t kv_chunk_tokens;  /* chosen chunk length (INT32_MAX = unsplit) */
-    int32_t num_ctas_cuda;    /* persistent CTAs that may run the warp body */
-    int32_t num_ctas_tensor;  /* persistent CTAs that may run the span body */
+    int32_t num_ctas_cuda;    /* persistent CTAs launched that may run the warp body */
+    int32_t num_ctas_tensor;  /* persistent CTAs launched that may run the span body */
     int32_t num_items_tensor; /* items routed to the span body */
     int32_t launches_append;  /* kernels asynclm_kv_append launches */
     int32_t launches_attn;    /* kernels asynclm_attn_mixed launches */

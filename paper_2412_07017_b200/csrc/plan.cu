@@ -1080,8 +1080,8 @@ extern "C" int asynclm_plan(const asynclm_shape* shape, const asynclm_plan_optio
     int max_chunk = 0;
     for (const Item& it : items) max_chunk = std::max(max_chunk, it.kv1 - it.kv0);
     info.kv_chunk_tokens = fixed_chunk > 0 ? fixed_chunk : (d.num_split_units ? max_chunk : INT32_MAX);
-    info.num_ctas_cuda = ctas_cuda;
-    info.num_ctas_tensor = ctas_tensor;
+    info.num_ctas_cuda = grid_cuda;
+    info.num_ctas_tensor = grid_tensor;
     info.num_items_tensor = d.num_items_tensor;
     info.launches_append = T > 0 ? 1 : 0;
     // span tiles and decode rows share one fused launch when a step has both

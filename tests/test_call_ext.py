@@ -85,6 +85,10 @@ def test_a_small_plan_holds_headers_of_the_ctas_it_uses_only():
     p = B.plan_host(W.Shape(8, 2, 64, 16), 40, [0, 1, 2], [100, 200], [0, 7, 20], list(range(20)))
     used = int(p.items()["cta"].max()) + 1
     assert 0 < used < 148 and 384 * used <= p.info["device_bytes_used"] < 384 * 148
+    assert p.info["num_ctas_cuda"] == p.info["num_ctas_tensor"] == used
+    n = 300      # sequences whose work is queued: every CTA takes part
+    p = B.plan_host(W.Shape(8, 2, 64, 16), 20 * n, list(range(n + 1)), [300] * n, [20 * k for k in range(n + 1)], list(range(20 * n)))
+    assert (p.items()["cta"] < 0).any() and p.info["num_ctas_cuda"] == 148
 
 
 @pytest.mark.gpu
