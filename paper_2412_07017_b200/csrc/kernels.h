@@ -22,7 +22,10 @@ cudaError_t driver_function(const char* name, Fn* fn) {
 // all in one allocation or one registration.
 void* page_locked_on_device(const void* host, size_t bytes);
 
-// The packed plan from page-locked host memory into the device workspace, by a kernel.
+// The packed plan from page-locked host memory into the device workspace, by a kernel, for plans of these sizes.  Smaller ones belong to
+// steps that the host bounds, where the question whether the workspace is page-locked costs more than the copy does; of larger ones the bus
+// takes most of the time either way (none was measured: 2 MB are pages of 7 million tokens).
+constexpr size_t kUploadMinBytes = 32 << 10, kUploadMaxBytes = 2 << 20;
 cudaError_t upload_plan(void* dev, const void* host, size_t bytes, cudaStream_t stream);
 
 cudaError_t launch_kv_append(const DevPlan& p, const void* k_new, const void* v_new, void* kv_pool,

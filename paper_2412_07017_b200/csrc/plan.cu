@@ -270,12 +270,6 @@ void cut_and_deal(const std::vector<int>& unit_ids, std::vector<UnitBuild>& unit
     cta_indptr[(size_t)n_ctas] = at;
 }
 
-
-// Plans of these sizes are uploaded by a kernel (see plan_upload.cu).  Smaller ones belong to steps that the host bounds, where the question
-// whether the workspace is page-locked costs more than the copy does; of larger ones the bus takes most of the time either way
-// (none was measured: 2 MB are pages of 7 million tokens).
-constexpr size_t kUploadMinBytes = 32 << 10, kUploadMaxBytes = 2 << 20;
-
 // Costs of the attention kernels on B200 as the packing sees them, in nanoseconds, used only to size the span
 // CTAs.  At head_dim 128 they are those of an earlier form of the span body with 128-key tiles, which the margins
 // below were chosen with; the present body takes, per 128 keys with one | two row tiles, 0.9 | 1.55 us on a CTA

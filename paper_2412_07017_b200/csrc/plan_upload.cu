@@ -17,12 +17,13 @@ namespace asynclm {
 
 namespace {
 
-constexpr int kUploadThreads = 256, kUploadAhead = 8;      // 16-byte vectors that a thread requests ahead of the wait
+constexpr int kUploadCtas = 148, kUploadThreads = 256, kUploadAhead = 4;      // 16-byte vectors of a thread, at most, all requested ahead of the wait
+static_assert(kUploadMaxBytes <= (size_t)16 * kUploadCtas * kUploadThreads * kUploadAhead, "the largest plan is read in one pass");
 
 __global__ void __launch_bounds__(kUploadThreads)
 plan_upload_kernel(uint4* __restrict__ dev, const uint4* host, int n) {
     const int step = gridDim.x * kUploadThreads;
-    int i = blockIdx.x * kUploadThreads + threadIdx.x;
+    const int i = blockIdx.x * kUploadThreads + threadIdx.x;
     uint4 v[kUploadAhead];
 #pragma unroll
     for (int k = 0; k < kUploadAhead; ++k)
@@ -31,7 +32,6 @@ plan_upload_kernel(uint4* __restrict__ dev, const uint4* host, int n) {
 #pragma unroll
     for (int k = 0; k < kUploadAhead; ++k)
         if (i + k * step < n) dev[i + k * step] = v[k];
-    for (i += kUploadAhead * step; i < n; i += step) dev[i] = ld_host_v4(host + i);
     // No early trigger: the kernels behind read the plan ahead of their own wait (see PlanUse).
 }
 
@@ -61,8 +61,9 @@ void* page_locked_on_device(const void* host, size_t bytes) {
 }
 
 cudaError_t upload_plan(void* dev, const void* host, size_t bytes, cudaStream_t stream) {
+    if (bytes > kUploadMaxBytes) return cudaErrorInvalidValue;
     const int n = (int)(bytes / 16);      // (the sections of a plan are multiples of 256 bytes)
-    const int blocks = std::min(148, (n + kUploadThreads - 1) / kUploadThreads);
+    const int blocks = std::min(kUploadCtas, (n + kUploadThreads - 1) / kUploadThreads);
     return launch_pdl(plan_upload_kernel, dim3(blocks), dim3(kUploadThreads), 0, stream, (uint4*)dev, (const uint4*)host, n);
 }
 

@@ -1,5 +1,7 @@
 """Plans of middling size are uploaded by a kernel out of a page-locked workspace, and the kernels behind read them ahead of
 their wait for the one in front: whatever comes first behind an upload sees that plan and no older one."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -57,6 +59,62 @@ def bits(x):
     return x.view(torch.int16).cpu()
 
 
+def blob_bytes(plan):
+    """Bytes of the plan itself: the device workspace without the partial rows behind it."""
+    rows, a256 = plan.info["partial_rows"] * SHAPE.num_q_heads // SHAPE.num_kv_heads, lambda x: -(-x // 256) * 256
+    return plan.info["device_bytes_used"] - a256(rows * SHAPE.head_dim * 4) - a256(rows * 4)
+
+
+KERNEL, COPY = 0, 1      # of CUgraphNodeType
+
+
+def nodes_of(call):
+    """What `call(stream)` enqueues: the types of the nodes that it leaves in a capture."""
+    import torch
+    cu, s, graph, n = ctypes.CDLL("libcuda.so.1"), torch.cuda.Stream(), ctypes.c_void_p(), ctypes.c_size_t()
+    raw = ctypes.c_void_p(s.cuda_stream)
+    assert cu.cuStreamBeginCapture_v2(raw, 2) == 0      # (relaxed: the mode does not matter to what is called here)
+    try:
+        call(s)
+    finally:
+        assert cu.cuStreamEndCapture(raw, ctypes.byref(graph)) == 0
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes, kind = (ctypes.c_void_p * n.value)(), ctypes.c_int()
+    assert cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for node in nodes:
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        kinds.append(kind.value)
+    assert cu.cuGraphDestroy(graph) == 0
+    return kinds
+
+
+@pytest.mark.parametrize("want", [32768 - 256, 32768, 32768 + 4096, 300 << 10, (600 << 10) + 256, (1 << 20) + 512, (2 << 20) - 256, 2 << 20, (2 << 20) + 256])
+def test_plans_of_middling_size_go_by_kernel_and_arrive_whole(want):
+    """Plans of `want` bytes, by page table entries that no key needs yet (4 bytes each, sections of 256)."""
+    import torch
+    t = Batch()
+    few = 4 if want < 65536 else 24      # sequences (24 have a plan of 83 712 bytes at least)
+    qi, ctx, pi = t.qi[:few + 1], t.ctx[:few], t.pi[:few + 1].copy()
+    ids = t.ids(0)
+    dry = lambda n: B.plan_host(SHAPE, t.pages, qi, ctx, np.append(pi[:-1], n).astype(np.int32), np.resize(ids, n))
+    at = int(pi[-1]) + (want - blob_bytes(dry(int(pi[-1])))) // 4
+    pi[-1] = at
+    ids = np.resize(ids, at)
+    host, dev = B.workspace_size(SHAPE, t.pages, few, few, at)
+    dev_ws = torch.full((dev,), 0xA5, dtype=torch.uint8, device="cuda")
+    ws = torch.zeros(host, dtype=torch.uint8).pin_memory()
+    plan_of = lambda s=None: B.asynclm_plan(SHAPE, t.pages, qi, ctx, pi, ids, stream=s, host_ws=ws, dev_ws=dev_ws)
+    torch.cuda.synchronize()
+    assert nodes_of(plan_of) == [KERNEL if 32768 <= want <= 2 << 20 else COPY]
+    assert (dev_ws == 0xA5).all()
+    plan = plan_of()
+    torch.cuda.synchronize()
+    assert blob_bytes(plan) == want
+    start = plan.info["host_bytes_used"] - want - -(-plan.info["num_items"] // 64) * 256      # behind the plan: the CTA of each item
+    assert torch.equal(dev_ws[:want].cpu(), ws[start:start + want]) and (dev_ws[want:] == 0xA5).all()
+
+
 @pytest.mark.parametrize("kind", ["calls", "step", "rope", "attention", "static"])
 def test_steps_in_a_row_see_their_own_plan(kind):
     """One device workspace, planned anew ahead of every step without waiting for anything, page-locked against pageable memory
@@ -67,7 +125,7 @@ def test_steps_in_a_row_see_their_own_plan(kind):
     for k in range(6):
         pool, out = t.pool.clone(), torch.empty_like(t.q)
         plan = t.plan(t.ids(k), torch.empty(t.host_bytes, dtype=torch.uint8))
-        assert plan.info["device_bytes_used"] > 40000
+        assert blob_bytes(plan) >= 32768      # by kernel, from page-locked memory
         torch.cuda.synchronize()
         t.call(plan, kind, pool, out)
         torch.cuda.synchronize()
