@@ -72,10 +72,11 @@ def test_swap_out_and_in_are_bit_copies(Hq, Hkv, d):
 @pytest.mark.gpu
 @pytest.mark.parametrize("hk,pages,memory", [(1, 1, "pinned"), (1, 511, "pinned"), (1, 512, "pinned"), (1, 513, "pinned"),
                                              (1, 960, "pinned"), (1, 961, "pinned"), (3, 170, "pinned"), (3, 171, "pinned"),
-                                             (1, 512, "pageable"), (1, 961, "pageable"), (1, 300, "part of a larger one"), (1, 300, "captured")])
+                                             (1, 300, "pinned"), (1, 512, "pageable"), (1, 961, "pageable"), (1, 300, "captured")])
 def test_swaps_in_place_and_through_staging(hk, pages, memory):
     """Images up to and beyond 2 MB (4096 bytes a page and head) and page ids up to and beyond those that parameters hold, behind
-    one another in one stream."""
+    one another in one stream.  What is left in the staging buffer says which way they went: nothing of a swap in place, the image of
+    the others, and behind it the ids where they were copied."""
     import torch
     shape, num = W.Shape(8, hk, 64, 16), 1200
     g = np.random.default_rng(pages)
@@ -86,6 +87,7 @@ def test_swaps_in_place_and_through_staging(hk, pages, memory):
     trap.swap_in(want, new, want_image)
     src, dst = torch.from_numpy(pool.view(np.int16)).cuda(), torch.zeros(pool.shape, dtype=torch.int16, device="cuda")
     staging = torch.empty(B.kv_swap_staging_bytes(shape, num, pages), dtype=torch.uint8, device="cuda")
+    staging.fill_(0xA5)
     whole = torch.full((pages + 2,) + pool.shape[1:], 77, dtype=torch.int16)
     whole = whole if memory == "pageable" else whole.pin_memory()
     image = whole[1:-1]
@@ -113,3 +115,34 @@ def test_swaps_in_place_and_through_staging(hk, pages, memory):
     torch.cuda.synchronize()
     assert np.array_equal(image.numpy().view(np.uint16), want_image) and (whole[0] == 77).all() and (whole[-1] == 77).all()
     assert np.array_equal(dst.cpu().numpy().view(np.uint16), want) and np.array_equal(src.cpu().numpy().view(np.uint16), pool)
+    used = staging.cpu().numpy()
+    image_bytes = want_image.nbytes
+    in_place = memory == "pinned" and image_bytes <= 2 << 20
+    ids_copied = memory == "captured" or pages > 960
+    assert (used[:image_bytes] == 0xA5).all() if in_place else np.array_equal(used[:image_bytes].view(np.uint16), want_image.reshape(-1))
+    assert np.array_equal(used[image_bytes:image_bytes + 4 * pages].view(np.int32), new) if ids_copied else (used[image_bytes:] == 0xA5).all()
+
+
+@pytest.mark.gpu
+def test_an_image_in_two_registrations_is_refused():
+    """Page-locked in two parts that no single range covers: no kernel touches it, and the copy refuses it."""
+    import torch
+    shape, num, pages = W.Shape(8, 1, 64, 16), 200, 100
+    pool = torch.ones((num, 2, 1, 16, 64), dtype=torch.int16, device="cuda")
+    staging = torch.zeros(B.kv_swap_staging_bytes(shape, num, pages), dtype=torch.uint8, device="cuda")
+    base = torch.zeros(pages * 4096 + 8192, dtype=torch.uint8)
+    base, rt = base[-base.data_ptr() % 4096:], torch.cuda.cudart()
+    image, ids, cut = base[:pages * 4096], np.arange(pages, dtype=np.int32), 32768
+    parts = [(image.data_ptr(), cut), (image.data_ptr() + cut, pages * 4096 - cut)]
+    torch.cuda.synchronize()
+    for p, n in parts:
+        assert int(rt.cudaHostRegister(p, n, 0)) == 0
+    try:
+        for call in (B.asynclm_kv_swap_out, B.asynclm_kv_swap_in):
+            with pytest.raises(B.AsynclmError, match="CUDA"):
+                call(shape, num, ids, pool, staging, image)
+        torch.cuda.synchronize()
+    finally:
+        for p, n in parts:
+            rt.cudaHostUnregister(p)
+    assert not image.any() and (pool == 1).all()
