@@ -326,8 +326,8 @@ __device__ __forceinline__ void tc_body(const DevPlan& p, const CUtensorMap* spa
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int Hq = p.num_q_heads, Hkv = p.num_kv_heads;
-    // The plan was uploaded before the kernel in front of this one started, so it may be read before
-    // pdl_wait(); everything else (pool, q, outputs) is touched only after it.
+    // The plan is there when this kernel starts (behind an upload by kernel the first launch starts when that has completed: PlanUse),
+    // so it may be read before pdl_wait(); everything else (pool, q, outputs) is touched only after it.
     const int32_t* head = p.cta_heads + (size_t)blockIdx.x * kHeadWords;
     const int i0 = head[0], i1 = head[1];
     const Work* head_work = reinterpret_cast<const Work*>(head + kHeadWorkTensor);      // = p.works[i0]

@@ -508,8 +508,8 @@ __device__ __forceinline__ void decode_body(const DevPlan& p, const CUtensorMap*
             pages_cur = head[kHeadPagesCuda + lane];
             if constexpr (APPEND) unappended_from = cur.kv_limit0 - 1 - (cur.q_row0 - cur.q_seq0);
         }
-        // The plan was uploaded before the kernel in front of this one started, so all of the above
-        // overlaps that kernel's tail; the pool, Q and the queue are touched only from here on.
+        // The plan is there when this kernel starts (behind an upload by kernel the first launch starts when that has completed: PlanUse),
+        // so all of the above overlaps the tail of the kernel in front; the pool, Q and the queue are touched only from here on.
         pdl_wait();
         if (cur.kv_end == 0) cur = take();      // a CTA that came from span tiles starts on the queue
         while (cur.kv_end > 0 && ok) {

@@ -30,7 +30,7 @@ kv_append_kernel(DevPlan p, const uint4* __restrict__ k_new, const uint4* __rest
         const int r = (int)(rest >> 1);
         // the planner resolved the row's page and slot (position ctx_b + i through the page table), so
         // the slot and the source row are fetched side by side instead of through four dependent loads
-        const int64_t ps = __ldg(p.row_slot + r);      // the plan was uploaded before the kernel in front of this one started
+        const int64_t ps = __ldg(p.row_slot + r);      // the plan is there when this kernel starts (see PlanUse)
         if (first) pdl_wait();                         // the rows and the pool belong to the kernels in front until those have completed
         first = false;
         const uint4 val = ldg_nc_v4((which ? v_new : k_new) + ((size_t)r * p.num_kv_heads + h) * vpr + vec);
